@@ -180,40 +180,51 @@ class _Site:
     pass
 
 
+class _Inputs:
+    """Everything a case draws from its seed: the binding, the activations and every site's weights and adapters."""
+
+    def __init__(self, case, seed):
+        gen = torch.Generator(device="cuda").manual_seed(int(seed))
+
+        def normal(*shape, std=1.0):
+            return torch.randn(shape, generator=gen, device="cuda", dtype=torch.float32).mul_(std).to(torch.bfloat16)
+
+        T, entries = case["tokens"], _entries(case)
+        self.entry = _binding(case, np.random.Generator(np.random.Philox(key=[int(seed), 1])))
+        self.x, self.sites = {}, []
+        for name, k, n, src in _sites(case):
+            if src not in self.x:
+                self.x[src] = normal(T, k)
+            s = _Site()
+            s.name, s.k, s.n, s.src = name, k, n, src
+            s.W0 = normal(n, k, std=STD)
+            s.A = [normal(r, k, std=STD) for _, _, r in entries]
+            s.B = [normal(n, r, std=STD) for _, _, r in entries]
+            if case["kind"] == "publish":
+                s.new = (normal(entries[0][2], k, std=STD), normal(n, entries[0][2], std=STD))
+            if case["kind"] == "train":
+                s.dy = normal(T, n)
+            self.sites.append(s)
+
+
 def prepare(case, seed):
     """Weights, adapters registered in their tables, activations and the binding of the batch."""
-    gen = torch.Generator(device="cuda").manual_seed(int(seed))
-    rng = np.random.Generator(np.random.Philox(key=[int(seed), 1]))
-    T, kind, entries = case["tokens"], case["kind"], _entries(case)
-
-    def normal(*shape, std=1.0):
-        return torch.randn(shape, generator=gen, device="cuda", dtype=torch.float32).mul_(std).to(torch.bfloat16)
-
-    entry = _binding(case, rng)
+    kind, T, entries, inputs = case["kind"], case["tokens"], _entries(case), _Inputs(case, seed)
+    entry = inputs.entry
     ints = lambda a: torch.from_numpy(np.ascontiguousarray(a, dtype=np.int32)).cuda()  # noqa: E731
-    state = dict(case=case, sites=[], x={})
-    for name, k, n, src in _sites(case):
-        if src not in state["x"]:
-            state["x"][src] = normal(T, k)
-        s = _Site()
-        s.name, s.src = name, src
-        s.W0 = normal(n, k, std=STD)
-        s.table = Table(k, n, max_slots=len(entries) + SPARE_SLOTS)
-        s.A = [normal(r, k, std=STD) for _, _, r in entries]
-        s.B = [normal(n, r, std=STD) for _, _, r in entries]
+    state = dict(case=case, sites=inputs.sites, x=inputs.x)
+    for s in inputs.sites:
+        s.table = Table(s.k, s.n, max_slots=len(entries) + SPARE_SLOTS)
         slots = [s.table.register_adapter(a, v, A, B, SCALE) for (a, v, _), A, B in zip(entries, s.A, s.B)]
         if kind == "publish":
             for a in range(case["adapters"]):
                 s.table.publish(a, 1)
-            s.new = (normal(entries[0][2], k, std=STD), normal(n, entries[0][2], std=STD))
         if kind == "train":
             s.W0T = s.W0.t().contiguous()
-            s.dy = normal(T, n)
-            s.table_T = Table(n, k, max_slots=len(entries) + SPARE_SLOTS)
+            s.table_T = Table(s.n, s.k, max_slots=len(entries) + SPARE_SLOTS)
             s.slots_T = [s.table_T.register_adapter_transposed(a, v, A, B, SCALE) for (a, v, _), A, B in zip(entries, s.A, s.B)]
-            s.dA = torch.zeros((s.table.max_slots, 64, k), dtype=torch.float32, device="cuda")
-            s.dB = torch.zeros((s.table.max_slots, n, 64), dtype=torch.float32, device="cuda")
-        state["sites"].append(s)
+            s.dA = torch.zeros((s.table.max_slots, 64, s.k), dtype=torch.float32, device="cuda")
+            s.dB = torch.zeros((s.table.max_slots, s.n, 64), dtype=torch.float32, device="cuda")
     state["version"] = 1
     # every site registered its entries in the same order, so the slot of an entry is the same everywhere
     slot_of = lambda e: np.where(e < 0, -1, np.asarray(slots, dtype=np.int32)[e])  # noqa: E731
@@ -296,3 +307,45 @@ def tolerance(case) -> dict:
     # by rel 1.7e-3 and max 6e-3 at most.  dA and dB are float32 sums of products with bf16-rounded u: rel 1.8e-3, but an element
     # near zero is a sum that cancels, so its error is up to 0.037 of the matrix's root mean square.
     return {"rel": 7e-3, "max": 0.15} if case["kind"] == "train" else {"rel": 7e-3, "max": 0.025}
+
+
+def exact(case, seed):
+    """What run() returns for these inputs, in 64 bits: entry e is in slot e (the first registrations of an empty table)."""
+    inputs, entries, kind = _Inputs(case, seed), _entries(case), case["kind"]
+    wide = lambda t: t.to(torch.float64)  # noqa: E731
+
+    def rows(entry, e):
+        return torch.from_numpy(np.flatnonzero(entry == e)).cuda()
+
+    def layer(x, W, A, B, entry):
+        x = wide(x)
+        y = x @ wide(W).t()
+        for e in range(len(A)):
+            at = rows(entry, e)
+            y[at] += SCALE * ((x[at] @ wide(A[e]).t()) @ wide(B[e]).t())
+        return y
+
+    out = []
+    for s in inputs.sites:
+        x, A = inputs.x[s.src], list(s.A)
+        B = list(s.B)
+        if kind == "publish":
+            A[0], B[0] = s.new
+        y = layer(x, s.W0, A, B, inputs.entry)
+        if kind == "dual":
+            y = (y, layer(x, s.W0, A, B, np.where(inputs.entry == 0, len(entries) - 1, inputs.entry)))
+        out.append(y)
+    if kind == "host":
+        return out[0].cpu()
+    if kind == "train":
+        for s in reversed(inputs.sites):
+            x, dy = wide(inputs.x[s.src]), wide(s.dy)
+            out.append(layer(s.dy, s.W0.t(), [B.t() for B in s.B], [A.t() for A in s.A], inputs.entry))
+            dA = torch.zeros((len(entries) + SPARE_SLOTS, 64, s.k), dtype=torch.float64, device="cuda")
+            dB = torch.zeros((len(entries) + SPARE_SLOTS, s.n, 64), dtype=torch.float64, device="cuda")
+            for e, (_, _, r) in enumerate(entries):
+                at = rows(inputs.entry, e)
+                dA[e, :r] = SCALE * ((dy[at] @ wide(s.B[e])).t() @ x[at])
+                dB[e, :, :r] = SCALE * (dy[at].t() @ (x[at] @ wide(s.A[e]).t()))
+            out += [dA, dB]
+    return out
