@@ -11,29 +11,146 @@ namespace {
 
 inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 
-// Workspace layout of the prefill path: [PlanWord][tile_identity][u blocks][gathered x (perm form only)];
-// the decode path uses [PlanWord][..][u fp32 16x64].
+// Workspace of the GEMM path (lml_bind.cu): [plan of every row tile][slot per row, both bindings]
+// [u blocks, one or two sets].  A row tile has room for the chunks of `slots` slots of the widest rank, whatever the table
+// holds when the call comes; calls of more than kSlabTiles row tiles work in slabs, so the blocks stay bounded.
 struct WsLayout {
-    size_t plan_off, ident_off, u_off, xg_off, total;
+    size_t plan_off, rows_off, rows2_off, u_off, u2_off, total;
+    int cap;   // chunks per row tile
 };
-WsLayout ws_layout(const lml_table* t, int T, int G, int u_sets = 1)
+WsLayout ws_layout(const lml_table* t, int T, int slots, int u_sets = 1)
 {
     WsLayout w;
-    w.plan_off = 0;
     const size_t num_m = (size_t)(T + kTileM - 1) / kTileM;
-    w.ident_off = round_up(sizeof(PlanWord), 256);
-    w.u_off = round_up(w.ident_off + (num_m + 1) * sizeof(int32_t), 1024);
-    size_t u_bytes = (size_t)u_sets * (num_m + (size_t)(G > 0 ? G : 1)) * kTileM * kRankPad * sizeof(__nv_bfloat16);
-    w.xg_off = w.u_off + round_up(u_bytes, 1024);
-    w.total = w.xg_off + round_up((size_t)T * t->d_in * sizeof(__nv_bfloat16), 1024);
+    const size_t slab = num_m < (size_t)kSlabTiles ? num_m : (size_t)kSlabTiles;
+    if (slots > t->max_slots) slots = t->max_slots;
+    if (slots < 1) slots = 1;
+    w.cap = slots * (kRankPad / kChunk);
+    w.plan_off = 0;
+    w.rows_off = round_up(slab * sizeof(TilePlan), 256);
+    w.rows2_off = w.rows_off + round_up((size_t)T, 256);
+    w.u_off = round_up(w.rows2_off + round_up((size_t)T, 256), 1024);
+    const size_t u_bytes = slab * (size_t)w.cap * kUBlockBytes;
+    w.u2_off = w.u_off + u_bytes;
+    w.total = w.u_off + (size_t)u_sets * u_bytes;
     return w;
+}
+// (a dual call's rows can use a slot per segment and binding)
+WsLayout dual_layout(const lml_table* t, int T, int G) { return ws_layout(t, T, G > kMaxSlots ? kMaxSlots : 2 * G, 2); }
+
+// Workspace of the backward pass: two sets of piece blocks.
+size_t backward_ws_bytes(int T, int G)
+{
+    const size_t num_m = (size_t)(T + kTileM - 1) / kTileM;
+    return 2 * (num_m + (size_t)(G > 0 ? G : 1)) * kTileM * kRankPad * sizeof(__nv_bfloat16);
+}
+
+// One projection of a call on the GEMM path.
+struct GemmCall {
+    lml_table* t;
+    const void* W0;
+    void* y;
+    const int32_t* ids;     // per token, or per segment
+    uint8_t* ws;
+    WsLayout layout;
+};
+
+// The GEMM path: the rows stay in their order; one launch binds them and computes u (unless the GEMM does both itself),
+// one launch multiplies.  P > 1: projections of the same x.  ids2 / y2: the second binding of a dual call.
+cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, RowMode mode, const int32_t* seg_offsets, int G,
+                          const int32_t* perm, const int32_t* ids2, void* y2, bool by_adapter, cudaStream_t stream, int* launches)
+{
+    lml_table* t0 = calls[0].t;
+    const int num_m = (T + kTileM - 1) / kTileM;
+    const bool dual = y2 != nullptr;
+    SlotSnapshot snap[LML_MAX_PROJECTIONS];
+    BindArgs b;
+    GemmArgs g;
+    int d_outs[LML_MAX_PROJECTIONS], most_chunks = 1;
+    TmapCache* caches[LML_MAX_PROJECTIONS];
+    const CUtensorMap* tmaps_A[LML_MAX_PROJECTIONS];
+    *launches = 0;
+    g.lora = mode != kRowsNone;
+    b.rows.mode = mode; b.rows.ids = calls[0].ids; b.rows.ids2 = ids2; b.rows.seg_offsets = seg_offsets; b.rows.G = G;
+    b.d_in = g.d_in = t0->d_in; b.P = g.P = P;
+    for (int p = 0; p < P; ++p) {
+        const GemmCall& c = calls[p];
+        snap[p] = snapshot_locked(c.t);
+        b.snap[p] = snap[p];
+        caches[p] = &c.t->tmaps;
+        tmaps_A[p] = &c.t->tmap_A;
+        d_outs[p] = c.t->d_out;
+        int live = 0;   // chunks of all live slots: no tile needs more
+        for (int s = 0; s < c.t->max_slots; ++s) live += chunks_of_rank(snap[p].rank[s]);
+        const int cap = live < c.layout.cap ? (live > 0 ? live : 1) : c.layout.cap;
+        most_chunks = cap > most_chunks ? cap : most_chunks;
+        BindPart& bp = b.part[p];
+        bp.A = c.t->arena.A; bp.ids = c.ids; bp.adapter_map = by_adapter ? c.t->arena.adapter_map : nullptr; bp.status = c.t->arena.status;
+        bp.plan = reinterpret_cast<TilePlan*>(c.ws + c.layout.plan_off);
+        bp.u = reinterpret_cast<__nv_bfloat16*>(c.ws + c.layout.u_off);
+        bp.u2 = reinterpret_cast<__nv_bfloat16*>(c.ws + c.layout.u2_off);
+        bp.cap = cap;
+        GemmProj& gp = g.proj[p];
+        gp.W0 = c.W0; gp.y = c.y; gp.d_out = c.t->d_out; gp.ar = &c.t->arena; gp.snap = &snap[p];
+        gp.plan = bp.plan; gp.u = bp.u; gp.cap = cap;
+    }
+    g.num_sms = t0->num_sms;
+    if (mode == kRowsSegments && (perm || G > kBindSegs || num_m > kSlabTiles)) {   // a slot per row first
+        int8_t* rows = reinterpret_cast<int8_t*>(calls[0].ws + calls[0].layout.rows_off);
+        int8_t* rows2 = dual ? reinterpret_cast<int8_t*>(calls[0].ws + calls[0].layout.rows2_off) : nullptr;
+        const cudaError_t e = launch_rows_from_segments(t0->arena, snap[0], seg_offsets, calls[0].ids, ids2, G, perm, T, rows, rows2, stream);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+        b.rows.mode = kRowsGiven; b.rows.rows = rows; b.rows.rows2 = rows2;
+    }
+    for (int r0 = 0; r0 < T; r0 += kSlabTiles * kTileM) {
+        const int rows = T - r0 < kSlabTiles * kTileM ? T - r0 : kSlabTiles * kTileM;
+        b.T = g.T = rows;
+        b.x = g.x = static_cast<const __nv_bfloat16*>(x) + (size_t)r0 * t0->d_in;
+        for (int p = 0; p < P; ++p) {
+            if (mode == kRowsTokens) b.part[p].ids = calls[p].ids + r0;
+            g.proj[p].y = static_cast<__nv_bfloat16*>(calls[p].y) + (size_t)r0 * d_outs[p];
+        }
+        if (r0 > 0 && b.rows.rows) b.rows.rows += kSlabTiles * kTileM;
+        if (r0 > 0 && b.rows.rows2) b.rows.rows2 += kSlabTiles * kTileM;
+        g.shape = gemm_pick_shape(rows, t0->d_in, d_outs, P, t0->num_sms, t0->split_bn, t0->split_s);
+        // With whole-K tiles and few row tiles the shrink runs inside the GEMM kernel (on the CTAs that own the fewest tiles,
+        // ahead of their tiles); otherwise a launch goes first and the GEMM is its programmatic dependent.
+        g.fused = mode == kRowsSegments && !dual && P == 1 && T == rows && t0->fuse_shrink &&
+                  gemm_can_fuse_shrink(g.shape, T, t0->d_out, G, b.rows.mode == kRowsSegments, b.part[0].cap, t0->num_sms);
+        if (g.fused) g.rows = b.rows;
+        b.x_flag = g.x_flag = nullptr;
+        if (mode != kRowsNone && !g.fused && bind_starts_gemm_early(rows, P, t0->num_sms)) {
+            b.x_flag = g.x_flag = t0->arena.status + 8;
+            b.share_sm = g.share_sm = g.shape.split > 1 &&
+                g.shape.ctas + bind_ctas_early(rows, t0->d_in, P, most_chunks, t0->num_sms) > t0->num_sms;
+            std::lock_guard<std::mutex> lock(t0->mu);
+            if (++t0->next_call == 0u) ++t0->next_call;
+            b.call_id = g.call_id = t0->next_call;
+        }
+        if (dual) {
+            // (split-K: an accumulator per binding; whole-K tiles: the second output is the first plus the difference)
+            b.second = g.shape.split > 1 ? 1 : 2;
+            g.u2 = b.part[0].u2;
+            g.y2 = static_cast<__nv_bfloat16*>(y2) + (size_t)r0 * d_outs[0];
+        }
+        if (mode != kRowsNone && !g.fused) {
+            const cudaError_t e = launch_bind_shrink(b, tmaps_A, caches[0], t0->num_sms, stream);
+            if (e != cudaSuccess) return e;
+            ++*launches;
+        }
+        const cudaError_t e = launch_gemm_sm100(t0->tmap_A, caches, g, stream);
+        if (e != cudaSuccess) return e;
+        ++*launches;
+    }
+    return cudaSuccess;
 }
 
 }  // namespace
 
 static void free_table_resources(lml_table* t)
 {
-    cudaFree(t->arena.A); cudaFree(t->arena.B); cudaFree(t->arena.Bc); cudaFree(t->arena.status); cudaFree(t->arena.adapter_map); cudaFree(t->arena.tile_flags); cudaFree(t->arena.dec_u);
+    cudaFree(t->arena.A); cudaFree(t->arena.B); cudaFree(t->arena.Bc); cudaFree(t->arena.Bk); cudaFree(t->arena.status); cudaFree(t->arena.adapter_map); cudaFree(t->arena.tile_flags); cudaFree(t->arena.dec_u);
     if (t->copy_in) cudaStreamDestroy(t->copy_in);
     if (t->copy_out) cudaStreamDestroy(t->copy_out);
     if (t->ev_begin) cudaEventDestroy(t->ev_begin);
@@ -93,6 +210,9 @@ lml_status lml_table_create(lml_table** out, int device, int d_in, int d_out, in
     const size_t bc_bytes = (size_t)max_slots * d_out * kRankCompact * sizeof(__nv_bfloat16);
     ok = ok && cudaMalloc(&t->arena.Bc, bc_bytes) == cudaSuccess;
     ok = ok && cudaMemset(t->arena.Bc, 0, bc_bytes) == cudaSuccess;
+    const size_t bk_bytes = (size_t)max_slots * kRankPad * b_rows_padded(d_out) * sizeof(__nv_bfloat16);
+    ok = ok && cudaMalloc(&t->arena.Bk, bk_bytes) == cudaSuccess;
+    ok = ok && cudaMemset(t->arena.Bk, 0, bk_bytes) == cudaSuccess;   // (the rows past d_out stay zero)
     ok = ok && cudaMalloc(&t->arena.status, 256) == cudaSuccess;
     ok = ok && cudaMalloc(&t->arena.adapter_map, kMaxAdapterIds * sizeof(int32_t)) == cudaSuccess;
     ok = ok && cudaMemset(t->arena.A, 0, a_bytes) == cudaSuccess;
@@ -108,21 +228,11 @@ lml_status lml_table_create(lml_table** out, int device, int d_in, int d_out, in
     ok = ok && shrink_init() == cudaSuccess;
     ok = ok && decode_init() == cudaSuccess;
     ok = ok && aux_init() == cudaSuccess;
-    ok = ok && encode_tmap_3d(&t->tmap_B256, t->arena.B, kRankPad, (uint64_t)d_out, (uint64_t)max_slots,
-                              kRankPad * 2, (uint64_t)d_out * kRankPad * 2, 64, 256, 1);
-    ok = ok && encode_tmap_3d(&t->tmap_B128, t->arena.B, kRankPad, (uint64_t)d_out, (uint64_t)max_slots,
-                              kRankPad * 2, (uint64_t)d_out * kRankPad * 2, 64, 128, 1);
+    ok = ok && bind_init() == cudaSuccess;
     ok = ok && encode_tmap_3d(&t->tmap_A, t->arena.A, (uint64_t)d_in, kRankPad, (uint64_t)max_slots, (uint64_t)d_in * 2,
-                              (uint64_t)d_in * kRankPad * 2, 64, 64, 1);
+                              (uint64_t)d_in * kRankPad * 2, 64, kChunk, 1);
     gemm_split_override(&t->split_bn, &t->split_s);   // the test knobs are read here, never on the hot path
     if (const char* e = getenv("LML_FUSE_SHRINK")) t->fuse_shrink = e[0] != '0';
-    // (two row tiles where the rows of x are short enough for the GEMM's CTAs to get resident beside the binding kernel's:
-    // 256 tokens 29 / 45 us against 34 / 50 on the grouped path on 4096 x 4096 / 11008 x 4096; from 512 tokens on, and on
-    // 4096 x 11008 from 256 on, a piece per slot and tile costs the GEMM more than grouping the rows)
-    t->one_tile_tokens = d_in <= 4096 ? 2 * kTileM : kTileM;
-    if (const char* e = getenv("LML_ONE_TILE")) t->one_tile_tokens = e[0] != '0' ? t->one_tile_tokens : 0;
-    if (const char* e = getenv("LML_ONE_TILE_TOKENS")) t->one_tile_tokens = atoi(e) < 0 ? 0 : (atoi(e) > 8 * kTileM ? 8 * kTileM : atoi(e));
-    if (const char* e = getenv("LML_BIND_THREADS")) t->bind_threads = atoi(e);
     if (const char* e = getenv("LML_DECODE_BLOCK_TOKENS")) t->dec_block_tokens = atoi(e) < 0 ? 0 : (atoi(e) > kDecMaxBlocks * kDecodeMaxT ? kDecMaxBlocks * kDecodeMaxT : atoi(e));
     ok = ok && cudaEventCreateWithFlags(&t->ev_map, cudaEventDisableTiming) == cudaSuccess;
     ok = ok && cudaStreamCreateWithFlags(&t->copy_in, cudaStreamNonBlocking) == cudaSuccess;
@@ -403,88 +513,39 @@ lml_status lora_mixed_linear(lml_table* t, const void* x, const void* W0, int T,
     if (G == 0) perm = nullptr;   // without adapters the row order is irrelevant
     const WsLayout ws = ws_layout(t, T, G);
     const bool decode = T <= kDecodeMaxT;
-    const size_t need = decode ? ws.xg_off : (perm ? ws.total : ws.xg_off);
-    const bool need_ws = G > 0 || (!decode && perm);
-    if (need_ws && (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < need))
+    if (G > 0 && (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < ws.total))
         return LML_ERR_WORKSPACE;
     cudaStream_t stream = (cudaStream_t)stream_v;
-    const SlotSnapshot snap = snapshot_locked(t);
     DeviceGuard guard(t->device);
     if (!guard.ok) return LML_ERR_CUDA;
-    uint8_t* wsb = static_cast<uint8_t*>(workspace);
     int launches = 0;
     cudaError_t e = cudaSuccess;
 
     if (decode) {
+        const SlotSnapshot snap = snapshot_locked(t);
         DecodeArgs a;
         a.x = x; a.W0 = W0; a.y = y; a.perm = perm; a.seg_offsets = seg_offsets; a.slot_ids = slot_ids;
         a.T = T; a.d_in = t->d_in; a.d_out = t->d_out; a.G = G; a.num_sms = t->num_sms;
         e = launch_decode(t->arena, snap, a, stream, &launches);
     } else {
-        const void* xg = x;
-        int32_t* tile_identity = nullptr;
-        if (perm) {
-            tile_identity = reinterpret_cast<int32_t*>(wsb + ws.ident_off);
-            e = launch_gather_rows(x, perm, T, t->d_in, wsb + ws.xg_off, tile_identity, true, t->arena.status, stream);
-            if (e == cudaSuccess) { ++launches; xg = wsb + ws.xg_off; }
-        }
-        PlanWord* plan = reinterpret_cast<PlanWord*>(wsb + ws.plan_off);
-        __nv_bfloat16* u_blocks = reinterpret_cast<__nv_bfloat16*>(wsb + ws.u_off);
-        // With whole-K tiles the shrink runs inside the GEMM kernel (on the CTAs that own the fewest tiles, ahead of
-        // their tiles); otherwise a shrink kernel goes first and the GEMM is its programmatic dependent.
-        const bool fused = G > 0 && t->fuse_shrink &&
-                           gemm_can_fuse_shrink(T, t->d_in, t->d_out, G, t->num_sms, t->split_bn, t->split_s);
-        if (e == cudaSuccess && G > 0 && !fused) {
-            e = launch_shrink_pieces(t->arena, snap, xg, T, t->d_in, seg_offsets, slot_ids, G, x, tile_identity, plan,
-                                     u_blocks, stream, perm ? 2 : 0);
-            if (e == cudaSuccess) ++launches;
-        }
-        if (e == cudaSuccess) {
-            GemmArgs a;
-            a.fused_shrink = fused;
-            a.x = xg; a.x_in_place = x; a.tile_identity = tile_identity; a.W0 = W0; a.y = y; a.perm = perm; a.seg_offsets = seg_offsets; a.slot_ids = slot_ids;
-            a.plan = plan; a.u_blocks = u_blocks ? u_blocks : reinterpret_cast<const __nv_bfloat16*>(x);
-            a.T = T; a.d_in = t->d_in; a.d_out = t->d_out; a.G = G; a.num_sms = t->num_sms;
-            a.overlap_with_previous = G > 0;
-            a.split_bn = t->split_bn; a.split_s = t->split_s;
-            if (G == 0) a.u_blocks = reinterpret_cast<const __nv_bfloat16*>(W0);   // never read; map needs a valid base
-            e = launch_gemm_sm100(t->arena, snap, t->tmap_B256, t->tmap_B128, t->tmap_A, &t->tmaps, a, stream);
-            if (e == cudaSuccess) ++launches;
-        }
+        const GemmCall c = {t, W0, y, slot_ids, static_cast<uint8_t*>(workspace), ws};
+        e = run_gemm_path(&c, 1, x, T, G > 0 ? kRowsSegments : kRowsNone, seg_offsets, G, perm, nullptr, nullptr, false, stream, &launches);
     }
     t->last_launches = launches;
     if (e != cudaSuccess) { cudaGetLastError(); return LML_ERR_CUDA; }
     return LML_OK;
 }
 
-// Segments of a token-form call: one per slot and one for "none" on the grouped path; on the path that keeps the
-// tokens in their order, one per slot and row tile at most, and one more.
-static int tokens_segments(const lml_table* t, int T)
-{
-    if (T > t->one_tile_tokens) return t->max_slots + 1;
-    return ((T + kTileM - 1) / kTileM) * t->max_slots + 1;
-}
-
 size_t lml_tokens_workspace_bytes(const lml_table* t, int max_tokens)
 {
     if (!t || max_tokens < 0 || max_tokens > kMaxTokens) return 0;
-    // (the largest of the layouts that a call of up to max_tokens tokens can take)
-    size_t best = 0;
-    const int candidates[2] = {max_tokens, max_tokens < t->one_tile_tokens ? max_tokens : t->one_tile_tokens};
-    for (int T : candidates) {
-        const int G = tokens_segments(t, T);
-        size_t n = ws_layout(t, T, G).total;
-        n += round_up((size_t)T * 4 + 4, 1024);               // perm
-        n += 2 * round_up((size_t)(G + 1) * 4, 1024);         // seg_offsets, seg_slot_ids
-        best = n > best ? n : best;
-    }
-    return best;
+    return ws_layout(t, max_tokens, t->max_slots).total;
 }
 
 size_t lml_dual_workspace_bytes(const lml_table* t, int max_tokens, int max_segments)
 {
     if (!t || max_tokens < 0 || max_segments < 0 || max_tokens > kMaxTokens) return 0;
-    return ws_layout(t, max_tokens, max_segments, 3).total;
+    return dual_layout(t, max_tokens, max_segments).total;
 }
 
 lml_status lora_mixed_linear_dual(lml_table* t, const void* x, const void* W0, int T, const int32_t* seg_offsets,
@@ -500,8 +561,7 @@ lml_status lora_mixed_linear_dual(lml_table* t, const void* x, const void* W0, i
         // One launch of the decode kernel with the two bindings as two projections over the same W0: half of the CTAs
         // per binding, each half exactly a single call (so y_a and y_b are bit for bit those of two calls).  The two
         // halves walk the same rows of W0 at the same time, so the second reader of a line finds it in L2.
-        const WsLayout ws1 = ws_layout(t, T, G);
-        if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < ws1.xg_off) return LML_ERR_WORKSPACE;
+        if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < ws_layout(t, T, G).total) return LML_ERR_WORKSPACE;
         const SlotSnapshot snap = snapshot_locked(t);
         DeviceGuard guard(t->device);
         if (!guard.ok) return LML_ERR_CUDA;
@@ -519,49 +579,13 @@ lml_status lora_mixed_linear_dual(lml_table* t, const void* x, const void* W0, i
         if (e != cudaSuccess) { cudaGetLastError(); return LML_ERR_CUDA; }
         return LML_OK;
     }
-    const WsLayout ws = ws_layout(t, T, G, 3);
-    const size_t need = perm ? ws.total : ws.xg_off;
-    if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < need) return LML_ERR_WORKSPACE;
-    cudaStream_t stream = (cudaStream_t)stream_v;
-    const SlotSnapshot snap = snapshot_locked(t);
+    const WsLayout ws = dual_layout(t, T, G);
+    if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < ws.total) return LML_ERR_WORKSPACE;
     DeviceGuard guard(t->device);
     if (!guard.ok) return LML_ERR_CUDA;
-    uint8_t* wsb = static_cast<uint8_t*>(workspace);
     int launches = 0;
-    cudaError_t e = cudaSuccess;
-    const void* xg = x;
-    int32_t* tile_identity = nullptr;
-    if (perm) {
-        tile_identity = reinterpret_cast<int32_t*>(wsb + ws.ident_off);
-        e = launch_gather_rows(x, perm, T, t->d_in, wsb + ws.xg_off, tile_identity, true, t->arena.status, stream);
-        if (e == cudaSuccess) { ++launches; xg = wsb + ws.xg_off; }
-    }
-    PlanWord* plan = reinterpret_cast<PlanWord*>(wsb + ws.plan_off);
-    __nv_bfloat16* u_blocks = reinterpret_cast<__nv_bfloat16*>(wsb + ws.u_off);
-    const size_t num_m = (size_t)(T + kTileM - 1) / kTileM;
-    const size_t set_elems = (num_m + (size_t)G) * kTileM * kRankPad;
-    // three sets of u blocks: scale.x.A^T under the first slots (set 0) and its negation (set 2), written by
-    // one shrink pass, and under the second slots (set 1), by a second pass that runs beside the first:
-    // the second output is the first accumulator plus (second delta - first delta)
-    e = launch_shrink_pieces(t->arena, snap, xg, T, t->d_in, seg_offsets, slot_ids_a, G, x, tile_identity, plan, u_blocks,
-                             stream, false, u_blocks + 2 * set_elems);
-    if (e == cudaSuccess) {
-        ++launches;
-        e = launch_shrink_pieces(t->arena, snap, xg, T, t->d_in, seg_offsets, slot_ids_b, G, x, tile_identity, plan,
-                                 u_blocks + set_elems, stream, true);
-        if (e == cudaSuccess) ++launches;
-    }
-    if (e == cudaSuccess) {
-        GemmArgs a;
-        a.x = xg; a.x_in_place = x; a.tile_identity = tile_identity; a.W0 = W0; a.y = y_a; a.perm = perm;
-        a.seg_offsets = seg_offsets; a.slot_ids = slot_ids_a; a.slot_ids2 = slot_ids_b; a.y2 = y_b;
-        a.plan = plan; a.u_blocks = u_blocks;
-        a.T = T; a.d_in = t->d_in; a.d_out = t->d_out; a.G = G; a.num_sms = t->num_sms;
-        a.overlap_with_previous = true;
-        a.split_bn = t->split_bn; a.split_s = t->split_s;   // (few tokens: the split-K kernel, both bindings' accumulators side by side)
-        e = launch_gemm_sm100(t->arena, snap, t->tmap_B256, t->tmap_B128, t->tmap_A, &t->tmaps, a, stream);
-        if (e == cudaSuccess) ++launches;
-    }
+    const GemmCall c = {t, W0, y_a, slot_ids_a, static_cast<uint8_t*>(workspace), ws};
+    const cudaError_t e = run_gemm_path(&c, 1, x, T, kRowsSegments, seg_offsets, G, perm, slot_ids_b, y_b, false, (cudaStream_t)stream_v, &launches);
     t->last_launches = launches;
     if (e != cudaSuccess) { cudaGetLastError(); return LML_ERR_CUDA; }
     return LML_OK;
@@ -570,7 +594,7 @@ lml_status lora_mixed_linear_dual(lml_table* t, const void* x, const void* W0, i
 size_t lml_backward_workspace_bytes(const lml_table* t, int max_tokens, int max_segments)
 {
     if (!t || max_tokens < 0 || max_segments < 0 || max_tokens > kMaxTokens) return 0;
-    return ws_layout(t, max_tokens, max_segments, 2).xg_off;
+    return backward_ws_bytes(max_tokens, max_segments);
 }
 
 lml_status lora_mixed_linear_backward_adapters(lml_table* t, lml_table* t_T, const void* x, const void* dy, int T,
@@ -584,27 +608,23 @@ lml_status lora_mixed_linear_backward_adapters(lml_table* t, lml_table* t_T, con
     if (!x || !dy || !seg_offsets || !slot_ids || !slot_ids_T || !dA || !dB || !aligned16(x) || !aligned16(dy) ||
         !aligned16(dA) || !aligned16(dB))
         return LML_ERR_INVALID_ARG;
-    const WsLayout ws = ws_layout(t, T, G, 2);
-    if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < ws.xg_off) return LML_ERR_WORKSPACE;
+    if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < backward_ws_bytes(T, G)) return LML_ERR_WORKSPACE;
     cudaStream_t stream = (cudaStream_t)stream_v;
     const SlotSnapshot snap = snapshot_locked(t);
     const SlotSnapshot snap_T = snapshot_locked(t_T);
     DeviceGuard guard(t->device);
     if (!guard.ok) return LML_ERR_CUDA;
-    uint8_t* wsb = static_cast<uint8_t*>(workspace);
-    PlanWord* plan = reinterpret_cast<PlanWord*>(wsb + ws.plan_off);
-    __nv_bfloat16* u_blocks = reinterpret_cast<__nv_bfloat16*>(wsb + ws.u_off);
+    __nv_bfloat16* u_blocks = static_cast<__nv_bfloat16*>(workspace);
     const size_t num_m = (size_t)(T + kTileM - 1) / kTileM;
     const size_t set_elems = (num_m + (size_t)G) * kTileM * kRankPad;
     int launches = 0;
     // set 0: scale.(x.A^T) per position (the forward shrink); set 1: scale.(dy.B), the same pass on the
     // transposed table, whose "A" is B^T
-    cudaError_t e = launch_shrink_pieces(t->arena, snap, x, T, t->d_in, seg_offsets, slot_ids, G, x, nullptr, plan, u_blocks, stream);
+    cudaError_t e = launch_shrink_pieces(t->arena, snap, x, T, t->d_in, seg_offsets, slot_ids, G, u_blocks, stream);
     if (e == cudaSuccess) {
         ++launches;
         // (a further pass of the same call: it runs beside the first)
-        e = launch_shrink_pieces(t_T->arena, snap_T, dy, T, t_T->d_in, seg_offsets, slot_ids_T, G, dy, nullptr, plan,
-                                 u_blocks + set_elems, stream, 1);
+        e = launch_shrink_pieces(t_T->arena, snap_T, dy, T, t_T->d_in, seg_offsets, slot_ids_T, G, u_blocks + set_elems, stream, 1);
     }
     if (e == cudaSuccess) {
         ++launches;
@@ -627,14 +647,12 @@ static lml_status tokens_impl(lml_table* t, const void* x, const void* W0, int T
     if (!workspace || (reinterpret_cast<uintptr_t>(workspace) & 255u) || workspace_bytes < lml_tokens_workspace_bytes(t, T))
         return LML_ERR_WORKSPACE;
     cudaStream_t stream = (cudaStream_t)stream_v;
-    uint8_t* wsb = static_cast<uint8_t*>(workspace);
     if (T <= kDecodeMaxT) {
         // Up to 16 tokens need no grouping: the decode kernel handles every row of x on its own, so it reads
         // the slot ids directly.  One launch.
         const SlotSnapshot snap = snapshot_locked(t);
         DeviceGuard guard(t->device);
         if (!guard.ok) return LML_ERR_CUDA;
-        const WsLayout ws = ws_layout(t, T, 1);
         DecodeArgs a;
         a.x = x; a.W0 = W0; a.y = y; a.perm = nullptr; a.seg_offsets = nullptr; a.slot_ids = nullptr;
         a.token_slots = token_slots;
@@ -659,7 +677,6 @@ static lml_status tokens_impl(lml_table* t, const void* x, const void* W0, int T
         const SlotSnapshot snap = snapshot_locked(t);
         DeviceGuard guard(t->device);
         if (!guard.ok) return LML_ERR_CUDA;
-        const WsLayout ws = ws_layout(t, T, 1);
         const int nb = (T + kDecodeMaxT - 1) / kDecodeMaxT;
         SlotSnapshot snaps[kDecMaxBlocks];
         DecodeArgs args[kDecMaxBlocks];
@@ -683,49 +700,14 @@ static lml_status tokens_impl(lml_table* t, const void* x, const void* W0, int T
         if (e != cudaSuccess) { cudaGetLastError(); return LML_ERR_CUDA; }
         return LML_OK;
     }
-    // Prefill: the segmentation pass writes perm and the segment arrays behind the layer's own workspace,
-    // and the layer call follows on the same stream.
-    const int G = tokens_segments(t, T);
-    const size_t base = ws_layout(t, T, G).total;
-    int32_t* perm = reinterpret_cast<int32_t*>(wsb + base);
-    int32_t* seg_offsets = reinterpret_cast<int32_t*>(wsb + base + round_up((size_t)T * 4 + 4, 1024));
-    int32_t* seg_ids = seg_offsets + round_up((size_t)(G + 1) * 4, 1024) / 4;
-    if (T <= t->one_tile_tokens) {
-        // One row tile: the tokens stay where they are.  One launch binds them and writes, per distinct slot of the
-        // batch, a block of u whose rows are the slot's tokens (zeros elsewhere); the GEMM then adds block x B per
-        // slot.  No grouping, no row copy: two launches instead of four (21 against 30 us at 128 tokens on 4096 x 4096,
-        // 32 against 41 on 11008 x 4096, 38 against 46 on 4096 x 11008).
-        const SlotSnapshot snap = snapshot_locked(t);
-        DeviceGuard guard(t->device);
-        if (!guard.ok) return LML_ERR_CUDA;
-        const WsLayout ws = ws_layout(t, T, G);
-        PlanWord* plan = reinterpret_cast<PlanWord*>(wsb + ws.plan_off);
-        __nv_bfloat16* u_blocks = reinterpret_cast<__nv_bfloat16*>(wsb + ws.u_off);
-        int launches = 0;
-        cudaError_t e = launch_bind_shrink_tile(t->arena, snap, token_slots, T, t->d_in, x, seg_offsets, seg_ids, G, plan,
-                                                u_blocks, t->bind_threads > 0 ? t->bind_threads : (t->d_in > 4096 ? 1024 : 512), stream, by_adapter);
-        if (e == cudaSuccess) {
-            ++launches;
-            GemmArgs a;
-            a.fused_shrink = false;
-            a.x = x; a.x_in_place = x; a.tile_identity = nullptr; a.W0 = W0; a.y = y; a.perm = nullptr;
-            a.seg_offsets = seg_offsets; a.slot_ids = seg_ids;
-            a.plan = plan; a.u_blocks = u_blocks;
-            a.T = T; a.d_in = t->d_in; a.d_out = t->d_out; a.G = G; a.num_sms = t->num_sms;
-            a.overlap_with_previous = true;
-            a.split_bn = t->split_bn; a.split_s = t->split_s;
-            e = launch_gemm_sm100(t->arena, snap, t->tmap_B256, t->tmap_B128, t->tmap_A, &t->tmaps, a, stream);
-            if (e == cudaSuccess) ++launches;
-        }
-        t->last_launches = launches;
-        if (e != cudaSuccess) { cudaGetLastError(); return LML_ERR_CUDA; }
-        return LML_OK;
-    }
-    lml_status st = segment_tokens_impl(t, token_slots, T, perm, seg_offsets, seg_ids, stream_v, by_adapter);
-    if (st != LML_OK) return st;
-    st = lora_mixed_linear(t, x, W0, T, seg_offsets, seg_ids, G, perm, y, workspace, base, stream_v);
-    if (st == LML_OK) t->last_launches += 1;
-    return st;
+    DeviceGuard guard(t->device);
+    if (!guard.ok) return LML_ERR_CUDA;
+    int launches = 0;
+    const GemmCall c = {t, W0, y, token_slots, static_cast<uint8_t*>(workspace), ws_layout(t, T, t->max_slots)};
+    const cudaError_t e = run_gemm_path(&c, 1, x, T, kRowsTokens, nullptr, 0, nullptr, nullptr, nullptr, by_adapter, stream, &launches);
+    t->last_launches = launches;
+    if (e != cudaSuccess) { cudaGetLastError(); return LML_ERR_CUDA; }
+    return LML_OK;
 }
 
 lml_status lora_mixed_linear_tokens(lml_table* t, const void* x, const void* W0, int T, const int32_t* token_slots,
@@ -747,8 +729,7 @@ size_t lml_multi_workspace_bytes(lml_table* const* tables, int P, int max_tokens
     size_t n = 0;
     for (int p = 0; p < P; ++p) {
         if (!tables[p]) return 0;
-        const size_t b = lml_tokens_workspace_bytes(tables[p], max_tokens);
-        n = b > n ? b : n;
+        n += round_up(lml_tokens_workspace_bytes(tables[p], max_tokens), 1024);   // (a part of its own for every projection)
     }
     return n;
 }
@@ -781,7 +762,6 @@ lml_status lora_mixed_linear_multi(lml_table* const* tables, int P, const void* 
         SlotSnapshot snaps[kDecMaxBlocks];
         DecodeArgs args[kDecMaxBlocks];
         const Arena* ars[kDecMaxBlocks];
-        const WsLayout ws = ws_layout(tables[0], T, 1);
         int n = 0;
         for (int p = 0; p < P; ++p) {
             const SlotSnapshot snap = snapshot_locked(tables[p]);
@@ -805,7 +785,24 @@ lml_status lora_mixed_linear_multi(lml_table* const* tables, int P, const void* 
         for (int p = 0; p < P; ++p) tables[p]->last_launches = p == 0 ? 1 : 0;
         return LML_OK;
     }
-    // one projection after the other: larger batches (the GEMM path), a single projection, or a table named twice
+    if (P > 1 && T > kDecodeMaxT) {
+        // One launch binds the rows of all projections and computes their u, one multiplies: the projections' tiles share
+        // the last wave, and the chain of small launches is paid once.
+        DeviceGuard guard(tables[0]->device);
+        if (!guard.ok) return LML_ERR_CUDA;
+        GemmCall calls[LML_MAX_PROJECTIONS];
+        size_t off = 0;
+        for (int p = 0; p < P; ++p) {
+            calls[p] = GemmCall{tables[p], W0[p], y[p], token_slots[p], static_cast<uint8_t*>(workspace) + off, ws_layout(tables[p], T, tables[p]->max_slots)};
+            off += round_up(calls[p].layout.total, 1024);
+        }
+        int launches = 0;
+        const cudaError_t e = run_gemm_path(calls, P, x, T, kRowsTokens, nullptr, 0, nullptr, nullptr, nullptr, false, stream, &launches);
+        if (e != cudaSuccess) { cudaGetLastError(); return LML_ERR_CUDA; }
+        for (int p = P - 1; p >= 0; --p) tables[p]->last_launches = p == 0 ? launches : 0;
+        return LML_OK;
+    }
+    // one projection after the other: a single projection, or a table named twice in a decode call
     for (int p = 0; p < P; ++p) {
         const lml_status st = tokens_impl(tables[p], x, W0[p], T, token_slots[p], y[p], workspace, workspace_bytes, stream_v, false);
         if (st != LML_OK) return st;
@@ -962,7 +959,8 @@ lml_status lml_device_status(lml_table* t, uint32_t* flags_out, void* stream_v)
     if (ok && (v & LML_FLAG_TIMEOUT)) {
         // a launch gave up on a wait: its counters may have been left behind, so the decode kernel's exchange blocks
         // start over (only then: in normal operation nothing here touches memory that a call in flight uses)
-        ok = cudaMemsetAsync(t->arena.dec_u, 0, (size_t)kDecMaxBlocks * kDecExchStride * sizeof(unsigned long long), stream) == cudaSuccess;
+        ok = cudaMemsetAsync(t->arena.status + 8, 0, 2 * sizeof(uint32_t), stream) == cudaSuccess;
+        ok = ok && cudaMemsetAsync(t->arena.dec_u, 0, (size_t)kDecMaxBlocks * kDecExchStride * sizeof(unsigned long long), stream) == cudaSuccess;
         ok = ok && cudaStreamSynchronize(stream) == cudaSuccess;
     }
     if (!ok) { cudaGetLastError(); return LML_ERR_CUDA; }

@@ -1,46 +1,66 @@
-// Small helper kernels: adapter packing (register_adapter), token segmentation, row gather.
+// Small helper kernels: adapter packing (register_adapter), token segmentation, host staging; the adapter gradients.
 #include "lml_internal.cuh"
 #include "lml_ptx_sm100.cuh"
 
 namespace lml {
 
 // ---------------------------------------------------------------------------------------------
-// register_adapter: copy A[rank][d_in] and B[d_out][rank] into the arena, zero-padded to rank 64,
+// register_adapter: copy A[rank][d_in] and B[d_out][rank] into the arena, zero-padded to whole chunks of 16,
 // so that every kernel can read fixed-shape, 16-byte aligned rows.
 // ---------------------------------------------------------------------------------------------
+// Eight columns of one row of B (row n, columns 8g ...) into the three places that hold it: the padded row, the compact row
+// of narrow adapters, and the chunk that the GEMM multiplies.
+__device__ __forceinline__ void store_b_group(__nv_bfloat16* dstB, __nv_bfloat16* dstBc, __nv_bfloat16* dstBk, int n_pad, bool compact,
+                                              long long n, int g, const uint4& v)
+{
+    *reinterpret_cast<uint4*>(dstB + n * kRankPad + g * 8) = v;
+    if (compact) *reinterpret_cast<uint4*>(dstBc + n * kRankCompact + g * 8) = v;
+    *reinterpret_cast<uint4*>(dstBk + (size_t)(g >> 1) * n_pad * kChunk + chunk_elem((int)n, (g & 1) * 8)) = v;
+}
+__device__ __forceinline__ uint4 pack_u16x8(const unsigned short (&e)[8])
+{
+    return make_uint4(e[0] | ((uint32_t)e[1] << 16), e[2] | ((uint32_t)e[3] << 16), e[4] | ((uint32_t)e[5] << 16),
+                      e[6] | ((uint32_t)e[7] << 16));
+}
+
+// Only the rows of A and columns of B that are read are written: the chunks of 16 that the rank needs.
 __global__ void __launch_bounds__(256) pack_adapter_kernel(__nv_bfloat16* __restrict__ dstA,
                                                            __nv_bfloat16* __restrict__ dstB,
                                                            __nv_bfloat16* __restrict__ dstBc,
+                                                           __nv_bfloat16* __restrict__ dstBk, int n_pad,
                                                            const __nv_bfloat16* __restrict__ A,
                                                            const __nv_bfloat16* __restrict__ B,
                                                            int rank, int d_in, int d_out)
 {
-    const long long nA8 = (long long)kRankPad * (d_in / 8);   // uint4 chunks of the padded A
-    const long long nB = (long long)d_out * kRankPad;         // elements of the padded B
+    const int cols = chunks_of_rank(rank) * kChunk, groups = cols / 8;
+    const int k8 = d_in / 8;
+    const long long nA = (long long)rank * k8, nA8 = (long long)cols * k8;   // uint4 chunks of A, and with its padding
+    const long long nB8 = (long long)d_out * groups;
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    const int k8 = d_in / 8;
-    for (long long i = tid; i < nA8; i += stride) {
-        int j = (int)(i / k8);
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (j < rank) v = reinterpret_cast<const uint4*>(A)[i];   // same linear index: rows are contiguous
-        reinterpret_cast<uint4*>(dstA)[i] = v;
-    }
+    for (long long i = tid; i < nA8; i += stride)   // same linear index: rows are contiguous
+        reinterpret_cast<uint4*>(dstA)[i] = i < nA ? __ldg(reinterpret_cast<const uint4*>(A) + i) : make_uint4(0, 0, 0, 0);
     const unsigned short* Bs = reinterpret_cast<const unsigned short*>(B);
-    unsigned short* Bd = reinterpret_cast<unsigned short*>(dstB);
-    for (long long i = tid; i < nB; i += stride) {
-        int j = (int)(i % kRankPad);
-        long long n = i / kRankPad;
-        Bd[i] = (j < rank) ? Bs[n * rank + j] : (unsigned short)0;
-    }
-    if (rank <= kRankCompact) {   // the compact copy: [d_out][kRankCompact]
-        unsigned short* Bcd = reinterpret_cast<unsigned short*>(dstBc);
-        for (long long i = tid; i < (long long)d_out * kRankCompact; i += stride) {
-            const int j = (int)(i % kRankCompact);
-            const long long n = i / kRankCompact;
-            Bcd[i] = (j < rank) ? Bs[n * rank + j] : (unsigned short)0;
+    for (long long i = tid; i < nB8; i += stride) {
+        const int g = (int)(i % groups);
+        const long long n = i / groups;
+        uint4 v;
+        if ((rank & 7) == 0) {   // rows of B are 16-byte aligned
+            v = g * 8 < rank ? __ldg(reinterpret_cast<const uint4*>(Bs + n * rank + g * 8)) : make_uint4(0, 0, 0, 0);
+        } else {
+            unsigned short e[8];
+#pragma unroll
+            for (int j = 0; j < 8; ++j) e[j] = g * 8 + j < rank ? Bs[n * rank + g * 8 + j] : (unsigned short)0;
+            v = pack_u16x8(e);
         }
+        store_b_group(dstB, dstBc, dstBk, n_pad, rank <= kRankCompact, n, g, v);
     }
+}
+
+static int pack_blocks(long long work)
+{
+    const long long blocks = (work + 255) / 256;
+    return (int)(blocks > 1184 ? 1184 : (blocks < 1 ? 1 : blocks));
 }
 
 cudaError_t launch_pack_adapter(const Arena& ar, int slot, const void* A, const void* B, int rank,
@@ -48,12 +68,12 @@ cudaError_t launch_pack_adapter(const Arena& ar, int slot, const void* A, const 
 {
     __nv_bfloat16* dstA = ar.A + (size_t)slot * kRankPad * d_in;
     __nv_bfloat16* dstB = ar.B + (size_t)slot * d_out * kRankPad;
-    long long work = (long long)d_out * kRankPad;
-    int blocks = (int)((work + 255) / 256);
-    if (blocks > 1184) blocks = 1184;
     __nv_bfloat16* dstBc = ar.Bc + (size_t)slot * d_out * kRankCompact;
-    pack_adapter_kernel<<<blocks, 256, 0, stream>>>(dstA, dstB, dstBc, (const __nv_bfloat16*)A,
-                                                    (const __nv_bfloat16*)B, rank, d_in, d_out);
+    const int n_pad = b_rows_padded(d_out);
+    __nv_bfloat16* dstBk = ar.Bk + (size_t)slot * kRankPad * n_pad;
+    const long long work = (long long)chunks_of_rank(rank) * 2 * (d_in > d_out ? d_in : d_out);
+    pack_adapter_kernel<<<pack_blocks(work), 256, 0, stream>>>(dstA, dstB, dstBc, dstBk, n_pad, (const __nv_bfloat16*)A,
+                                                               (const __nv_bfloat16*)B, rank, d_in, d_out);
     return cudaGetLastError();
 }
 
@@ -256,216 +276,6 @@ cudaError_t launch_segment_tokens(const Arena& ar, const SlotSnapshot& snap, con
 }
 
 // ---------------------------------------------------------------------------------------------
-// Token-form calls of a row tile or two (T <= 128 or 256) that are too long for the decode kernel: binding and shrink in
-// one launch, with no grouping and no row copy.  The GEMM adds, per LoRA piece of a row tile, the product of a whole
-// 128 x 64 block of u with the slot's B; which rows of the block are non-zero is the block's own business.  So the
-// tokens stay in their order: the distinct live slots of a tile's tokens, in ascending order, become the tile's
-// "segments" (the k-th is given the row range [128 m + k, 128 m + k + 1), the tile's last one the rest of the tile:
-// ranges that lie in their tile and satisfy the layer's checks; the GEMM only asks which tile a range meets; a tile
-// without any slot gets one segment without a slot), numbered through the tiles, and the block of segment g of tile m,
-// block m + g as on the grouped path, holds scale * x_t . A_slot^T in the tile's rows t that are bound to that slot and
-// zeros everywhere else.  (The kernel serves up to eight tiles; beyond two the GEMM's extra pieces, one per slot and
-// tile, cost more than grouping the rows: 54.9 against 48.2 us at 1024 tokens on 4096 x 4096.)
-// One CTA per row: it works out the slot sets of its tile and of the tiles before it, computes its row's dot
-// products (up to sixteen columns j at a time, one or two warps per column, each on its part of the row; the row of x
-// in shared memory when it fits) and writes its row of every block.  The GEMM that follows (216 KB of shared memory and
-// 18K registers per CTA) gets resident beside this kernel's CTAs, and starts on its base k-blocks, only where they leave
-// it room: 512 threads of at most 64 registers and a row of x of at most 8 KB do (d_in <= 4096); a wider row does not
-// fit beside the GEMM anyway, and 1024 threads finish it sooner.  Measured, us per call at 128 tokens on 4096 x 4096 /
-// 11008 x 4096 / 4096 x 11008: 256 threads 23.9 / 32.1 / 47.7, 512 threads 21.2 / 32.2 / 40.2, 1024 threads 24.4 / 39.6 /
-// 37.8; 512 threads with sixteen loads in flight per lane (128 registers) 25.2 / 39.9 / 40.8.  (A small persistent grid
-// on the SMs that the GEMM leaves free was measured too: beside the GEMM's stream every dependent load takes
-// microseconds, 37 against 21 us per call.)
-constexpr int kBindMaxSmemCols = 20480;   // a row of x up to this width is staged in shared memory (40 KB)
-constexpr int kBindMaxTiles = 8;          // row tiles of a call at most
-
-template <int kThreads>
-__global__ void __launch_bounds__(kThreads) bind_shrink_tile_kernel(
-    const __grid_constant__ SlotSnapshot snap, const __nv_bfloat16* __restrict__ arenaA,
-    const int32_t* __restrict__ token_slots, int T, int K, const __nv_bfloat16* __restrict__ x,
-    int32_t* __restrict__ seg_offsets, int32_t* __restrict__ seg_slot_ids, int G, PlanWord* __restrict__ plan,
-    __nv_bfloat16* __restrict__ u_blocks, uint32_t* __restrict__ status, const int32_t* __restrict__ adapter_map, int in_smem)
-{
-    constexpr int kWarps = kThreads / 32;
-    constexpr int kCols = kWarps < 16 ? kWarps : 16;   // columns worked on side by side
-    constexpr int kParts = kWarps / kCols;             // warps per column, each on its part of the row
-    extern __shared__ uint4 bind_x_s[];
-    __shared__ unsigned mask_s[kBindMaxTiles][2];
-    __shared__ int my_slot_s, bad_s;
-    __shared__ float dots_s[kRankPad];
-    __shared__ float part_s[kParts][kRankPad];
-    const int row = blockIdx.x, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int tile = row / kTileM, r_in_tile = row % kTileM, num_m = (T + kTileM - 1) / kTileM;
-    if (tid < 2 * kBindMaxTiles) (&mask_s[0][0])[tid] = 0u;
-    if (tid == 0) { my_slot_s = -1; bad_s = 0; }
-    ptx::grid_dependency_wait();      // launched as a programmatic dependent: whatever ran before is complete now
-    ptx::grid_launch_dependents();    // the GEMM may get resident where there is room; it waits for this grid before its pieces
-    __syncthreads();
-    const int nch = K / 8;
-    const uint4* xr = reinterpret_cast<const uint4*>(x + (size_t)row * K);
-    if (row < T && in_smem)   // (does not depend on the binding: goes out with the ids)
-        for (int c = tid; c < nch; c += kThreads) bind_x_s[c] = __ldg(xr + c);
-    // the slot sets of this row's tile and of the tiles before it (their sizes place this tile's segments and blocks)
-    const bool closes = tile == num_m - 1 && r_in_tile == 0;   // the CTA that also closes the segment arrays
-    const int ids_end = min(T, (tile + 1) * kTileM);
-    for (int i = tid; i < ids_end; i += kThreads) {
-        int s = __ldg(token_slots + i);
-        if (adapter_map) s = resolve_adapter(snap, adapter_map, s);
-        const bool bad_id = s < -1 || s >= snap.max_slots || (s >= 0 && snap.rank[s] == 0);
-        if (bad_id) { bad_s = 1; s = -1; }
-        if (s >= 0) atomicOr(&mask_s[i / kTileM][s >> 5], 1u << (s & 31));
-        if (i == row) my_slot_s = s;
-    }
-    __syncthreads();
-    // A tile's segments: one per distinct live slot of the tile, in ascending order; a tile without any gets one
-    // segment without a slot, so that every tile's rows belong to segments of its own.
-    auto tile_mask = [&](int m) { return (unsigned long long)mask_s[m][0] | ((unsigned long long)mask_s[m][1] << 32); };
-    int base = 0;   // segments of the tiles before this one
-    for (int m = 0; m < tile; ++m) base += max(1, __popcll(tile_mask(m)));
-    const unsigned long long mask = tile_mask(tile);
-    const int Gp = __popcll(mask);
-    if (r_in_tile == 0) {
-        if (tid == 0 && bad_s && closes) atomicOr(status, LML_FLAG_BAD_SLOT);   // (this CTA has seen every id)
-        const int nseg = max(1, Gp);
-        for (int k = tid; k < nseg; k += kThreads) {
-            int slot = -1;
-            if (k < Gp) {   // the k-th live slot of the tile
-                unsigned long long mm = mask;
-                for (int q = 0; q < k; ++q) mm &= mm - 1ull;
-                slot = __ffsll((long long)mm) - 1;
-            }
-            seg_offsets[base + k] = tile * kTileM + k;
-            seg_slot_ids[base + k] = slot;
-        }
-        if (closes) {
-            for (int g = base + nseg + tid; g <= G; g += kThreads) {
-                seg_offsets[g] = T;
-                if (g < G) seg_slot_ids[g] = -1;
-            }
-            if (tid == 0) plan->lora_ok = 1;
-        }
-    }
-    const int my_slot = row < T ? my_slot_s : -1;
-    const int g_mine = my_slot >= 0 ? __popcll(mask & ((1ull << my_slot) - 1ull)) : -1;
-    const int rank = my_slot >= 0 ? (int)snap.rank[my_slot] : 0;
-    // this row's dot products: the warps w, w + kCols, ... take the columns j = w, w + kCols, ..., each its part of the
-    // row; a lane sums the 8-element chunks lane, lane + 32, ... of the part in order, the warp adds its lanes up with
-    // the butterfly, and the parts are added in a fixed order
-    const int part = (nch + kParts - 1) / kParts;
-    const int h = warp / kCols, c_begin = min(nch, h * part), c_end = min(nch, c_begin + part);
-    for (int j = warp % kCols; j < rank; j += kCols) {
-        const uint4* ar = reinterpret_cast<const uint4*>(arenaA + ((size_t)my_slot * kRankPad + j) * K);
-        float acc = 0.f;
-        for (int c0 = c_begin + lane; c0 < c_end; c0 += 32 * 8) {
-            uint4 av[8];
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int c = c0 + 32 * i;
-                av[i] = c < c_end ? __ldg(ar + c) : make_uint4(0, 0, 0, 0);
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-                const int c = c0 + 32 * i;
-                if (c < c_end) {
-                    const uint4 xv = in_smem ? bind_x_s[c] : __ldg(xr + c);
-                    float p = 0.f;
-                    p = fmaf(bf16_lo(xv.x), bf16_lo(av[i].x), p); p = fmaf(bf16_hi(xv.x), bf16_hi(av[i].x), p);
-                    p = fmaf(bf16_lo(xv.y), bf16_lo(av[i].y), p); p = fmaf(bf16_hi(xv.y), bf16_hi(av[i].y), p);
-                    p = fmaf(bf16_lo(xv.z), bf16_lo(av[i].z), p); p = fmaf(bf16_hi(xv.z), bf16_hi(av[i].z), p);
-                    p = fmaf(bf16_lo(xv.w), bf16_lo(av[i].w), p); p = fmaf(bf16_hi(xv.w), bf16_hi(av[i].w), p);
-                    acc += p;
-                }
-            }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-        if (lane == 0) part_s[h][j] = acc;
-    }
-    __syncthreads();
-    if (tid < kRankPad) {
-        float v = 0.f;
-        if (tid < rank) {
-#pragma unroll
-            for (int q = 0; q < kParts; ++q) v += part_s[q][tid];
-            v *= snap.scale[my_slot];
-        }
-        dots_s[tid] = v;
-    }
-    __syncthreads();
-    // this row of every block: the dot products in its own block, zeros in the others (pairs of columns per thread)
-    for (int i = tid; i < Gp * (kRankPad / 2); i += kThreads) {
-        const int g = i / (kRankPad / 2), c2 = i % (kRankPad / 2);
-        __nv_bfloat162 v = __floats2bfloat162_rn(0.f, 0.f);
-        if (g == g_mine) v = __floats2bfloat162_rn(dots_s[2 * c2], dots_s[2 * c2 + 1]);
-        reinterpret_cast<__nv_bfloat162*>(u_blocks + ((size_t)(tile + base + g) * kTileM + r_in_tile) * kRankPad)[c2] = v;
-    }
-}
-
-cudaError_t launch_bind_shrink_tile(const Arena& ar, const SlotSnapshot& snap, const int32_t* token_slots, int T, int d_in,
-                                    const void* x, int32_t* seg_offsets, int32_t* seg_slot_ids, int G, PlanWord* plan,
-                                    void* u_blocks, int threads, cudaStream_t stream, bool by_adapter)
-{
-    const int in_smem = d_in <= kBindMaxSmemCols ? 1 : 0;   // (reading x through L1 instead was measured: 2 - 7 us slower per call)
-    const size_t smem = in_smem ? (size_t)d_in * 2 : 0;   // (at most 40 KB: no opt-in needed)
-    auto launch = [&](auto kernel, int nthreads) {
-        cudaLaunchConfig_t cfg = {};
-        cudaLaunchAttribute attr[1];
-        pdl_config(cfg, attr, dim3((unsigned)(((T + kTileM - 1) / kTileM) * kTileM)), dim3((unsigned)nthreads), smem, stream);
-        return cudaLaunchKernelEx(&cfg, kernel, snap, (const __nv_bfloat16*)ar.A, token_slots, T, d_in,
-                                  (const __nv_bfloat16*)x, seg_offsets, seg_slot_ids, G, plan, (__nv_bfloat16*)u_blocks, ar.status,
-                                  by_adapter ? (const int32_t*)ar.adapter_map : (const int32_t*)nullptr, in_smem);
-    };
-    if (threads >= 1024) return launch(bind_shrink_tile_kernel<1024>, 1024);
-    if (threads >= 512) return launch(bind_shrink_tile_kernel<512>, 512);
-    return launch(bind_shrink_tile_kernel<256>, 256);
-}
-
-// ---------------------------------------------------------------------------------------------
-// Row gather for the perm form of the prefill call: x_grouped[p][:] = x[perm[p]][:].
-// Batches usually arrive with each request's tokens together, so the grouping perm is the
-// identity over long stretches.  A 128-row tile whose perm is the identity is not copied: the
-// kernel marks it in tile_identity[] and the kernels that follow read (and write) those rows in
-// place, with TMA, as if no perm had been given.
-// ---------------------------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) gather_rows_kernel(const uint4* __restrict__ x,
-                                                          const int32_t* __restrict__ perm, int T, int k8,
-                                                          uint4* __restrict__ out, int32_t* __restrict__ tile_identity,
-                                                          int allow_skip, uint32_t* __restrict__ status)
-{
-    ptx::grid_dependency_wait();
-    ptx::grid_launch_dependents();
-    const int m = blockIdx.y;             // 128-row tile
-    const int p0 = m * kTileM;
-    const int rows = min(kTileM, T - p0);
-    // every CTA of the tile takes the same decision from the same 128 perm entries
-    int mine = (int)threadIdx.x < rows ? __ldg(perm + p0 + threadIdx.x) : p0 + (int)threadIdx.x;
-    const int not_identity = __syncthreads_or(mine != p0 + (int)threadIdx.x);
-    const bool skip = allow_skip && !not_identity;
-    if (blockIdx.x == 0 && threadIdx.x == 0) tile_identity[m] = skip ? 1 : 0;
-    if (skip) return;
-    for (int r = blockIdx.x; r < rows; r += gridDim.x) {
-        const int p = p0 + r;
-        int row = __ldg(perm + p);
-        const bool ok = row >= 0 && row < T;
-        if (!ok && threadIdx.x == 0) atomicOr(status, LML_FLAG_BAD_PERM);
-        const uint4* src = x + (size_t)(ok ? row : 0) * k8;
-        uint4* dst = out + (size_t)p * k8;
-        for (int i = threadIdx.x; i < k8; i += blockDim.x) dst[i] = ok ? ldg_nc_v4(src + i) : make_uint4(0, 0, 0, 0);
-    }
-}
-
-cudaError_t launch_gather_rows(const void* x, const int32_t* perm, int T, int d_in, void* x_grouped,
-                               int32_t* tile_identity, bool allow_skip, uint32_t* status, cudaStream_t stream)
-{
-    dim3 grid(32, (T + kTileM - 1) / kTileM);   // 32 CTAs share a tile's 128 rows
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[1];
-    pdl_config(cfg, attr, grid, dim3(128), 0, stream);
-    return cudaLaunchKernelEx(&cfg, gather_rows_kernel, (const uint4*)x, perm, T, d_in / 8, (uint4*)x_grouped,
-                              tile_identity, allow_skip ? 1 : 0, status);
-}
-
-// ---------------------------------------------------------------------------------------------
 // Transposed registration for the backward pass: the gradient with respect to x of the layer
 // (d_in = K, d_out = N, adapter A [r][K], B [N][r]) is the layer itself on the transposed problem
 // (d_in = N, d_out = K, base weight W0^T, adapter A' = B^T [r][N], B' = A^T [K][r]).  This kernel
@@ -474,6 +284,7 @@ cudaError_t launch_gather_rows(const void* x, const int32_t* perm, int T, int d_
 __global__ void __launch_bounds__(256) pack_adapter_transposed_kernel(__nv_bfloat16* __restrict__ dstA,
                                                                       __nv_bfloat16* __restrict__ dstB,
                                                                       __nv_bfloat16* __restrict__ dstBc,
+                                                                      __nv_bfloat16* __restrict__ dstBk, int k_pad,
                                                                       const __nv_bfloat16* __restrict__ A,
                                                                       const __nv_bfloat16* __restrict__ B,
                                                                       int rank, int K, int N)
@@ -481,26 +292,21 @@ __global__ void __launch_bounds__(256) pack_adapter_transposed_kernel(__nv_bfloa
     const unsigned short* As = reinterpret_cast<const unsigned short*>(A);
     const unsigned short* Bs = reinterpret_cast<const unsigned short*>(B);
     unsigned short* Ad = reinterpret_cast<unsigned short*>(dstA);   // [64][N]: A'[j][n] = B[n][j]
-    unsigned short* Bd = reinterpret_cast<unsigned short*>(dstB);   // [K][64]: B'[k][j] = A[j][k]
+    const int cols = chunks_of_rank(rank) * kChunk, groups = cols / 8;
     const long long stride = (long long)gridDim.x * blockDim.x;
     const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    for (long long i = tid; i < (long long)kRankPad * N; i += stride) {
+    for (long long i = tid; i < (long long)cols * N; i += stride) {
         const int j = (int)(i / N);
         const long long n = i % N;
         Ad[i] = j < rank ? Bs[n * rank + j] : (unsigned short)0;
     }
-    for (long long i = tid; i < (long long)K * kRankPad; i += stride) {
-        const int j = (int)(i % kRankPad);
-        const long long k = i / kRankPad;
-        Bd[i] = j < rank ? As[(long long)j * K + k] : (unsigned short)0;
-    }
-    if (rank <= kRankCompact) {   // the compact copy of B': [K][kRankCompact]
-        unsigned short* Bcd = reinterpret_cast<unsigned short*>(dstBc);
-        for (long long i = tid; i < (long long)K * kRankCompact; i += stride) {
-            const int j = (int)(i % kRankCompact);
-            const long long k = i / kRankCompact;
-            Bcd[i] = j < rank ? As[(long long)j * K + k] : (unsigned short)0;
-        }
+    for (long long i = tid; i < (long long)K * groups; i += stride) {   // B'[k][j] = A[j][k]
+        const int g = (int)(i / K);
+        const long long k = i % K;
+        unsigned short e[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) e[j] = g * 8 + j < rank ? As[(long long)(g * 8 + j) * K + k] : (unsigned short)0;
+        store_b_group(dstB, dstBc, dstBk, k_pad, rank <= kRankCompact, k, g, pack_u16x8(e));
     }
 }
 
@@ -509,12 +315,12 @@ cudaError_t launch_pack_adapter_transposed(const Arena& arT, int slot, const voi
 {
     __nv_bfloat16* dstA = arT.A + (size_t)slot * kRankPad * N;   // the transposed table has d_in = N ...
     __nv_bfloat16* dstB = arT.B + (size_t)slot * K * kRankPad;   // ... and d_out = K
-    long long work = (long long)(K > N ? K : N) * kRankPad;
-    int blocks = (int)((work + 255) / 256);
-    if (blocks > 1184) blocks = 1184;
     __nv_bfloat16* dstBc = arT.Bc + (size_t)slot * K * kRankCompact;
-    pack_adapter_transposed_kernel<<<blocks, 256, 0, stream>>>(dstA, dstB, dstBc, (const __nv_bfloat16*)A,
-                                                               (const __nv_bfloat16*)B, rank, K, N);
+    const int k_pad = b_rows_padded(K);
+    __nv_bfloat16* dstBk = arT.Bk + (size_t)slot * kRankPad * k_pad;
+    const long long work = (long long)chunks_of_rank(rank) * kChunk * (K > N ? K : N);
+    pack_adapter_transposed_kernel<<<pack_blocks(work), 256, 0, stream>>>(dstA, dstB, dstBc, dstBk, k_pad, (const __nv_bfloat16*)A,
+                                                                          (const __nv_bfloat16*)B, rank, K, N);
     return cudaGetLastError();
 }
 

@@ -1,31 +1,32 @@
-// Prefill path: y = bf16( x.W0^T + sum over pieces u_piece.B_slot^T ) on the sm_100a tensor cores.
+// Prefill path: y = bf16( x.W0^T + sum over chunks u_chunk.B_chunk^T ) on the sm_100a tensor cores.
 //
 // One persistent CTA per SM, 6 warps:
 //   warp 0   TMA producer: streams 128x64 tiles of x and BNx64 tiles of W0 (128-byte swizzle) into
-//            a ring of shared-memory stages; after the last k-block of a tile it appends one
-//            stage per LoRA piece of that tile: the piece's 128x64 block of u and the BNx64 block
-//            of the slot's packed B.  So the LoRA expand is just more K for the same accumulator:
-//            [x | u_1 | u_2 ...] . [W0 ; B_s1 ; B_s2 ...].
+//            a ring of shared-memory stages; after the last k-block of a tile it appends the tile's LoRA
+//            chunks (lml_bind.cu), up to four to a stage: per chunk the 128x16 block of u and the BNx16
+//            block of the slot's packed B, two contiguous pieces.  So the LoRA expand is just more K for
+//            the same accumulator: [x | u_1 | u_2 ...] . [W0 ; B_1 ; B_2 ...], and costs what the ranks of the tile's slots need.
 //   warp 1   MMA issuer: one lane issues tcgen05.mma (M=128, N=BN, K=16) per 16 columns of a stage
 //            into one of two TMEM accumulators and commits to the stage's "empty" barrier.
 //   warps 2-5 epilogue: tcgen05.ld the accumulator (each warp its 32 TMEM lanes = 32 rows), round to
-//            bf16 once, stage 32x32 chunks in shared memory and write them with TMA stores (or
-//            row-scattered 16-byte stores when a perm is given).  Runs one tile behind the MMA
-//            warp thanks to the second accumulator.
+//            bf16 once, stage 32x32 chunks in shared memory and write them with TMA stores.  Runs one tile
+//            behind the MMA warp thanks to the second accumulator.
+// Several projections of the same x share a launch: their tiles are numbered through, so that the last wave of
+// tiles is shared as well.
 // Dual form (two slot bindings of the same segments, two outputs): the base product is computed once.
 // The epilogue reads the first output out of the accumulator and tells the MMA thread; that thread
 // then adds (second binding's delta - first binding's delta) on top, as further K-steps whose u
-// operands come from two more sets of u blocks (second slots; first slots negated), and the epilogue
-// reads the second output.  The producer slips those stages into the middle of the next tile's
-// k-blocks, by when the first read is long done.
-// Fused shrink (the plain call): no shrink kernel runs before this one.  The CTAs at the end of the grid, which
-// own the fewest output tiles, first compute u = scale * x.A^T for a row tile each, as 128 x 64 tcgen05 products
-// (x k-blocks against the A k-blocks of the segments that touch the tile, side by side in an accumulator), write
-// the u blocks and raise the row tile's flag in the table's device memory; a producer waits for that flag (a
-// bounded wait) before it loads the tile's u blocks.  The table's epoch, advanced by the last CTA of every such
-// call, tells this call's flags from the last call's.
+// operands come from a second set of u blocks, and the epilogue reads the second output.  The producer slips
+// those stages into the middle of the next tile's k-blocks, by when the first read is long done.
+// Fused shrink (the plain call on a few row tiles): no launch goes ahead of this one.  Every CTA works out the slots of
+// all row tiles; the CTAs at the end of the grid, which own the fewest output tiles, first compute u = scale * x.A^T,
+// four chunks of a row tile to a pass, as 128 x 64 tcgen05 products, write the u blocks and raise the pass's flag in the
+// table's device memory; a producer waits for a tile's flags (a bounded wait) before it loads the tile's u blocks.  The
+// table's epoch, advanced by the last CTA of every such call, tells this call's flags from the last call's.
+// Early start (few rows): the kernel begins while the work before the call is still running.  It asks for the first stages'
+// W0, which is frozen, and reads x once bind_shrink, which waits for that work, has raised a word for it (a bounded wait).
 // For few tokens (tiles far fewer than SMs) a split-K variant follows below: a cluster of CTAs shares a
-// tile and exchanges partial sums through distributed shared memory; it also has a shrink mode.
+// tile and exchanges partial sums through distributed shared memory.
 // Every wait is bounded; on give-up the CTA sets LML_FLAG_TIMEOUT, drains and frees its TMEM.
 #include <cstdio>
 #include <cstdlib>
@@ -41,9 +42,10 @@ using namespace ptx;
 constexpr int kBM = kTileM;   // 128
 constexpr int kBK = 64;       // bf16 elements per 128-byte swizzled row
 constexpr int kGemmThreads = 192;
-constexpr int kSegCache = 256;            // segments cached in shared memory
 constexpr int kEpiChunkCols = 32;
 constexpr int kEpiBufBytes = 32 * kEpiChunkCols * 2;   // 2 KB: 32 rows x 64 B
+
+constexpr int kFuseTilesInKernel = 80;    // row tiles of a call whose shrink runs inside the kernel (the per-tile tables in shared memory)
 
 template <int BN> struct GemmCfg {
     static constexpr int kABytes = kBM * kBK * 2;
@@ -52,7 +54,11 @@ template <int BN> struct GemmCfg {
     static constexpr int kStages = (BN == 256) ? 4 : (BN == 128 ? 6 : 8);
     static constexpr int kEpiBytes = 4 * 2 * kEpiBufBytes;
     static constexpr int kTmemCols = 2 * BN;
-    static constexpr int kCtrlBytes = 256 + (kSegCache + 1) * 4 + 2 * kSegCache + 512 + 1040;   // barriers + segment cache (two slot arrays) + shrink plan + its per-tile table
+    static constexpr int kCtrlBytes = 256 + (kBindSegs + 1) * 4 + kBindSegs + 4 + 512 + kFuseTilesInKernel * 10 + 8 + kMaxChunks * 4;   // barriers; fused shrink: segment cache, shrink plan, per-tile masks and first passes; the first tile's chunks
+    // The split-K kernel: no staging for the epilogue.  The ring also takes the partial sums that the CTAs exchange; where
+    // they fit, a shorter one leaves the launch that computes u room on the same SM, so that the two run side by side.
+    static constexpr int kSplitStagesShort = BN == 256 ? 3 : (BN == 128 ? 4 : 5);
+    static constexpr int split_smem(int stages) { return 1024 + stages * kStageBytes + 256 + 2 * kMaxChunks * 4; }
     static constexpr int kSmemBytes = 1024 + kStages * kStageBytes + kEpiBytes + ((kCtrlBytes + 15) & ~15);
 };
 
@@ -62,11 +68,12 @@ struct GemmCtrl {
     uint64_t tmem_full[2];
     uint64_t tmem_empty[2];
     uint64_t tmem_read1[2];   // dual form: the first output of the tile has been read out of the accumulator
+    uint64_t plan_full;       // the list of chunks is in shared memory
     uint32_t tmem_base;
     int abort;
     uint32_t stage_info[8];   // written by the producer: k-steps (0..4) | kStage* flags
-    int32_t piece[4];         // shrink form of the split-K kernel: found, slot, first row, end row of the CTA's piece
     int32_t pad[2];
+    int32_t listed[2];        // entries of the list (per binding)
 };
 // stage_info flags
 constexpr uint32_t kStageCommit = 0x100u;   // after this stage the accumulator holds an output: commit it to the epilogue
@@ -76,63 +83,147 @@ constexpr uint32_t kStageDelta = 0x800u;    // dual form: first stage of a tile'
 
 static_assert(sizeof(GemmCtrl) <= 256, "control block");
 constexpr uint32_t kStageBoth = 0x2000u;    // split-K dual form: the stage's product goes into both bindings' accumulators
-constexpr uint32_t kStageShrink = 0x1000u;  // a stage of a shrink pass: x tile and bits 16..18 blocks of A; as many 128 x 64 products
+constexpr uint32_t kStageChunks = 0x4000u;  // LoRA chunks (no-swizzle operands), a K-step each
 
-// Fused shrink (the plain call on whole-K tiles): the CTAs at the end of the grid, which own one tile fewer than
-// the others or none more, first compute u = scale * x.A^T for a row tile each: one pass multiplies the tile's x
-// k-blocks with the A blocks of up to BN / 64 segments that touch the tile (128 x 64 tcgen05 products side by side
-// in an accumulator), its epilogue writes the u blocks and raises the tile's flag in the table's device memory.
-constexpr int kShrMaxPasses = 8;
-constexpr int kFuseTilesInKernel = 512;   // row tiles of a call whose shrink runs inside the kernel (the per-tile table in shared memory)
+// Fused shrink: a pass computes up to four chunks of a row tile, x[tile].A^T over all of K, two k-blocks to a stage.
+constexpr int kShrMaxPasses = 4;
+constexpr int kShrChunks = 4;
 struct ShrPass {
     int32_t m;          // row tile
-    int32_t n;          // pieces in this pass
+    int32_t n;          // chunks in this pass
+    int32_t first;      // number of the first among the tile's chunks
     int32_t flag;       // the pass's number among all passes of the call: the flag it raises
-    int32_t g[4];       // segment of each piece
-    int32_t slot[4];
+    int32_t slot[kShrChunks];
+    int32_t c[kShrChunks];
 };
 struct ShrPlan {
     int32_t npass;
-    int32_t lora_ok;
     int32_t epoch;
-    int32_t pad;
+    int32_t pad[2];
     ShrPass pass[kShrMaxPasses];
 };
 static_assert(sizeof(ShrPlan) <= 512, "shrink plan");
 
-struct GemmParams {
-    const int32_t* seg_offsets;
-    const int32_t* slot_ids;
-    const int32_t* perm;
-    const int32_t* tile_identity;   // perm form: tiles whose rows stayed in place (read tmap_x0, store with TMA)
-    const PlanWord* plan;
-    const int32_t* slot_ids2;   // dual form: the second slot per segment (else null)
-    __nv_bfloat16* y2;          // dual form: the second output
-    int u_set_rows;             // dual form: rows between the three sets of u blocks (first slots, second slots, minus first)
-    __nv_bfloat16* y;
-    uint32_t* status;
-    int T, K, N, G;
-    int num_m, num_n;
-    int fused;                  // the shrink runs inside this kernel (else a shrink kernel ran before it)
-    int32_t* tile_flags;        // fused: [row tile] = epoch + 1 once the tile's u blocks are written
-    uint32_t* fuse_sync;        // fused: [0] the table's epoch, [1] CTAs that have finished (the last one advances the epoch)
-    __nv_bfloat16* u_out;       // fused: the u blocks, for writing
+struct alignas(64) GemmPart {
+    CUtensorMap w, y;
+    const __nv_bfloat16* bk;            // the table's packed B, by chunk
+    const TilePlan* plan;               // [row tile] its chunks
+    const __nv_bfloat16* u;
+    __nv_bfloat16* y_ptr;
+    unsigned long long live;            // slots that hold an adapter
+    unsigned long long nch[2];          // ... their chunks less one, two bits each
+    int N, num_n, n_pad, cap;           // n_pad: rows of a chunk of B in memory
+    int tile0;                          // number of its first tile
 };
+struct alignas(64) GemmParams {
+    CUtensorMap x, a, y2;
+    GemmPart part[LML_MAX_PROJECTIONS];
+    const __nv_bfloat16* u2;            // dual form (else null): the second set of u blocks
+    __nv_bfloat16* y2_ptr;              // dual form: the second output
+    uint32_t* status;
+    int T, K, P;
+    int num_m, num_tiles;
+    int x_bytes;                // of one copy of x (a k-block of a row tile)
+    int stages;                 // split-K kernel: stages of the ring
+    int lora;                   // the call has adapters
+    int fused;                  // the shrink runs inside this kernel (else a bind_shrink launch came before it)
+    RowSource rows;             // fused: where the slot of a row comes from
+    int32_t* tile_flags;        // fused: [pass] = epoch + 1 once its u blocks are written
+    uint32_t* x_flag;           // early start (else null): [0] == call_id: x may be read; [1] CTAs that have finished
+    uint32_t call_id;
+    uint32_t* fuse_sync;        // fused: [0] the table's epoch, [1] CTAs that have finished (the last one advances the epoch)
+};
+__device__ __forceinline__ int slot_chunks(const GemmPart& pt, int slot)
+{
+    return 1 + (int)((pt.nch[slot >> 5] >> (2 * (slot & 31))) & 3ull);
+}
+__device__ __forceinline__ int mask_chunks(const GemmPart& pt, unsigned long long mask)
+{
+    int n = 0;
+    for (; mask; mask &= mask - 1ull) n += slot_chunks(pt, __ffsll((long long)mask) - 1);
+    return n;
+}
+// Early start: W0 is on its way already; x may be read once the launch that this one overlaps with says so (bounded wait).
+__device__ __forceinline__ bool wait_x(const GemmParams& p, volatile int* abort)
+{
+    const long long t0 = clock64();
+    while (ld_acquire_gpu_u32(p.x_flag) != p.call_id) {
+        if (*abort) return false;
+        if (clock64() - t0 > (1ll << 31)) { *abort = 1; return false; }
+    }
+    fence_proxy_async_all();
+    return true;
+}
+// A give-up before x: the copies of W0 that are on their way land (again a bounded wait) before the CTA leaves.
+__device__ __forceinline__ void drain_ahead(GemmCtrl* ctrl, int ahead)
+{
+    volatile int never = 0;
+    for (int i = 0; i < ahead; ++i) {
+        mbar_arrive(smem_u32(&ctrl->full[i]));
+        mbar_wait(smem_u32(&ctrl->full[i]), 0u, &never);
+    }
+}
+// ... and its last CTA clears the word: a replay of the same call finds it cleared.
+__device__ __forceinline__ void leave_early_start(const GemmParams& p)
+{
+    if (p.x_flag && atomicAdd(p.x_flag + 1, 1u) == gridDim.x * gridDim.y * gridDim.z - 1) {
+        p.x_flag[1] = 0u;
+        p.x_flag[0] = 0u;
+    }
+}
+// the projection that a tile belongs to
+__device__ __forceinline__ int part_of(const GemmParams& p, int tile)
+{
+    int i = 0;
+    while (i + 1 < p.P && tile >= p.part[i + 1].tile0) ++i;
+    return i;
+}
+// A whole warp copies the part of a tile's plan that concerns this CTA into shared memory, number << 16 | chunk word:
+// chunks that rows use under the bindings `who` and (rank, S) its share of them.  Returns how many.
+__device__ __forceinline__ int list_chunks(const TilePlan* plan, uint32_t who, int rank, int S, int lane, uint32_t* out)
+{
+    uint32_t e = __ldg(&plan->chunk[lane]);   // (goes out with the count; what lies past it is not used)
+    const int count = __ldg(&plan->count);
+    int n = 0;
+    for (int i0 = 0; i0 < count; i0 += 32) {
+        const int i = i0 + lane;
+        if (i0 > 0) e = i < count ? (uint32_t)__ldg(&plan->chunk[i]) : 0u;
+        const bool keep = i < count && (e & who) && (S == 1 || (int)((e & 0xffu) + ((e >> 8) & 0xfu)) % S == rank);
+        const uint32_t m = __ballot_sync(0xffffffffu, keep);
+        if (keep) out[n + __popc(m & ((1u << lane) - 1u))] = ((uint32_t)i << 16) | e;
+        n += __popc(m);
+    }
+    return n;
+}
+// One chunk of a stage: the block of u (number `index` of row tile m) and the chunk's rows of B for columns
+// [n * BN, + BN), each contiguous.  entry = slot | chunk << 8.
+template <int BN>
+__device__ __forceinline__ void load_chunk(const GemmPart& pt, const __nv_bfloat16* u, int m, int n, uint32_t entry, int index, int k,
+                                           uint32_t a_dst, uint32_t b_dst, uint32_t bar)
+{
+    mbar_expect_tx(bar, kUBlockBytes + BN * kChunk * 2);
+    bulk_load(a_dst + (uint32_t)(k * kUBlockBytes), u + ((size_t)m * pt.cap + index) * (kTileM * kChunk), kUBlockBytes, bar);
+    const size_t chunk = (size_t)(entry & 0xffu) * (kRankPad / kChunk) + (size_t)((entry >> 8) & 0xfu);
+    bulk_load(b_dst + (uint32_t)(k * BN * kChunk * 2), pt.bk + (chunk * pt.n_pad + (size_t)n * BN) * kChunk, BN * kChunk * 2, bar);
+}
+// Early start: the live slots' rows of B for this CTA's columns start on their way into L2 (a hint; the warps that will
+// run the epilogue have nothing else to do).  rank, S: this CTA's share of the chunks.
+template <int BN>
+__device__ __forceinline__ void prefetch_b(const GemmPart& pt, int n, int lane, int rank, int S)
+{
+    for (int i = lane; i < kMaxChunks; i += 32) {
+        const int s = i / (kRankPad / kChunk), c = i % (kRankPad / kChunk);
+        if (((pt.live >> s) & 1ull) && c < slot_chunks(pt, s) && (s + c) % S == rank)
+            bulk_prefetch_to_l2(pt.bk + ((size_t)i * pt.n_pad + (size_t)n * BN) * kChunk, BN * kChunk * 2);
+    }
+}
 
 template <int BN>
-__global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
-    const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_x0,
-    const __grid_constant__ CUtensorMap tmap_w,
-    const __grid_constant__ CUtensorMap tmap_u, const __grid_constant__ CUtensorMap tmap_b,
-    const __grid_constant__ CUtensorMap tmap_y, const __grid_constant__ CUtensorMap tmap_y2,
-    const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ SlotSnapshot snap, const GemmParams p)
+__global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const __grid_constant__ GemmParams p,
+                                                                          const __grid_constant__ SlotSnapshot snap)
 {
     using Cfg = GemmCfg<BN>;
-    // One piece to a pass: a pass with one piece moves two k-blocks per stage and takes about as long as an output
-    // tile; more pieces side by side (up to BN / 64 fit an accumulator) halve that rate, and every CTA's first
-    // tile would wait for the longest pass.  A row tile's pieces run on different CTAs instead.
-    constexpr int kShrPerPass = 1;
-    const bool dual = p.slot_ids2 != nullptr;
+    const bool dual = p.u2 != nullptr;
     extern __shared__ uint8_t smem_raw[];
     // 128-byte swizzled tiles need 1024-byte alignment
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -141,16 +232,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
     const uint32_t epi_addr = tiles_addr + Cfg::kStages * Cfg::kStageBytes;
     uint8_t* epi_ptr = tiles_ptr + Cfg::kStages * Cfg::kStageBytes;
     GemmCtrl* ctrl = reinterpret_cast<GemmCtrl*>(epi_ptr + Cfg::kEpiBytes);
-    int32_t* seg_cache = reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(ctrl) + 256);
-    int8_t* slot_cache = reinterpret_cast<int8_t*>(seg_cache + kSegCache + 1);
-    int8_t* slot_cache2 = slot_cache + kSegCache;   // dual form: the second slot per segment
-    ShrPlan* shr = reinterpret_cast<ShrPlan*>(slot_cache2 + kSegCache);
-    uint16_t* shr_base = reinterpret_cast<uint16_t*>(reinterpret_cast<uint8_t*>(shr) + 512);   // [row tile] first pass; kFuseTilesInKernel + 1 entries
+    ShrPlan* shr = reinterpret_cast<ShrPlan*>(reinterpret_cast<uint8_t*>(ctrl) + 256);
+    unsigned long long* tile_mask = reinterpret_cast<unsigned long long*>(reinterpret_cast<uint8_t*>(shr) + 512);   // [row tile] the slots in use
+    int32_t* seg_cache = reinterpret_cast<int32_t*>(tile_mask + kFuseTilesInKernel);
+    uint16_t* shr_base = reinterpret_cast<uint16_t*>(seg_cache + kBindSegs + 1);   // [row tile] first pass; kFuseTilesInKernel + 1 entries
+    int8_t* slot_cache = reinterpret_cast<int8_t*>(shr_base + kFuseTilesInKernel + 2);
+    uint32_t* list0 = reinterpret_cast<uint32_t*>(slot_cache + kBindSegs);   // chunks of the CTA's first tile
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int num_tiles = p.num_m * p.num_n;
+    const int num_tiles = p.num_tiles;
     const int num_kb = (p.K + kBK - 1) / kBK;
-    const bool seg_cached = p.G <= kSegCache;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < Cfg::kStages; ++s) {
@@ -162,25 +253,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
             mbar_init(smem_u32(&ctrl->tmem_empty[a]), 4);
             mbar_init(smem_u32(&ctrl->tmem_read1[a]), 4);
         }
+        mbar_init(smem_u32(&ctrl->plan_full), 1);
         ctrl->abort = 0;
         fence_mbar_init();
     }
     if (warp == 0 && lane == 0) {
-        prefetch_tmap(&tmap_x0);
-        prefetch_tmap(&tmap_x); prefetch_tmap(&tmap_w); prefetch_tmap(&tmap_u);
-        prefetch_tmap(&tmap_b); prefetch_tmap(&tmap_y);
-        if (dual) prefetch_tmap(&tmap_y2);
-    }
-    if (seg_cached && p.G > 0) {
-        for (int g = threadIdx.x; g <= p.G; g += kGemmThreads) seg_cache[g] = __ldg(p.seg_offsets + g);
-        for (int g = threadIdx.x; g < p.G; g += kGemmThreads) {
-            int s = __ldg(p.slot_ids + g);
-            slot_cache[g] = (int8_t)((s >= 0 && s < snap.max_slots && snap.rank[s] > 0) ? s : -1);
-            if (dual) {
-                const int s2 = __ldg(p.slot_ids2 + g);
-                slot_cache2[g] = (int8_t)((s2 >= 0 && s2 < snap.max_slots && snap.rank[s2] > 0) ? s2 : -1);
-            }
-        }
+        prefetch_tmap(&p.x);
+        for (int i = 0; i < p.P; ++i) { prefetch_tmap(&p.part[i].w); prefetch_tmap(&p.part[i].y); }
+        if (dual) prefetch_tmap(&p.y2);
     }
     if (warp == 1) tmem_alloc(smem_u32(&ctrl->tmem_base), Cfg::kTmemCols);
     tc_fence_before();
@@ -188,51 +268,59 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
     tc_fence_after();
     const uint32_t tmem_base = ctrl->tmem_base;
     volatile int* abort = &ctrl->abort;
-    if (p.G == 0 || p.fused) {   // no shrink kernel ran before this one in the call: wait for foreign work here
+    if (!p.lora || p.fused) {   // no launch of this call came before this one: wait for foreign work here
         grid_dependency_wait();
         grid_launch_dependents();
     }
+    const bool by_segment = p.rows.mode == kRowsSegments;
     if (p.fused) {
-        // The segment arrays are checked here (every CTA reaches the same verdict from its own copy), and the CTA's
-        // shrink passes are laid out: row tiles grid-1-blockIdx, +grid, ... (the CTAs at the end of the grid own
-        // the fewest output tiles), and for each the live segments that touch it, kShrPerPass to a pass.
+        // Every CTA works out the slots of all row tiles from its own copy of the segment arrays (checked here: all reach
+        // the same verdict) or from the slot per row.
         int bad_off = 0, bad_slot = 0;
-        for (int g = threadIdx.x; g < p.G; g += kGemmThreads) {
-            const int s0 = seg_cache[g], s1 = seg_cache[g + 1];
-            if (s1 < s0 || s0 < 0 || s1 > p.T) bad_off = 1;
-            const int sl = __ldg(p.slot_ids + g);
-            if (sl != -1 && s1 > s0 && slot_rank(snap, sl) == 0) bad_slot = 1;   // an empty segment may name anything
-        }
-        if (threadIdx.x == 0 && (seg_cache[0] != 0 || seg_cache[p.G] != p.T)) bad_off = 1;
-        bad_off = __syncthreads_or(bad_off);
-        bad_slot = __syncthreads_or(bad_slot);
-        // Passes of every row tile: its live pieces, kShrPerPass to a pass (threads share the tiles out) ...
-        auto live_pieces = [&](int m, int skip, int take, ShrPass* out) -> int {   // counts the tile's pieces; fills `out` with pieces skip .. skip+take-1
-            const int row0 = m * kBM, row1 = min(row0 + kBM, p.T);
-            int lo = 0, hi = p.G;
-            while (lo < hi) { const int mid = (lo + hi) >> 1; if (seg_cache[mid + 1] > row0) hi = mid; else lo = mid + 1; }
-            int c = 0;
-            for (int g = lo; g < p.G && seg_cache[g] < row1; ++g) {
-                const int sl = slot_cache[g];
-                if (sl < 0 || min(seg_cache[g + 1], row1) <= max(seg_cache[g], row0)) continue;
-                if (out && c >= skip && c < skip + take) { out->g[c - skip] = g; out->slot[c - skip] = sl; }
-                ++c;
+        for (int m = threadIdx.x; m < p.num_m; m += kGemmThreads) tile_mask[m] = 0ull;
+        if (by_segment) {
+            const int G = p.rows.G;
+            for (int g = threadIdx.x; g <= G; g += kGemmThreads) seg_cache[g] = __ldg(p.rows.seg_offsets + g);
+            for (int g = threadIdx.x; g < G; g += kGemmThreads) {
+                const int s = __ldg(p.rows.ids + g);
+                slot_cache[g] = (int8_t)(slot_rank(snap, s) > 0 ? s : (s == -1 ? -1 : -2));
             }
-            return c;
-        };
-        for (int m = threadIdx.x; m < p.num_m; m += kGemmThreads)
-            shr_base[m + 1] = (uint16_t)(bad_off ? 0 : (live_pieces(m, 0, 0, nullptr) + kShrPerPass - 1) / kShrPerPass);
-        __syncthreads();
-        if (threadIdx.x == 0) {
-            if (blockIdx.x == 0) {
+            __syncthreads();
+            for (int g = threadIdx.x; g < G; g += kGemmThreads) {
+                const int s0 = seg_cache[g], s1 = seg_cache[g + 1];
+                if (s1 < s0 || s0 < 0 || s1 > p.T) bad_off = 1;
+                if (slot_cache[g] == -2 && s1 > s0) bad_slot = 1;   // an empty segment may name anything
+            }
+            if (threadIdx.x == 0 && (seg_cache[0] != 0 || seg_cache[G] != p.T)) bad_off = 1;
+            bad_off = __syncthreads_or(bad_off);
+            bad_slot = __syncthreads_or(bad_slot);
+            if (!bad_off)
+                for (int g = threadIdx.x; g < G; g += kGemmThreads) {
+                    const int s0 = seg_cache[g], s1 = seg_cache[g + 1], s = slot_cache[g];
+                    if (s >= 0 && s1 > s0)
+                        for (int m = s0 / kBM; m <= (s1 - 1) / kBM; ++m) atomicOr(&tile_mask[m], 1ull << s);
+                }
+            if (threadIdx.x == 0 && blockIdx.x == 0) {
                 const unsigned f = (bad_off ? LML_FLAG_BAD_OFFSETS : 0u) | (bad_slot ? LML_FLAG_BAD_SLOT : 0u);
                 if (f) atomicOr(p.status, f);
             }
-            shr->lora_ok = bad_off ? 0 : 1;
+        } else {
+            __syncthreads();
+            for (int row = threadIdx.x; row < p.T; row += kGemmThreads) {
+                const int s = p.rows.rows[row];
+                if (slot_rank(snap, s) > 0) atomicOr(&tile_mask[row / kBM], 1ull << s);
+            }
+        }
+        __syncthreads();
+        const GemmPart& pt = p.part[0];
+        for (int m = threadIdx.x; m < p.num_m; m += kGemmThreads)
+            shr_base[m + 1] = (uint16_t)((mask_chunks(pt, tile_mask[m]) + kShrChunks - 1) / kShrChunks);
+        __syncthreads();
+        if (threadIdx.x == 0) {
+            // The passes are numbered through all row tiles (shr_base[m] = first pass of tile m); pass i is the work of CTA
+            // grid-1 - (i mod grid): the CTAs at the end of the grid own the fewest output tiles, and the passes of a row
+            // tile run side by side on different CTAs.
             shr->epoch = (int32_t)(*reinterpret_cast<volatile uint32_t*>(p.fuse_sync));
-            // ... numbered through all row tiles (shr_base[m] = first pass of tile m); pass i is the work of CTA
-            // grid-1 - (i mod grid): the CTAs at the end of the grid own the fewest output tiles, and the passes
-            // of a row tile with many pieces run side by side on different CTAs
             shr_base[0] = 0;
             for (int m = 0; m < p.num_m; ++m) shr_base[m + 1] = (uint16_t)(shr_base[m] + shr_base[m + 1]);
             const int total = shr_base[p.num_m];
@@ -240,9 +328,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
             for (int i = (int)gridDim.x - 1 - (int)blockIdx.x; i < total && np < kShrMaxPasses; i += (int)gridDim.x) {
                 while (shr_base[m + 1] <= i) ++m;
                 ShrPass& ps = shr->pass[np++];
-                ps.m = m; ps.flag = i;
-                const int c = live_pieces(m, (i - shr_base[m]) * kShrPerPass, kShrPerPass, &ps);
-                ps.n = min(kShrPerPass, c - (i - shr_base[m]) * kShrPerPass);
+                ps.m = m; ps.flag = i; ps.n = 0;
+                ps.first = (i - shr_base[m]) * kShrChunks;
+                int at = 0;
+                for (unsigned long long mk = tile_mask[m]; mk; mk &= mk - 1ull) {
+                    const int s = __ffsll((long long)mk) - 1;
+                    for (int c = 0; c < slot_chunks(pt, s); ++c, ++at)
+                        if (at >= ps.first && at < ps.first + kShrChunks) { ps.slot[ps.n] = s; ps.c[ps.n] = c; ++ps.n; }
+                }
             }
             shr->npass = np;
         }
@@ -259,7 +352,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
         // into the middle of the NEXT tile's k-blocks (or follow the last tile), where the MMA thread
         // does not have to wait for that.
         if (lane == 0) {
-            bool lora = false, lora_known = (p.G == 0);
+            bool lora = false, lora_known = !p.lora;
+            // the CTA's first tile: its chunks are listed in shared memory
+            const GemmPart* const list0_part = &p.part[part_of(p, (int)blockIdx.x)];
+            const int list0_m = ((int)blockIdx.x - list0_part->tile0) % p.num_m, list0_n = ((int)blockIdx.x - list0_part->tile0) / p.num_m;
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -268,20 +364,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
             };
             auto advance = [&]() { if (++stage == Cfg::kStages) { stage = 0; phase ^= 1u; } };
             auto learn_lora = [&]() {
-                // Everything the shrink kernel wrote (plan word, u blocks) is first touched after the
+                // Everything the launch before this one wrote (plans, u blocks) is first touched after the
                 // base k-blocks of the first tile are already in flight.
                 if (!lora_known) {
-                    if (p.fused) lora = shr->lora_ok != 0;
-                    else {
+                    if (!p.fused) {   // (warp 2 has waited for that launch, and has let the next one go)
+                        ok = mbar_wait(smem_u32(&ctrl->plan_full), 0u, abort);
                         grid_dependency_wait();
-                        grid_launch_dependents();
-                        lora = p.plan->lora_ok != 0;
                     }
+                    lora = true;
                     lora_known = true;
                 }
             };
-            // fused shrink: the u blocks of row tile m are written by another CTA of this grid, which raises the
-            // tile's flag when they are complete (bounded wait; the flag's writer runs its shrink passes first thing)
+            // fused shrink: the u blocks of row tile m are written by other CTAs of this grid, which raise the
+            // passes' flags when they are complete (bounded wait; the flags' writers run their passes first thing)
             int flag_seen_m = -1;
             auto wait_u = [&](int m) {
                 if (!p.fused || m == flag_seen_m) return;
@@ -292,64 +387,67 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
                         if (*abort) { ok = false; return; }
                         if (clock64() - t0 > (1ll << 31)) { *abort = 1; ok = false; return; }
                     }
-                fence_proxy_async_all();   // what those CTAs wrote with ordinary stores is read by TMA from here on
+                fence_proxy_async_all();   // what those CTAs wrote with ordinary stores is read by bulk copies from here on
                 flag_seen_m = m;
             };
-            // slot of segment g as far as tile rows [row0, row1) are concerned; -1 = no piece
-            auto piece_slot = [&](int g, int row0, int row1, bool second) -> int {
-                int s0, s1, s;
-                if (seg_cached) { s0 = seg_cache[g]; s1 = seg_cache[g + 1]; s = second ? slot_cache2[g] : slot_cache[g]; }
-                else {
-                    s0 = __ldg(p.seg_offsets + g); s1 = __ldg(p.seg_offsets + g + 1);
-                    s = __ldg((second ? p.slot_ids2 : p.slot_ids) + g);
-                    if (slot_rank(snap, s) == 0) s = -1;
-                }
-                if (min(s1, row1) <= max(s0, row0)) return -1;
-                return s;
-            };
-            auto segment_range = [&](int row0, int row1, int& g_first, int& g_end) {
-                if (seg_cached) {
-                    int lo = 0, hi = p.G;
-                    while (lo < hi) { int mid = (lo + hi) >> 1; if (seg_cache[mid + 1] > row0) hi = mid; else lo = mid + 1; }
-                    g_first = lo;
-                    g_end = g_first;
-                    while (g_end < p.G && seg_cache[g_end] < row1) ++g_end;
-                } else {
-                    g_first = seg_upper(p.seg_offsets, p.G, row0);
-                    g_end = g_first;
-                    while (g_end < p.G && __ldg(p.seg_offsets + g_end) < row1) ++g_end;
-                }
-            };
-            // one stage per piece of a tile from one of the three sets of u blocks; `flags_first` go on the
-            // first stage emitted, `flags_last` on the last; returns how many stages went out
-            auto emit_pieces = [&](int m, int n, int set, bool second, uint32_t acc_flag, uint32_t flags_first,
-                                   uint32_t flags_last, bool count_only) -> int {
-                const int row0 = m * kBM, row1 = min(row0 + kBM, p.T);
-                int g_first = 0, g_end = 0, count = 0, last_piece = -1;
-                if (lora) {
-                    segment_range(row0, row1, g_first, g_end);
-                    for (int g = g_first; g < g_end; ++g) if (piece_slot(g, row0, row1, second) >= 0) { last_piece = g; ++count; }
-                }
-                if (count_only) return count;
-                if (count > 0) wait_u(m);
-                if (!ok) return count;
+            // The chunks of row tile m that rows use under the bindings `who`, up to four to a stage; `flags_first` go on the
+            // first stage, `flags_last` on the last.  They are listed in the tile's plan; with the fused shrink, they follow
+            // from the tile's slots.
+            auto emit_chunks = [&](const GemmPart& pt, const __nv_bfloat16* u, int m, int n, uint32_t who, uint32_t acc_flag,
+                                   uint32_t flags_first, uint32_t flags_last) {
+                wait_u(m);
+                int index = -1, c = 0, at = 0;
+                const bool listed = !p.fused && &pt == list0_part && m == list0_m && n == list0_n;
+                unsigned long long mk = p.fused ? tile_mask[m] : 0ull;
+                const TilePlan* plan = pt.plan + m;
+                const int count = p.fused ? 0 : (listed ? ctrl->listed[0] : __ldg(&plan->count));
+                auto next = [&]() -> int {   // the next chunk, or -1; index is its number
+                    if (p.fused) {
+                        if (!mk) return -1;
+                        const int s = __ffsll((long long)mk) - 1, e = s | (c << 8);
+                        if (++c == slot_chunks(pt, s)) { c = 0; mk &= mk - 1ull; }
+                        ++index;
+                        return e;
+                    }
+                    while (listed && at < count) {
+                        const uint32_t e = list0[at++];
+                        index = (int)(e >> 16);
+                        if (e & who) return (int)(e & 0xffffu);
+                    }
+                    if (listed) return -1;
+                    while (++index < count) {
+                        const int e = __ldg(&plan->chunk[index]);
+                        if ((uint32_t)e & who) return e;
+                    }
+                    return -1;
+                };
                 bool first = true;
-                for (int g = g_first; g < g_end && ok; ++g) {
-                    const int s = piece_slot(g, row0, row1, second);
-                    if (s < 0) continue;
+                int e = next();
+                while (e >= 0 && ok) {
                     ok = acquire();
                     if (!ok) break;
-                    const uint32_t a_dst = tiles_addr + stage * Cfg::kStageBytes;
-                    const uint32_t bar = smem_u32(&ctrl->full[stage]);
-                    const uint32_t ksteps = (uint32_t)((snap.rank[s] + 15) >> 4);
-                    ctrl->stage_info[stage] = ksteps | acc_flag | (first ? flags_first : 0u) | (g == last_piece ? flags_last : 0u);
+                    const uint32_t a_dst = tiles_addr + stage * Cfg::kStageBytes, bar = smem_u32(&ctrl->full[stage]);
+                    int k = 0;
+                    while (k < 4 && e >= 0) {
+                        load_chunk<BN>(pt, u, m, n, (uint32_t)e, index, k++, a_dst, a_dst + Cfg::kABytes, bar);
+                        e = next();
+                    }
+                    ctrl->stage_info[stage] = (uint32_t)k | acc_flag | kStageChunks | (first ? flags_first : 0u) | (e < 0 ? flags_last : 0u);
                     first = false;
-                    mbar_arrive_expect_tx(bar, Cfg::kStageBytes);
-                    tma_load_2d(a_dst, &tmap_u, bar, 0, set * p.u_set_rows + (m + g) * kBM);
-                    tma_load_3d(a_dst + Cfg::kABytes, &tmap_b, bar, 0, n * BN, s);
+                    mbar_arrive(bar);
                     advance();
                 }
-                return count;
+            };
+            // whether any rows of tile m use a slot under the bindings `who`
+            auto has_chunks = [&](const GemmPart& pt, int m, int n, uint32_t who) -> bool {
+                if (!lora) return false;
+                if (p.fused) return tile_mask[m] != 0ull;
+                const bool listed = &pt == list0_part && m == list0_m && n == list0_n;
+                const TilePlan* plan = pt.plan + m;
+                const int count = listed ? ctrl->listed[0] : __ldg(&plan->count);
+                if (!dual) return count > 0;
+                for (int i = 0; i < count; ++i) if ((listed ? list0[i] : (uint32_t)__ldg(&plan->chunk[i])) & who) return true;
+                return false;
             };
             // a stage without operands: only its flags matter to the MMA thread
             auto emit_marker = [&](uint32_t info) {
@@ -359,72 +457,89 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
                 mbar_arrive(smem_u32(&ctrl->full[stage]));
                 advance();
             };
-            // the delta stages of tile (m, n) on accumulator flag acc_flag
+            // dual form: the delta stages of tile (m, n) on accumulator flag acc_flag
             auto emit_delta = [&](int m, int n, uint32_t acc_flag) {
-                const int n_new = emit_pieces(m, n, 1, true, acc_flag, 0u, 0u, true);
-                const int n_old = emit_pieces(m, n, 2, false, acc_flag, 0u, 0u, true);
-                if (n_new + n_old == 0) { emit_marker(acc_flag | kStageDelta | kStageCommit); return; }
-                emit_pieces(m, n, 1, true, acc_flag, kStageDelta, n_old == 0 ? kStageCommit : 0u, false);
-                if (ok && n_old > 0) emit_pieces(m, n, 2, false, acc_flag, n_new == 0 ? kStageDelta : 0u, kStageCommit, false);
+                if (!has_chunks(p.part[0], m, n, kChunkFirst | kChunkSecond)) { emit_marker(acc_flag | kStageDelta | kStageCommit); return; }
+                emit_chunks(p.part[0], p.u2, m, n, kChunkFirst | kChunkSecond, acc_flag, kStageDelta, kStageCommit);
             };
             int ordinal = 0, prev_m = -1, prev_n = -1;
             // this CTA's shrink passes: a pass is num_kb stages of [x k-block | A k-blocks of its pieces]
             for (int ps = 0; p.fused && ps < shr->npass && ok; ++ps, ++ordinal) {
                 const ShrPass& sp = shr->pass[ps];
                 const uint32_t acc_flag = (ordinal & 1) ? kStageAcc1 : 0u;
-                const bool in_place = p.tile_identity && __ldg(p.tile_identity + sp.m);
-                // (a pass with one piece moves 24 KB per k-block: two k-blocks share a stage, so that as many bytes
-                // are on their way as in the tiles' stages)
-                const int sub_bytes = Cfg::kABytes + sp.n * (64 * kBK * 2);
+                // (a k-block of a pass is at most 24 KB: two share a stage, so that as many bytes are on their way
+                // as in the tiles' stages)
+                const int sub_bytes = Cfg::kABytes + sp.n * (kChunk * kBK * 2);
                 const int per_stage = 2 * sub_bytes <= Cfg::kStageBytes ? 2 : 1;
                 for (int kb = 0; kb < num_kb && ok; kb += per_stage) {
                     ok = acquire();
                     if (!ok) break;
                     const int nsub = min(per_stage, num_kb - kb);
                     const uint32_t bar = smem_u32(&ctrl->full[stage]);
-                    ctrl->stage_info[stage] = 4u | acc_flag | kStageShrink | ((uint32_t)sp.n << 16) | ((uint32_t)nsub << 20) |
+                    ctrl->stage_info[stage] = 4u | acc_flag | ((uint32_t)sp.n << 16) | ((uint32_t)nsub << 20) |
                                               (kb == 0 ? kStageFresh : 0u) | (kb + nsub >= num_kb ? kStageCommit : 0u);
-                    mbar_arrive_expect_tx(bar, (uint32_t)(nsub * sub_bytes));
+                    mbar_arrive_expect_tx(bar, (uint32_t)(nsub * (p.x_bytes + sp.n * (kChunk * kBK * 2))));
                     for (int j = 0; j < nsub; ++j) {
                         const uint32_t a_dst = tiles_addr + stage * Cfg::kStageBytes + j * sub_bytes;
-                        if (in_place) tma_load_2d(a_dst, &tmap_x0, bar, (kb + j) * kBK, sp.m * kBM);
-                        else tma_load_2d(a_dst, &tmap_x, bar, (kb + j) * kBK, sp.m * kBM);
+                        tma_load_2d(a_dst, &p.x, bar, (kb + j) * kBK, sp.m * kBM);
                         for (int i = 0; i < sp.n; ++i)
-                            tma_load_3d(a_dst + Cfg::kABytes + i * (64 * kBK * 2), &tmap_a, bar, (kb + j) * kBK, 0, sp.slot[i]);
+                            tma_load_3d(a_dst + Cfg::kABytes + i * (kChunk * kBK * 2), &p.a, bar, (kb + j) * kBK, sp.c[i] * kChunk, sp.slot[i]);
                     }
                     advance();
                 }
             }
+            int ahead = 0;   // early start: k-blocks of the first tile whose W0 has been asked for already
+            if (p.x_flag) {
+                const GemmPart& pt = *list0_part;
+                ahead = min(Cfg::kStages, num_kb);
+                for (int kb = 0; kb < ahead; ++kb) {
+                    const uint32_t bar = smem_u32(&ctrl->full[kb]);
+                    mbar_expect_tx(bar, Cfg::kBBytes);
+                    tma_load_2d(tiles_addr + kb * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, kb * kBK, list0_n * BN);
+                }
+                ok = wait_x(p, abort);
+                if (!ok) drain_ahead(ctrl, ahead);
+            }
+            // k-blocks [k0, k1) of a tile; the ring's place lives in registers here (the lambdas above hold it by reference)
+            auto base_blocks = [&](const CUtensorMap* w, int row0, int col0, int k0, int k1, uint32_t acc_flag, uint32_t flags_last, int have_w) {
+                int st = stage;
+                uint32_t ph = phase;
+                bool good = ok;
+                for (int kb = k0; kb < k1; ++kb) {
+                    good = mbar_wait(smem_u32(&ctrl->empty[st]), ph ^ 1u, abort);
+                    if (!good) break;
+                    const uint32_t a_dst = tiles_addr + st * Cfg::kStageBytes;
+                    const uint32_t bar = smem_u32(&ctrl->full[st]);
+                    ctrl->stage_info[st] = 4u | acc_flag | (kb == 0 ? kStageFresh : 0u) | (kb == num_kb - 1 ? flags_last : 0u);
+                    mbar_arrive_expect_tx(bar, (uint32_t)(p.x_bytes + (kb < have_w ? 0 : Cfg::kBBytes)));
+                    tma_load_2d(a_dst, &p.x, bar, kb * kBK, row0);
+                    if (kb >= have_w) tma_load_2d(a_dst + Cfg::kABytes, w, bar, kb * kBK, col0);
+                    if (++st == Cfg::kStages) { st = 0; ph ^= 1u; }
+                }
+                stage = st; phase = ph; ok = good;
+            };
             for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++ordinal) {
-                const int m = tile % p.num_m, n = tile / p.num_m;
+                const GemmPart& pt = p.part[part_of(p, tile)];
+                const int m = (tile - pt.tile0) % p.num_m, n = (tile - pt.tile0) / p.num_m;
                 const int row0 = m * kBM;
                 const uint32_t acc_flag = (ordinal & 1) ? kStageAcc1 : 0u;
-                const bool in_place = p.tile_identity && __ldg(p.tile_identity + m);   // rows of x never copied
-                int pieces = 0;
-                for (int kb = 0; kb < num_kb && ok; ++kb) {
-                    if (kb == num_kb - 1) {
-                        learn_lora();
-                        pieces = emit_pieces(m, n, 0, false, acc_flag, 0u, 0u, true);
-                    }
-                    if (dual && prev_m >= 0 && kb == min((num_kb + 1) / 2, num_kb - 1)) {
-                        learn_lora();
-                        emit_delta(prev_m, prev_n, acc_flag ^ kStageAcc1);
-                        if (!ok) break;
-                    }
-                    ok = acquire();
+                const int mid = min((num_kb + 1) / 2, num_kb - 1);
+                int from = 0;
+                if (dual && prev_m >= 0) {
+                    base_blocks(&pt.w, row0, n * BN, 0, mid, acc_flag, 0u, 0);
+                    from = mid;
                     if (!ok) break;
-                    const uint32_t a_dst = tiles_addr + stage * Cfg::kStageBytes;
-                    const uint32_t bar = smem_u32(&ctrl->full[stage]);
-                    ctrl->stage_info[stage] = 4u | acc_flag | (kb == 0 ? kStageFresh : 0u) |
-                                              ((kb == num_kb - 1 && pieces == 0) ? kStageCommit : 0u);
-                    mbar_arrive_expect_tx(bar, Cfg::kStageBytes);
-                    // two call sites on purpose: each names its tensor map as a kernel-parameter constant
-                    if (in_place) tma_load_2d(a_dst, &tmap_x0, bar, kb * kBK, row0);
-                    else tma_load_2d(a_dst, &tmap_x, bar, kb * kBK, row0);
-                    tma_load_2d(a_dst + Cfg::kABytes, &tmap_w, bar, kb * kBK, n * BN);
-                    advance();
+                    learn_lora();
+                    if (ok) emit_delta(prev_m, prev_n, acc_flag ^ kStageAcc1);
+                    if (!ok) break;
                 }
-                if (ok && pieces > 0) emit_pieces(m, n, 0, false, acc_flag, 0u, kStageCommit, false);
+                base_blocks(&pt.w, row0, n * BN, from, num_kb - 1, acc_flag, 0u, ordinal == 0 ? ahead : 0);
+                if (!ok) break;
+                learn_lora();
+                if (!ok) break;
+                const bool chunks = has_chunks(pt, m, n, kChunkFirst);
+                base_blocks(&pt.w, row0, n * BN, num_kb - 1, num_kb, acc_flag, chunks ? 0u : kStageCommit, ordinal == 0 ? ahead : 0);
+                if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, acc_flag, 0u, kStageCommit);
                 prev_m = m; prev_n = n;
             }
             if (ok && dual && prev_m >= 0) {
@@ -447,14 +562,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
             uint32_t empty_ph0 = 0, empty_ph1 = 0, read1_ph0 = 0, read1_ph1 = 0;
             bool ok = true;
             // one stage: ksteps MMAs into d_tmem, then the stage goes back to the producer
-            auto issue = [&](uint32_t d_tmem, int ksteps, uint32_t& accumulate) {
+            auto issue = [&](uint32_t d_tmem, int ksteps, bool chunks, uint32_t& accumulate) {
                 const uint32_t a_addr = tiles_addr + stage * Cfg::kStageBytes;
-                const uint64_t adesc = umma_desc_k128(a_addr);
-                const uint64_t bdesc = umma_desc_k128(a_addr + Cfg::kABytes);
+                const uint64_t adesc = chunks ? umma_desc_k16(a_addr) : umma_desc_k128(a_addr);
+                const uint64_t bdesc = chunks ? umma_desc_k16(a_addr + Cfg::kABytes) : umma_desc_k128(a_addr + Cfg::kABytes);
+                // 16 bf16 columns = 32 bytes further along the swizzled row: +2 in 16-byte units; a chunk is a block of its own
+                const uint64_t astep = chunks ? kUBlockBytes / 16 : 2, bstep = chunks ? BN * kChunk * 2 / 16 : 2;
 #pragma unroll 4
                 for (int k = 0; k < ksteps; ++k) {
-                    // 16 bf16 columns = 32 bytes further along the swizzled row: +2 in 16-byte units
-                    umma_bf16(d_tmem, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, accumulate);
+                    umma_bf16(d_tmem, adesc + (uint64_t)k * astep, bdesc + (uint64_t)k * bstep, idesc, accumulate);
                     accumulate = 1;
                 }
                 umma_commit(smem_u32(&ctrl->empty[stage]));
@@ -468,7 +584,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
                     if (!ok) break;
                     const uint32_t info = ctrl->stage_info[stage];
                     more = (info & kStageCommit) == 0;
-                    issue(d_tmem, (int)(info & 0xffu), accumulate);
+                    issue(d_tmem, (int)(info & 0xffu), (info & kStageChunks) != 0, accumulate);
                 }
                 if (ok) umma_commit(smem_u32(&ctrl->tmem_full[acc]));
             };
@@ -484,9 +600,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
                 flagged_stages(acc, accumulate);
             };
             int ordinal = 0;
-            // this CTA's shrink passes: per stage, one 128 x 64 product per piece, side by side in the accumulator
+            // this CTA's shrink passes: 128 x (16 per chunk) products
             for (int ps = 0; p.fused && ps < shr->npass && ok; ++ps, ++ordinal) {
-                constexpr uint32_t idesc64 = umma_idesc_bf16(kBM, 64);
                 const int acc = ordinal & 1;
                 uint32_t& eph = acc ? empty_ph1 : empty_ph0;
                 ok = mbar_wait(smem_u32(&ctrl->tmem_empty[acc]), eph ^ 1u, abort);
@@ -500,19 +615,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
                     if (!ok) break;
                     const uint32_t info = ctrl->stage_info[stage];
                     more = (info & kStageCommit) == 0;
-                    const int npc = (int)((info >> 16) & 7u), nsub = (int)((info >> 20) & 3u);
-                    const int sub_bytes = Cfg::kABytes + npc * (64 * kBK * 2);
+                    const int nch = (int)((info >> 16) & 7u), nsub = (int)((info >> 20) & 3u);
+                    const int sub_bytes = Cfg::kABytes + nch * (kChunk * kBK * 2);
+                    const uint32_t idesc_n = umma_idesc_bf16(kBM, nch * kChunk);
                     tc_fence_after();
                     for (int j = 0; j < nsub; ++j) {
                         const uint32_t a_addr = tiles_addr + stage * Cfg::kStageBytes + j * sub_bytes;
                         const uint64_t adesc = umma_desc_k128(a_addr);
-                        for (int i = 0; i < npc; ++i) {
-                            const uint64_t bdesc = umma_desc_k128(a_addr + Cfg::kABytes + i * (64 * kBK * 2));
+                        const uint64_t bdesc = umma_desc_k128(a_addr + Cfg::kABytes);
 #pragma unroll
-                            for (int k = 0; k < 4; ++k)
-                                umma_bf16(d_tmem + (uint32_t)(64 * i), adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc64,
-                                          (!fresh || k > 0) ? 1u : 0u);
-                        }
+                        for (int k = 0; k < 4; ++k)
+                            umma_bf16(d_tmem, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc_n, (!fresh || k > 0) ? 1u : 0u);
                         fresh = false;
                     }
                     umma_commit(smem_u32(&ctrl->empty[stage]));
@@ -534,7 +647,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
                     if (dual && ordinal > 0 && kb == mid) { delta_stages(acc ^ 1); if (!ok) break; }
                     ok = mbar_wait(smem_u32(&ctrl->full[stage]), phase, abort);
                     if (!ok) break;
-                    issue(d_tmem, 4, accumulate);
+                    issue(d_tmem, 4, false, accumulate);
                 }
                 if (!ok) break;
                 if (dual && ordinal > 0 && mid == num_kb - 1) { delta_stages(acc ^ 1); if (!ok) break; }
@@ -552,8 +665,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
         uint32_t full_ph0 = 0, full_ph1 = 0;
         int buf = 0;
         bool ok = true;
-        // this CTA's shrink passes: scale, zero the rows outside the segment, round, write the u blocks; after a
-        // tile's last pass its flag goes up (release: the four warps' stores are complete)
+        if (p.lora && !p.fused && warp == 2) {   // nothing else to do yet: the first tile's chunks, as soon as they are known
+            const GemmPart& pt = p.part[part_of(p, (int)blockIdx.x)];
+            if (p.x_flag) prefetch_b<BN>(pt, ((int)blockIdx.x - pt.tile0) / p.num_m, lane, 0, 1);
+            grid_dependency_wait();
+            grid_launch_dependents();
+            const int n = list_chunks(pt.plan + ((int)blockIdx.x - pt.tile0) % p.num_m, kChunkFirst | kChunkSecond, 0, 1, lane, list0);
+            __syncwarp();
+            if (lane == 0) { ctrl->listed[0] = n; mbar_arrive(smem_u32(&ctrl->plan_full)); }
+        }
+        // this CTA's shrink passes: scale, zero the rows of other slots, round, write the u blocks; then the pass's
+        // flag goes up (release: the four warps' stores are complete)
         for (int ps = 0; p.fused && ps < shr->npass && ok; ++ps) {
             const ShrPass& sp = shr->pass[ps];
             uint32_t& fph = acc ? full_ph1 : full_ph0;
@@ -562,26 +684,36 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
             fph ^= 1u;
             tc_fence_after();
             const int pos = sp.m * kBM + q * 32 + lane;
-            const int row0 = sp.m * kBM, row1 = min(row0 + kBM, p.T);
-            for (int i = 0; i < sp.n; ++i) {
-                const int g = sp.g[i];
-                const bool mine = pos >= max(seg_cache[g], row0) && pos < min(seg_cache[g + 1], row1);
-                const float sc = mine ? snap.scale[sp.slot[i]] : 0.f;
-                __nv_bfloat16* out = p.u_out + ((size_t)(sp.m + g) * kBM + q * 32 + lane) * kRankPad;
+            int my_slot = -1;
+            if (pos < p.T) {
+                if (by_segment) {
+                    int lo = 0, hi = p.rows.G;
+                    while (lo < hi) { const int mid = (lo + hi) >> 1; if (seg_cache[mid + 1] > pos) hi = mid; else lo = mid + 1; }
+                    if (lo < p.rows.G) my_slot = slot_cache[lo];
+                } else my_slot = p.rows.rows[pos];
+            }
+#pragma unroll 1
+            for (int i0 = 0; i0 < sp.n; i0 += 2) {   // two chunks, 32 columns at a time
+                uint32_t r[32];
+                tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + kChunk * i0), r);
+                tmem_ld_wait();
 #pragma unroll
-                for (int c = 0; c < 2; ++c) {
-                    uint32_t r[32];
-                    tmem_ld_32x32(tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN + 64 * i + 32 * c), r);
-                    tmem_ld_wait();
+                for (int ii = 0; ii < 2; ++ii) {
+                    const int i = i0 + ii;
+                    if (i >= sp.n) continue;
+                    const bool mine = my_slot == sp.slot[i];
+                    const float sc = snap.scale[sp.slot[i]];
+                    __nv_bfloat16* out = const_cast<__nv_bfloat16*>(p.part[0].u) + ((size_t)sp.m * p.part[0].cap + sp.first + i) * (kTileM * kChunk) + chunk_elem(q * 32 + lane, 0);
 #pragma unroll
-                    for (int j = 0; j < 4; ++j) {
+                    for (int j = 0; j < 2; ++j) {
+                        const int b = ii * 16 + j * 8;
                         uint4 v;
-                        v.x = pack_bf16(__uint_as_float(r[8 * j + 0]) * sc, __uint_as_float(r[8 * j + 1]) * sc);
-                        v.y = pack_bf16(__uint_as_float(r[8 * j + 2]) * sc, __uint_as_float(r[8 * j + 3]) * sc);
-                        v.z = pack_bf16(__uint_as_float(r[8 * j + 4]) * sc, __uint_as_float(r[8 * j + 5]) * sc);
-                        v.w = pack_bf16(__uint_as_float(r[8 * j + 6]) * sc, __uint_as_float(r[8 * j + 7]) * sc);
-                        if (!mine) v = make_uint4(0, 0, 0, 0);   // (0 * garbage may be a NaN)
-                        *reinterpret_cast<uint4*>(out + c * 32 + j * 8) = v;
+                        v.x = pack_bf16(__uint_as_float(r[b + 0]) * sc, __uint_as_float(r[b + 1]) * sc);
+                        v.y = pack_bf16(__uint_as_float(r[b + 2]) * sc, __uint_as_float(r[b + 3]) * sc);
+                        v.z = pack_bf16(__uint_as_float(r[b + 4]) * sc, __uint_as_float(r[b + 5]) * sc);
+                        v.w = pack_bf16(__uint_as_float(r[b + 6]) * sc, __uint_as_float(r[b + 7]) * sc);
+                        if (!mine) v = make_uint4(0, 0, 0, 0);
+                        *reinterpret_cast<uint4*>(out + j * 64) = v;
                     }
                 }
             }
@@ -595,9 +727,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
             acc ^= 1;
         }
         for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
-            const int m = tile % p.num_m, n = tile / p.num_m;
+            const GemmPart& pt = p.part[part_of(p, tile)];
+            const int m = (tile - pt.tile0) % p.num_m, n = (tile - pt.tile0) / p.num_m;
             const int row_base = m * kBM + q * 32;
-            const bool scatter = p.perm != nullptr && !(p.tile_identity && __ldg(p.tile_identity + m));
             for (int pass = 0; pass < (dual ? 2 : 1) && ok; ++pass) {
                 uint32_t& fph = acc ? full_ph1 : full_ph0;
                 ok = mbar_wait_warp(smem_u32(&ctrl->tmem_full[acc]), fph, abort);
@@ -605,7 +737,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
                 fph ^= 1u;
                 tc_fence_after();
                 const bool last_pass = pass == (dual ? 1 : 0);
-                __nv_bfloat16* yout = pass == 0 ? p.y : p.y2;
                 const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
 #pragma unroll 1
                 for (int c = 0; c < BN / kEpiChunkCols; ++c) {
@@ -620,7 +751,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
                         if (lane == 0) mbar_arrive(smem_u32(last_pass ? &ctrl->tmem_empty[acc] : &ctrl->tmem_read1[acc]));
                     }
                     const int col0 = n * BN + c * kEpiChunkCols;
-                    if (col0 >= p.N || row_base >= p.T) continue;   // nothing of this chunk is inside y
+                    if (col0 >= pt.N || row_base >= p.T) continue;   // nothing of this chunk is inside y
                     // the buffer we are about to overwrite must have been read by its earlier store
                     if (lane == 0) tma_store_wait_read<1>();
                     __syncwarp();
@@ -637,32 +768,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
                         const int phys = j ^ ((lane >> 1) & 3);
                         *reinterpret_cast<uint4*>(bp + lane * 64 + phys * 16) = v;
                     }
-                    if (!scatter) {
-                        fence_proxy_async_smem();
-                        __syncwarp();
-                        if (lane == 0) {
-                            // two call sites on purpose: each names its tensor map as a kernel-parameter constant
-                            if (pass == 0) tma_store_2d(&tmap_y, ba, col0, row_base);
-                            else tma_store_2d(&tmap_y2, ba, col0, row_base);
-                            tma_store_commit();
-                        }
-                    } else {
-                        __syncwarp();
-                        // scatter: 4 lanes write one 64-byte row piece; 8 rows per pass
-#pragma unroll
-                        for (int sp = 0; sp < 4; ++sp) {
-                            const int rr = sp * 8 + (lane >> 2), j = lane & 3;
-                            const int pos = row_base + rr;
-                            if (pos < p.T && col0 + j * 8 < p.N) {
-                                const int row = __ldg(p.perm + pos);
-                                if (row >= 0 && row < p.T) {
-                                    const int phys = j ^ ((rr >> 1) & 3);
-                                    uint4 v = *reinterpret_cast<const uint4*>(bp + rr * 64 + phys * 16);
-                                    *reinterpret_cast<uint4*>(yout + (size_t)row * p.N + col0 + j * 8) = v;
-                                }
-                            }
-                        }
-                        __syncwarp();
+                    fence_proxy_async_smem();
+                    __syncwarp();
+                    if (lane == 0) {
+                        if (pass == 0) tma_store_2d(&pt.y, ba, col0, row_base);
+                        else tma_store_2d(&p.y2, ba, col0, row_base);
+                        tma_store_commit();
                     }
                     buf ^= 1;
                 }
@@ -674,6 +785,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
 
     __syncthreads();
     if (threadIdx.x == 0 && ctrl->abort) atomicOr(p.status, LML_FLAG_TIMEOUT);
+    if (threadIdx.x == 0) leave_early_start(p);
     if (threadIdx.x == 0 && p.fused) {
         // the last CTA to finish moves the table's epoch on: the flags of this call mean nothing to the next one
         __threadfence();
@@ -691,7 +803,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
 // ---- split-K variant for few tokens ---------------------------------------------------------------------
 // With a few hundred tokens or fewer the layer is bound by the read of W0, and 128 x 256 tiles give far
 // fewer CTAs than the machine has SMs.  Here a cluster of S CTAs shares one tile: CTA r multiplies its
-// share of the k-blocks (and of the tile's LoRA pieces, which are just more K) into its own TMEM
+// share of the k-blocks (and of the tile's LoRA chunks, which are just more K) into its own TMEM
 // accumulator, so S times as many SMs stream W0.  The partial sums are then exchanged through
 // distributed shared memory: the tile's eight 32-column chunks are dealt out to the CTAs, every CTA
 // writes each chunk of its partial sums into the owner's (by then idle) stage memory, and the owner adds
@@ -701,16 +813,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(
 // side-band word.
 constexpr int kSplitMaxS = 8;
 
-__device__ __forceinline__ void st_shared_cluster_v4(uint32_t cluster_addr, uint32_t a, uint32_t b, uint32_t c, uint32_t d)
-{
-    asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(cluster_addr), "r"(a), "r"(b), "r"(c), "r"(d) : "memory");
-}
-
 template <int BN>
-__global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel(
-    const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_x0,
-    const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_u,
-    const __grid_constant__ CUtensorMap tmap_b, const __grid_constant__ SlotSnapshot snap, const GemmParams p)
+__global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel(const __grid_constant__ GemmParams p)
 {
     using Cfg = GemmCfg<BN>;
     constexpr int kSplitChunks = BN / kEpiChunkCols;   // 32-column chunks of the tile: 4 or 8
@@ -718,48 +822,36 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
     const uint32_t raw_addr = smem_u32(smem_raw);
     const uint32_t tiles_addr = (raw_addr + 1023u) & ~1023u;
     uint8_t* tiles_ptr = smem_raw + (tiles_addr - raw_addr);
-    uint8_t* epi_ptr = tiles_ptr + Cfg::kStages * Cfg::kStageBytes;
-    GemmCtrl* ctrl = reinterpret_cast<GemmCtrl*>(epi_ptr + Cfg::kEpiBytes);
-    int32_t* seg_cache = reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(ctrl) + 256);
-    int8_t* slot_cache = reinterpret_cast<int8_t*>(seg_cache + kSegCache + 1);
-    int8_t* slot_cache2 = slot_cache + kSegCache;   // dual form: the second slot per segment
+    GemmCtrl* ctrl = reinterpret_cast<GemmCtrl*>(tiles_ptr + p.stages * Cfg::kStageBytes);
+    uint32_t* lists = reinterpret_cast<uint32_t*>(reinterpret_cast<uint8_t*>(ctrl) + 256);   // this CTA's chunks, per binding
     // Dual form (two bindings of the same segments, two outputs): the k-blocks pass through shared memory once and
     // are multiplied into two accumulators (with few tokens the tensor cores have time to spare: the kernel is
     // bound by the read of W0); each binding's pieces go to its own accumulator, and the exchange runs twice.
-    const bool dual = p.slot_ids2 != nullptr;
+    const bool dual = p.u2 != nullptr;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int S = (int)gridDim.x, rank = (int)blockIdx.x;   // the cluster spans the grid's x dimension
-    const int n = (int)blockIdx.y;
     const int m = (int)blockIdx.z;
+    // (column tiles are numbered through the projections; tile0 counts row tiles too)
+    const GemmPart& pt = p.part[part_of(p, (int)blockIdx.y * p.num_m)];
+    const int n = (int)blockIdx.y - pt.tile0 / p.num_m;
     const int num_kb = (p.K + kBK - 1) / kBK;
-    const bool seg_cached = p.G <= kSegCache;
     // chunks of the tile's 256 columns that CTA r reduces: [first(r), first(r + 1))
     auto first_chunk = [&](int r) { return r * kSplitChunks / S; };
     const int cpr = (kSplitChunks + S - 1) / S;   // most chunks any CTA owns
 
     if (threadIdx.x == 0) {
-        for (int s = 0; s < Cfg::kStages; ++s) {
+        for (int s = 0; s < p.stages; ++s) {
             mbar_init(smem_u32(&ctrl->full[s]), 1);
             mbar_init(smem_u32(&ctrl->empty[s]), 1);
         }
         mbar_init(smem_u32(&ctrl->tmem_full[0]), 1);
+        mbar_init(smem_u32(&ctrl->plan_full), 1);
         ctrl->abort = 0;
         fence_mbar_init();
     }
     if (warp == 0 && lane == 0) {
-        prefetch_tmap(&tmap_x0); prefetch_tmap(&tmap_x); prefetch_tmap(&tmap_w); prefetch_tmap(&tmap_u); prefetch_tmap(&tmap_b);
-    }
-    if (seg_cached && p.G > 0) {
-        for (int g = threadIdx.x; g <= p.G; g += kGemmThreads) seg_cache[g] = __ldg(p.seg_offsets + g);
-        for (int g = threadIdx.x; g < p.G; g += kGemmThreads) {
-            int s = __ldg(p.slot_ids + g);
-            slot_cache[g] = (int8_t)((s >= 0 && s < snap.max_slots && snap.rank[s] > 0) ? s : -1);
-            if (dual) {
-                const int s2 = __ldg(p.slot_ids2 + g);
-                slot_cache2[g] = (int8_t)((s2 >= 0 && s2 < snap.max_slots && snap.rank[s2] > 0) ? s2 : -1);
-            }
-        }
+        prefetch_tmap(&p.x); prefetch_tmap(&pt.w);
     }
     if (warp == 1) tmem_alloc(smem_u32(&ctrl->tmem_base), dual ? 2 * BN : BN);
     tc_fence_before();
@@ -767,7 +859,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
     tc_fence_after();
     const uint32_t tmem_base = ctrl->tmem_base;
     volatile int* abort = &ctrl->abort;
-    if (p.G == 0) {   // no shrink kernel ran before this one in the call: wait for foreign work here
+    if (!p.lora) {   // no launch of this call came before this one: wait for foreign work here
         grid_dependency_wait();
         grid_launch_dependents();
     }
@@ -779,70 +871,55 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
             uint32_t phase = 0;
             bool ok = true;
             auto acquire = [&]() -> bool { return mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, abort); };
-            auto advance = [&]() { if (++stage == Cfg::kStages) { stage = 0; phase ^= 1u; } };
-            const int row0 = m * kBM, row1 = min(row0 + kBM, p.T);
-            const bool in_place = p.tile_identity && __ldg(p.tile_identity + m);
+            auto advance = [&]() { if (++stage == p.stages) { stage = 0; phase ^= 1u; } };
+            const int row0 = m * kBM;
             const int kb0 = rank * num_kb / S, kb1 = (rank + 1) * num_kb / S;
-            auto piece_slot = [&](int g, bool second) -> int {
-                int s0, s1, s;
-                if (seg_cached) { s0 = seg_cache[g]; s1 = seg_cache[g + 1]; s = second ? slot_cache2[g] : slot_cache[g]; }
-                else {
-                    s0 = __ldg(p.seg_offsets + g); s1 = __ldg(p.seg_offsets + g + 1);
-                    s = __ldg((second ? p.slot_ids2 : p.slot_ids) + g);
-                    if (slot_rank(snap, s) == 0) s = -1;
+            // base k-blocks first: they do not depend on the launch that precedes this one
+            int ahead = 0;   // early start: k-blocks whose W0 has been asked for already
+            if (p.x_flag) {
+                ahead = min(p.stages, kb1 - kb0);
+                for (int i = 0; i < ahead; ++i) {
+                    const uint32_t bar = smem_u32(&ctrl->full[i]);
+                    mbar_expect_tx(bar, Cfg::kBBytes);
+                    tma_load_2d(tiles_addr + i * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, (kb0 + i) * kBK, n * BN);
                 }
-                return min(s1, row1) <= max(s0, row0) ? -1 : s;
-            };
-            // base k-blocks first: they do not depend on the shrink kernel that precedes this one
+                ok = wait_x(p, abort);
+                if (!ok) drain_ahead(ctrl, ahead);
+            }
             for (int kb = kb0; kb < kb1 && ok; ++kb) {
                 ok = acquire();
                 if (!ok) break;
                 const uint32_t a_dst = tiles_addr + stage * Cfg::kStageBytes;
                 const uint32_t bar = smem_u32(&ctrl->full[stage]);
                 ctrl->stage_info[stage] = 4u | (dual ? kStageBoth : 0u);
-                mbar_arrive_expect_tx(bar, Cfg::kStageBytes);
-                if (in_place) tma_load_2d(a_dst, &tmap_x0, bar, kb * kBK, row0);
-                else tma_load_2d(a_dst, &tmap_x, bar, kb * kBK, row0);
-                tma_load_2d(a_dst + Cfg::kABytes, &tmap_w, bar, kb * kBK, n * BN);
+                const bool have_w = kb - kb0 < ahead;
+                mbar_arrive_expect_tx(bar, (uint32_t)(p.x_bytes + (have_w ? 0 : Cfg::kBBytes)));
+                tma_load_2d(a_dst, &p.x, bar, kb * kBK, row0);
+                if (!have_w) tma_load_2d(a_dst + Cfg::kABytes, &pt.w, bar, kb * kBK, n * BN);
                 advance();
             }
-            // this CTA's share of the tile's LoRA pieces
-            bool lora = false;
-            if (p.G > 0) {
+            // This CTA's share of the tile's LoRA chunks: chunk c of slot s goes to CTA (s + c) mod S.  Which CTA adds a
+            // row's LoRA term depends only on the row's own slot, so a row's bits do not change with what other rows
+            // are bound to.
+            if (p.lora && ok) {
+                ok = mbar_wait(smem_u32(&ctrl->plan_full), 0u, abort);   // (warp 2 has waited for that launch)
                 grid_dependency_wait();
-                grid_launch_dependents();
-                lora = p.plan->lora_ok != 0;
-            }
-            if (lora && ok) {
-                int g_first, g_end;
-                if (seg_cached) {
-                    int lo = 0, hi = p.G;
-                    while (lo < hi) { int mid = (lo + hi) >> 1; if (seg_cache[mid + 1] > row0) hi = mid; else lo = mid + 1; }
-                    g_first = lo;
-                    g_end = g_first;
-                    while (g_end < p.G && seg_cache[g_end] < row1) ++g_end;
-                } else {
-                    g_first = seg_upper(p.seg_offsets, p.G, row0);
-                    g_end = g_first;
-                    while (g_end < p.G && __ldg(p.seg_offsets + g_end) < row1) ++g_end;
-                }
-                // segment g's piece goes to CTA g mod S: which CTA adds a row's LoRA term depends only on the
-                // row's own segment, so a row's bits do not change with what other segments are bound to
-                for (int side = 0; side < (dual ? 2 : 1) && ok; ++side)
-                    for (int g = g_first; g < g_end && ok; ++g) {
-                        if (g % S != rank) continue;
-                        const int s = piece_slot(g, side == 1);
-                        if (s < 0) continue;
+                for (int side = 0; side < (dual ? 2 : 1) && ok; ++side) {
+                    const __nv_bfloat16* u = side ? p.u2 : pt.u;
+                    const uint32_t* list = lists + side * kMaxChunks;
+                    const int count = ctrl->listed[side];
+                    for (int i = 0; i < count && ok; i += 4) {
                         ok = acquire();
                         if (!ok) break;
-                        const uint32_t a_dst = tiles_addr + stage * Cfg::kStageBytes;
-                        const uint32_t bar = smem_u32(&ctrl->full[stage]);
-                        ctrl->stage_info[stage] = (uint32_t)((snap.rank[s] + 15) >> 4) | (side ? kStageAcc1 : 0u);
-                        mbar_arrive_expect_tx(bar, Cfg::kStageBytes);
-                        tma_load_2d(a_dst, &tmap_u, bar, 0, side * p.u_set_rows + (m + g) * kBM);   // (the second binding's u blocks: the second set)
-                        tma_load_3d(a_dst + Cfg::kABytes, &tmap_b, bar, 0, n * BN, s);
+                        const uint32_t a_dst = tiles_addr + stage * Cfg::kStageBytes, bar = smem_u32(&ctrl->full[stage]);
+                        const int nk = min(4, count - i);
+                        for (int k = 0; k < nk; ++k)
+                            load_chunk<BN>(pt, u, m, n, list[i + k] & 0xffffu, (int)(list[i + k] >> 16), k, a_dst, a_dst + Cfg::kABytes, bar);
+                        ctrl->stage_info[stage] = (uint32_t)nk | kStageChunks | (side ? kStageAcc1 : 0u);
+                        mbar_arrive(bar);
                         advance();
                     }
+                }
             }
             if (ok) {   // end of this CTA's K: a stage without operands
                 ok = acquire();
@@ -853,7 +930,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
                 }
             }
             // leave the role only after every load has landed and been consumed
-            for (int i = 0; i < Cfg::kStages && ok; ++i) { ok = acquire(); advance(); }
+            for (int i = 0; i < p.stages && ok; ++i) { ok = acquire(); advance(); }
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
@@ -868,26 +945,28 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
                 const uint32_t info = ctrl->stage_info[stage];
                 more = (info & kStageCommit) == 0;
                 const int ksteps = (int)(info & 0xffu);
+                const bool chunks = (info & kStageChunks) != 0;
                 const uint32_t a_addr = tiles_addr + stage * Cfg::kStageBytes;
-                const uint64_t adesc = umma_desc_k128(a_addr);
-                const uint64_t bdesc = umma_desc_k128(a_addr + Cfg::kABytes);
+                const uint64_t adesc = chunks ? umma_desc_k16(a_addr) : umma_desc_k128(a_addr);
+                const uint64_t bdesc = chunks ? umma_desc_k16(a_addr + Cfg::kABytes) : umma_desc_k128(a_addr + Cfg::kABytes);
+                const uint64_t astep = chunks ? kUBlockBytes / 16 : 2, bstep = chunks ? BN * kChunk * 2 / 16 : 2;
                 tc_fence_after();
                 if ((info & kStageAcc1) == 0) {
 #pragma unroll 4
                     for (int k = 0; k < ksteps; ++k) {
-                        umma_bf16(tmem_base, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, accumulate);
+                        umma_bf16(tmem_base, adesc + (uint64_t)k * astep, bdesc + (uint64_t)k * bstep, idesc, accumulate);
                         accumulate = 1;
                     }
                 }
                 if (info & (kStageAcc1 | kStageBoth)) {   // the second binding's accumulator
 #pragma unroll 4
                     for (int k = 0; k < ksteps; ++k) {
-                        umma_bf16(tmem_base + (uint32_t)BN, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc, accumulate2);
+                        umma_bf16(tmem_base + (uint32_t)BN, adesc + (uint64_t)k * astep, bdesc + (uint64_t)k * bstep, idesc, accumulate2);
                         accumulate2 = 1;
                     }
                 }
                 umma_commit(smem_u32(&ctrl->empty[stage]));
-                if (++stage == Cfg::kStages) { stage = 0; phase ^= 1u; }
+                if (++stage == p.stages) { stage = 0; phase ^= 1u; }
             }
             if (ok) umma_commit(smem_u32(&ctrl->tmem_full[0]));
             ctrl->pad[0] = (int32_t)accumulate;    // 0: this CTA had no K at all, its accumulator holds nothing
@@ -898,13 +977,24 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
     __syncwarp();   // (the producer's and the MMA issuer's other lanes waited here: the cluster barrier wants whole warps)
     bool ok = true;
     if (warp >= 2) {
+        if (p.lora && warp == 2) {   // nothing else to do yet: this CTA's share of the tile's chunks, as soon as they are known
+            if (p.x_flag) prefetch_b<BN>(pt, n, lane, rank, S);
+            grid_dependency_wait();
+            grid_launch_dependents();
+            for (int side = 0; side < (dual ? 2 : 1); ++side) {
+                const int c = list_chunks(pt.plan + m, side ? kChunkSecond : kChunkFirst, rank, S, lane, lists + side * kMaxChunks);
+                if (lane == 0) ctrl->listed[side] = c;
+            }
+            __syncwarp();
+            if (lane == 0) mbar_arrive(smem_u32(&ctrl->plan_full));
+        }
         ok = mbar_wait_warp(smem_u32(&ctrl->tmem_full[0]), 0u, abort);   // this CTA's MMAs are complete: so are its loads
         tc_fence_after();
     }
     const int q = warp & 3;   // TMEM lane quarter an epilogue warp may read
     const int row = q * 32 + lane;
     for (int o = 0; o < (dual ? 2 : 1); ++o) {   // one exchange per output
-    __nv_bfloat16* const yout = o ? p.y2 : p.y;
+    __nv_bfloat16* const yout = o ? p.y2_ptr : pt.y_ptr;
     cluster_sync_all();   // every CTA of the cluster is done with its stage memory (and with the exchange before this one)
     if (warp >= 2 && ok) {
         const bool have = ctrl->pad[o] != 0;
@@ -933,10 +1023,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
     cluster_sync_all();   // all contributions have arrived
     if (warp >= 2 && ok) {
         const int pos = m * kBM + row;
-        const bool scatter = p.perm != nullptr && !(p.tile_identity && __ldg(p.tile_identity + m));
-        int out_row = pos;
-        if (pos < p.T && scatter) out_row = __ldg(p.perm + pos);
-        const bool row_ok = pos < p.T && out_row >= 0 && out_row < p.T;
+        const bool row_ok = pos < p.T;
         const int c_first = first_chunk(rank), c_end = first_chunk(rank + 1);
 #pragma unroll 1
         for (int c = c_first; c < c_end; ++c) {
@@ -955,19 +1042,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
             if (!row_ok) continue;
 #pragma unroll
             for (int j = 0; j < 4; ++j) {
-                if (col0 + j * 8 >= p.N) continue;
+                if (col0 + j * 8 >= pt.N) continue;
                 uint4 v;
                 v.x = pack_bf16(acc[8 * j + 0], acc[8 * j + 1]);
                 v.y = pack_bf16(acc[8 * j + 2], acc[8 * j + 3]);
                 v.z = pack_bf16(acc[8 * j + 4], acc[8 * j + 5]);
                 v.w = pack_bf16(acc[8 * j + 6], acc[8 * j + 7]);
-                *reinterpret_cast<uint4*>(yout + (size_t)out_row * p.N + col0 + j * 8) = v;
+                *reinterpret_cast<uint4*>(yout + (size_t)pos * pt.N + col0 + j * 8) = v;
             }
         }
     }
     }   // outputs
     __syncthreads();
     if (threadIdx.x == 0 && ctrl->abort) atomicOr(p.status, LML_FLAG_TIMEOUT);
+    if (threadIdx.x == 0) leave_early_start(p);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, dual ? 2 * BN : BN);
@@ -1030,35 +1118,24 @@ bool encode_tmap_3d(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, 
 
 cudaError_t gemm_sm100_init(int /*device*/)
 {
-    cudaError_t e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    cudaError_t e = cudaFuncSetAttribute(lora_gemm_sm100_splitk_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         GemmCfg<64>::split_smem(GemmCfg<64>::kStages));
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<64>::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          GemmCfg<256>::kSmemBytes);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(lora_gemm_sm100_splitk_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             GemmCfg<256>::kSmemBytes);
+                             GemmCfg<256>::split_smem(GemmCfg<256>::kStages));
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(lora_gemm_sm100_splitk_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             GemmCfg<128>::kSmemBytes);
+                             GemmCfg<128>::split_smem(GemmCfg<128>::kStages));
     if (e != cudaSuccess) return e;
     return cudaFuncSetAttribute(lora_gemm_sm100_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 GemmCfg<128>::kSmemBytes);
 }
 
-int gemm_pick_bn(int T, int d_out, int num_sms)
-{
-    const int num_m = (T + kBM - 1) / kBM;
-    const int tiles256 = num_m * ((d_out + 255) / 256), tiles128 = num_m * ((d_out + 127) / 128);
-    // Rounds of tiles over the SMs times the cost of a tile: a 128-column tile takes about 0.82 of the
-    // time of a 256-column one (measured: the narrow kernel needs 1.64 times as long for the same work).
-    const float t256 = (float)((tiles256 + num_sms - 1) / num_sms);
-    const float t128 = 0.82f * (float)((tiles128 + num_sms - 1) / num_sms);
-    return t256 <= t128 ? 256 : 128;
-}
-
-// Split-K choice for few tokens: tile width and how many CTAs share a tile (split 0: do not use it).
-// It pays while the 128-column tiles are too few to keep most SMs busy.  Of the shapes whose clusters all
-// fit the machine at once, take the one with the most CTAs, and among equals the smaller cluster (less
-// to exchange); every CTA keeps at least two k-blocks, and the exchange area must fit the stage memory.
-struct SplitChoice { int bn, split; };
 // The table's override (LML_GEMM_SPLIT, read once when the table is created; a test knob): "<bn>x<split>"
 // forces that shape, 0 switches the split-K kernel off.  Returns false when the variable is not set.
 bool gemm_split_override(int* bn_out, int* split_out)
@@ -1067,7 +1144,7 @@ bool gemm_split_override(int* bn_out, int* split_out)
     const char* e = getenv("LML_GEMM_SPLIT");
     if (!e) return false;
     int bn = 0, sp = 0;
-    if (sscanf(e, "%dx%d", &bn, &sp) == 2 && (bn == 128 || bn == 256) && sp >= 2 && sp <= kSplitMaxS &&
+    if (sscanf(e, "%dx%d", &bn, &sp) == 2 && (bn == 64 || bn == 128 || bn == 256) && sp >= 1 && sp <= kSplitMaxS &&
         sp * ((bn / 32 + sp - 1) / sp) * 16384 <= GemmCfg<128>::kStages * GemmCfg<128>::kStageBytes) {
         *bn_out = bn; *split_out = sp;
     } else {
@@ -1076,42 +1153,71 @@ bool gemm_split_override(int* bn_out, int* split_out)
     return true;
 }
 
-static SplitChoice gemm_pick_split(int T, int d_in, int d_out, int num_sms, int forced_bn, int forced_split)
+static int gemm_stages(int bn) { return bn == 256 ? GemmCfg<256>::kStages : (bn == 128 ? GemmCfg<128>::kStages : GemmCfg<64>::kStages); }
+static int gemm_stages_short(int bn)
 {
-    static int max_clusters[2][kSplitMaxS + 1];
+    return bn == 256 ? GemmCfg<256>::kSplitStagesShort : (bn == 128 ? GemmCfg<128>::kSplitStagesShort : GemmCfg<64>::kSplitStagesShort);
+}
+static int gemm_stage_bytes(int bn) { return (kBM + bn) * kBK * 2; }
+static int gemm_exchange_bytes(int bn, int split) { return split * ((bn / 32 + split - 1) / split) * 16384; }
+
+// The shape of a call: the smallest estimated time (us) over whole-K tiles of three widths and over the splits that the
+// machine can hold.  More tiles than SMs: rounds of tiles times the tensor time of a k-block.  Fewer: a CTA's k-blocks come
+// through its ring at one round of the ring per trip to memory, 1.5 us while W0 streams (measured at 128 tokens, us per
+// k-block: 256 columns whole-K 0.37, 128 columns 0.265; with the short rings of the split-K kernel 0.52 and 0.40).
+GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, int num_sms, int split_bn, int split_s)
+{
+    static int max_clusters[3][kSplitMaxS + 1];   // for 64, 128 and 256 columns
     static std::once_flag probed;
-    if (forced_bn >= 0) return {forced_bn, forced_split};
     std::call_once(probed, [&]() {   // clusters of each size that can be resident together
-        for (int w = 0; w < 2; ++w)
+        for (int w = 0; w < 3; ++w)
             for (int S = 2; S <= kSplitMaxS; ++S) {
                 cudaLaunchConfig_t cfg = {};
                 cfg.gridDim = dim3(S, num_sms / S, 1);
                 cfg.blockDim = dim3(kGemmThreads);
-                cfg.dynamicSmemBytes = w ? GemmCfg<256>::kSmemBytes : GemmCfg<128>::kSmemBytes;
+                cfg.dynamicSmemBytes = w == 2 ? GemmCfg<256>::split_smem(GemmCfg<256>::kStages)
+                                              : (w == 1 ? GemmCfg<128>::split_smem(GemmCfg<128>::kStages) : GemmCfg<64>::split_smem(GemmCfg<64>::kStages));
                 cudaLaunchAttribute attr[1];
                 attr[0].id = cudaLaunchAttributeClusterDimension;
                 attr[0].val.clusterDim.x = S; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
                 cfg.attrs = attr; cfg.numAttrs = 1;
                 int n = 0;
-                cudaError_t e = w ? cudaOccupancyMaxActiveClusters(&n, lora_gemm_sm100_splitk_kernel<256>, &cfg)
-                                  : cudaOccupancyMaxActiveClusters(&n, lora_gemm_sm100_splitk_kernel<128>, &cfg);
+                cudaError_t e = w == 2 ? cudaOccupancyMaxActiveClusters(&n, lora_gemm_sm100_splitk_kernel<256>, &cfg)
+                                       : (w == 1 ? cudaOccupancyMaxActiveClusters(&n, lora_gemm_sm100_splitk_kernel<128>, &cfg)
+                                                 : cudaOccupancyMaxActiveClusters(&n, lora_gemm_sm100_splitk_kernel<64>, &cfg));
                 if (e != cudaSuccess) { n = 0; (void)cudaGetLastError(); }
                 max_clusters[w][S] = n;
             }
     });
     const int num_m = (T + kBM - 1) / kBM, num_kb = (d_in + kBK - 1) / kBK;
-    if (num_m * ((d_out + 127) / 128) * 4 > num_sms * 3) return {0, 0};   // enough tiles without splitting
-    SplitChoice best = {0, 0};
-    int best_ctas = 0;
-    for (int S = 2; S <= kSplitMaxS; ++S)
-        for (int w = 0; w < 2; ++w) {
-            const int bn = w ? 256 : 128;
-            const int tiles = num_m * ((d_out + bn - 1) / bn);
-            const int cpr = (bn / 32 + S - 1) / S;
-            if (tiles > max_clusters[w][S] || num_kb < 2 * S) continue;
-            if (S * cpr * 16384 > GemmCfg<128>::kStages * GemmCfg<128>::kStageBytes) continue;
-            if (tiles * S > best_ctas) { best_ctas = tiles * S; best = {bn, S}; }
+    auto tiles_of = [&](int bn) {
+        int tiles = 0;
+        for (int p = 0; p < P; ++p) tiles += num_m * ((d_outs[p] + bn - 1) / bn);
+        return tiles;
+    };
+    if (split_bn > 0) return {split_bn, split_s, tiles_of(split_bn) * split_s};
+    const bool crowded = tiles_of(256) > num_sms;
+    GemmShape best = {256, 1, tiles_of(256)};
+    float best_us = 1e30f;
+    for (int w = 2; w >= (crowded ? 1 : 0); --w) {
+        const int bn = 64 << w, tiles = tiles_of(bn);
+        for (int S = 1; S <= (split_bn == 0 ? 1 : kSplitMaxS); ++S) {
+            if (S > 1 && (max_clusters[w][S] <= 0 || num_kb < 8 * S || gemm_exchange_bytes(bn, S) > gemm_stages(bn) * gemm_stage_bytes(bn))) continue;
+            // (a cluster needs its CTAs on one part of the chip: with the last places taken by other work it waits)
+            const int fit = S > 1 ? max_clusters[w][S] - (S > 3 ? 1 : 0) : num_sms;
+            if (S > 1 && tiles > fit) continue;
+            const int waves = (tiles + fit - 1) / fit;
+            float us;
+            if (crowded) {
+                us = (float)(waves * num_kb) * (w == 2 ? 0.31f : 0.254f);
+            } else {
+                const int stages = S > 1 && tiles * S > num_sms - 40 ? gemm_stages_short(bn) : gemm_stages(bn);
+                us = (w == 2 ? 12.5f : (w == 1 ? 10.f : 8.f)) + (S > 1 ? 1.f : 0.f) +
+                     (float)waves * (float)((num_kb + S - 1) / S) * 1.55f / (float)stages;
+            }
+            if (us < best_us * 0.999f) { best_us = us; best = {bn, S, tiles * S}; }
         }
+    }
     return best;
 }
 
@@ -1138,87 +1244,87 @@ bool TmapCache::get_2d(CUtensorMap* out, const void* base, uint64_t inner, uint6
     return true;
 }
 
-// Whether the shrink can run inside the GEMM kernel for this call: whole-K tiles, the segment arrays in the
-// kernel's shared-memory cache, a flag per row tile in the table's array, and no CTA with more shrink passes
-// than its plan holds (worst case: every segment touches every one of its row tiles).
-bool gemm_can_fuse_shrink(int T, int d_in, int d_out, int G, int num_sms, int split_bn, int split_s)
+// Whether the shrink can run inside the GEMM kernel for this call: whole-K tiles, few enough row tiles for its tables, and
+// the passes on CTAs with a tile's time to spare.  A shrink pass takes about as long as an output tile, whatever its width.
+// It pays where some CTAs have that time and the others do not reach their first chunks before it is over: 256-column
+// tiles in more than one wave, and few enough passes (every segment boundary inside a row tile can add one) that no CTA gets two.
+bool gemm_can_fuse_shrink(const GemmShape& shape, int T, int d_out, int G, bool in_segment_order, int cap, int num_sms)
 {
-    if (G <= 0 || G > kSegCache) return false;
-    if (gemm_pick_split(T, d_in, d_out, num_sms, split_bn, split_s).split) return false;
-    // A shrink pass takes about as long as an output tile, whatever its width.  It pays where some CTAs have a
-    // tile's time to spare and the others do not reach their first pieces before it is over: 256-column tiles in
-    // more than one wave, and few enough passes that no CTA gets two.
-    if (gemm_pick_bn(T, d_out, num_sms) != 256) return false;
+    if (G <= 0 || (in_segment_order && G > kBindSegs)) return false;
+    if (shape.split != 1 || shape.bn != 256) return false;
     const int num_m = (T + kBM - 1) / kBM, num_n = (d_out + 255) / 256;
     if (num_m > kFuseTilesInKernel || num_m * num_n <= num_sms) return false;
-    const int worst_passes = num_m + G;   // (every segment boundary inside a row tile adds a piece)
+    int worst_passes = num_m * ((cap + kShrChunks - 1) / kShrChunks);
+    if (in_segment_order && num_m + G < worst_passes) worst_passes = num_m + G;
     return worst_passes <= num_sms / 2;
 }
 
-cudaError_t launch_gemm_sm100(const Arena& ar, const SlotSnapshot& snap, const CUtensorMap& tmap_B256,
-                              const CUtensorMap& tmap_B128, const CUtensorMap& tmap_A, TmapCache* cache, const GemmArgs& a,
-                              cudaStream_t stream)
+cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* caches, const GemmArgs& a, cudaStream_t stream)
 {
-    const bool dual = a.slot_ids2 != nullptr;
-    if (dual && (a.G <= 0 || !a.y2)) return cudaErrorInvalidValue;
-    const SplitChoice sc = gemm_pick_split(a.T, a.d_in, a.d_out, a.num_sms, a.split_bn, a.split_s);
-    const int split = sc.split;
-    const int bn = split ? sc.bn : gemm_pick_bn(a.T, a.d_out, a.num_sms);
-    const int num_m = (a.T + kBM - 1) / kBM;
-    const int num_n = (a.d_out + bn - 1) / bn;
-    TmapCache local;   // (a call without a table-owned cache encodes its maps afresh)
-    TmapCache* tc = cache ? cache : &local;
-    CUtensorMap tx, tx0, tw, tu, ty, ty2;
-    const CUtensorMap& tb = bn == 256 ? tmap_B256 : tmap_B128;
-    const uint64_t u_set_rows = (uint64_t)(num_m + (a.G > 0 ? a.G : 1)) * kBM;
-    const uint64_t u_rows = u_set_rows * (dual ? 3 : 1);
-    const uint64_t xs = (uint64_t)a.d_in * 2, ys = (uint64_t)a.d_out * 2;
-    if (!tc->get_2d(&tx, a.x, (uint64_t)a.d_in, (uint64_t)a.T, xs, kBK, kBM)) return cudaErrorInvalidValue;
-    if (!tc->get_2d(&tx0, a.x_in_place ? a.x_in_place : a.x, (uint64_t)a.d_in, (uint64_t)a.T, xs, kBK, kBM)) return cudaErrorInvalidValue;
-    if (!tc->get_2d(&tw, a.W0, (uint64_t)a.d_in, (uint64_t)a.d_out, xs, kBK, (uint32_t)bn)) return cudaErrorInvalidValue;
-    if (!tc->get_2d(&tu, a.u_blocks, kRankPad, u_rows, kRankPad * 2, kBK, kBM)) return cudaErrorInvalidValue;
-    if (!split) {   // (the split-K kernel stores its outputs with plain stores)
-        if (!tc->get_2d(&ty, a.y, (uint64_t)a.d_out, (uint64_t)a.T, ys, kEpiChunkCols, 32)) return cudaErrorInvalidValue;
-        if (!tc->get_2d(&ty2, dual ? a.y2 : a.y, (uint64_t)a.d_out, (uint64_t)a.T, ys, kEpiChunkCols, 32)) return cudaErrorInvalidValue;
-    }
+    const bool dual = a.u2 != nullptr;
+    if (dual && (!a.lora || !a.y2 || a.P != 1 || a.fused)) return cudaErrorInvalidValue;
+    const int bn = a.shape.bn, split = a.shape.split;
+    if (a.fused && (split != 1 || bn != 256 || a.P != 1)) return cudaErrorInvalidValue;   // (the caller asked gemm_can_fuse_shrink first)
     GemmParams p;
-    p.seg_offsets = a.seg_offsets; p.slot_ids = a.slot_ids; p.perm = a.perm; p.plan = a.plan;
-    p.tile_identity = a.tile_identity;
-    p.y = (__nv_bfloat16*)a.y; p.status = ar.status;
-    p.slot_ids2 = a.slot_ids2; p.y2 = (__nv_bfloat16*)a.y2; p.u_set_rows = (int)u_set_rows;
-    p.T = a.T; p.K = a.d_in; p.N = a.d_out; p.G = a.G; p.num_m = num_m; p.num_n = num_n;
-    p.fused = (a.fused_shrink && !split && !dual) ? 1 : 0;
-    p.tile_flags = ar.tile_flags; p.fuse_sync = ar.status + 4; p.u_out = const_cast<__nv_bfloat16*>(a.u_blocks);
-    if (a.fused_shrink && !p.fused) return cudaErrorInvalidValue;   // (the caller asked gemm_can_fuse_shrink first)
+    p.num_m = (a.T + kBM - 1) / kBM;
+    const uint64_t xs = (uint64_t)a.d_in * 2;
+    if (!caches[0]->get_2d(&p.x, a.x, (uint64_t)a.d_in, (uint64_t)a.T, xs, kBK, (uint32_t)x_box_rows(a.T))) return cudaErrorInvalidValue;
+    p.x_bytes = x_box_rows(a.T) * kBK * 2;
+    p.a = tmap_A;
+    int tiles = 0, columns = 0;
+    for (int i = 0; i < a.P; ++i) {
+        const GemmProj& pr = a.proj[i];
+        GemmPart& pt = p.part[i];
+        const uint64_t ys = (uint64_t)pr.d_out * 2;
+        if (!caches[i]->get_2d(&pt.w, pr.W0, (uint64_t)a.d_in, (uint64_t)pr.d_out, xs, kBK, (uint32_t)bn)) return cudaErrorInvalidValue;
+        if (split == 1) {   // (the split-K kernel stores its outputs with plain stores)
+            if (!caches[i]->get_2d(&pt.y, pr.y, (uint64_t)pr.d_out, (uint64_t)a.T, ys, kEpiChunkCols, 32)) return cudaErrorInvalidValue;
+        } else {
+            pt.y = pt.w;
+        }
+        pt.bk = pr.ar->Bk; pt.plan = pr.plan; pt.u = pr.u; pt.y_ptr = (__nv_bfloat16*)pr.y;
+        pt.live = pt.nch[0] = pt.nch[1] = 0ull;
+        for (int s = 0; s < pr.snap->max_slots; ++s)
+            if (pr.snap->rank[s] > 0) {
+                pt.live |= 1ull << s;
+                pt.nch[s >> 5] |= (unsigned long long)(chunks_of_rank(pr.snap->rank[s]) - 1) << (2 * (s & 31));
+            }
+        pt.N = pr.d_out; pt.num_n = (pr.d_out + bn - 1) / bn; pt.n_pad = b_rows_padded(pr.d_out); pt.cap = pr.cap;
+        pt.tile0 = tiles;
+        tiles += p.num_m * pt.num_n;
+        columns += pt.num_n;
+    }
+    p.y2 = p.part[0].y;
+    if (dual && split == 1 &&
+        !caches[0]->get_2d(&p.y2, a.y2, (uint64_t)a.proj[0].d_out, (uint64_t)a.T, (uint64_t)a.proj[0].d_out * 2, kEpiChunkCols, 32)) return cudaErrorInvalidValue;
+    p.u2 = a.u2; p.y2_ptr = (__nv_bfloat16*)a.y2;
+    p.status = a.proj[0].ar->status;
+    p.T = a.T; p.K = a.d_in; p.P = a.P; p.num_tiles = tiles;
+    p.lora = a.lora ? 1 : 0; p.fused = a.fused ? 1 : 0; p.rows = a.rows;
+    p.x_flag = a.x_flag; p.call_id = a.call_id;
+    p.tile_flags = a.proj[0].ar->tile_flags; p.fuse_sync = a.proj[0].ar->status + 4;
     cudaLaunchConfig_t cfg = {};
-    cfg.blockDim = dim3(kGemmThreads);
-    cfg.stream = stream;
     cudaLaunchAttribute attr[2];
-    int nattr = 0;
-    {   // with adapters the predecessor is the shrink kernel of this call, else the kernel waits at its top
-        attr[nattr].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[nattr].val.programmaticStreamSerializationAllowed = 1;
-        ++nattr;
+    // with adapters the predecessor is the bind_shrink launch of this call, else the kernel waits at its top
+    pdl_config(cfg, attr, dim3((unsigned)(tiles < a.num_sms ? tiles : a.num_sms)), dim3(kGemmThreads),
+               bn == 256 ? GemmCfg<256>::kSmemBytes : (bn == 128 ? GemmCfg<128>::kSmemBytes : GemmCfg<64>::kSmemBytes), stream);
+    p.stages = 0;
+    if (split > 1) {
+        p.stages = a.share_sm && gemm_exchange_bytes(bn, split) <= gemm_stages_short(bn) * gemm_stage_bytes(bn) ? gemm_stages_short(bn) : gemm_stages(bn);
+        cfg.dynamicSmemBytes = GemmCfg<64>::split_smem(0) + p.stages * gemm_stage_bytes(bn);
+        cfg.gridDim = dim3(split, columns, p.num_m);
+        attr[1].id = cudaLaunchAttributeClusterDimension;
+        attr[1].val.clusterDim.x = split;
+        attr[1].val.clusterDim.y = 1;
+        attr[1].val.clusterDim.z = 1;
+        cfg.numAttrs = 2;
+        if (bn == 256) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_splitk_kernel<256>, p);
+        if (bn == 64) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_splitk_kernel<64>, p);
+        return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_splitk_kernel<128>, p);
     }
-    if (split) {
-        cfg.gridDim = dim3(split, num_n, num_m);
-        cfg.dynamicSmemBytes = bn == 256 ? GemmCfg<256>::kSmemBytes : GemmCfg<128>::kSmemBytes;
-        attr[nattr].id = cudaLaunchAttributeClusterDimension;
-        attr[nattr].val.clusterDim.x = split;
-        attr[nattr].val.clusterDim.y = 1;
-        attr[nattr].val.clusterDim.z = 1;
-        ++nattr;
-        cfg.attrs = attr;
-        cfg.numAttrs = nattr;
-        if (bn == 256) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_splitk_kernel<256>, tx, tx0, tw, tu, tb, snap, p);
-        return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_splitk_kernel<128>, tx, tx0, tw, tu, tb, snap, p);
-    }
-    cfg.gridDim = dim3(min(num_m * num_n, a.num_sms));
-    cfg.dynamicSmemBytes = bn == 256 ? GemmCfg<256>::kSmemBytes : GemmCfg<128>::kSmemBytes;
-    cfg.attrs = attr;
-    cfg.numAttrs = nattr;
-    if (bn == 256) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<256>, tx, tx0, tw, tu, tb, ty, ty2, tmap_A, snap, p);
-    return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<128>, tx, tx0, tw, tu, tb, ty, ty2, tmap_A, snap, p);
+    if (bn == 256) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<256>, p, *a.proj[0].snap);
+    if (bn == 64) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<64>, p, *a.proj[0].snap);
+    return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<128>, p, *a.proj[0].snap);
 }
 
 }  // namespace lml

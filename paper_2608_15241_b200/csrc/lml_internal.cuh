@@ -17,6 +17,11 @@ constexpr int kMaxSlots = LML_MAX_SLOTS;
 constexpr int kRankPad = 64;          // adapters are stored zero-padded to this rank
 constexpr int kRankCompact = 16;      // ... and B a second time, padded to this rank only, where the rank allows
 constexpr int kTileM = 128;           // token rows per GEMM tile and per shrink piece block
+constexpr int kChunk = 16;            // the LoRA product is computed in chunks of 16 of a slot's columns: one K-step of the tensor cores
+constexpr int kMaxChunks = kMaxSlots * (kRankPad / kChunk);   // chunks of a row tile at most
+constexpr int kUBlockBytes = kTileM * kChunk * 2;             // u of one row tile and chunk
+constexpr int kSlabTiles = 512;       // row tiles worked on at a time: longer calls run in slabs of this many, so that the u blocks stay bounded
+constexpr int kBindSegs = 256;        // segments that the kernels look up in shared memory; more are turned into a slot per row first
 constexpr int kDecodeMaxT = LML_DECODE_MAX_TOKENS;
 constexpr int kMaxAdapterIds = LML_MAX_ADAPTER_IDS;
 constexpr int kFuseMaxTiles = 4096;   // row tiles of a call whose shrink can run inside the GEMM kernel (524288 tokens)   // adapter ids that can be resolved on the device
@@ -32,23 +37,20 @@ struct SlotSnapshot {
 
 // Device-resident pieces of a table.
 struct Arena {
-    __nv_bfloat16* A;   // [max_slots][kRankPad][d_in]   rows >= rank are zero
-    __nv_bfloat16* B;   // [max_slots][d_out][kRankPad]  columns >= rank are zero
+    __nv_bfloat16* A;   // [max_slots][kRankPad][d_in]   rows >= rank are zero (as far as the last chunk of 16 that the rank needs)
+    __nv_bfloat16* B;   // [max_slots][d_out][kRankPad]  columns >= rank are zero (likewise)
     __nv_bfloat16* Bc;  // [max_slots][d_out][kRankCompact]: the same rows, 32 bytes each, for slots of rank <= kRankCompact
                         // (what the decode kernel reads: it needs a row's real columns only, a quarter of the padded row)
+    __nv_bfloat16* Bk;  // [max_slots][4 chunks][b_rows_padded(d_out)][kChunk] for the GEMM: a chunk is 16 of the slot's columns, its rows in the
+                        // no-swizzle operand order of the tensor cores (see chunk_elem), so that the rows of an output tile are one
+                        // contiguous piece and a slot costs the chunks its rank needs and no more
     uint32_t* status;   // sticky LML_FLAG_* bits
-    int32_t* tile_flags;    // [kFuseMaxTiles] fused shrink of the prefill GEMM: row tile m's u blocks are written (= epoch + 1; the epoch is word 4 of status)
+    int32_t* tile_flags;    // [kFuseMaxTiles] fused shrink of the prefill GEMM: the u blocks of pass i are written (= epoch + 1; the epoch is word 4 of status)
     int32_t* adapter_map;   // [kMaxAdapterIds] serving entry of each adapter id: slot | generation << 8, -1 = none; written by lml_publish
     unsigned long long* dec_u;   // [kDecMaxBlocks][kDecExchStride] the decode kernel's exchange blocks, one per part of a launch that works on this table
 };
 
 inline int32_t adapter_map_word(int slot, uint16_t gen) { return (int32_t)((uint32_t)slot | ((uint32_t)gen << 8)); }
-
-// Workspace header written by the shrink kernels and read by the kernels that follow.
-struct PlanWord {
-    int32_t lora_ok;    // 1 = seg_offsets well formed, expand steps may run
-    int32_t pad[63];
-};
 
 // ---- kernel launchers (each enqueues on `stream` and returns the launch error) ------------
 
@@ -78,42 +80,113 @@ cudaError_t launch_segment_tokens(const Arena& ar, const SlotSnapshot& snap, con
                                   int T, int32_t* perm, int32_t* seg_offsets, int32_t* seg_slot_ids,
                                   cudaStream_t stream, bool by_adapter = false);   // by_adapter: the ids are adapter ids, resolved through ar.adapter_map
 
-// u blocks: block b = (tile m) + (segment g) holds the 128 x 64 bf16 values scale*(x.A^T) of
+// u blocks of the backward pass: block b = (tile m) + (segment g) holds the 128 x 64 bf16 values scale*(x.A^T) of
 // the rows of tile m that belong to segment g, zero elsewhere.
-// x_in_place / tile_identity: rows of tiles marked identity are read from x_in_place instead of x.
 cudaError_t launch_shrink_pieces(const Arena& ar, const SlotSnapshot& snap, const void* x, int T,
                                  int d_in, const int32_t* seg_offsets, const int32_t* slot_ids, int G,
-                                 const void* x_in_place, const int32_t* tile_identity, PlanWord* plan,
-                                 __nv_bfloat16* u_blocks, cudaStream_t stream, int chained = 0,   // 1: a further pass of the same call, may run beside the one before; 2: behind the call's row-gather kernel
-                                 __nv_bfloat16* u_blocks_neg = nullptr);                              // optional second copy of the blocks, negated
+                                 __nv_bfloat16* u_blocks, cudaStream_t stream,
+                                 int chained = 0);   // 1: a further pass of the same call, may run beside the one before
 
-// tile_identity[m] = 1: tile m's perm is the identity, its rows were not copied and stay in place.
-// token-form calls of one row tile: binding and shrink in one launch, tokens in their order (see the kernel)
-cudaError_t launch_bind_shrink_tile(const Arena& ar, const SlotSnapshot& snap, const int32_t* token_slots, int T, int d_in,
-                                    const void* x, int32_t* seg_offsets, int32_t* seg_slot_ids, int G, PlanWord* plan,
-                                    void* u_blocks, int threads, cudaStream_t stream, bool by_adapter);
-cudaError_t launch_gather_rows(const void* x, const int32_t* perm, int T, int d_in, void* x_grouped,
-                               int32_t* tile_identity, bool allow_skip, uint32_t* status, cudaStream_t stream);
+// ---- binding and shrink of the GEMM path ----------------------------------------------------------
+// The rows stay where they are.  Of every 128-row tile the GEMM needs to know which slots its rows use and,
+// per chunk of 16 columns of each of those slots, the block u = scale * x.A^T of the tile, zero in the rows that are
+// bound to another slot.  A tile's blocks are numbered by slot, then by chunk; it has room for `cap` of them.
 
-struct GemmArgs {
-    const void* x;            // rows in position order (already gathered when perm is used)
-    const void* x_in_place;   // perm form: the caller's x, read for tiles whose perm is the identity
-    const int32_t* tile_identity;   // perm form: 1 per 128-row tile that was left in place, else NULL
+__host__ __device__ __forceinline__ int chunks_of_rank(int rank) { return (rank + kChunk - 1) / kChunk; }
+// element (row, column) of a chunk's block: 8 x 8 core matrices of 128 contiguous bytes, the two of a row group side by side
+__host__ __device__ __forceinline__ size_t chunk_elem(int row, int col)
+{
+    return (size_t)(row >> 3) * 128 + (size_t)(col >> 3) * 64 + (size_t)(row & 7) * 8 + (size_t)(col & 7);
+}
+// rows of x that a copy of one row tile brings in: a call of a single tile moves its own rows only (the others' products are
+// not stored, whatever the shared memory under them holds)
+inline int x_box_rows(int T) { return T >= kTileM ? kTileM : (T + 7) / 8 * 8; }
+inline int b_rows_padded(int d_out) { return (d_out + 255) / 256 * 256; }
+
+// What bind_shrink writes for the GEMM, per row tile: the tile's chunks in the order of their blocks.
+struct alignas(16) TilePlan {
+    int32_t count;
+    int32_t pad[3];
+    uint16_t chunk[kMaxChunks];   // slot | chunk << 8 | kChunkFirst, kChunkSecond
+};
+constexpr uint32_t kChunkFirst = 0x1000u, kChunkSecond = 0x2000u;   // rows use the slot under the first / second binding
+
+enum RowMode { kRowsNone = 0, kRowsTokens = 1, kRowsSegments = 2, kRowsGiven = 3 };
+// Where the slot of a row comes from: an id per token, the segment arrays (G <= kBindSegs), or a slot per row that
+// launch_rows_from_segments has written.
+struct RowSource {
+    int mode = kRowsNone;
+    const int32_t* ids = nullptr;    // segments: per segment (BindPart has the ids of the bind_shrink launch)
+    const int32_t* ids2 = nullptr;   // dual calls: the second binding (segments)
+    const int32_t* seg_offsets = nullptr;
+    int G = 0;
+    const int8_t* rows = nullptr;
+    const int8_t* rows2 = nullptr;
+};
+// One projection's share of a launch.
+struct BindPart {
+    const __nv_bfloat16* A;
+    const int32_t* ids;           // per token, or per segment
+    const int32_t* adapter_map;   // null: the ids are slots; else adapter ids, resolved through the table's device map
+    uint32_t* status;
+    TilePlan* plan;               // [row tile]
+    __nv_bfloat16* u;
+    __nv_bfloat16* u2;            // dual calls: a second set of blocks
+    int cap;
+    int pad;
+};
+struct BindArgs {
+    const void* x;
+    int T, d_in, P;
+    RowSource rows;
+    int second = 0;   // dual calls, what u2 holds: 1 the second binding's blocks, 2 second minus first
+    // early start of the GEMM (see bind_starts_gemm_early): the word that says "x may be read" and this call's value of it
+    uint32_t* x_flag = nullptr;
+    uint32_t call_id = 0;
+    bool share_sm = false;   // the GEMM's CTAs and this launch's have to fit an SM together
+    BindPart part[LML_MAX_PROJECTIONS];
+    SlotSnapshot snap[LML_MAX_PROJECTIONS];
+};
+// slot per row (int8, -1 = none) of a segment call with a row permutation or with many segments; checks the arrays and raises the flags
+cudaError_t launch_rows_from_segments(const Arena& ar, const SlotSnapshot& snap, const int32_t* seg_offsets, const int32_t* slot_ids,
+                                      const int32_t* slot_ids2, int G, const int32_t* perm, int T, int8_t* rows, int8_t* rows2,
+                                      cudaStream_t stream);
+cudaError_t bind_init();
+
+// One projection of a GEMM launch.
+struct GemmProj {
     const void* W0;
     void* y;
-    const int32_t* perm;      // NULL or position -> output row
-    const int32_t* seg_offsets;
-    const int32_t* slot_ids;
-    const PlanWord* plan;
-    const __nv_bfloat16* u_blocks;
-    const int32_t* slot_ids2 = nullptr;   // dual form: second slot per segment; u_blocks then holds three sets of
-    void* y2 = nullptr;                   // (num_m + G) blocks: first slots, second slots, first slots negated
-    int T, d_in, d_out, G;
-    int num_sms;
-    bool fused_shrink = false;         // no shrink kernel ran: the GEMM kernel computes the u blocks itself (see gemm_can_fuse_shrink)
-    int split_bn = -1, split_s = -1;   // the table's split-K override: -1 = the library chooses, 0 = off, else the forced shape
-    bool overlap_with_previous;   // launch as a programmatic dependent of the shrink kernel before it
+    int d_out;
+    const Arena* ar;
+    const SlotSnapshot* snap;
+    const TilePlan* plan;
+    const __nv_bfloat16* u;
+    int cap;
 };
+// What the library takes for a call: width of an output tile and CTAs that share one (1: whole-K tiles), CTAs in all.
+struct GemmShape { int bn, split, ctas; };
+struct GemmArgs {
+    const void* x;
+    int T, d_in, P;
+    bool lora;                // the call has adapters (a bind_shrink launch came before, unless fused)
+    GemmProj proj[LML_MAX_PROJECTIONS];
+    GemmShape shape;
+    // dual form (one projection): the second set of u blocks, the second output
+    const __nv_bfloat16* u2 = nullptr;
+    void* y2 = nullptr;
+    // fused shrink (one projection): no bind_shrink launch; the kernel binds the rows and computes the u blocks itself
+    bool fused = false;
+    RowSource rows;
+    uint32_t* x_flag = nullptr;   // early start: [0] holds call_id once x may be read, [1] CTAs that have finished (the last one clears both)
+    uint32_t call_id = 0;
+    bool share_sm = false;        // as in BindArgs
+    int num_sms;
+};
+// split_bn, split_s: the table's override (-1 = the library chooses, 0 = whole-K tiles, else the forced shape)
+GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, int num_sms, int split_bn, int split_s);
+// whether the shrink of a plain call of this size and shape runs inside the GEMM kernel; cap: chunks per tile at most
+bool gemm_can_fuse_shrink(const GemmShape& shape, int T, int d_out, int G, bool in_segment_order, int cap, int num_sms);
 // Tensor maps of caller buffers, kept per table and found again by (pointer, shape, box).
 struct TmapCache {
     static constexpr int kEntries = 32;
@@ -126,15 +199,17 @@ struct TmapCache {
                 uint32_t box_inner, uint32_t box_outer);
 };
 bool gemm_split_override(int* bn_out, int* split_out);
-// tmap_B256 / tmap_B128: the table's maps of its packed B arena for 256- and 128-column tiles.
-// Returns cudaErrorInvalidValue if a tensor map cannot be encoded.
-bool gemm_can_fuse_shrink(int T, int d_in, int d_out, int G, int num_sms, int split_bn, int split_s);
-// tmap_A: the table's map of its packed A arena ([max_slots][64][d_in], box 64 x 64 x 1), for the fused shrink.
-cudaError_t launch_gemm_sm100(const Arena& ar, const SlotSnapshot& snap, const CUtensorMap& tmap_B256,
-                              const CUtensorMap& tmap_B128, const CUtensorMap& tmap_A, TmapCache* cache, const GemmArgs& a,
-                              cudaStream_t stream);
+// bind_starts_gemm_early: for calls of few rows the GEMM may start while the work before the call is still running; it then
+// reads nothing but W0 until bind_shrink, which waits for that work, has said that x may be read.
+bool bind_starts_gemm_early(int T, int P, int num_sms);
+int bind_ctas_early(int T, int d_in, int P, int cap, int num_sms);   // ... and how many CTAs bind_shrink has then
+// tmap_A[p]: the map of projection p's packed A arena ([max_slots][64][d_in], box 64 x 16 x 1)
+cudaError_t launch_bind_shrink(const BindArgs& a, const CUtensorMap* const* tmap_A, TmapCache* cache, int num_sms, cudaStream_t stream);
+// tmap_A: the same of the (first) table, for the fused shrink; caches[p]: the tensor maps of the buffers of projection p.
+// Returns cudaErrorInvalidValue if one cannot be encoded.
+cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* caches, const GemmArgs& a, cudaStream_t stream);
 cudaError_t gemm_sm100_init(int device);
-cudaError_t shrink_init();   // both set the dynamic shared memory attributes of their kernels
+cudaError_t shrink_init();   // these set the dynamic shared memory attributes of their kernels
 bool encode_tmap_2d(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer,
                     uint64_t row_stride_bytes, uint32_t box_inner, uint32_t box_outer);
 bool encode_tmap_3d(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2,
@@ -217,8 +292,7 @@ __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint3
         : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
 }
 
-// Segment lookup shared by the kernels.  seg_offsets is assumed monotone (the shrink kernel
-// validates it and clears PlanWord::lora_ok otherwise); all results are clamped so that a
+// Segment lookup shared by the kernels.  seg_offsets is assumed monotone; all results are clamped so that a
 // malformed array can only produce wrong-but-in-range indices.
 //
 // first segment whose end lies beyond `pos`

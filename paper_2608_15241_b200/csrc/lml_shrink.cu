@@ -1,12 +1,11 @@
-// LoRA shrink for the prefill path: u = scale_s * (x . A_s^T), written as bf16 "piece blocks"
-// that the GEMM kernel consumes as extra tensor-core K-steps.
+// LoRA shrink for the backward pass: u = scale_s * (x . A_s^T), written as bf16 "piece blocks"
+// that the gradient kernel contracts with x and dy.
 //
 // A piece is the intersection of a 128-row tile m with a segment g whose slot is live.  Its
 // block index is b = m + g, which is unique because segments are ordered row ranges: a later
 // segment cannot reach into an earlier tile.  Block b holds 128 x 64 bf16: row i is
 // scale * x[m*128+i] . A_s^T (columns >= rank are zero) when that row belongs to segment g
-// and zero otherwise, so one UMMA of the whole block with B_s adds exactly the segment's LoRA
-// term to the tile.
+// and zero otherwise, so the whole tile can be multiplied.
 //
 // The contraction runs on mma.sync m16n8k16 with operands loaded straight from global memory
 // by 128-bit loads: a dot product does not care about the order of k, so lane (g, t) takes
@@ -44,18 +43,12 @@ __global__ void __launch_bounds__(kShrinkWarps * 32, NB <= 2 ? 2 : 1) shrink_pie
     const __grid_constant__ SlotSnapshot snap, const __nv_bfloat16* __restrict__ arenaA,
     uint32_t* __restrict__ status, const __nv_bfloat16* __restrict__ x, int T, int K,
     const int32_t* __restrict__ seg_offsets, const int32_t* __restrict__ slot_ids, int G,
-    const __nv_bfloat16* __restrict__ x_in_place, const int32_t* __restrict__ tile_identity,
-    PlanWord* __restrict__ plan, __nv_bfloat16* __restrict__ u_blocks, int num_tiles, int chained,
-    __nv_bfloat16* __restrict__ u_blocks_neg)   // optional second copy of the blocks with the sign flipped
+    __nv_bfloat16* __restrict__ u_blocks, int num_tiles, int chained)
 {
-    // chained 0: launched with a full dependency on the work before it, so nothing to wait for; the GEMM that
-    // follows may start its main loop right away.  chained 1: this is a further shrink pass of the same call,
+    // chained 0: launched with a full dependency on the work before it, so nothing to wait for.  chained 1: this is a further shrink pass of the same call,
     // launched as a programmatic dependent of the first, which had that full dependency: the passes run side by
     // side; one CTA then stays until the pass before is complete, so that whoever waits for this grid has
-    // waited for all of them.  chained 2: the predecessor is the call's own short row-gather kernel; launched
-    // as its programmatic dependent (the launch latency hides behind it), every CTA waits for it here before
-    // it lets the GEMM go, so that the GEMM finds the gathered rows complete as well.
-    if (chained == 2) ptx::grid_dependency_wait();
+    // waited for all of them.
     ptx::grid_launch_dependents();
     extern __shared__ float shrink_smem[];
     using S = ShrinkSmem<NB>;
@@ -69,7 +62,7 @@ __global__ void __launch_bounds__(kShrinkWarps * 32, NB <= 2 ? 2 : 1) shrink_pie
     const int b = blockIdx.y, sub = blockIdx.x;
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
-    // One CTA validates the segment arrays for the whole call.
+    // One CTA checks the segment arrays for the whole call.
     if (b == 0 && sub == 0 && ks == 0) {
         if (chained == 1 && tid == 0) ptx::grid_dependency_wait();
         int bad_off = 0, bad_slot = 0;
@@ -83,7 +76,6 @@ __global__ void __launch_bounds__(kShrinkWarps * 32, NB <= 2 ? 2 : 1) shrink_pie
         bad_off = __syncthreads_or(bad_off);
         bad_slot = __syncthreads_or(bad_slot);
         if (tid == 0) {
-            plan->lora_ok = bad_off ? 0 : 1;
             unsigned f = (bad_off ? LML_FLAG_BAD_OFFSETS : 0u) | (bad_slot ? LML_FLAG_BAD_SLOT : 0u);
             if (f) atomicOr(status, f);
         }
@@ -124,25 +116,20 @@ __global__ void __launch_bounds__(kShrinkWarps * 32, NB <= 2 ? 2 : 1) shrink_pie
     const int nblk = ((int)snap.rank[slot] + 7) >> 3;
     const int p0 = m * kTileM + sub * kShrinkRows;
     uint4* out = reinterpret_cast<uint4*>(u_blocks + ((size_t)b * kTileM + sub * kShrinkRows) * kRankPad);
-    uint4* out_neg = u_blocks_neg ? reinterpret_cast<uint4*>(u_blocks_neg + ((size_t)b * kTileM + sub * kShrinkRows) * kRankPad) : nullptr;
 
     if (p0 + kShrinkRows <= plo || p0 >= phi) {   // no row of this slab is in the piece
-        if (ks == 0) {   // 32 rows x 128 B = 256 x 16 B
-            out[tid] = make_uint4(0, 0, 0, 0);
-            if (out_neg) out_neg[tid] = make_uint4(0, 0, 0, 0);
-        }
+        if (ks == 0) out[tid] = make_uint4(0, 0, 0, 0);   // 32 rows x 128 B = 256 x 16 B
         return;
     }
 
     const int gq = lane >> 2, tq = lane & 3;
-    const __nv_bfloat16* xsrc = (tile_identity && __ldg(tile_identity + m)) ? x_in_place : x;   // in-place tiles were never copied
     const __nv_bfloat16* xr[4];
     bool xv[4];
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
         const int p = p0 + gq + 8 * i;
         xv[i] = p >= plo && p < phi;
-        xr[i] = xsrc + (size_t)(xv[i] ? p : 0) * K + tq * 8;
+        xr[i] = x + (size_t)(xv[i] ? p : 0) * K + tq * 8;
     }
     const __nv_bfloat16* Abase = arenaA + ((size_t)slot * kRankPad + gq) * K + tq * 8;
 
@@ -222,7 +209,6 @@ __global__ void __launch_bounds__(kShrinkWarps * 32, NB <= 2 ? 2 : 1) shrink_pie
         o.x = pack_bf16(v[0] * sc, v[1] * sc); o.y = pack_bf16(v[2] * sc, v[3] * sc);
         o.z = pack_bf16(v[4] * sc, v[5] * sc); o.w = pack_bf16(v[6] * sc, v[7] * sc);
         out[row * 8 + (tid & 7)] = o;
-        if (out_neg) out_neg[row * 8 + (tid & 7)] = make_uint4(o.x ^ 0x80008000u, o.y ^ 0x80008000u, o.z ^ 0x80008000u, o.w ^ 0x80008000u);
     }
     cluster.sync();   // peers stay alive until their partials have been read
 }
@@ -230,8 +216,7 @@ __global__ void __launch_bounds__(kShrinkWarps * 32, NB <= 2 ? 2 : 1) shrink_pie
 template <int NB>
 static cudaError_t launch_shrink_nb(const Arena& ar, const SlotSnapshot& snap, const void* x, int T, int d_in,
                                     const int32_t* seg_offsets, const int32_t* slot_ids, int G,
-                                    const void* x_in_place, const int32_t* tile_identity, PlanWord* plan,
-                                    __nv_bfloat16* u_blocks, cudaStream_t stream, int chained, __nv_bfloat16* u_blocks_neg)
+                                    __nv_bfloat16* u_blocks, cudaStream_t stream, int chained)
 {
     const int num_tiles = (T + kTileM - 1) / kTileM;
     int ks = (d_in + 1023) / 1024;
@@ -253,9 +238,8 @@ static cudaError_t launch_shrink_nb(const Arena& ar, const SlotSnapshot& snap, c
     const __nv_bfloat16* arenaA = ar.A;
     uint32_t* status = ar.status;
     const __nv_bfloat16* xb = (const __nv_bfloat16*)x;
-    const __nv_bfloat16* xip = (const __nv_bfloat16*)x_in_place;
     return cudaLaunchKernelEx(&cfg, shrink_pieces_kernel<NB>, snap, arenaA, status, xb, T, d_in, seg_offsets,
-                              slot_ids, G, xip, tile_identity, plan, u_blocks, num_tiles, chained, u_blocks_neg);
+                              slot_ids, G, u_blocks, num_tiles, chained);
 }
 
 cudaError_t shrink_init()
@@ -269,14 +253,13 @@ cudaError_t shrink_init()
 
 cudaError_t launch_shrink_pieces(const Arena& ar, const SlotSnapshot& snap, const void* x, int T,
                                  int d_in, const int32_t* seg_offsets, const int32_t* slot_ids, int G,
-                                 const void* x_in_place, const int32_t* tile_identity, PlanWord* plan,
-                                 __nv_bfloat16* u_blocks, cudaStream_t stream, int chained, __nv_bfloat16* u_blocks_neg)
+                                 __nv_bfloat16* u_blocks, cudaStream_t stream, int chained)
 {
     int max_rank = 0;
     for (int i = 0; i < snap.max_slots; ++i) max_rank = snap.rank[i] > max_rank ? snap.rank[i] : max_rank;
     if (max_rank <= 16)
-        return launch_shrink_nb<2>(ar, snap, x, T, d_in, seg_offsets, slot_ids, G, x_in_place, tile_identity, plan, u_blocks, stream, chained, u_blocks_neg);
-    return launch_shrink_nb<8>(ar, snap, x, T, d_in, seg_offsets, slot_ids, G, x_in_place, tile_identity, plan, u_blocks, stream, chained, u_blocks_neg);
+        return launch_shrink_nb<2>(ar, snap, x, T, d_in, seg_offsets, slot_ids, G, u_blocks, stream, chained);
+    return launch_shrink_nb<8>(ar, snap, x, T, d_in, seg_offsets, slot_ids, G, u_blocks, stream, chained);
 }
 
 }  // namespace lml

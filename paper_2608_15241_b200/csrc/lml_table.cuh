@@ -17,12 +17,9 @@ struct lml_table {
     } entries[lml::kMaxSlots];
     uint16_t next_gen = 0;
     lml::Arena arena{};
-    CUtensorMap tmap_B256, tmap_B128;   // packed B arena as [max_slots][d_out][64], boxes 64 x 256 x 1 and 64 x 128 x 1
-    CUtensorMap tmap_A;                 // packed A arena as [max_slots][64][d_in], box 64 x 64 x 1
+    CUtensorMap tmap_A;                 // packed A arena as [max_slots][64][d_in], box 64 x 16 x 1
     bool fuse_shrink = true;            // LML_FUSE_SHRINK=0 when the table was created: always the separate shrink kernel (a test knob)
     lml::TmapCache tmaps;               // tensor maps of the caller's buffers seen so far
-    int bind_threads = 0;               // LML_BIND_THREADS as it stood when the table was created (0: the library chooses; a test knob)
-    int one_tile_tokens = lml::kTileM;  // token-form calls of up to this many tokens (beyond the decode kernel's range) keep the tokens in their order: one or two row tiles, set when the table is created; LML_ONE_TILE=0 or LML_ONE_TILE_TOKENS=n at that time change it (test knobs)
     int dec_block_tokens = -1;          // token-form calls of up to this many tokens run as blocks of 16 on the decode kernel; -1: the library's own limit (LML_DECODE_BLOCK_TOKENS as it stood when the table was created)
     int split_bn = -1, split_s = -1;    // LML_GEMM_SPLIT as it stood when the table was created (-1: not set)
     // Retiring a serving entry clears its word of the device map with a kernel on a stream; the event marks
@@ -30,6 +27,7 @@ struct lml_table {
     cudaEvent_t ev_map = nullptr;
     bool map_clear_recorded = false;
     int last_launches = 0;
+    uint32_t next_call = 0;             // numbers the calls whose GEMM starts early (never 0)
     // host-buffer form of large calls: the copies of x in and of y out run on two streams of the table's own,
     // chunk by chunk beside the layer (created with the table: the call itself creates nothing)
     static constexpr int kHostChunks = 8;
