@@ -122,8 +122,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         b.x_flag = g.x_flag = nullptr;
         if (mode != kRowsNone && !g.fused && bind_starts_gemm_early(rows, P, t0->num_sms)) {
             b.x_flag = g.x_flag = t0->arena.status + 8;
-            b.share_sm = g.share_sm = g.shape.split > 1 &&
-                g.shape.ctas + bind_ctas_early(rows, t0->d_in, P, most_chunks, t0->num_sms) > t0->num_sms;
+            b.share_sm = g.share_sm = g.shape.ctas + bind_ctas_early(rows, t0->d_in, P, most_chunks, t0->num_sms) > t0->num_sms;
             std::lock_guard<std::mutex> lock(t0->mu);
             if (++t0->next_call == 0u) ++t0->next_call;
             b.call_id = g.call_id = t0->next_call;

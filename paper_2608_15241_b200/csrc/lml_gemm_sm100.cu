@@ -1203,16 +1203,18 @@ GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, int num_sms
         const int bn = 64 << w, tiles = tiles_of(bn);
         for (int S = 1; S <= (split_bn == 0 ? 1 : kSplitMaxS); ++S) {
             if (S > 1 && (max_clusters[w][S] <= 0 || num_kb < 8 * S || gemm_exchange_bytes(bn, S) > gemm_stages(bn) * gemm_stage_bytes(bn))) continue;
-            // (a cluster needs its CTAs on one part of the chip: with the last places taken by other work it waits)
-            const int fit = S > 1 ? max_clusters[w][S] - (S > 3 ? 1 : 0) : num_sms;
+            // (a cluster needs its CTAs on one part of the chip: where they do not all find a place beside bind_shrink's, about
+            // 40 CTAs, some wait for it to end)
+            const int fit = S > 1 ? max_clusters[w][S] : num_sms;
             if (S > 1 && tiles > fit) continue;
+            const bool beside = tiles * num_sms <= fit * (num_sms - 40);
             const int waves = (tiles + fit - 1) / fit;
             float us;
             if (crowded) {
                 us = (float)(waves * num_kb) * (w == 2 ? 0.31f : 0.254f);
             } else {
-                const int stages = S > 1 && tiles * S > num_sms - 40 ? gemm_stages_short(bn) : gemm_stages(bn);
-                us = (w == 2 ? 12.5f : (w == 1 ? 10.f : 8.f)) + (S > 1 ? 1.f : 0.f) +
+                const int stages = S > 1 && !beside ? gemm_stages_short(bn) : gemm_stages(bn);
+                us = (w == 2 ? 12.5f : (w == 1 ? 10.f : 8.f)) + (S > 1 ? 1.f : 0.f) + (S > 1 && !beside ? 4.f : 0.f) +
                      (float)waves * (float)((num_kb + S - 1) / S) * 1.55f / (float)stages;
             }
             if (us < best_us * 0.999f) { best_us = us; best = {bn, S, tiles * S}; }
