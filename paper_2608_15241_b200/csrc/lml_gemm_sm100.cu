@@ -576,6 +576,26 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                 umma_commit(smem_u32(&ctrl->empty[stage]));
                 if (++stage == Cfg::kStages) { stage = 0; phase ^= 1u; }
             };
+            // `count` k-blocks without a side-band word: the loop that the tensor cores wait for; its state lives in registers
+            auto base_stages = [&](uint32_t d_tmem, int count, uint32_t& accumulate) {
+                int st = stage;
+                uint32_t ph = phase, on = accumulate;
+                bool good = true;
+                const uint64_t adesc0 = umma_desc_k128(tiles_addr), bdesc0 = umma_desc_k128(tiles_addr + Cfg::kABytes);
+                const uint32_t full0 = smem_u32(&ctrl->full[0]), empty0 = smem_u32(&ctrl->empty[0]);
+                for (int i = 0; i < count; ++i) {
+                    good = mbar_wait(full0 + 8u * (uint32_t)st, ph, abort);
+                    if (!good) break;
+                    const uint64_t at = (uint64_t)((uint32_t)st * (uint32_t)(Cfg::kStageBytes / 16));
+#pragma unroll
+                    for (int k = 0; k < 4; ++k)
+                        umma_bf16(d_tmem, adesc0 + at + (uint64_t)(k * 2), bdesc0 + at + (uint64_t)(k * 2), idesc, k == 0 ? on : 1u);
+                    on = 1u;
+                    umma_commit(empty0 + 8u * (uint32_t)st);
+                    if (++st == Cfg::kStages) { st = 0; ph ^= 1u; }
+                }
+                stage = st; phase = ph; accumulate = on; ok = good;
+            };
             // stages with a side-band word, up to and including the one that completes an output
             auto flagged_stages = [&](int acc, uint32_t& accumulate) {
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
@@ -642,15 +662,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                 tc_fence_after();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(acc * BN);
                 uint32_t accumulate = 0;
-                const int mid = min((num_kb + 1) / 2, num_kb - 1);
-                for (int kb = 0; kb < num_kb - 1 && ok; ++kb) {
-                    if (dual && ordinal > 0 && kb == mid) { delta_stages(acc ^ 1); if (!ok) break; }
-                    ok = mbar_wait(smem_u32(&ctrl->full[stage]), phase, abort);
+                int from = 0;
+                if (dual && ordinal > 0) {
+                    from = min((num_kb + 1) / 2, num_kb - 1);
+                    base_stages(d_tmem, from, accumulate);
+                    if (ok) delta_stages(acc ^ 1);
                     if (!ok) break;
-                    issue(d_tmem, 4, false, accumulate);
                 }
+                base_stages(d_tmem, num_kb - 1 - from, accumulate);
                 if (!ok) break;
-                if (dual && ordinal > 0 && mid == num_kb - 1) { delta_stages(acc ^ 1); if (!ok) break; }
                 flagged_stages(acc, accumulate);   // the last k-block and the tile's LoRA pieces
             }
             if (ok && dual && ordinal > 0) delta_stages((ordinal - 1) & 1);
