@@ -113,7 +113,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         }
         if (r0 > 0 && b.rows.rows) b.rows.rows += kSlabTiles * kTileM;
         if (r0 > 0 && b.rows.rows2) b.rows.rows2 += kSlabTiles * kTileM;
-        g.shape = gemm_pick_shape(rows, t0->d_in, d_outs, P, t0->num_sms, t0->split_bn, t0->split_s);
+        g.shape = gemm_pick_shape(rows, t0->d_in, d_outs, P, dual, t0->num_sms, t0->split_bn, t0->split_s);
         // With whole-K tiles and few row tiles the shrink runs inside the GEMM kernel (on the CTAs that own the fewest tiles,
         // ahead of their tiles); otherwise a launch goes first and the GEMM is its programmatic dependent.
         g.fused = mode == kRowsSegments && !dual && P == 1 && T == rows && t0->fuse_shrink &&

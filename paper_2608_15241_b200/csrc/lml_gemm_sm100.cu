@@ -42,17 +42,21 @@ using namespace ptx;
 constexpr int kBM = kTileM;   // 128
 constexpr int kBK = 64;       // bf16 elements per 128-byte swizzled row
 constexpr int kGemmThreads = 192;
+constexpr int kGemmThreadsTall = 320;
 constexpr int kEpiChunkCols = 32;
 constexpr int kEpiBufBytes = 32 * kEpiChunkCols * 2;   // 2 KB: 32 rows x 64 B
 
 constexpr int kFuseTilesInKernel = 80;    // row tiles of a call whose shrink runs inside the kernel (the per-tile tables in shared memory)
 
-template <int BN> struct GemmCfg {
-    static constexpr int kABytes = kBM * kBK * 2;
+template <int BN, bool kTall = false> struct GemmCfg {
+    static constexpr int kRowTiles = kTall ? 2 : 1;
+    static constexpr int kXBytes = kBM * kBK * 2;             // a k-block of one row tile
+    static constexpr int kABytes = kRowTiles * kXBytes;
     static constexpr int kBBytes = BN * kBK * 2;
     static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kStages = (BN == 256) ? 4 : (BN == 128 ? 6 : 8);
-    static constexpr int kEpiBytes = 4 * 2 * kEpiBufBytes;
+    static constexpr int kStages = kTall ? 3 : ((BN == 256) ? 4 : (BN == 128 ? 6 : 8));
+    static constexpr int kEpiBufs = kTall ? 1 : 2;
+    static constexpr int kEpiBytes = 4 * kRowTiles * kEpiBufs * kEpiBufBytes;
     static constexpr int kTmemCols = 2 * BN;
     static constexpr int kCtrlBytes = 256 + (kBindSegs + 1) * 4 + kBindSegs + 4 + 512 + kFuseTilesInKernel * 10 + 8 + kMaxChunks * 4;   // barriers; fused shrink: segment cache, shrink plan, per-tile masks and first passes; the first tile's chunks
     // The split-K kernel: no staging for the epilogue.  The ring also takes the partial sums that the CTAs exchange; where
@@ -83,6 +87,7 @@ constexpr uint32_t kStageDelta = 0x800u;    // dual form: first stage of a tile'
 
 static_assert(sizeof(GemmCtrl) <= 256, "control block");
 constexpr uint32_t kStageBoth = 0x2000u;    // split-K dual form: the stage's product goes into both bindings' accumulators
+constexpr uint32_t kStageMore0 = 0x8000u, kStageMore1 = 0x10000u;   // tall tiles, on the last k-block: LoRA stages follow for the first / second row tile
 constexpr uint32_t kStageChunks = 0x4000u;  // LoRA chunks (no-swizzle operands), a K-step each
 
 // Fused shrink: a pass computes up to four chunks of a row tile, x[tile].A^T over all of K, two k-blocks to a stage.
@@ -218,12 +223,18 @@ __device__ __forceinline__ void prefetch_b(const GemmPart& pt, int n, int lane, 
     }
 }
 
-template <int BN>
-__global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const __grid_constant__ GemmParams p,
-                                                                          const __grid_constant__ SlotSnapshot snap)
+// kTall: a tile is two row tiles high (256 x 256).  Both accumulators belong to the tile, each row tile has four epilogue
+// warps of its own, and a stage holds two tiles of x beside one of W0: 64 KB for 1024 cycles of the tensor cores where the
+// single tile moves 48 KB for 512, so the ring covers twice the latency of a copy with the same shared memory (2048 x 4096 x
+// 4096 without adapters 55.9 -> 50.4 us, 0.82 of the 1665 TFLOP/s that a plain library product reaches here).  (No dual form.)
+template <int BN, bool kTall>
+__global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lora_gemm_sm100_kernel(
+    const __grid_constant__ GemmParams p, const __grid_constant__ SlotSnapshot snap)
 {
-    using Cfg = GemmCfg<BN>;
-    const bool dual = p.u2 != nullptr;
+    using Cfg = GemmCfg<BN, kTall>;
+    constexpr int kRowTiles = Cfg::kRowTiles;
+    constexpr int kThreads = kTall ? kGemmThreadsTall : kGemmThreads;
+    const bool dual = !kTall && p.u2 != nullptr;
     extern __shared__ uint8_t smem_raw[];
     // 128-byte swizzled tiles need 1024-byte alignment
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -242,6 +253,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int num_tiles = p.num_tiles;
     const int num_kb = (p.K + kBK - 1) / kBK;
+    const int num_mt = (p.num_m + kRowTiles - 1) / kRowTiles;   // tiles along the rows
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < Cfg::kStages; ++s) {
@@ -277,16 +289,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
         // Every CTA works out the slots of all row tiles from its own copy of the segment arrays (checked here: all reach
         // the same verdict) or from the slot per row.
         int bad_off = 0, bad_slot = 0;
-        for (int m = threadIdx.x; m < p.num_m; m += kGemmThreads) tile_mask[m] = 0ull;
+        for (int m = threadIdx.x; m < p.num_m; m += kThreads) tile_mask[m] = 0ull;
         if (by_segment) {
             const int G = p.rows.G;
-            for (int g = threadIdx.x; g <= G; g += kGemmThreads) seg_cache[g] = __ldg(p.rows.seg_offsets + g);
-            for (int g = threadIdx.x; g < G; g += kGemmThreads) {
+            for (int g = threadIdx.x; g <= G; g += kThreads) seg_cache[g] = __ldg(p.rows.seg_offsets + g);
+            for (int g = threadIdx.x; g < G; g += kThreads) {
                 const int s = __ldg(p.rows.ids + g);
                 slot_cache[g] = (int8_t)(slot_rank(snap, s) > 0 ? s : (s == -1 ? -1 : -2));
             }
             __syncthreads();
-            for (int g = threadIdx.x; g < G; g += kGemmThreads) {
+            for (int g = threadIdx.x; g < G; g += kThreads) {
                 const int s0 = seg_cache[g], s1 = seg_cache[g + 1];
                 if (s1 < s0 || s0 < 0 || s1 > p.T) bad_off = 1;
                 if (slot_cache[g] == -2 && s1 > s0) bad_slot = 1;   // an empty segment may name anything
@@ -295,7 +307,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             bad_off = __syncthreads_or(bad_off);
             bad_slot = __syncthreads_or(bad_slot);
             if (!bad_off)
-                for (int g = threadIdx.x; g < G; g += kGemmThreads) {
+                for (int g = threadIdx.x; g < G; g += kThreads) {
                     const int s0 = seg_cache[g], s1 = seg_cache[g + 1], s = slot_cache[g];
                     if (s >= 0 && s1 > s0)
                         for (int m = s0 / kBM; m <= (s1 - 1) / kBM; ++m) atomicOr(&tile_mask[m], 1ull << s);
@@ -306,14 +318,14 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             }
         } else {
             __syncthreads();
-            for (int row = threadIdx.x; row < p.T; row += kGemmThreads) {
+            for (int row = threadIdx.x; row < p.T; row += kThreads) {
                 const int s = p.rows.rows[row];
                 if (slot_rank(snap, s) > 0) atomicOr(&tile_mask[row / kBM], 1ull << s);
             }
         }
         __syncthreads();
         const GemmPart& pt = p.part[0];
-        for (int m = threadIdx.x; m < p.num_m; m += kGemmThreads)
+        for (int m = threadIdx.x; m < p.num_m; m += kThreads)
             shr_base[m + 1] = (uint16_t)((mask_chunks(pt, tile_mask[m]) + kShrChunks - 1) / kShrChunks);
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -355,7 +367,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             bool lora = false, lora_known = !p.lora;
             // the CTA's first tile: its chunks are listed in shared memory
             const GemmPart* const list0_part = &p.part[part_of(p, (int)blockIdx.x)];
-            const int list0_m = ((int)blockIdx.x - list0_part->tile0) % p.num_m, list0_n = ((int)blockIdx.x - list0_part->tile0) / p.num_m;
+            const int list0_m = ((int)blockIdx.x - list0_part->tile0) % num_mt * kRowTiles, list0_n = ((int)blockIdx.x - list0_part->tile0) / num_mt;
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -469,7 +481,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                 const uint32_t acc_flag = (ordinal & 1) ? kStageAcc1 : 0u;
                 // (a k-block of a pass is at most 24 KB: two share a stage, so that as many bytes are on their way
                 // as in the tiles' stages)
-                const int sub_bytes = Cfg::kABytes + sp.n * (kChunk * kBK * 2);
+                const int sub_bytes = Cfg::kXBytes + sp.n * (kChunk * kBK * 2);
                 const int per_stage = 2 * sub_bytes <= Cfg::kStageBytes ? 2 : 1;
                 for (int kb = 0; kb < num_kb && ok; kb += per_stage) {
                     ok = acquire();
@@ -483,7 +495,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                         const uint32_t a_dst = tiles_addr + stage * Cfg::kStageBytes + j * sub_bytes;
                         tma_load_2d(a_dst, &p.x, bar, (kb + j) * kBK, sp.m * kBM);
                         for (int i = 0; i < sp.n; ++i)
-                            tma_load_3d(a_dst + Cfg::kABytes + i * (kChunk * kBK * 2), &p.a, bar, (kb + j) * kBK, sp.c[i] * kChunk, sp.slot[i]);
+                            tma_load_3d(a_dst + Cfg::kXBytes + i * (kChunk * kBK * 2), &p.a, bar, (kb + j) * kBK, sp.c[i] * kChunk, sp.slot[i]);
                     }
                     advance();
                 }
@@ -510,9 +522,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                     if (!good) break;
                     const uint32_t a_dst = tiles_addr + st * Cfg::kStageBytes;
                     const uint32_t bar = smem_u32(&ctrl->full[st]);
+                    const bool second = kTall && row0 + kBM < p.T;
                     ctrl->stage_info[st] = 4u | acc_flag | (kb == 0 ? kStageFresh : 0u) | (kb == num_kb - 1 ? flags_last : 0u);
-                    mbar_arrive_expect_tx(bar, (uint32_t)(p.x_bytes + (kb < have_w ? 0 : Cfg::kBBytes)));
+                    mbar_arrive_expect_tx(bar, (uint32_t)(p.x_bytes + (second ? p.x_bytes : 0) + (kb < have_w ? 0 : Cfg::kBBytes)));
                     tma_load_2d(a_dst, &p.x, bar, kb * kBK, row0);
+                    if (second) tma_load_2d(a_dst + Cfg::kXBytes, &p.x, bar, kb * kBK, row0 + kBM);
                     if (kb >= have_w) tma_load_2d(a_dst + Cfg::kABytes, w, bar, kb * kBK, col0);
                     if (++st == Cfg::kStages) { st = 0; ph ^= 1u; }
                 }
@@ -520,7 +534,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             };
             for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++ordinal) {
                 const GemmPart& pt = p.part[part_of(p, tile)];
-                const int m = (tile - pt.tile0) % p.num_m, n = (tile - pt.tile0) / p.num_m;
+                const int m = (tile - pt.tile0) % num_mt * kRowTiles, n = (tile - pt.tile0) / num_mt;
                 const int row0 = m * kBM;
                 const uint32_t acc_flag = (ordinal & 1) ? kStageAcc1 : 0u;
                 const int mid = min((num_kb + 1) / 2, num_kb - 1);
@@ -538,8 +552,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                 learn_lora();
                 if (!ok) break;
                 const bool chunks = has_chunks(pt, m, n, kChunkFirst);
-                base_blocks(&pt.w, row0, n * BN, num_kb - 1, num_kb, acc_flag, chunks ? 0u : kStageCommit, ordinal == 0 ? ahead : 0);
-                if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, acc_flag, 0u, kStageCommit);
+                if constexpr (kTall) {
+                    const bool chunks1 = m + 1 < p.num_m && has_chunks(pt, m + 1, n, kChunkFirst);
+                    base_blocks(&pt.w, row0, n * BN, num_kb - 1, num_kb, 0u, (chunks ? kStageMore0 : 0u) | (chunks1 ? kStageMore1 : 0u), ordinal == 0 ? ahead : 0);
+                    if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, 0u, 0u, kStageCommit);
+                    if (ok && chunks1) emit_chunks(pt, pt.u, m + 1, n, kChunkFirst, 0u, 0u, kStageCommit);
+                } else {
+                    base_blocks(&pt.w, row0, n * BN, num_kb - 1, num_kb, acc_flag, chunks ? 0u : kStageCommit, ordinal == 0 ? ahead : 0);
+                    if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, acc_flag, 0u, kStageCommit);
+                }
                 prev_m = m; prev_n = n;
             }
             if (ok && dual && prev_m >= 0) {
@@ -577,7 +598,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                 if (++stage == Cfg::kStages) { stage = 0; phase ^= 1u; }
             };
             // `count` k-blocks without a side-band word: the loop that the tensor cores wait for; its state lives in registers
-            auto base_stages = [&](uint32_t d_tmem, int count, uint32_t& accumulate) {
+            // (tall tiles: both halves, the second's product right behind the first's)
+            auto base_stages = [&](uint32_t d_tmem, int count, uint32_t& accumulate, bool second) {
                 int st = stage;
                 uint32_t ph = phase, on = accumulate;
                 bool good = true;
@@ -590,6 +612,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
                         umma_bf16(d_tmem, adesc0 + at + (uint64_t)(k * 2), bdesc0 + at + (uint64_t)(k * 2), idesc, k == 0 ? on : 1u);
+                    if (kTall && second) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            umma_bf16(d_tmem + (uint32_t)BN, adesc0 + at + (uint64_t)(Cfg::kXBytes / 16 + k * 2), bdesc0 + at + (uint64_t)(k * 2), idesc, k == 0 ? on : 1u);
+                    }
                     on = 1u;
                     umma_commit(empty0 + 8u * (uint32_t)st);
                     if (++st == Cfg::kStages) { st = 0; ph ^= 1u; }
@@ -636,13 +663,13 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                     const uint32_t info = ctrl->stage_info[stage];
                     more = (info & kStageCommit) == 0;
                     const int nch = (int)((info >> 16) & 7u), nsub = (int)((info >> 20) & 3u);
-                    const int sub_bytes = Cfg::kABytes + nch * (kChunk * kBK * 2);
+                    const int sub_bytes = Cfg::kXBytes + nch * (kChunk * kBK * 2);
                     const uint32_t idesc_n = umma_idesc_bf16(kBM, nch * kChunk);
                     tc_fence_after();
                     for (int j = 0; j < nsub; ++j) {
                         const uint32_t a_addr = tiles_addr + stage * Cfg::kStageBytes + j * sub_bytes;
                         const uint64_t adesc = umma_desc_k128(a_addr);
-                        const uint64_t bdesc = umma_desc_k128(a_addr + Cfg::kABytes);
+                        const uint64_t bdesc = umma_desc_k128(a_addr + Cfg::kXBytes);
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
                             umma_bf16(d_tmem, adesc + (uint64_t)(k * 2), bdesc + (uint64_t)(k * 2), idesc_n, (!fresh || k > 0) ? 1u : 0u);
@@ -653,7 +680,29 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                 }
                 if (ok) umma_commit(smem_u32(&ctrl->tmem_full[acc]));
             }
-            for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++ordinal) {
+            for (int tile = blockIdx.x; kTall && tile < num_tiles && ok; tile += gridDim.x) {
+                const GemmPart& pt = p.part[part_of(p, tile)];
+                const bool second = (tile - pt.tile0) % num_mt * kRowTiles + 1 < p.num_m;
+                ok = mbar_wait(smem_u32(&ctrl->tmem_empty[0]), empty_ph0 ^ 1u, abort);
+                if (ok && second) ok = mbar_wait(smem_u32(&ctrl->tmem_empty[1]), empty_ph1 ^ 1u, abort);
+                if (!ok) break;
+                empty_ph0 ^= 1u;
+                if (second) empty_ph1 ^= 1u;
+                tc_fence_after();
+                uint32_t accumulate = 0;
+                base_stages(tmem_base, num_kb - 1, accumulate, second);
+                if (!ok) break;
+                ok = mbar_wait(smem_u32(&ctrl->full[stage]), phase, abort);
+                if (!ok) break;
+                const uint32_t info = ctrl->stage_info[stage];
+                base_stages(tmem_base, 1, accumulate, second);
+                if (info & kStageMore0) flagged_stages(0, accumulate);
+                else umma_commit(smem_u32(&ctrl->tmem_full[0]));
+                if (!ok || !second) continue;
+                if (info & kStageMore1) flagged_stages(1, accumulate);
+                else umma_commit(smem_u32(&ctrl->tmem_full[1]));
+            }
+            for (int tile = blockIdx.x; !kTall && tile < num_tiles && ok; tile += gridDim.x, ++ordinal) {
                 const int acc = ordinal & 1;
                 uint32_t& eph = acc ? empty_ph1 : empty_ph0;
                 ok = mbar_wait(smem_u32(&ctrl->tmem_empty[acc]), eph ^ 1u, abort);
@@ -665,11 +714,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                 int from = 0;
                 if (dual && ordinal > 0) {
                     from = min((num_kb + 1) / 2, num_kb - 1);
-                    base_stages(d_tmem, from, accumulate);
+                    base_stages(d_tmem, from, accumulate, false);
                     if (ok) delta_stages(acc ^ 1);
                     if (!ok) break;
                 }
-                base_stages(d_tmem, num_kb - 1 - from, accumulate);
+                base_stages(d_tmem, num_kb - 1 - from, accumulate, false);
                 if (!ok) break;
                 flagged_stages(acc, accumulate);   // the last k-block and the tile's LoRA pieces
             }
@@ -679,18 +728,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
         // ------------------------------------------------------------------ epilogue warps
         const int q = warp & 3;                 // TMEM lane quarter this warp may read
         const int ew = warp - 2;
-        const uint32_t buf_addr0 = epi_addr + (uint32_t)(ew * 2 * kEpiBufBytes);
-        uint8_t* buf_ptr0 = epi_ptr + ew * 2 * kEpiBufBytes;
+        const int group = ew >> 2;              // tall tiles: the row tile, and accumulator, of these four warps
+        constexpr int kBufs = Cfg::kEpiBufs;    // staging buffers of a warp
+        const uint32_t buf_addr0 = epi_addr + (uint32_t)(ew * kBufs * kEpiBufBytes);
+        uint8_t* buf_ptr0 = epi_ptr + ew * kBufs * kEpiBufBytes;
         int acc = 0;
         uint32_t full_ph0 = 0, full_ph1 = 0;
         int buf = 0;
         bool ok = true;
         if (p.lora && !p.fused && warp == 2) {   // nothing else to do yet: the first tile's chunks, as soon as they are known
             const GemmPart& pt = p.part[part_of(p, (int)blockIdx.x)];
-            if (p.x_flag) prefetch_b<BN>(pt, ((int)blockIdx.x - pt.tile0) / p.num_m, lane, 0, 1);
+            if (p.x_flag) prefetch_b<BN>(pt, ((int)blockIdx.x - pt.tile0) / num_mt, lane, 0, 1);
             grid_dependency_wait();
             grid_launch_dependents();
-            const int n = list_chunks(pt.plan + ((int)blockIdx.x - pt.tile0) % p.num_m, kChunkFirst | kChunkSecond, 0, 1, lane, list0);
+            const int n = list_chunks(pt.plan + ((int)blockIdx.x - pt.tile0) % num_mt * kRowTiles, kChunkFirst | kChunkSecond, 0, 1, lane, list0);
             __syncwarp();
             if (lane == 0) { ctrl->listed[0] = n; mbar_arrive(smem_u32(&ctrl->plan_full)); }
         }
@@ -698,6 +749,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
         // flag goes up (release: the four warps' stores are complete)
         for (int ps = 0; p.fused && ps < shr->npass && ok; ++ps) {
             const ShrPass& sp = shr->pass[ps];
+            if (kTall && (ps & 1) != group) { acc ^= 1; continue; }
             uint32_t& fph = acc ? full_ph1 : full_ph0;
             ok = mbar_wait_warp(smem_u32(&ctrl->tmem_full[acc]), fph, abort);
             if (!ok) break;
@@ -742,13 +794,17 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             if (lane == 0) mbar_arrive(smem_u32(&ctrl->tmem_empty[acc]));
             fence_proxy_async_all();   // the blocks will be read by TMA
             __threadfence();
-            asm volatile("bar.sync 1, 128;" ::: "memory");   // the four epilogue warps
-            if (warp == 2 && lane == 0) st_release_gpu_s32(p.tile_flags + sp.flag, shr->epoch + 1);
+            asm volatile("bar.sync %0, 128;" ::"r"(1 + group) : "memory");   // the four epilogue warps of the accumulator
+            if ((ew & 3) == 0 && lane == 0) st_release_gpu_s32(p.tile_flags + sp.flag, shr->epoch + 1);
             acc ^= 1;
         }
         for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
             const GemmPart& pt = p.part[part_of(p, tile)];
-            const int m = (tile - pt.tile0) % p.num_m, n = (tile - pt.tile0) / p.num_m;
+            const int m = (tile - pt.tile0) % num_mt * kRowTiles + group, n = (tile - pt.tile0) / num_mt;
+            if (kTall) {
+                acc = group;
+                if (m >= p.num_m) continue;
+            }
             const int row_base = m * kBM + q * 32;
             for (int pass = 0; pass < (dual ? 2 : 1) && ok; ++pass) {
                 uint32_t& fph = acc ? full_ph1 : full_ph0;
@@ -773,7 +829,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                     const int col0 = n * BN + c * kEpiChunkCols;
                     if (col0 >= pt.N || row_base >= p.T) continue;   // nothing of this chunk is inside y
                     // the buffer we are about to overwrite must have been read by its earlier store
-                    if (lane == 0) tma_store_wait_read<1>();
+                    if (lane == 0) tma_store_wait_read<kBufs - 1>();
                     __syncwarp();
                     uint8_t* bp = buf_ptr0 + buf * kEpiBufBytes;
                     const uint32_t ba = buf_addr0 + (uint32_t)(buf * kEpiBufBytes);
@@ -795,7 +851,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                         else tma_store_2d(&p.y2, ba, col0, row_base);
                         tma_store_commit();
                     }
-                    buf ^= 1;
+                    buf = kBufs == 2 ? buf ^ 1 : 0;
                 }
             }
             acc ^= 1;
@@ -1141,9 +1197,11 @@ cudaError_t gemm_sm100_init(int /*device*/)
     cudaError_t e = cudaFuncSetAttribute(lora_gemm_sm100_splitk_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          GemmCfg<64>::split_smem(GemmCfg<64>::kStages));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<64>::kSmemBytes);
+    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<64>::kSmemBytes);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<256, true>::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          GemmCfg<256>::kSmemBytes);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(lora_gemm_sm100_splitk_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1152,7 +1210,7 @@ cudaError_t gemm_sm100_init(int /*device*/)
     e = cudaFuncSetAttribute(lora_gemm_sm100_splitk_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              GemmCfg<128>::split_smem(GemmCfg<128>::kStages));
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(lora_gemm_sm100_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(lora_gemm_sm100_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 GemmCfg<128>::kSmemBytes);
 }
 
@@ -1164,8 +1222,8 @@ bool gemm_split_override(int* bn_out, int* split_out)
     const char* e = getenv("LML_GEMM_SPLIT");
     if (!e) return false;
     int bn = 0, sp = 0;
-    if (sscanf(e, "%dx%d", &bn, &sp) == 2 && (bn == 64 || bn == 128 || bn == 256) && sp >= 1 && sp <= kSplitMaxS &&
-        sp * ((bn / 32 + sp - 1) / sp) * 16384 <= GemmCfg<128>::kStages * GemmCfg<128>::kStageBytes) {
+    if (sscanf(e, "%dx%d", &bn, &sp) == 2 && (bn == 64 || bn == 128 || bn == 256 || (bn == 512 && sp == 1)) && sp >= 1 && sp <= kSplitMaxS &&
+        (sp == 1 ? 0 : sp) * ((bn / 32 + sp - 1) / sp) * 16384 <= GemmCfg<128>::kStages * GemmCfg<128>::kStageBytes) {
         *bn_out = bn; *split_out = sp;
     } else {
         *bn_out = 0; *split_out = 0;
@@ -1185,7 +1243,7 @@ static int gemm_exchange_bytes(int bn, int split) { return split * ((bn / 32 + s
 // machine can hold.  More tiles than SMs: rounds of tiles times the tensor time of a k-block.  Fewer: a CTA's k-blocks come
 // through its ring at one round of the ring per trip to memory, 1.5 us while W0 streams (measured at 128 tokens, us per
 // k-block: 256 columns whole-K 0.37, 128 columns 0.265; with the short rings of the split-K kernel 0.52 and 0.40).
-GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, int num_sms, int split_bn, int split_s)
+GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, int num_sms, int split_bn, int split_s)
 {
     static int max_clusters[3][kSplitMaxS + 1];   // for 64, 128 and 256 columns
     static std::once_flag probed;
@@ -1215,9 +1273,15 @@ GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, int num_sms
         for (int p = 0; p < P; ++p) tiles += num_m * ((d_outs[p] + bn - 1) / bn);
         return tiles;
     };
-    if (split_bn > 0) return {split_bn, split_s, tiles_of(split_bn) * split_s};
+    if (split_bn == 512 && !dual) {   // (a test knob: tall tiles)
+        int tiles = 0;
+        for (int p = 0; p < P; ++p) tiles += (num_m + 1) / 2 * ((d_outs[p] + 255) / 256);
+        return {256, 1, tiles, true};
+    }
+    if (split_bn == 512) split_bn = 0;
+    if (split_bn > 0) return {split_bn, split_s, tiles_of(split_bn) * split_s, false};
     const bool crowded = tiles_of(256) > num_sms;
-    GemmShape best = {256, 1, tiles_of(256)};
+    GemmShape best = {256, 1, tiles_of(256), false};
     float best_us = 1e30f;
     for (int w = 2; w >= (crowded ? 1 : 0); --w) {
         const int bn = 64 << w, tiles = tiles_of(bn);
@@ -1231,14 +1295,22 @@ GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, int num_sms
             const int waves = (tiles + fit - 1) / fit;
             float us;
             if (crowded) {
-                us = (float)(waves * num_kb) * (w == 2 ? 0.31f : 0.254f);
+                us = (float)(waves * num_kb) * (w == 2 ? 0.415f : 0.34f);
             } else {
                 const int stages = S > 1 && !beside ? gemm_stages_short(bn) : gemm_stages(bn);
                 us = (w == 2 ? 12.5f : (w == 1 ? 10.f : 8.f)) + (S > 1 ? 1.f : 0.f) + (S > 1 && !beside ? 4.f : 0.f) +
                      (float)waves * (float)((num_kb + S - 1) / S) * 1.55f / (float)stages;
             }
-            if (us < best_us * 0.999f) { best_us = us; best = {bn, S, tiles * S}; }
+            if (us < best_us * 0.999f) { best_us = us; best = {bn, S, tiles * S, false}; }
         }
+    }
+    if (crowded && !dual && num_m > 1 && best.split == 1) {
+        // Tall tiles: 0.71 us per k-block against twice 0.415 (2048 tokens, us per call without adapters, single / tall:
+        // 4096 x 4096 55.9 / 50.4, 4096 x 11008 145.5 / 127.0; 8192 tokens, 11008 x 4096 581 / 546).
+        int tiles = 0;
+        for (int p = 0; p < P; ++p) tiles += (num_m + 1) / 2 * ((d_outs[p] + 255) / 256);
+        const float us = (float)((tiles + num_sms - 1) / num_sms) * ((float)num_kb * 0.71f);
+        if (us < best_us) best = {256, 1, tiles, true};
     }
     return best;
 }
@@ -1275,9 +1347,11 @@ bool gemm_can_fuse_shrink(const GemmShape& shape, int T, int d_out, int G, bool 
     if (G <= 0 || (in_segment_order && G > kBindSegs)) return false;
     if (shape.split != 1 || shape.bn != 256) return false;
     const int num_m = (T + kBM - 1) / kBM, num_n = (d_out + 255) / 256;
-    if (num_m > kFuseTilesInKernel || num_m * num_n <= num_sms) return false;
+    if (num_m > kFuseTilesInKernel || (!shape.tall && num_m * num_n <= num_sms)) return false;
     int worst_passes = num_m * ((cap + kShrChunks - 1) / kShrChunks);
     if (in_segment_order && num_m + G < worst_passes) worst_passes = num_m + G;
+    // (tall tiles: only as many passes as there are CTAs with a tile less than the others, or none)
+    if (shape.tall) return worst_passes <= num_sms - (shape.ctas - 1) % num_sms - 1;
     return worst_passes <= num_sms / 2;
 }
 
@@ -1313,7 +1387,7 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
             }
         pt.N = pr.d_out; pt.num_n = (pr.d_out + bn - 1) / bn; pt.n_pad = b_rows_padded(pr.d_out); pt.cap = pr.cap;
         pt.tile0 = tiles;
-        tiles += p.num_m * pt.num_n;
+        tiles += (a.shape.tall ? (p.num_m + 1) / 2 : p.num_m) * pt.num_n;
         columns += pt.num_n;
     }
     p.y2 = p.part[0].y;
@@ -1328,8 +1402,10 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     // with adapters the predecessor is the bind_shrink launch of this call, else the kernel waits at its top
-    pdl_config(cfg, attr, dim3((unsigned)(tiles < a.num_sms ? tiles : a.num_sms)), dim3(kGemmThreads),
-               bn == 256 ? GemmCfg<256>::kSmemBytes : (bn == 128 ? GemmCfg<128>::kSmemBytes : GemmCfg<64>::kSmemBytes), stream);
+    const bool tall = a.shape.tall;
+    // (tall tiles with the shrink inside: the SMs without a tile take its passes)
+    pdl_config(cfg, attr, dim3((unsigned)(tiles < a.num_sms && !(tall && a.fused) ? tiles : a.num_sms)), dim3(tall ? kGemmThreadsTall : kGemmThreads),
+               tall ? GemmCfg<256, true>::kSmemBytes : bn == 256 ? GemmCfg<256>::kSmemBytes : (bn == 128 ? GemmCfg<128>::kSmemBytes : GemmCfg<64>::kSmemBytes), stream);
     p.stages = 0;
     if (split > 1) {
         p.stages = a.share_sm && gemm_exchange_bytes(bn, split) <= gemm_stages_short(bn) * gemm_stage_bytes(bn) ? gemm_stages_short(bn) : gemm_stages(bn);
@@ -1344,9 +1420,10 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
         if (bn == 64) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_splitk_kernel<64>, p);
         return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_splitk_kernel<128>, p);
     }
-    if (bn == 256) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<256>, p, *a.proj[0].snap);
-    if (bn == 64) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<64>, p, *a.proj[0].snap);
-    return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<128>, p, *a.proj[0].snap);
+    if (tall) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<256, true>, p, *a.proj[0].snap);
+    if (bn == 256) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<256, false>, p, *a.proj[0].snap);
+    if (bn == 64) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<64, false>, p, *a.proj[0].snap);
+    return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<128, false>, p, *a.proj[0].snap);
 }
 
 }  // namespace lml

@@ -164,8 +164,9 @@ struct GemmProj {
     const __nv_bfloat16* u;
     int cap;
 };
-// What the library takes for a call: width of an output tile and CTAs that share one (1: whole-K tiles), CTAs in all.
-struct GemmShape { int bn, split, ctas; };
+// What the library takes for a call: width of an output tile and CTAs that share one (1: whole-K tiles), CTAs in all, and
+// whether a whole-K tile is two row tiles high.
+struct GemmShape { int bn, split, ctas; bool tall; };
 struct GemmArgs {
     const void* x;
     int T, d_in, P;
@@ -184,7 +185,7 @@ struct GemmArgs {
     int num_sms;
 };
 // split_bn, split_s: the table's override (-1 = the library chooses, 0 = whole-K tiles, else the forced shape)
-GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, int num_sms, int split_bn, int split_s);
+GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, int num_sms, int split_bn, int split_s);
 // whether the shrink of a plain call of this size and shape runs inside the GEMM kernel; cap: chunks per tile at most
 bool gemm_can_fuse_shrink(const GemmShape& shape, int T, int d_out, int G, bool in_segment_order, int cap, int num_sms);
 // Tensor maps of caller buffers, kept per table and found again by (pointer, shape, box).
