@@ -322,11 +322,24 @@ def _ptr(t) -> int:
     return 0 if t is None else int(t.data_ptr())
 
 
+_current_raw_stream = None
+
+
 def _stream(stream) -> int:
-    import torch
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return int(stream.cuda_stream)
+    if stream is not None:
+        return int(stream.cuda_stream)
+    # the current stream of the current device, as a number: torch.cuda.current_stream() builds a Stream object for it at
+    # every call (1.5 us of a small call's 17 us)
+    global _current_raw_stream
+    if _current_raw_stream is None:
+        import torch
+        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+        if raw is None:
+            _current_raw_stream = lambda: torch.cuda.current_stream().cuda_stream  # noqa: E731
+        else:
+            device = torch.cuda.current_device
+            _current_raw_stream = lambda: raw(device())  # noqa: E731
+    return int(_current_raw_stream())
 
 
 def fuse_projection_adapters(parts):
