@@ -207,10 +207,12 @@ lml_status lml_segment_tokens(lml_table* t, const int32_t* token_slots, int T, i
  * a small exchange block that belongs to the table, so two decode calls on the SAME table must not overlap on the GPU:
  * put them on one stream or order them; a CTA whose peers are late computes their share itself,
  * so the call completes even when the grid cannot be resident all at once); larger T runs the
- * TMA / tcgen05 GEMM with the LoRA expand as extra tensor-core K-steps.
- * W0 is the frozen base weight: it must not be written by the operation that immediately precedes
- * the call on `stream` (the decode kernel starts fetching W0 while the kernel before it is still
- * draining; x, the segment arrays and the adapters are read only after that kernel has finished).
+ * TMA / tcgen05 GEMM with the LoRA expand as extra tensor-core K-steps (the rows of x stay in
+ * their order, with or without perm; rows that a malformed perm does not name get base output).
+ * W0 is the frozen base weight: it must not be written by work on `stream` that may still be running
+ * when the call is reached (the decode kernel, and the GEMM of a call of few rows, start fetching W0
+ * while the kernel before them is still draining; x, the segment arrays and the adapters are read only
+ * after that kernel has finished).
  * Errors: INVALID_ARG, WORKSPACE, CUDA.
  */
 lml_status lora_mixed_linear(lml_table* t, const void* x, const void* W0, int T,
@@ -274,13 +276,10 @@ lml_status lora_mixed_linear_backward_adapters(lml_table* t, lml_table* t_T, con
  * T <= 16: one launch; the decode kernel treats every row on its own and reads the ids itself, no
  * grouping is computed.  A few blocks of 16 tokens (T <= 48 where d_in * d_out <= 2^24; else T <= 32 where d_in > 4096) are
  * one launch of the same kernel, an equal share of its CTAs per block: every block's rows are bit for
- * bit those of a decode call on that block, and W0 still leaves HBM once.  Beyond that, up to one
- * row tile (T <= 128; two tiles, T <= 256, where d_in <= 4096): two launches, the tokens staying in
- * their order; the first binds them and writes, per row tile and distinct slot, the slot's rows of
- * the shrink result, the GEMM adds them slot by slot.  Larger T: the segmentation pass runs into the
- * tail of the workspace and the perm form of lora_mixed_linear follows on the same stream; results
- * are then identical to lml_segment_tokens followed by lora_mixed_linear (on the other paths they
- * agree with it to fp32 summation order and the bf16 rounding of u).  workspace: device, 256-byte aligned, at least
+ * bit those of a decode call on that block, and W0 still leaves HBM once.  Beyond that: two launches, the
+ * tokens staying in their order; the first binds them and writes, per row tile and 16 columns of every slot
+ * in use, the rows' shrink result, the GEMM adds them.  Results agree with lml_segment_tokens followed by
+ * lora_mixed_linear to fp32 summation order and the bf16 rounding of u.  workspace: device, 256-byte aligned, at least
  * lml_tokens_workspace_bytes(t, T) bytes.  Errors: INVALID_ARG, WORKSPACE, CUDA.
  */
 size_t lml_tokens_workspace_bytes(const lml_table* t, int max_tokens);
@@ -302,8 +301,9 @@ lml_status lora_mixed_linear_tokens(lml_table* t, const void* x, const void* W0,
  * projection are bit for bit those of lora_mixed_linear_tokens on that projection, and the fixed cost of a
  * call (the wait for the preceding work, the fetch of x, the tail) is paid once.  A single projection, or a
  * table named twice, runs as one decode call per projection.
- * T > 16: the projections run one after the other on `stream`, each exactly as
- * lora_mixed_linear_tokens(tables[p], ...).
+ * T > 16: two launches for all projections, one that binds the rows and computes every projection's shrink
+ * result, one GEMM over all projections' tiles; results per projection agree with
+ * lora_mixed_linear_tokens(tables[p], ...) to fp32 summation order and the bf16 rounding of u.
  * Every projection's CTAs count themselves in that table's exchange block, as in a decode call: two calls
  * that share a table must not overlap on the GPU.  Device-detected errors set the flags of the table they
  * concern.
