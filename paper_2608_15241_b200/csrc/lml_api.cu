@@ -663,9 +663,9 @@ static lml_status tokens_impl(lml_table* t, const void* x, const void* W0, int T
         if (e != cudaSuccess) { cudaGetLastError(); return LML_ERR_CUDA; }
         return LML_OK;
     }
-    // (measured on B200 against the one-tile path below, us per call at 20 / 32 / 48 / 64 tokens: 4096 x 4096 13.3 / 13.8 /
-    // 19.8 / 24.1 against 19.1 / 20.1 / 20.6 / 20.6; 11008 x 4096 33.5 / 31.5 against 29.2 / 29.7; 4096 x 11008 31.4 / 32.0
-    // against 27.4 / 35.4: every block's CTAs take all of W0 in from L2, which a wide output pays for at once)
+    // (us per call at 20 / 32 / 48 / 64 tokens: 4096 x 4096 13.3 / 13.8 / 19.8 / 24.1 as blocks against 18.4 on the GEMM path at
+    // 64; 11008 x 4096 33.5 / 31.5 against 27.8; 4096 x 11008 31.4 / 32.0 against 33.9 at 128: every block's CTAs take all of
+    // W0 in from L2, which a wide output pays for at once)
     const bool small_layer = (long long)t->d_in * t->d_out <= (1ll << 24);
     const int block_limit = t->dec_block_tokens >= 0 ? t->dec_block_tokens
                                                      : (small_layer ? 3 : (t->d_in > 4096 ? 2 : 1)) * kDecodeMaxT;
