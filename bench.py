@@ -166,8 +166,8 @@ class Rotation:
     def step(self, i):
         """Whole hot path from one slot id per token: token segmentation + layer, through the call a
         serving loop makes (lora_mixed_linear_tokens).  Up to 16 tokens that is one launch (the decode
-        kernel binds every row to its slot itself); above, the segmentation kernel, the row gather, the
-        shrink kernel and the GEMM."""
+        kernel binds every row to its slot itself); above, the kernel that binds the rows and computes the
+        shrink, and the GEMM."""
         from paper_2608_15241_b200 import binding as b
         s = self.sets[i % self.R]
         t = s["table"]

@@ -35,6 +35,8 @@ WsLayout ws_layout(const lml_table* t, int T, int slots, int u_sets = 1)
     w.total = w.u_off + (size_t)u_sets * u_bytes;
     return w;
 }
+// (calls of one row tile have room for u as two bf16 values)
+WsLayout tokens_layout(const lml_table* t, int T) { return ws_layout(t, T, t->max_slots, T <= kTileM ? 2 : 1); }
 // (a dual call's rows can use a slot per segment and binding)
 WsLayout dual_layout(const lml_table* t, int T, int G) { return ws_layout(t, T, G > kMaxSlots ? kMaxSlots : 2 * G, 2); }
 
@@ -56,9 +58,11 @@ struct GemmCall {
 };
 
 // The GEMM path: the rows stay in their order; one launch binds them and computes u (unless the GEMM does both itself),
-// one launch multiplies.  P > 1: projections of the same x.  ids2 / y2: the second binding of a dual call.
+// one launch multiplies.  P > 1: projections of the same x.  ids2 / y2: the second binding of a dual call.  precise: u goes
+// into the product as two bf16 values (16 bits of significand), a further K-step per chunk.
 cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, RowMode mode, const int32_t* seg_offsets, int G,
-                          const int32_t* perm, const int32_t* ids2, void* y2, bool by_adapter, cudaStream_t stream, int* launches)
+                          const int32_t* perm, const int32_t* ids2, void* y2, bool by_adapter, cudaStream_t stream, int* launches,
+                          bool precise = false)
 {
     lml_table* t0 = calls[0].t;
     const int num_m = (T + kTileM - 1) / kTileM;
@@ -92,7 +96,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         bp.cap = cap;
         GemmProj& gp = g.proj[p];
         gp.W0 = c.W0; gp.y = c.y; gp.d_out = c.t->d_out; gp.ar = &c.t->arena; gp.snap = &snap[p];
-        gp.plan = bp.plan; gp.u = bp.u; gp.cap = cap;
+        gp.plan = bp.plan; gp.u = bp.u; gp.u_lo = precise ? bp.u2 : nullptr; gp.cap = cap;
     }
     g.num_sms = t0->num_sms;
     if (mode == kRowsSegments && (perm || G > kBindSegs || num_m > kSlabTiles)) {   // a slot per row first
@@ -127,6 +131,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
             if (++t0->next_call == 0u) ++t0->next_call;
             b.call_id = g.call_id = t0->next_call;
         }
+        if (precise) b.second = 3;
         if (dual) {
             // (split-K: an accumulator per binding; whole-K tiles: the second output is the first plus the difference)
             b.second = g.shape.split > 1 ? 1 : 2;
@@ -538,7 +543,8 @@ lml_status lora_mixed_linear(lml_table* t, const void* x, const void* W0, int T,
 size_t lml_tokens_workspace_bytes(const lml_table* t, int max_tokens)
 {
     if (!t || max_tokens < 0 || max_tokens > kMaxTokens) return 0;
-    return ws_layout(t, max_tokens, t->max_slots).total;
+    // (more than one tile takes at least as much as one with two values)
+    return tokens_layout(t, max_tokens).total;
 }
 
 size_t lml_dual_workspace_bytes(const lml_table* t, int max_tokens, int max_segments)
@@ -637,6 +643,16 @@ lml_status lora_mixed_linear_backward_adapters(lml_table* t, lml_table* t_T, con
     return LML_OK;
 }
 
+// Token-form calls of up to this many tokens run as blocks of 16 on the decode kernel.
+// (us per call at 20 / 32 / 48 / 64 tokens: 4096 x 4096 13.3 / 13.8 / 19.8 / 24.1 as blocks against 18.4 on the GEMM path at
+// 64; 11008 x 4096 33.5 / 31.5 against 27.8; 4096 x 11008 31.4 / 32.0 against 33.9 at 128: every block's CTAs take all of
+// W0 in from L2, which a wide output pays for at once)
+static int decode_block_limit(const lml_table* t)
+{
+    const bool small_layer = (long long)t->d_in * t->d_out <= (1ll << 24);
+    return t->dec_block_tokens >= 0 ? t->dec_block_tokens : (small_layer ? 3 : (t->d_in > 4096 ? 2 : 1)) * kDecodeMaxT;
+}
+
 static lml_status tokens_impl(lml_table* t, const void* x, const void* W0, int T, const int32_t* token_slots, void* y,
                               void* workspace, size_t workspace_bytes, void* stream_v, bool by_adapter)
 {
@@ -663,12 +679,7 @@ static lml_status tokens_impl(lml_table* t, const void* x, const void* W0, int T
         if (e != cudaSuccess) { cudaGetLastError(); return LML_ERR_CUDA; }
         return LML_OK;
     }
-    // (us per call at 20 / 32 / 48 / 64 tokens: 4096 x 4096 13.3 / 13.8 / 19.8 / 24.1 as blocks against 18.4 on the GEMM path at
-    // 64; 11008 x 4096 33.5 / 31.5 against 27.8; 4096 x 11008 31.4 / 32.0 against 33.9 at 128: every block's CTAs take all of
-    // W0 in from L2, which a wide output pays for at once)
-    const bool small_layer = (long long)t->d_in * t->d_out <= (1ll << 24);
-    const int block_limit = t->dec_block_tokens >= 0 ? t->dec_block_tokens
-                                                     : (small_layer ? 3 : (t->d_in > 4096 ? 2 : 1)) * kDecodeMaxT;
+    const int block_limit = decode_block_limit(t);
     if (T <= block_limit) {
         // A few blocks of 16 tokens: one launch of the decode kernel with the blocks as its parts, an equal share of the
         // CTAs each.  The shares walk W0 together, so a line leaves HBM once and the other readers find it in L2; no
@@ -702,7 +713,7 @@ static lml_status tokens_impl(lml_table* t, const void* x, const void* W0, int T
     DeviceGuard guard(t->device);
     if (!guard.ok) return LML_ERR_CUDA;
     int launches = 0;
-    const GemmCall c = {t, W0, y, token_slots, static_cast<uint8_t*>(workspace), ws_layout(t, T, t->max_slots)};
+    const GemmCall c = {t, W0, y, token_slots, static_cast<uint8_t*>(workspace), tokens_layout(t, T)};
     const cudaError_t e = run_gemm_path(&c, 1, x, T, kRowsTokens, nullptr, 0, nullptr, nullptr, nullptr, by_adapter, stream, &launches);
     t->last_launches = launches;
     if (e != cudaSuccess) { cudaGetLastError(); return LML_ERR_CUDA; }
@@ -790,13 +801,17 @@ lml_status lora_mixed_linear_multi(lml_table* const* tables, int P, const void* 
         DeviceGuard guard(tables[0]->device);
         if (!guard.ok) return LML_ERR_CUDA;
         GemmCall calls[LML_MAX_PROJECTIONS];
+        // A call of its own would run as blocks of 16 tokens on the decode kernel, which keeps u in fp32: the shared launches
+        // carry it as two bf16 values then.
+        bool precise = false;
         size_t off = 0;
         for (int p = 0; p < P; ++p) {
-            calls[p] = GemmCall{tables[p], W0[p], y[p], token_slots[p], static_cast<uint8_t*>(workspace) + off, ws_layout(tables[p], T, tables[p]->max_slots)};
+            calls[p] = GemmCall{tables[p], W0[p], y[p], token_slots[p], static_cast<uint8_t*>(workspace) + off, tokens_layout(tables[p], T)};
+            precise = precise || T <= decode_block_limit(tables[p]);
             off += round_up(calls[p].layout.total, 1024);
         }
         int launches = 0;
-        const cudaError_t e = run_gemm_path(calls, P, x, T, kRowsTokens, nullptr, 0, nullptr, nullptr, nullptr, false, stream, &launches);
+        const cudaError_t e = run_gemm_path(calls, P, x, T, kRowsTokens, nullptr, 0, nullptr, nullptr, nullptr, false, stream, &launches, precise);
         if (e != cudaSuccess) { cudaGetLastError(); return LML_ERR_CUDA; }
         for (int p = P - 1; p >= 0; --p) tables[p]->last_launches = p == 0 ? launches : 0;
         return LML_OK;

@@ -63,7 +63,7 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
     const int m = (int)blockIdx.z % B.num_m, pi = (int)blockIdx.z / B.num_m;
     const BindPart& part = L.part[pi];
     const SlotSnapshot& snap = L.snap[pi];
-    const bool dual = L.second != 0;
+    const bool dual = L.second == 1 || L.second == 2;
     const bool first_cta = r == 0 && blockIdx.y == 0;
     const int num_kb = (L.d_in + 63) / 64;
     const int kb0 = r * num_kb / S, kb1 = (r + 1) * num_kb / S, nkb = kb1 - kb0;
@@ -302,6 +302,11 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
             const uint2 zero = make_uint2(0u, 0u);
             const size_t at = ((size_t)m * part.cap + c0 + (piece >> 2)) * (kTileM * kChunk) + chunk_elem(tr, (piece & 3) * 4);
             *reinterpret_cast<uint2*>(part.u + at) = a ? val : zero;
+            if (L.second == 3) {
+                const uint2 lo = make_uint2(pack_bf16(v.x * sc - bf16_lo(val.x), v.y * sc - bf16_hi(val.x)),
+                                            pack_bf16(v.z * sc - bf16_lo(val.y), v.w * sc - bf16_hi(val.y)));
+                *reinterpret_cast<uint2*>(part.u2 + at) = a ? lo : zero;
+            }
             if (dual) {
                 // (the blocks of the second binding, or of the difference of the two)
                 const uint2 neg = make_uint2(val.x ^ 0x80008000u, val.y ^ 0x80008000u);

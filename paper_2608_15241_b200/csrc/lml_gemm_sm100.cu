@@ -114,6 +114,7 @@ struct alignas(64) GemmPart {
     const __nv_bfloat16* bk;            // the table's packed B, by chunk
     const TilePlan* plan;               // [row tile] its chunks
     const __nv_bfloat16* u;
+    const __nv_bfloat16* u_lo;          // or null: what u's bf16 values leave, a further K-step per chunk
     __nv_bfloat16* y_ptr;
     unsigned long long live;            // slots that hold an adapter
     unsigned long long nch[2];          // ... their chunks less one, two bits each
@@ -440,8 +441,9 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                     if (!ok) break;
                     const uint32_t a_dst = tiles_addr + stage * Cfg::kStageBytes, bar = smem_u32(&ctrl->full[stage]);
                     int k = 0;
-                    while (k < 4 && e >= 0) {
+                    while (k < (pt.u_lo ? 3 : 4) && e >= 0) {
                         load_chunk<BN>(pt, u, m, n, (uint32_t)e, index, k++, a_dst, a_dst + Cfg::kABytes, bar);
+                        if (pt.u_lo) load_chunk<BN>(pt, pt.u_lo, m, n, (uint32_t)e, index, k++, a_dst, a_dst + Cfg::kABytes, bar);
                         e = next();
                     }
                     ctrl->stage_info[stage] = (uint32_t)k | acc_flag | kStageChunks | (first ? flags_first : 0u) | (e < 0 ? flags_last : 0u);
@@ -984,13 +986,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
                     const __nv_bfloat16* u = side ? p.u2 : pt.u;
                     const uint32_t* list = lists + side * kMaxChunks;
                     const int count = ctrl->listed[side];
-                    for (int i = 0; i < count && ok; i += 4) {
+                    const int per = pt.u_lo ? 2 : 4;   // chunks to a stage
+                    for (int i = 0; i < count && ok; i += per) {
                         ok = acquire();
                         if (!ok) break;
                         const uint32_t a_dst = tiles_addr + stage * Cfg::kStageBytes, bar = smem_u32(&ctrl->full[stage]);
-                        const int nk = min(4, count - i);
-                        for (int k = 0; k < nk; ++k)
-                            load_chunk<BN>(pt, u, m, n, list[i + k] & 0xffffu, (int)(list[i + k] >> 16), k, a_dst, a_dst + Cfg::kABytes, bar);
+                        int nk = 0;
+                        for (int q = i; q < min(i + per, count); ++q) {
+                            load_chunk<BN>(pt, u, m, n, list[q] & 0xffffu, (int)(list[q] >> 16), nk++, a_dst, a_dst + Cfg::kABytes, bar);
+                            if (pt.u_lo) load_chunk<BN>(pt, pt.u_lo, m, n, list[q] & 0xffffu, (int)(list[q] >> 16), nk++, a_dst, a_dst + Cfg::kABytes, bar);
+                        }
                         ctrl->stage_info[stage] = (uint32_t)nk | kStageChunks | (side ? kStageAcc1 : 0u);
                         mbar_arrive(bar);
                         advance();
@@ -1378,7 +1383,7 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
         } else {
             pt.y = pt.w;
         }
-        pt.bk = pr.ar->Bk; pt.plan = pr.plan; pt.u = pr.u; pt.y_ptr = (__nv_bfloat16*)pr.y;
+        pt.bk = pr.ar->Bk; pt.plan = pr.plan; pt.u = pr.u; pt.u_lo = pr.u_lo; pt.y_ptr = (__nv_bfloat16*)pr.y;
         pt.live = pt.nch[0] = pt.nch[1] = 0ull;
         for (int s = 0; s < pr.snap->max_slots; ++s)
             if (pr.snap->rank[s] > 0) {

@@ -131,7 +131,7 @@ struct BindPart {
     uint32_t* status;
     TilePlan* plan;               // [row tile]
     __nv_bfloat16* u;
-    __nv_bfloat16* u2;            // dual calls: a second set of blocks
+    __nv_bfloat16* u2;            // a second set of blocks (see BindArgs::second)
     int cap;
     int pad;
 };
@@ -139,7 +139,8 @@ struct BindArgs {
     const void* x;
     int T, d_in, P;
     RowSource rows;
-    int second = 0;   // dual calls, what u2 holds: 1 the second binding's blocks, 2 second minus first
+    // what u2 holds: dual calls 1 the second binding's blocks, 2 second minus first; else 3 the rest of u beyond its bf16 value
+    int second = 0;
     // early start of the GEMM (see bind_starts_gemm_early): the word that says "x may be read" and this call's value of it
     uint32_t* x_flag = nullptr;
     uint32_t call_id = 0;
@@ -162,6 +163,7 @@ struct GemmProj {
     const SlotSnapshot* snap;
     const TilePlan* plan;
     const __nv_bfloat16* u;
+    const __nv_bfloat16* u_lo;   // or null: the rest of u, multiplied with the same B
     int cap;
 };
 // What the library takes for a call: width of an output tile and CTAs that share one (1: whole-K tiles), CTAs in all, and

@@ -183,3 +183,19 @@ def test_seven_b_class_qkv_decode():
     x, W, ents, tok = _case(0, K, Ns, ranks, scales, T, none_every=100)
     out, sep, flags = _run_multi(K, Ns, x, W, ents, tok, reorder=False)
     _check(out, sep, flags, x, W, ents, tok)
+
+
+@pytest.mark.parametrize("T", [17, 33, 48])
+@pytest.mark.parametrize("K,Ns", [(520, (264, 136, 1000)), (2048, (2056, 1032))])
+def test_projections_of_a_few_blocks_of_tokens_keep_u_beyond_bf16(T, K, Ns):
+    """17 - 48 tokens: a call of its own keeps u in fp32 (decode kernel); the shared launches carry it as two bf16 values, so
+    the outputs stay as close to the fp64 result."""
+    ranks = [(16, 64, 4, 8), (8, 16, 33, 1), (64, 33, 16, 2)][:len(Ns)]
+    scales = [(40.0, 50.0, 100.0, 40.0), (100.0, 20.0, 25.0, 300.0), (50.0, 15.0, 200.0, 100.0)][:len(Ns)]
+    x, W, ents, tok = _case(500 + T, K, Ns, ranks, scales, T)
+    out, sep, flags = _run_multi(K, Ns, x, W, ents, tok)
+    assert flags == [0] * len(Ns)
+    for p in range(len(Ns)):
+        ref, _ = oracle.forward(x, W[p], ents[p], np.arange(T + 1, dtype=np.int32), tok)
+        err = [np.linalg.norm(wl.bf16_bits_to_f64(y) - ref) / np.linalg.norm(ref) for y in (out[p], sep[p])]
+        assert err[0] <= 1.01 * err[1], (p, err)     # (both are the rounding of y; u rounded to bf16 would add 2^-9 / sqrt(3) of the LoRA term)
