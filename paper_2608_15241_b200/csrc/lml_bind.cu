@@ -107,12 +107,12 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
     int s_a = -1, s_b = -1;
     if (L.rows.mode == kRowsSegments) {
         int bad_off = 0;
-        for (int g = tid; g <= L.rows.G; g += kBindThreads) ctrl->seg[g] = __ldg(L.rows.seg_offsets + g);
+        for (int g = tid; g <= L.rows.G; g += kBindThreads) ctrl->seg[g] = ld_after_wait(L.rows.seg_offsets + g);
         for (int g = tid; g < L.rows.G; g += kBindThreads) {
-            const int s = __ldg(part.ids + g);
+            const int s = ld_after_wait(part.ids + g);
             ctrl->seg_slot[0][g] = (int8_t)(slot_rank(snap, s) > 0 ? s : (s == -1 ? -1 : -2));
             if (dual) {
-                const int s2 = __ldg(L.rows.ids2 + g);
+                const int s2 = ld_after_wait(L.rows.ids2 + g);
                 ctrl->seg_slot[1][g] = (int8_t)(slot_rank(snap, s2) > 0 ? s2 : (s2 == -1 ? -1 : -2));
             }
         }
@@ -139,7 +139,7 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
         const int row = m * kTileM + row_t;
         if (row < L.T) {
             if (L.rows.mode == kRowsTokens) {
-                s_a = __ldg(part.ids + row);
+                s_a = ld_after_wait(part.ids + row);
                 if (part.adapter_map) s_a = resolve_adapter(snap, part.adapter_map, s_a);
                 if (s_a != -1 && slot_rank(snap, s_a) == 0) { bad_slot = 1; s_a = -1; }
             } else {
@@ -416,32 +416,34 @@ __global__ void __launch_bounds__(1024) rows_from_segments_kernel(
     const bool cached = G <= kBindSegs;
     int bad_off = 0, bad_slot = 0, bad_perm = 0;
     for (int g = tid; g < G; g += blockDim.x) {
-        const int s0 = __ldg(seg_offsets + g), s1 = __ldg(seg_offsets + g + 1);
+        const int s0 = ld_after_wait(seg_offsets + g), s1 = ld_after_wait(seg_offsets + g + 1);
         if (cached) seg_s[g] = s0;
         if (s1 < s0 || s0 < 0 || s1 > T) bad_off = 1;
-        const int s = __ldg(slot_ids + g), s2 = slot_ids2 ? __ldg(slot_ids2 + g) : -1;
+        const int s = ld_after_wait(slot_ids + g), s2 = slot_ids2 ? ld_after_wait(slot_ids2 + g) : -1;
         if (s1 > s0 && ((s != -1 && slot_rank(snap, s) == 0) || (s2 != -1 && slot_rank(snap, s2) == 0))) bad_slot = 1;
     }
     if (tid == 0) {
-        const int last = __ldg(seg_offsets + G);
+        const int last = ld_after_wait(seg_offsets + G);
         if (cached) seg_s[G] = last;
-        if (__ldg(seg_offsets) != 0 || last != T) bad_off = 1;
+        if (ld_after_wait(seg_offsets) != 0 || last != T) bad_off = 1;
     }
     if (perm)   // (rows that a malformed perm does not name get no adapter)
         for (int i = tid; i < T; i += blockDim.x) { rows[i] = -1; if (rows2) rows2[i] = -1; }
     bad_off = __syncthreads_or(bad_off);
     for (int pos = tid; pos < T; pos += blockDim.x) {
-        const int row = perm ? __ldg(perm + pos) : pos;
+        const int row = perm ? ld_after_wait(perm + pos) : pos;
         if (row < 0 || row >= T) { bad_perm = 1; continue; }
         int s = -1, s2 = -1;
         if (!bad_off) {
             int lo = 0, hi = G;
-            if (cached) { while (lo < hi) { const int mid = (lo + hi) >> 1; if (seg_s[mid + 1] > pos) hi = mid; else lo = mid + 1; } }
-            else lo = seg_upper(seg_offsets, G, pos);
+            while (lo < hi) {
+                const int mid = (lo + hi) >> 1;
+                if ((cached ? seg_s[mid + 1] : ld_after_wait(seg_offsets + mid + 1)) > pos) hi = mid; else lo = mid + 1;
+            }
             if (lo < G) {
-                s = __ldg(slot_ids + lo);
+                s = ld_after_wait(slot_ids + lo);
                 if (slot_rank(snap, s) == 0) s = -1;
-                if (slot_ids2) { s2 = __ldg(slot_ids2 + lo); if (slot_rank(snap, s2) == 0) s2 = -1; }
+                if (slot_ids2) { s2 = ld_after_wait(slot_ids2 + lo); if (slot_rank(snap, s2) == 0) s2 = -1; }
             }
         }
         rows[row] = (int8_t)s;

@@ -188,12 +188,12 @@ __device__ __forceinline__ int part_of(const GemmParams& p, int tile)
 // chunks that rows use under the bindings `who` and (rank, S) its share of them.  Returns how many.
 __device__ __forceinline__ int list_chunks(const TilePlan* plan, uint32_t who, int rank, int S, int lane, uint32_t* out)
 {
-    uint32_t e = __ldg(&plan->chunk[lane]);   // (goes out with the count; what lies past it is not used)
-    const int count = __ldg(&plan->count);
+    uint32_t e = ld_after_wait(&plan->chunk[lane]);   // (goes out with the count; what lies past it is not used)
+    const int count = ld_after_wait(&plan->count);
     int n = 0;
     for (int i0 = 0; i0 < count; i0 += 32) {
         const int i = i0 + lane;
-        if (i0 > 0) e = i < count ? (uint32_t)__ldg(&plan->chunk[i]) : 0u;
+        if (i0 > 0) e = i < count ? ld_after_wait(&plan->chunk[i]) : 0u;
         const bool keep = i < count && (e & who) && (S == 1 || (int)((e & 0xffu) + ((e >> 8) & 0xfu)) % S == rank);
         const uint32_t m = __ballot_sync(0xffffffffu, keep);
         if (keep) out[n + __popc(m & ((1u << lane) - 1u))] = ((uint32_t)i << 16) | e;
@@ -293,9 +293,9 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
         for (int m = threadIdx.x; m < p.num_m; m += kThreads) tile_mask[m] = 0ull;
         if (by_segment) {
             const int G = p.rows.G;
-            for (int g = threadIdx.x; g <= G; g += kThreads) seg_cache[g] = __ldg(p.rows.seg_offsets + g);
+            for (int g = threadIdx.x; g <= G; g += kThreads) seg_cache[g] = ld_after_wait(p.rows.seg_offsets + g);
             for (int g = threadIdx.x; g < G; g += kThreads) {
-                const int s = __ldg(p.rows.ids + g);
+                const int s = ld_after_wait(p.rows.ids + g);
                 slot_cache[g] = (int8_t)(slot_rank(snap, s) > 0 ? s : (s == -1 ? -1 : -2));
             }
             __syncthreads();
@@ -413,7 +413,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                 const bool listed = !p.fused && &pt == list0_part && m == list0_m && n == list0_n;
                 unsigned long long mk = p.fused ? tile_mask[m] : 0ull;
                 const TilePlan* plan = pt.plan + m;
-                const int count = p.fused ? 0 : (listed ? ctrl->listed[0] : __ldg(&plan->count));
+                const int count = p.fused ? 0 : (listed ? ctrl->listed[0] : ld_after_wait(&plan->count));
                 auto next = [&]() -> int {   // the next chunk, or -1; index is its number
                     if (p.fused) {
                         if (!mk) return -1;
@@ -429,7 +429,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                     }
                     if (listed) return -1;
                     while (++index < count) {
-                        const int e = __ldg(&plan->chunk[index]);
+                        const int e = ld_after_wait(&plan->chunk[index]);
                         if ((uint32_t)e & who) return e;
                     }
                     return -1;
@@ -458,9 +458,9 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                 if (p.fused) return tile_mask[m] != 0ull;
                 const bool listed = &pt == list0_part && m == list0_m && n == list0_n;
                 const TilePlan* plan = pt.plan + m;
-                const int count = listed ? ctrl->listed[0] : __ldg(&plan->count);
+                const int count = listed ? ctrl->listed[0] : ld_after_wait(&plan->count);
                 if (!dual) return count > 0;
-                for (int i = 0; i < count; ++i) if ((listed ? list0[i] : (uint32_t)__ldg(&plan->chunk[i])) & who) return true;
+                for (int i = 0; i < count; ++i) if ((listed ? list0[i] : ld_after_wait(&plan->chunk[i])) & who) return true;
                 return false;
             };
             // a stage without operands: only its flags matter to the MMA thread

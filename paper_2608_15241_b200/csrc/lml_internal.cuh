@@ -284,6 +284,22 @@ __device__ __forceinline__ uint4 ldg_nc_v4(const void* p)
     return v;
 }
 
+// What an earlier grid of the stream writes while this one is already resident (ids, segment arrays, the plans of the row
+// tiles): read with ordinary loads, after griddepcontrol.wait.  The non-coherent path (__ldg) is for data that nobody writes
+// during the reading kernel's life; a line of an earlier call's values may wait in L1 there.
+__device__ __forceinline__ int ld_after_wait(const int32_t* p)
+{
+    int v;
+    asm volatile("ld.global.s32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+__device__ __forceinline__ uint32_t ld_after_wait(const uint16_t* p)
+{
+    uint16_t v;
+    asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
+    return v;
+}
+
 // D(16x8, fp32) += A(16x16, bf16, row) * B(16x8, bf16, col)
 __device__ __forceinline__ void mma_bf16_16816(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
                                                uint32_t a3, uint32_t b0, uint32_t b1)
