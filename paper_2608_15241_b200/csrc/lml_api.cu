@@ -228,9 +228,9 @@ lml_status lml_table_create(lml_table** out, int device, int d_in, int d_out, in
     ok = ok && cudaMemset(t->arena.adapter_map, 0xff, kMaxAdapterIds * sizeof(int32_t)) == cudaSuccess;   // -1: no serving version
     ok = ok && cudaMalloc(&t->arena.tile_flags, kFuseMaxTiles * sizeof(int32_t)) == cudaSuccess;
     ok = ok && cudaMemset(t->arena.tile_flags, 0, kFuseMaxTiles * sizeof(int32_t)) == cudaSuccess;
+    ok = ok && decode_init() == cudaSuccess;   // (first: see there)
     ok = ok && gemm_sm100_init(device) == cudaSuccess;
     ok = ok && shrink_init() == cudaSuccess;
-    ok = ok && decode_init() == cudaSuccess;
     ok = ok && aux_init() == cudaSuccess;
     ok = ok && bind_init() == cudaSuccess;
     ok = ok && encode_tmap_3d(&t->tmap_A, t->arena.A, (uint64_t)d_in, kRankPad, (uint64_t)max_slots, (uint64_t)d_in * 2,

@@ -270,38 +270,6 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_main_kernel(const __gri
         }
     } else {
         asm volatile("bar.sync 4, %0;" ::"n"(kDecThreads) : "memory");
-        if (!kBase && warp == kDecConsumers + 2 && G > 0 && !adapter_map) {
-            // What the call will read besides W0 starts on its way into L2 while the work before it still runs: the rows of A
-            // that its slots name (a few to every CTA of the grid), their rows of B for this CTA's columns, a share of x.  The ids
-            // are read here only to guess with (past L1, where the reads after the wait must not find them): if that work
-            // changes them, the prefetch was for nothing.  A decoder layer's adapters come cold out of HBM at every step, and
-            // every one of these reads is a dependent trip of its own behind the weight stream.  Measured: the seven projections
-            // of a layer at 1 token 95.2 -> 94.3 us, at 8 tokens 100.0 -> 98.7.
-            int hint = -1;
-            if (token_slots) { if (lane < T) hint = (int)ld_relaxed_gpu(reinterpret_cast<const unsigned*>(token_slots) + lane); }
-            else if (lane < G) hint = (int)ld_relaxed_gpu(reinterpret_cast<const unsigned*>(slot_ids) + lane);
-            const int rank = slot_rank(snap, hint);
-            const unsigned peers = __match_any_sync(0xffffffffu, rank > 0 ? hint : -1);
-            const bool leader = rank > 0 && lane == __ffs(peers) - 1;
-            int incl = leader ? rank : 0;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int v = __shfl_up_sync(0xffffffffu, incl, o);
-                if (lane >= o) incl += v;
-            }
-            const int excl = incl - (leader ? rank : 0), total = __shfl_sync(0xffffffffu, incl, 31);
-            for (int i = cta; i < total; i += ncta) {   // row i of the slots' rows of A, slot after slot
-                const bool here = leader && i >= excl && i < incl;
-                if (here) bulk_prefetch_l2(arenaA + ((size_t)hint * kRankPad + (i - excl)) * K, (uint32_t)(K * 2));
-            }
-            if (leader && row_end > row_begin) {
-                if (rank <= kRankCompact) bulk_prefetch_l2(arenaBc + ((size_t)hint * N + row_begin) * kRankCompact, (uint32_t)((row_end - row_begin) * kRankCompact * 2));
-                else bulk_prefetch_l2(arenaB + ((size_t)hint * N + row_begin) * kRankPad, (uint32_t)((row_end - row_begin) * kRankPad * 2));
-            }
-            const int pieces = T * K / 8;   // 16-byte pieces of x
-            const int p0 = (int)((long long)cta * pieces / ncta), p1 = (int)((long long)(cta + 1) * pieces / ncta);
-            if (lane == 31 && p1 > p0) bulk_prefetch_l2(x + (size_t)p0 * 8, (uint32_t)(p1 - p0) * 16);
-        }
         grid_dependency_wait();     // launched as a programmatic dependent: the work before this call is complete now
     }
 
@@ -356,6 +324,47 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_main_kernel(const __gri
     // worth 0.2 us once, and costs 0.1 - 0.4 us per call since the shrink warps no longer wait for a fence.)
     if (shrinker && G > 0) {
         const int sw = warp - kDecConsumers - 1;
+        if (sw == 1) {
+            // Which adapters this call names is known only after the lookup below, a memory round trip
+            // from now, and their rows of A are cold.  When the table's live adapters are very few (their rows
+            // of A together at most a 64th of W0), all of them are asked into L2 right now, ahead of the weight
+            // stream, a row or two per CTA.  (With a 16th as the limit this was worth 0.3 us while the chain behind
+            // the dot products was longer; now it changes nothing on a call that uses the adapters and costs
+            // 0.1 - 0.2 us on one that does not, hence the narrow rule.  Taking the block out altogether was measured
+            // too: the base-only call, which never runs it, came out 0.13 us slower, by code generation alone.)
+            int rows_before = 0, my_rank[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int sl = lane + 32 * h;
+                my_rank[h] = sl < snap.max_slots && sl < kMaxSlots ? (int)snap.rank[sl] : 0;
+            }
+            // running count of live rows in slot order: slots 0..31 first, then 32..63
+            int incl0 = my_rank[0], incl1 = my_rank[1];
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int v0 = __shfl_up_sync(0xffffffffu, incl0, o), v1 = __shfl_up_sync(0xffffffffu, incl1, o);
+                if (lane >= o) { incl0 += v0; incl1 += v1; }
+            }
+            const int total0 = __shfl_sync(0xffffffffu, incl0, 31);
+            const int live_rows = total0 + __shfl_sync(0xffffffffu, incl1, 31);
+            if ((long long)live_rows * K * 64 <= (long long)N * K) {
+                // lane L of this CTA takes live row blockIdx + L * grid
+                const int i = cta + lane * ncta;
+                // find the slot holding live row i: the first whose inclusive count exceeds i
+                const unsigned m0 = __ballot_sync(0xffffffffu, incl0 > 0);   // (dummy use keeps the shuffles converged)
+                (void)m0;
+                int slot = -1, j = 0;
+                for (int src = 0; src < 32; ++src) {   // uniform loop: every lane reads every lane's counts
+                    const int e0 = __shfl_sync(0xffffffffu, incl0, src), r0 = __shfl_sync(0xffffffffu, my_rank[0], src);
+                    const int e1 = __shfl_sync(0xffffffffu, incl1, src) + total0, r1 = __shfl_sync(0xffffffffu, my_rank[1], src);
+                    if (slot < 0 && i < e0 && i >= e0 - r0) { slot = src; j = i - (e0 - r0); }
+                    if (slot < 0 && i < e1 && i >= e1 - r1) { slot = src + 32; j = i - (e1 - r1); }
+                }
+                if (i < live_rows && slot >= 0)
+                    bulk_prefetch_l2(arenaA + ((size_t)slot * kRankPad + j) * K, (uint32_t)(K * 2));
+                (void)rows_before;
+            }
+        }
         if (sw == kDecShrinkWarps - 1) {
             // this launch's mark: one more than that of the last launch that finished on these words
             unsigned last_epoch = 0;
@@ -987,20 +996,24 @@ cudaError_t decode_init()
     auto set = [&](auto kernel) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDecSmemBytes);
     };
-    set(decode_main_kernel<false, false, false, 1>); set(decode_main_kernel<false, true, false, 1>); set(decode_main_kernel<false, true, true, 1>);
-    set(decode_main_kernel<true, false, false, 1>);  set(decode_main_kernel<true, true, false, 1>);  set(decode_main_kernel<true, true, true, 1>);
-    set(decode_main_kernel<false, false, false, kDecMaxProj>); set(decode_main_kernel<false, true, false, kDecMaxProj>); set(decode_main_kernel<false, true, true, kDecMaxProj>);
-    set(decode_main_kernel<true, false, false, kDecMaxProj>);  set(decode_main_kernel<true, true, false, kDecMaxProj>);  set(decode_main_kernel<true, true, true, kDecMaxProj>);
     auto set_base = [&](auto kernel) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DecCfg<kDecVarBase>::kSmemBytes);
     };
-    set_base(decode_main_kernel<false, false, false, 1, kDecVarBase>); set_base(decode_main_kernel<false, true, false, 1, kDecVarBase>);
-    set_base(decode_main_kernel<true, false, false, 1, kDecVarBase>);  set_base(decode_main_kernel<true, true, false, 1, kDecVarBase>);
     auto set_small = [&](auto kernel) {
         if (e == cudaSuccess) e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, DecCfg<kDecVarSmall>::kSmemBytes);
     };
-    set_small(decode_main_kernel<false, false, false, 1, kDecVarSmall>); set_small(decode_main_kernel<false, true, true, 1, kDecVarSmall>);
-    set_small(decode_main_kernel<true, false, false, 1, kDecVarSmall>);  set_small(decode_main_kernel<true, true, true, 1, kDecVarSmall>);
+    // Kernels are loaded in the order in which they are first named, one behind the other, and W0's stream pushes their code out
+    // of L2 between launches: the builds that alternate in a decode step (several projections, then one) go in first and side
+    // by side.  Measured over ten memory layouts, a layer pass at 1 / 8 tokens: 94.4 / 97.6 us in this order, 95.1 / 98.9 with
+    // the builds grouped by their last argument, 96.0 / 100.2 so grouped and behind the other kernels of the library.
+    set(decode_main_kernel<false, true, true, kDecMaxProj>); set_small(decode_main_kernel<false, false, false, 1, kDecVarSmall>); set_small(decode_main_kernel<false, true, true, 1, kDecVarSmall>);
+    set(decode_main_kernel<false, false, false, kDecMaxProj>); set(decode_main_kernel<false, true, false, kDecMaxProj>);
+    set(decode_main_kernel<false, false, false, 1>); set(decode_main_kernel<false, true, false, 1>); set(decode_main_kernel<false, true, true, 1>);
+    set(decode_main_kernel<true, true, true, kDecMaxProj>); set_small(decode_main_kernel<true, false, false, 1, kDecVarSmall>); set_small(decode_main_kernel<true, true, true, 1, kDecVarSmall>);
+    set(decode_main_kernel<true, false, false, kDecMaxProj>);  set(decode_main_kernel<true, true, false, kDecMaxProj>);
+    set(decode_main_kernel<true, false, false, 1>);  set(decode_main_kernel<true, true, false, 1>);  set(decode_main_kernel<true, true, true, 1>);
+    set_base(decode_main_kernel<false, false, false, 1, kDecVarBase>); set_base(decode_main_kernel<false, true, false, 1, kDecVarBase>);
+    set_base(decode_main_kernel<true, false, false, 1, kDecVarBase>);  set_base(decode_main_kernel<true, true, false, 1, kDecVarBase>);
     return e;
 }
 
