@@ -89,7 +89,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         const int cap = live < c.layout.cap ? (live > 0 ? live : 1) : c.layout.cap;
         most_chunks = cap > most_chunks ? cap : most_chunks;
         BindPart& bp = b.part[p];
-        bp.A = c.t->arena.A; bp.ids = c.ids; bp.adapter_map = by_adapter ? c.t->arena.adapter_map : nullptr; bp.status = c.t->arena.status;
+        bp.A = c.t->arena.A; bp.ids = c.ids; bp.adapter_map = by_adapter ? c.t->arena.adapter_map : nullptr; bp.status = c.t->arena.status; bp.nonfinite = c.t->arena.nonfinite;
         bp.plan = reinterpret_cast<TilePlan*>(c.ws + c.layout.plan_off);
         bp.u = reinterpret_cast<__nv_bfloat16*>(c.ws + c.layout.u_off);
         bp.u2 = reinterpret_cast<__nv_bfloat16*>(c.ws + c.layout.u2_off);
@@ -217,11 +217,14 @@ lml_status lml_table_create(lml_table** out, int device, int d_in, int d_out, in
     const size_t bk_bytes = (size_t)max_slots * kRankPad * b_rows_padded(d_out) * sizeof(__nv_bfloat16);
     ok = ok && cudaMalloc(&t->arena.Bk, bk_bytes) == cudaSuccess;
     ok = ok && cudaMemset(t->arena.Bk, 0, bk_bytes) == cudaSuccess;   // (the rows past d_out stay zero)
-    ok = ok && cudaMalloc(&t->arena.status, 256) == cudaSuccess;
+    // the status word and the kernels' counters; from word 10 on, in the sector of the words that an early start touches, Arena::nonfinite
+    constexpr size_t kStatusBytes = (11 + kMaxSlots) * sizeof(uint32_t);
+    ok = ok && cudaMalloc(&t->arena.status, kStatusBytes) == cudaSuccess;
+    t->arena.nonfinite = t->arena.status + 10;
     ok = ok && cudaMalloc(&t->arena.adapter_map, kMaxAdapterIds * sizeof(int32_t)) == cudaSuccess;
     ok = ok && cudaMemset(t->arena.A, 0, a_bytes) == cudaSuccess;
     ok = ok && cudaMemset(t->arena.B, 0, b_bytes) == cudaSuccess;
-    ok = ok && cudaMemset(t->arena.status, 0, 256) == cudaSuccess;
+    ok = ok && cudaMemset(t->arena.status, 0, kStatusBytes) == cudaSuccess;
     const size_t dec_u_bytes = (size_t)kDecMaxBlocks * kDecExchStride * sizeof(unsigned long long);
     ok = ok && cudaMalloc(&t->arena.dec_u, dec_u_bytes) == cudaSuccess;
     ok = ok && cudaMemset(t->arena.dec_u, 0, dec_u_bytes) == cudaSuccess;   // mark 0: written by no launch
@@ -290,7 +293,7 @@ lml_status register_adapter(lml_table* t, int adapter_id, int version, const voi
         cudaGetLastError();
         return LML_ERR_CUDA;
     }
-    if (launch_pack_adapter(t->arena, free_slot, A, B, rank, t->d_in, t->d_out, (cudaStream_t)stream) != cudaSuccess) {
+    if (launch_pack_adapter(t->arena, free_slot, (uint16_t)(t->next_gen + 1), A, B, rank, t->d_in, t->d_out, (cudaStream_t)stream) != cudaSuccess) {
         cudaGetLastError();
         return LML_ERR_CUDA;
     }
@@ -323,7 +326,7 @@ lml_status register_adapter_transposed(lml_table* t_T, int adapter_id, int versi
         cudaGetLastError();
         return LML_ERR_CUDA;
     }
-    if (launch_pack_adapter_transposed(t_T->arena, free_slot, A, B, rank, /*K=*/t_T->d_out, /*N=*/t_T->d_in,
+    if (launch_pack_adapter_transposed(t_T->arena, free_slot, (uint16_t)(t_T->next_gen + 1), A, B, rank, /*K=*/t_T->d_out, /*N=*/t_T->d_in,
                                        (cudaStream_t)stream) != cudaSuccess) {
         cudaGetLastError();
         return LML_ERR_CUDA;

@@ -9,13 +9,24 @@ namespace lml {
 // so that every kernel can read fixed-shape, 16-byte aligned rows.
 // ---------------------------------------------------------------------------------------------
 // Eight columns of one row of B (row n, columns 8g ...) into the three places that hold it: the padded row, the compact row
-// of narrow adapters, and the chunk that the GEMM multiplies.
+// of narrow adapters, and the chunk that the GEMM multiplies, which takes zeros for Inf and NaN and leaves a mark.
+__device__ __forceinline__ uint32_t finite_or_zero(uint32_t w)   // two bf16 values
+{
+    if ((w & 0x7f80u) == 0x7f80u) w &= 0xffff0000u;
+    if ((w & 0x7f800000u) == 0x7f800000u) w &= 0x0000ffffu;
+    return w;
+}
 __device__ __forceinline__ void store_b_group(__nv_bfloat16* dstB, __nv_bfloat16* dstBc, __nv_bfloat16* dstBk, int n_pad, bool compact,
-                                              long long n, int g, const uint4& v)
+                                              long long n, int g, const uint4& v, uint32_t* nonfinite, int slot, uint32_t tag)
 {
     *reinterpret_cast<uint4*>(dstB + n * kRankPad + g * 8) = v;
     if (compact) *reinterpret_cast<uint4*>(dstBc + n * kRankCompact + g * 8) = v;
-    *reinterpret_cast<uint4*>(dstBk + (size_t)(g >> 1) * n_pad * kChunk + chunk_elem((int)n, (g & 1) * 8)) = v;
+    const uint4 f = make_uint4(finite_or_zero(v.x), finite_or_zero(v.y), finite_or_zero(v.z), finite_or_zero(v.w));
+    if (f.x != v.x || f.y != v.y || f.z != v.z || f.w != v.w) {   // (the same words from every thread that finds one)
+        nonfinite[0] = 1u;
+        nonfinite[1 + slot] = tag;
+    }
+    *reinterpret_cast<uint4*>(dstBk + (size_t)(g >> 1) * n_pad * kChunk + chunk_elem((int)n, (g & 1) * 8)) = f;
 }
 __device__ __forceinline__ uint4 pack_u16x8(const unsigned short (&e)[8])
 {
@@ -30,7 +41,7 @@ __global__ void __launch_bounds__(256) pack_adapter_kernel(__nv_bfloat16* __rest
                                                            __nv_bfloat16* __restrict__ dstBk, int n_pad,
                                                            const __nv_bfloat16* __restrict__ A,
                                                            const __nv_bfloat16* __restrict__ B,
-                                                           int rank, int d_in, int d_out)
+                                                           int rank, int d_in, int d_out, uint32_t* __restrict__ nonfinite, int slot, uint32_t tag)
 {
     const int cols = chunks_of_rank(rank) * kChunk, groups = cols / 8;
     const int k8 = d_in / 8;
@@ -53,7 +64,7 @@ __global__ void __launch_bounds__(256) pack_adapter_kernel(__nv_bfloat16* __rest
             for (int j = 0; j < 8; ++j) e[j] = g * 8 + j < rank ? Bs[n * rank + g * 8 + j] : (unsigned short)0;
             v = pack_u16x8(e);
         }
-        store_b_group(dstB, dstBc, dstBk, n_pad, rank <= kRankCompact, n, g, v);
+        store_b_group(dstB, dstBc, dstBk, n_pad, rank <= kRankCompact, n, g, v, nonfinite, slot, tag);
     }
 }
 
@@ -63,7 +74,7 @@ static int pack_blocks(long long work)
     return (int)(blocks > 1184 ? 1184 : (blocks < 1 ? 1 : blocks));
 }
 
-cudaError_t launch_pack_adapter(const Arena& ar, int slot, const void* A, const void* B, int rank,
+cudaError_t launch_pack_adapter(const Arena& ar, int slot, uint16_t gen, const void* A, const void* B, int rank,
                                 int d_in, int d_out, cudaStream_t stream)
 {
     __nv_bfloat16* dstA = ar.A + (size_t)slot * kRankPad * d_in;
@@ -73,7 +84,7 @@ cudaError_t launch_pack_adapter(const Arena& ar, int slot, const void* A, const 
     __nv_bfloat16* dstBk = ar.Bk + (size_t)slot * kRankPad * n_pad;
     const long long work = (long long)chunks_of_rank(rank) * 2 * (d_in > d_out ? d_in : d_out);
     pack_adapter_kernel<<<pack_blocks(work), 256, 0, stream>>>(dstA, dstB, dstBc, dstBk, n_pad, (const __nv_bfloat16*)A,
-                                                               (const __nv_bfloat16*)B, rank, d_in, d_out);
+                                                               (const __nv_bfloat16*)B, rank, d_in, d_out, ar.nonfinite, slot, nonfinite_tag(gen));
     return cudaGetLastError();
 }
 
@@ -287,7 +298,7 @@ __global__ void __launch_bounds__(256) pack_adapter_transposed_kernel(__nv_bfloa
                                                                       __nv_bfloat16* __restrict__ dstBk, int k_pad,
                                                                       const __nv_bfloat16* __restrict__ A,
                                                                       const __nv_bfloat16* __restrict__ B,
-                                                                      int rank, int K, int N)
+                                                                      int rank, int K, int N, uint32_t* __restrict__ nonfinite, int slot, uint32_t tag)
 {
     const unsigned short* As = reinterpret_cast<const unsigned short*>(A);
     const unsigned short* Bs = reinterpret_cast<const unsigned short*>(B);
@@ -306,11 +317,11 @@ __global__ void __launch_bounds__(256) pack_adapter_transposed_kernel(__nv_bfloa
         unsigned short e[8];
 #pragma unroll
         for (int j = 0; j < 8; ++j) e[j] = g * 8 + j < rank ? As[(long long)(g * 8 + j) * K + k] : (unsigned short)0;
-        store_b_group(dstB, dstBc, dstBk, k_pad, rank <= kRankCompact, k, g, pack_u16x8(e));
+        store_b_group(dstB, dstBc, dstBk, k_pad, rank <= kRankCompact, k, g, pack_u16x8(e), nonfinite, slot, tag);
     }
 }
 
-cudaError_t launch_pack_adapter_transposed(const Arena& arT, int slot, const void* A, const void* B, int rank,
+cudaError_t launch_pack_adapter_transposed(const Arena& arT, int slot, uint16_t gen, const void* A, const void* B, int rank,
                                            int K, int N, cudaStream_t stream)
 {
     __nv_bfloat16* dstA = arT.A + (size_t)slot * kRankPad * N;   // the transposed table has d_in = N ...
@@ -320,7 +331,7 @@ cudaError_t launch_pack_adapter_transposed(const Arena& arT, int slot, const voi
     __nv_bfloat16* dstBk = arT.Bk + (size_t)slot * kRankPad * k_pad;
     const long long work = (long long)chunks_of_rank(rank) * kChunk * (K > N ? K : N);
     pack_adapter_transposed_kernel<<<pack_blocks(work), 256, 0, stream>>>(dstA, dstB, dstBc, dstBk, k_pad, (const __nv_bfloat16*)A,
-                                                                          (const __nv_bfloat16*)B, rank, K, N);
+                                                                          (const __nv_bfloat16*)B, rank, K, N, arT.nonfinite, slot, nonfinite_tag(gen));
     return cudaGetLastError();
 }
 

@@ -103,6 +103,7 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
 
     // ---- the slot of every row
     const int row_t = tid - 64;   // warps 2 .. 5: a row each
+    const uint32_t any_nonfinite = first_cta && row_t >= 0 ? ld_after_wait(part.nonfinite) : 0u;   // (used at the end)
     int bad_slot = 0;
     int s_a = -1, s_b = -1;
     if (L.rows.mode == kRowsSegments) {
@@ -328,6 +329,11 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
     }
     if (first && tid == 0)   // no chunks for this CTA: the tiles of x that went out early have to land before it leaves
         for (int i = 0; i < pre; ++i) { mbar_arrive(smem_u32(&ctrl->full[i])); mbar_wait(smem_u32(&ctrl->full[i]), 0u, abort); }
+    if (any_nonfinite) {
+        auto marked = [&](int slot) { return slot >= 0 && ld_after_wait(part.nonfinite + 1 + slot) == nonfinite_tag(snap.gen[slot]) ? slot : -1; };
+        part.plan[m].nonfinite_row[0][row_t] = (int8_t)marked(s_a);
+        part.plan[m].nonfinite_row[1][row_t] = (int8_t)marked(s_b);
+    }
     __syncthreads();
     if (tid == 0 && ctrl->abort) atomicOr(part.status, LML_FLAG_TIMEOUT);
     if (warp == 1) {

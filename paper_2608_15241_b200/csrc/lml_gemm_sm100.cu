@@ -27,6 +27,8 @@
 // W0, which is frozen, and reads x once bind_shrink, which waits for that work, has raised a word for it (a bounded wait).
 // For few tokens (tiles far fewer than SMs) a split-K variant follows below: a cluster of CTAs shares a
 // tile and exchanges partial sums through distributed shared memory.
+// B's chunks hold zeros where the adapter's B is Inf or NaN (every row of a tile meets the chunks of all its slots).  The terms
+// left out are added by the epilogue, element by element, to the rows that are bound to such a slot; other tiles pay one word.
 // Every wait is bounded; on give-up the CTA sets LML_FLAG_TIMEOUT, drains and frees its TMEM.
 #include <cstdio>
 #include <cstdlib>
@@ -78,6 +80,7 @@ struct GemmCtrl {
     uint32_t stage_info[8];   // written by the producer: k-steps (0..4) | kStage* flags
     int32_t pad[2];
     int32_t listed[2];        // entries of the list (per binding)
+    unsigned long long nonfinite;   // fused shrink: slots whose B holds Inf or NaN
 };
 // stage_info flags
 constexpr uint32_t kStageCommit = 0x100u;   // after this stage the accumulator holds an output: commit it to the epilogue
@@ -112,6 +115,8 @@ static_assert(sizeof(ShrPlan) <= 512, "shrink plan");
 struct alignas(64) GemmPart {
     CUtensorMap w, y;
     const __nv_bfloat16* bk;            // the table's packed B, by chunk
+    const __nv_bfloat16* b;             // ... and by row, as registered
+    const uint32_t* nonfinite;
     const TilePlan* plan;               // [row tile] its chunks
     const __nv_bfloat16* u;
     const __nv_bfloat16* u_lo;          // or null: what u's bf16 values leave, a further K-step per chunk
@@ -201,6 +206,41 @@ __device__ __forceinline__ int list_chunks(const TilePlan* plan, uint32_t who, i
     }
     return n;
 }
+// The terms of one row that the product with the chunks left out, 32 columns from col0: u_j B[n][j] where B is Inf or NaN.
+// u, u_more: the row of the slot's first block (u_more: to be added to it, or null); out: the row's outputs, bf16, 16-byte
+// pieces in an order given by piece_xor.
+__device__ __noinline__ void add_nonfinite(const GemmPart& pt, int slot, int col0, const __nv_bfloat16* u, const __nv_bfloat16* u_more,
+                                           uint8_t* out, int piece_xor)
+{
+    auto value = [](const __nv_bfloat16* p) { return __uint_as_float(ld_after_wait(reinterpret_cast<const uint16_t*>(p)) << 16); };
+    const int cols = slot_chunks(pt, slot) * kChunk;
+    for (int c = 0; c < kEpiChunkCols && col0 + c < pt.N; ++c) {
+        const __nv_bfloat16* b = pt.b + ((size_t)slot * pt.N + col0 + c) * kRankPad;
+        float sum = 0.f;
+        bool any = false;
+        for (int j = 0; j < cols; ++j) {
+            const float bv = value(b + j);
+            if (isfinite(bv)) continue;
+            const size_t at = (size_t)(j / kChunk) * (kTileM * kChunk) + chunk_elem(0, j % kChunk);
+            sum += (value(u + at) + (u_more ? value(u_more + at) : 0.f)) * bv;
+            any = true;
+        }
+        if (!any) continue;
+        __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(out + ((c >> 3) ^ piece_xor) * 16 + (c & 7) * 2);
+        *o = __float2bfloat16_rn(__bfloat162float(*o) + sum);
+    }
+}
+// number of the first of a slot's chunks among those of a tile
+__device__ __noinline__ int first_chunk_of(const TilePlan* plan, int slot)
+{
+    int i = 0;
+    while (i < kMaxChunks - 1 && (int)(ld_after_wait(&plan->chunk[i]) & 0xfffu) != slot) ++i;
+    return i;
+}
+__device__ __forceinline__ size_t u_row(const GemmPart& pt, int m, int index, int row)
+{
+    return ((size_t)m * pt.cap + index) * (kTileM * kChunk) + chunk_elem(row, 0);
+}
 // One chunk of a stage: the block of u (number `index` of row tile m) and the chunk's rows of B for columns
 // [n * BN, + BN), each contiguous.  entry = slot | chunk << 8.
 template <int BN>
@@ -268,6 +308,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
         }
         mbar_init(smem_u32(&ctrl->plan_full), 1);
         ctrl->abort = 0;
+        ctrl->nonfinite = 0ull;
         fence_mbar_init();
     }
     if (warp == 0 && lane == 0) {
@@ -290,6 +331,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
         // Every CTA works out the slots of all row tiles from its own copy of the segment arrays (checked here: all reach
         // the same verdict) or from the slot per row.
         int bad_off = 0, bad_slot = 0;
+        const uint32_t any_nonfinite = threadIdx.x < kMaxSlots ? ld_after_wait(p.part[0].nonfinite) : 0u;
         for (int m = threadIdx.x; m < p.num_m; m += kThreads) tile_mask[m] = 0ull;
         if (by_segment) {
             const int G = p.rows.G;
@@ -326,6 +368,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
         }
         __syncthreads();
         const GemmPart& pt = p.part[0];
+        if (any_nonfinite && ld_after_wait(pt.nonfinite + 1 + threadIdx.x) == nonfinite_tag(snap.gen[threadIdx.x])) atomicOr(&ctrl->nonfinite, 1ull << threadIdx.x);
         for (int m = threadIdx.x; m < p.num_m; m += kThreads)
             shr_base[m + 1] = (uint16_t)((mask_chunks(pt, tile_mask[m]) + kShrChunks - 1) / kShrChunks);
         __syncthreads();
@@ -737,6 +780,12 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
         int acc = 0;
         uint32_t full_ph0 = 0, full_ph1 = 0;
         int buf = 0;
+        auto row_slot = [&](int row) -> int {   // fused shrink: the slot of a row (< 0: none)
+            if (!by_segment) return p.rows.rows[row];
+            int lo = 0, hi = p.rows.G;
+            while (lo < hi) { const int mid = (lo + hi) >> 1; if (seg_cache[mid + 1] > row) hi = mid; else lo = mid + 1; }
+            return lo < p.rows.G ? slot_cache[lo] : -1;
+        };
         bool ok = true;
         if (p.lora && !p.fused && warp == 2) {   // nothing else to do yet: the first tile's chunks, as soon as they are known
             const GemmPart& pt = p.part[part_of(p, (int)blockIdx.x)];
@@ -746,6 +795,8 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
             const int n = list_chunks(pt.plan + ((int)blockIdx.x - pt.tile0) % num_mt * kRowTiles, kChunkFirst | kChunkSecond, 0, 1, lane, list0);
             __syncwarp();
             if (lane == 0) { ctrl->listed[0] = n; mbar_arrive(smem_u32(&ctrl->plan_full)); }
+        } else if (p.lora && !p.fused) {
+            grid_dependency_wait();   // (this warp reads the plans too)
         }
         // this CTA's shrink passes: scale, zero the rows of other slots, round, write the u blocks; then the pass's
         // flag goes up (release: the four warps' stores are complete)
@@ -758,14 +809,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
             fph ^= 1u;
             tc_fence_after();
             const int pos = sp.m * kBM + q * 32 + lane;
-            int my_slot = -1;
-            if (pos < p.T) {
-                if (by_segment) {
-                    int lo = 0, hi = p.rows.G;
-                    while (lo < hi) { const int mid = (lo + hi) >> 1; if (seg_cache[mid + 1] > pos) hi = mid; else lo = mid + 1; }
-                    if (lo < p.rows.G) my_slot = slot_cache[lo];
-                } else my_slot = p.rows.rows[pos];
-            }
+            const int my_slot = pos < p.T ? row_slot(pos) : -1;
 #pragma unroll 1
             for (int i0 = 0; i0 < sp.n; i0 += 2) {   // two chunks, 32 columns at a time
                 uint32_t r[32];
@@ -808,6 +852,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                 if (m >= p.num_m) continue;
             }
             const int row_base = m * kBM + q * 32;
+            const bool nonfinite = p.lora && (p.fused ? (tile_mask[m] & ctrl->nonfinite) != 0ull : ld_after_wait(pt.nonfinite) != 0u);
             for (int pass = 0; pass < (dual ? 2 : 1) && ok; ++pass) {
                 uint32_t& fph = acc ? full_ph1 : full_ph0;
                 ok = mbar_wait_warp(smem_u32(&ctrl->tmem_full[acc]), fph, abort);
@@ -815,6 +860,20 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                 fph ^= 1u;
                 tc_fence_after();
                 const bool last_pass = pass == (dual ? 1 : 0);
+                int nf_slot = -1;   // this row's slot, if its B holds Inf or NaN
+                size_t nf_u = 0;
+                if (nonfinite) {
+                    if (!p.fused) {
+                        nf_slot = ld_after_wait(&pt.plan[m].nonfinite_row[pass][q * 32 + lane]);
+                        if (nf_slot >= 0) nf_u = u_row(pt, m, first_chunk_of(pt.plan + m, nf_slot), q * 32 + lane);
+                    } else {
+                        const int s = row_base + lane < p.T ? row_slot(row_base + lane) : -1;
+                        if (s >= 0 && ((ctrl->nonfinite >> s) & 1ull)) {
+                            nf_slot = s;
+                            nf_u = u_row(pt, m, mask_chunks(pt, tile_mask[m] & ((1ull << s) - 1ull)), q * 32 + lane);
+                        }
+                    }
+                }
                 const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
 #pragma unroll 1
                 for (int c = 0; c < BN / kEpiChunkCols; ++c) {
@@ -846,6 +905,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                         const int phys = j ^ ((lane >> 1) & 3);
                         *reinterpret_cast<uint4*>(bp + lane * 64 + phys * 16) = v;
                     }
+                    if (nf_slot >= 0) add_nonfinite(pt, nf_slot, col0, pt.u + nf_u, pass ? p.u2 + nf_u : (pt.u_lo ? pt.u_lo + nf_u : nullptr), bp + lane * 64, (lane >> 1) & 3);
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) {
@@ -1056,7 +1116,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
     }
     // ---------------------------------------------------------------------- exchange and reduction
     __syncwarp();   // (the producer's and the MMA issuer's other lanes waited here: the cluster barrier wants whole warps)
-    bool ok = true;
+    bool ok = true, nonfinite = false;
     if (warp >= 2) {
         if (p.lora && warp == 2) {   // nothing else to do yet: this CTA's share of the tile's chunks, as soon as they are known
             if (p.x_flag) prefetch_b<BN>(pt, n, lane, rank, S);
@@ -1068,7 +1128,10 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
             }
             __syncwarp();
             if (lane == 0) mbar_arrive(smem_u32(&ctrl->plan_full));
+        } else if (p.lora) {
+            grid_dependency_wait();   // (this warp reads the plan too)
         }
+        if (p.lora) nonfinite = ld_after_wait(pt.nonfinite) != 0u;
         ok = mbar_wait_warp(smem_u32(&ctrl->tmem_full[0]), 0u, abort);   // this CTA's MMAs are complete: so are its loads
         tc_fence_after();
     }
@@ -1106,6 +1169,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
         const int pos = m * kBM + row;
         const bool row_ok = pos < p.T;
         const int c_first = first_chunk(rank), c_end = first_chunk(rank + 1);
+        const int nf_slot = nonfinite && row_ok ? ld_after_wait(&pt.plan[m].nonfinite_row[o][row]) : -1;   // this row's slot, if its B holds Inf or NaN
+        const size_t nf_u = nf_slot >= 0 ? u_row(pt, m, first_chunk_of(pt.plan + m, nf_slot), row) : 0;
 #pragma unroll 1
         for (int c = c_first; c < c_end; ++c) {
             float acc[32];
@@ -1131,6 +1196,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
                 v.w = pack_bf16(acc[8 * j + 6], acc[8 * j + 7]);
                 *reinterpret_cast<uint4*>(yout + (size_t)pos * pt.N + col0 + j * 8) = v;
             }
+            if (nf_slot >= 0)
+                add_nonfinite(pt, nf_slot, col0, (o ? p.u2 : pt.u) + nf_u, o || !pt.u_lo ? nullptr : pt.u_lo + nf_u, reinterpret_cast<uint8_t*>(yout + (size_t)pos * pt.N + col0), 0);
         }
     }
     }   // outputs
@@ -1383,7 +1450,7 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
         } else {
             pt.y = pt.w;
         }
-        pt.bk = pr.ar->Bk; pt.plan = pr.plan; pt.u = pr.u; pt.u_lo = pr.u_lo; pt.y_ptr = (__nv_bfloat16*)pr.y;
+        pt.bk = pr.ar->Bk; pt.b = pr.ar->B; pt.nonfinite = pr.ar->nonfinite; pt.plan = pr.plan; pt.u = pr.u; pt.u_lo = pr.u_lo; pt.y_ptr = (__nv_bfloat16*)pr.y;
         pt.live = pt.nch[0] = pt.nch[1] = 0ull;
         for (int s = 0; s < pr.snap->max_slots; ++s)
             if (pr.snap->rank[s] > 0) {

@@ -43,18 +43,22 @@ struct Arena {
                         // (what the decode kernel reads: it needs a row's real columns only, a quarter of the padded row)
     __nv_bfloat16* Bk;  // [max_slots][4 chunks][b_rows_padded(d_out)][kChunk] for the GEMM: a chunk is 16 of the slot's columns, its rows in the
                         // no-swizzle operand order of the tensor cores (see chunk_elem), so that the rows of an output tile are one
-                        // contiguous piece and a slot costs the chunks its rank needs and no more
+                        // contiguous piece and a slot costs the chunks its rank needs and no more.  Zero where B is Inf or NaN: every row
+                        // of an output tile meets the chunks of all slots of the tile, and 0 x Inf would reach the rows of other slots
+    uint32_t* nonfinite;    // [0] not 0: some registration's B held Inf or NaN; [1 + slot] nonfinite_tag() of the last such one in the slot.  The
+                            // GEMM adds those terms to the slot's own rows
     uint32_t* status;   // sticky LML_FLAG_* bits
     int32_t* tile_flags;    // [kFuseMaxTiles] fused shrink of the prefill GEMM: the u blocks of pass i are written (= epoch + 1; the epoch is word 4 of status)
     int32_t* adapter_map;   // [kMaxAdapterIds] serving entry of each adapter id: slot | generation << 8, -1 = none; written by lml_publish
     unsigned long long* dec_u;   // [kDecMaxBlocks][kDecExchStride] the decode kernel's exchange blocks, one per part of a launch that works on this table
 };
 
+__host__ __device__ inline uint32_t nonfinite_tag(uint16_t gen) { return 0x10000u | gen; }   // (0: nothing registered yet)
 inline int32_t adapter_map_word(int slot, uint16_t gen) { return (int32_t)((uint32_t)slot | ((uint32_t)gen << 8)); }
 
 // ---- kernel launchers (each enqueues on `stream` and returns the launch error) ------------
 
-cudaError_t launch_pack_adapter(const Arena& ar, int slot, const void* A, const void* B, int rank,
+cudaError_t launch_pack_adapter(const Arena& ar, int slot, uint16_t gen, const void* A, const void* B, int rank,
                                 int d_in, int d_out, cudaStream_t stream);
 
 cudaError_t launch_set_word(int32_t* dst, int32_t value, cudaStream_t stream);
@@ -68,7 +72,7 @@ cudaError_t launch_stage_host_inputs(const void* x_host, void* x_dev, size_t x_b
                                      int n_so, const int32_t* ids_host, int32_t* ids_dev, int n_ids,
                                      const int32_t* perm_host, int32_t* perm_dev, int n_perm, cudaStream_t stream);
 // (A', B') = (B^T, A^T) of a forward adapter A [rank][K], B [N][rank] into slot `slot` of the transposed table's arena
-cudaError_t launch_pack_adapter_transposed(const Arena& arT, int slot, const void* A, const void* B, int rank,
+cudaError_t launch_pack_adapter_transposed(const Arena& arT, int slot, uint16_t gen, const void* A, const void* B, int rank,
                                            int K, int N, cudaStream_t stream);
 // out_s += P_s^T . Q_s per slot (adapter gradients); mode 0: out[slot][j][c], mode 1: out[slot][c][j]
 cudaError_t launch_weight_grad(const SlotSnapshot& snap, const __nv_bfloat16* pieces, const void* Q, int T, int C,
@@ -108,6 +112,7 @@ struct alignas(16) TilePlan {
     int32_t count;
     int32_t pad[3];
     uint16_t chunk[kMaxChunks];   // slot | chunk << 8 | kChunkFirst, kChunkSecond
+    int8_t nonfinite_row[2][kTileM];   // [binding][row] the row's slot if its B holds Inf or NaN, else -1 (written only where the table has seen such a B)
 };
 constexpr uint32_t kChunkFirst = 0x1000u, kChunkSecond = 0x2000u;   // rows use the slot under the first / second binding
 
@@ -129,6 +134,7 @@ struct BindPart {
     const int32_t* ids;           // per token, or per segment
     const int32_t* adapter_map;   // null: the ids are slots; else adapter ids, resolved through the table's device map
     uint32_t* status;
+    const uint32_t* nonfinite;    // as in Arena
     TilePlan* plan;               // [row tile]
     __nv_bfloat16* u;
     __nv_bfloat16* u2;            // a second set of blocks (see BindArgs::second)
@@ -297,6 +303,14 @@ __device__ __forceinline__ uint32_t ld_after_wait(const uint16_t* p)
 {
     uint16_t v;
     asm volatile("ld.global.u16 %0, [%1];" : "=h"(v) : "l"(p) : "memory");
+    return v;
+}
+
+__device__ __forceinline__ uint32_t ld_after_wait(const uint32_t* p) { return (uint32_t)ld_after_wait(reinterpret_cast<const int32_t*>(p)); }
+__device__ __forceinline__ int ld_after_wait(const int8_t* p)
+{
+    int v;
+    asm volatile("ld.global.s8 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
     return v;
 }
 
