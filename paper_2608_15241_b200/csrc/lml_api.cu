@@ -15,7 +15,7 @@ inline size_t round_up(size_t v, size_t a) { return (v + a - 1) / a * a; }
 // [u blocks, one or two sets].  A row tile has room for the chunks of `slots` slots of the widest rank, whatever the table
 // holds when the call comes; calls of more than kSlabTiles row tiles work in slabs, so the blocks stay bounded.
 struct WsLayout {
-    size_t plan_off, rows_off, rows2_off, u_off, u2_off, total;
+    size_t plan_off, rows_off, rows2_off, u_off, u2_off, u3_off, total;   // (u2_off, u3_off: where the call has as many sets)
     int cap;   // chunks per row tile
 };
 WsLayout ws_layout(const lml_table* t, int T, int slots, int u_sets = 1)
@@ -32,11 +32,19 @@ WsLayout ws_layout(const lml_table* t, int T, int slots, int u_sets = 1)
     w.u_off = round_up(w.rows2_off + round_up((size_t)T, 256), 1024);
     const size_t u_bytes = slab * (size_t)w.cap * kUBlockBytes;
     w.u2_off = w.u_off + u_bytes;
+    w.u3_off = w.u2_off + u_bytes;
     w.total = w.u_off + (size_t)u_sets * u_bytes;
     return w;
 }
-// (calls of one row tile have room for u as two bf16 values)
-WsLayout tokens_layout(const lml_table* t, int T) { return ws_layout(t, T, t->max_slots, T <= kTileM ? 2 : 1); }
+// Calls of one row tile have room for u as three bf16 values (and longer ones take at least as much as those).
+WsLayout tokens_layout(const lml_table* t, int T)
+{
+    if (T <= kTileM) return ws_layout(t, T, t->max_slots, 3);
+    WsLayout w = ws_layout(t, T, t->max_slots);
+    const size_t one_tile = ws_layout(t, kTileM, t->max_slots, 3).total;
+    w.total = w.total > one_tile ? w.total : one_tile;
+    return w;
+}
 // (a dual call's rows can use a slot per segment and binding)
 WsLayout dual_layout(const lml_table* t, int T, int G) { return ws_layout(t, T, G > kMaxSlots ? kMaxSlots : 2 * G, 2); }
 
@@ -59,7 +67,7 @@ struct GemmCall {
 
 // The GEMM path: the rows stay in their order; one launch binds them and computes u (unless the GEMM does both itself),
 // one launch multiplies.  P > 1: projections of the same x.  ids2 / y2: the second binding of a dual call.  precise: u goes
-// into the product as two bf16 values (16 bits of significand), a further K-step per chunk.
+// into the product as three bf16 values that add up to its fp32 value, two further K-steps per chunk.
 cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, RowMode mode, const int32_t* seg_offsets, int G,
                           const int32_t* perm, const int32_t* ids2, void* y2, bool by_adapter, cudaStream_t stream, int* launches,
                           bool precise = false)
@@ -93,10 +101,11 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         bp.plan = reinterpret_cast<TilePlan*>(c.ws + c.layout.plan_off);
         bp.u = reinterpret_cast<__nv_bfloat16*>(c.ws + c.layout.u_off);
         bp.u2 = reinterpret_cast<__nv_bfloat16*>(c.ws + c.layout.u2_off);
+        bp.u3 = reinterpret_cast<__nv_bfloat16*>(c.ws + c.layout.u3_off);
         bp.cap = cap;
         GemmProj& gp = g.proj[p];
         gp.W0 = c.W0; gp.y = c.y; gp.d_out = c.t->d_out; gp.ar = &c.t->arena; gp.snap = &snap[p];
-        gp.plan = bp.plan; gp.u = bp.u; gp.u_lo = precise ? bp.u2 : nullptr; gp.cap = cap;
+        gp.plan = bp.plan; gp.u = bp.u; gp.u_mid = precise ? bp.u2 : nullptr; gp.u_lo = precise ? bp.u3 : nullptr; gp.cap = cap;
     }
     g.num_sms = t0->num_sms;
     if (mode == kRowsSegments && (perm || G > kBindSegs || num_m > kSlabTiles)) {   // a slot per row first
@@ -546,7 +555,6 @@ lml_status lora_mixed_linear(lml_table* t, const void* x, const void* W0, int T,
 size_t lml_tokens_workspace_bytes(const lml_table* t, int max_tokens)
 {
     if (!t || max_tokens < 0 || max_tokens > kMaxTokens) return 0;
-    // (more than one tile takes at least as much as one with two values)
     return tokens_layout(t, max_tokens).total;
 }
 
@@ -805,7 +813,7 @@ lml_status lora_mixed_linear_multi(lml_table* const* tables, int P, const void* 
         if (!guard.ok) return LML_ERR_CUDA;
         GemmCall calls[LML_MAX_PROJECTIONS];
         // A call of its own would run as blocks of 16 tokens on the decode kernel, which keeps u in fp32: the shared launches
-        // carry it as two bf16 values then.
+        // carry it as three bf16 values then, which is as many bits.
         bool precise = false;
         size_t off = 0;
         for (int p = 0; p < P; ++p) {

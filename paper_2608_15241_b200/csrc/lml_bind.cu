@@ -49,6 +49,19 @@ struct alignas(64) BindLaunch {
     int early;      // few rows: x is asked for before the ids are known, and A's rows into L2 before the wait for the preceding work
 };
 
+// Two fp32 values, each as three bf16 values of 8 bits that add up to it.  (The first is the largest bf16 value where rounding
+// would make Inf of a finite one; of an Inf or a NaN it is all there is.)
+__device__ __forceinline__ void split_bf16(float a, float b, uint32_t& hi, uint32_t& mid, uint32_t& lo)
+{
+    hi = pack_bf16(a, b);
+    if (isfinite(a) && (hi & 0x7fffu) == 0x7f80u) hi -= 1u;
+    if (isfinite(b) && (hi & 0x7fff0000u) == 0x7f800000u) hi -= 0x10000u;
+    a = isfinite(a) ? a - bf16_lo(hi) : 0.f;
+    b = isfinite(b) ? b - bf16_hi(hi) : 0.f;
+    mid = pack_bf16(a, b);
+    lo = pack_bf16(a - bf16_lo(mid), b - bf16_hi(mid));
+}
+
 __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_constant__ BindLaunch B)
 {
     const BindArgs& L = B.args;
@@ -298,16 +311,22 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
             const int slot = ctrl->list[c0 + (piece >> 2)] & 0xff;
             const float sc = snap.scale[slot];
             const int tr = r * rows + rr;
+            const int have = (int)snap.rank[slot] - (ctrl->list[c0 + (piece >> 2)] >> 8) * kChunk - (piece & 3) * 4;   // columns that the adapter has, of these and on
+            v = make_float4(have > 0 ? v.x * sc : 0.f, have > 1 ? v.y * sc : 0.f, have > 2 ? v.z * sc : 0.f, have > 3 ? v.w * sc : 0.f);   // (Inf in x times the padding of A: not into u)
             const bool a = ctrl->row[0][tr] == slot, b = dual && ctrl->row[1][tr] == slot;
-            const uint2 val = make_uint2(pack_bf16(v.x * sc, v.y * sc), pack_bf16(v.z * sc, v.w * sc));
             const uint2 zero = make_uint2(0u, 0u);
             const size_t at = ((size_t)m * part.cap + c0 + (piece >> 2)) * (kTileM * kChunk) + chunk_elem(tr, (piece & 3) * 4);
-            *reinterpret_cast<uint2*>(part.u + at) = a ? val : zero;
             if (L.second == 3) {
-                const uint2 lo = make_uint2(pack_bf16(v.x * sc - bf16_lo(val.x), v.y * sc - bf16_hi(val.x)),
-                                            pack_bf16(v.z * sc - bf16_lo(val.y), v.w * sc - bf16_hi(val.y)));
-                *reinterpret_cast<uint2*>(part.u2 + at) = a ? lo : zero;
+                uint2 hi, mid, lo;
+                split_bf16(v.x, v.y, hi.x, mid.x, lo.x);
+                split_bf16(v.z, v.w, hi.y, mid.y, lo.y);
+                *reinterpret_cast<uint2*>(part.u + at) = a ? hi : zero;
+                *reinterpret_cast<uint2*>(part.u2 + at) = a ? mid : zero;
+                *reinterpret_cast<uint2*>(part.u3 + at) = a ? lo : zero;
+                continue;
             }
+            const uint2 val = make_uint2(pack_bf16(v.x, v.y), pack_bf16(v.z, v.w));
+            *reinterpret_cast<uint2*>(part.u + at) = a ? val : zero;
             if (dual) {
                 // (the blocks of the second binding, or of the difference of the two)
                 const uint2 neg = make_uint2(val.x ^ 0x80008000u, val.y ^ 0x80008000u);

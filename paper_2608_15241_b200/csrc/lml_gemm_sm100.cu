@@ -91,6 +91,7 @@ constexpr uint32_t kStageDelta = 0x800u;    // dual form: first stage of a tile'
 static_assert(sizeof(GemmCtrl) <= 256, "control block");
 constexpr uint32_t kStageBoth = 0x2000u;    // split-K dual form: the stage's product goes into both bindings' accumulators
 constexpr uint32_t kStageMore0 = 0x8000u, kStageMore1 = 0x10000u;   // tall tiles, on the last k-block: LoRA stages follow for the first / second row tile
+constexpr uint32_t kStageOneB = 0x1000u;    // a LoRA chunk whose u is three blocks: a K-step each, with the same block of B
 constexpr uint32_t kStageChunks = 0x4000u;  // LoRA chunks (no-swizzle operands), a K-step each
 
 // Fused shrink: a pass computes up to four chunks of a row tile, x[tile].A^T over all of K, two k-blocks to a stage.
@@ -119,7 +120,8 @@ struct alignas(64) GemmPart {
     const uint32_t* nonfinite;
     const TilePlan* plan;               // [row tile] its chunks
     const __nv_bfloat16* u;
-    const __nv_bfloat16* u_lo;          // or null: what u's bf16 values leave, a further K-step per chunk
+    const __nv_bfloat16* u_mid;         // or null: what u's bf16 values leave of the fp32 u, two further K-steps per chunk
+    const __nv_bfloat16* u_lo;
     __nv_bfloat16* y_ptr;
     unsigned long long live;            // slots that hold an adapter
     unsigned long long nch[2];          // ... their chunks less one, two bits each
@@ -207,10 +209,10 @@ __device__ __forceinline__ int list_chunks(const TilePlan* plan, uint32_t who, i
     return n;
 }
 // The terms of one row that the product with the chunks left out, 32 columns from col0: u_j B[n][j] where B is Inf or NaN.
-// u, u_more: the row of the slot's first block (u_more: to be added to it, or null); out: the row's outputs, bf16, 16-byte
+// u, u_more, u_rest: the row of the slot's first block (the others: to be added to it, or null); out: the row's outputs, bf16, 16-byte
 // pieces in an order given by piece_xor.
 __device__ __noinline__ void add_nonfinite(const GemmPart& pt, int slot, int col0, const __nv_bfloat16* u, const __nv_bfloat16* u_more,
-                                           uint8_t* out, int piece_xor)
+                                           const __nv_bfloat16* u_rest, uint8_t* out, int piece_xor)
 {
     auto value = [](const __nv_bfloat16* p) { return __uint_as_float(ld_after_wait(reinterpret_cast<const uint16_t*>(p)) << 16); };
     const int cols = slot_chunks(pt, slot) * kChunk;
@@ -222,7 +224,7 @@ __device__ __noinline__ void add_nonfinite(const GemmPart& pt, int slot, int col
             const float bv = value(b + j);
             if (isfinite(bv)) continue;
             const size_t at = (size_t)(j / kChunk) * (kTileM * kChunk) + chunk_elem(0, j % kChunk);
-            sum += (value(u + at) + (u_more ? value(u_more + at) : 0.f)) * bv;
+            sum += (value(u + at) + (u_more ? value(u_more + at) : 0.f) + (u_rest ? value(u_rest + at) : 0.f)) * bv;
             any = true;
         }
         if (!any) continue;
@@ -251,6 +253,14 @@ __device__ __forceinline__ void load_chunk(const GemmPart& pt, const __nv_bfloat
     bulk_load(a_dst + (uint32_t)(k * kUBlockBytes), u + ((size_t)m * pt.cap + index) * (kTileM * kChunk), kUBlockBytes, bar);
     const size_t chunk = (size_t)(entry & 0xffu) * (kRankPad / kChunk) + (size_t)((entry >> 8) & 0xfu);
     bulk_load(b_dst + (uint32_t)(k * BN * kChunk * 2), pt.bk + (chunk * pt.n_pad + (size_t)n * BN) * kChunk, BN * kChunk * 2, bar);
+}
+// ... and the other two blocks of a u of three
+__device__ __forceinline__ void load_u_rest(const GemmPart& pt, int m, int index, uint32_t a_dst, uint32_t bar)
+{
+    const size_t at = ((size_t)m * pt.cap + index) * (kTileM * kChunk);
+    mbar_expect_tx(bar, 2 * kUBlockBytes);
+    bulk_load(a_dst + kUBlockBytes, pt.u_mid + at, kUBlockBytes, bar);
+    bulk_load(a_dst + 2 * kUBlockBytes, pt.u_lo + at, kUBlockBytes, bar);
 }
 // Early start: the live slots' rows of B for this CTA's columns start on their way into L2 (a hint; the warps that will
 // run the epilogue have nothing else to do).  rank, S: this CTA's share of the chunks.
@@ -484,12 +494,12 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                     if (!ok) break;
                     const uint32_t a_dst = tiles_addr + stage * Cfg::kStageBytes, bar = smem_u32(&ctrl->full[stage]);
                     int k = 0;
-                    while (k < (pt.u_lo ? 3 : 4) && e >= 0) {
+                    while (k < 4 && e >= 0) {
                         load_chunk<BN>(pt, u, m, n, (uint32_t)e, index, k++, a_dst, a_dst + Cfg::kABytes, bar);
-                        if (pt.u_lo) load_chunk<BN>(pt, pt.u_lo, m, n, (uint32_t)e, index, k++, a_dst, a_dst + Cfg::kABytes, bar);
+                        if (pt.u_lo) { load_u_rest(pt, m, index, a_dst, bar); k = 4; }   // (a stage to itself)
                         e = next();
                     }
-                    ctrl->stage_info[stage] = (uint32_t)k | acc_flag | kStageChunks | (first ? flags_first : 0u) | (e < 0 ? flags_last : 0u);
+                    ctrl->stage_info[stage] = (pt.u_lo ? 3u | kStageOneB : (uint32_t)k) | acc_flag | kStageChunks | (first ? flags_first : 0u) | (e < 0 ? flags_last : 0u);
                     first = false;
                     mbar_arrive(bar);
                     advance();
@@ -628,12 +638,12 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
             uint32_t empty_ph0 = 0, empty_ph1 = 0, read1_ph0 = 0, read1_ph1 = 0;
             bool ok = true;
             // one stage: ksteps MMAs into d_tmem, then the stage goes back to the producer
-            auto issue = [&](uint32_t d_tmem, int ksteps, bool chunks, uint32_t& accumulate) {
+            auto issue = [&](uint32_t d_tmem, int ksteps, bool chunks, bool one_b, uint32_t& accumulate) {
                 const uint32_t a_addr = tiles_addr + stage * Cfg::kStageBytes;
                 const uint64_t adesc = chunks ? umma_desc_k16(a_addr) : umma_desc_k128(a_addr);
                 const uint64_t bdesc = chunks ? umma_desc_k16(a_addr + Cfg::kABytes) : umma_desc_k128(a_addr + Cfg::kABytes);
                 // 16 bf16 columns = 32 bytes further along the swizzled row: +2 in 16-byte units; a chunk is a block of its own
-                const uint64_t astep = chunks ? kUBlockBytes / 16 : 2, bstep = chunks ? BN * kChunk * 2 / 16 : 2;
+                const uint64_t astep = chunks ? kUBlockBytes / 16 : 2, bstep = one_b ? 0 : (chunks ? BN * kChunk * 2 / 16 : 2);
 #pragma unroll 4
                 for (int k = 0; k < ksteps; ++k) {
                     umma_bf16(d_tmem, adesc + (uint64_t)k * astep, bdesc + (uint64_t)k * bstep, idesc, accumulate);
@@ -676,7 +686,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                     if (!ok) break;
                     const uint32_t info = ctrl->stage_info[stage];
                     more = (info & kStageCommit) == 0;
-                    issue(d_tmem, (int)(info & 0xffu), (info & kStageChunks) != 0, accumulate);
+                    issue(d_tmem, (int)(info & 0xffu), (info & kStageChunks) != 0, (info & kStageOneB) != 0, accumulate);
                 }
                 if (ok) umma_commit(smem_u32(&ctrl->tmem_full[acc]));
             };
@@ -821,15 +831,17 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                     if (i >= sp.n) continue;
                     const bool mine = my_slot == sp.slot[i];
                     const float sc = snap.scale[sp.slot[i]];
+                    const int have = (int)snap.rank[sp.slot[i]] - sp.c[i] * kChunk;   // columns that the adapter has, of these (Inf in x times the padding of A: not into u)
+                    auto at = [&](int b, int col) { return col < have ? __uint_as_float(r[b + col]) * sc : 0.f; };
                     __nv_bfloat16* out = const_cast<__nv_bfloat16*>(p.part[0].u) + ((size_t)sp.m * p.part[0].cap + sp.first + i) * (kTileM * kChunk) + chunk_elem(q * 32 + lane, 0);
 #pragma unroll
                     for (int j = 0; j < 2; ++j) {
-                        const int b = ii * 16 + j * 8;
+                        const int b = ii * 16, c = j * 8;
                         uint4 v;
-                        v.x = pack_bf16(__uint_as_float(r[b + 0]) * sc, __uint_as_float(r[b + 1]) * sc);
-                        v.y = pack_bf16(__uint_as_float(r[b + 2]) * sc, __uint_as_float(r[b + 3]) * sc);
-                        v.z = pack_bf16(__uint_as_float(r[b + 4]) * sc, __uint_as_float(r[b + 5]) * sc);
-                        v.w = pack_bf16(__uint_as_float(r[b + 6]) * sc, __uint_as_float(r[b + 7]) * sc);
+                        v.x = pack_bf16(at(b, c + 0), at(b, c + 1));
+                        v.y = pack_bf16(at(b, c + 2), at(b, c + 3));
+                        v.z = pack_bf16(at(b, c + 4), at(b, c + 5));
+                        v.w = pack_bf16(at(b, c + 6), at(b, c + 7));
                         if (!mine) v = make_uint4(0, 0, 0, 0);
                         *reinterpret_cast<uint4*>(out + j * 64) = v;
                     }
@@ -905,7 +917,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                         const int phys = j ^ ((lane >> 1) & 3);
                         *reinterpret_cast<uint4*>(bp + lane * 64 + phys * 16) = v;
                     }
-                    if (nf_slot >= 0) add_nonfinite(pt, nf_slot, col0, pt.u + nf_u, pass ? p.u2 + nf_u : (pt.u_lo ? pt.u_lo + nf_u : nullptr), bp + lane * 64, (lane >> 1) & 3);
+                    if (nf_slot >= 0) add_nonfinite(pt, nf_slot, col0, pt.u + nf_u, pass ? p.u2 + nf_u : (pt.u_mid ? pt.u_mid + nf_u : nullptr), pt.u_lo ? pt.u_lo + nf_u : nullptr, bp + lane * 64, (lane >> 1) & 3);
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) {
@@ -1046,7 +1058,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
                     const __nv_bfloat16* u = side ? p.u2 : pt.u;
                     const uint32_t* list = lists + side * kMaxChunks;
                     const int count = ctrl->listed[side];
-                    const int per = pt.u_lo ? 2 : 4;   // chunks to a stage
+                    const int per = pt.u_lo ? 1 : 4;   // chunks to a stage
                     for (int i = 0; i < count && ok; i += per) {
                         ok = acquire();
                         if (!ok) break;
@@ -1054,9 +1066,9 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
                         int nk = 0;
                         for (int q = i; q < min(i + per, count); ++q) {
                             load_chunk<BN>(pt, u, m, n, list[q] & 0xffffu, (int)(list[q] >> 16), nk++, a_dst, a_dst + Cfg::kABytes, bar);
-                            if (pt.u_lo) load_chunk<BN>(pt, pt.u_lo, m, n, list[q] & 0xffffu, (int)(list[q] >> 16), nk++, a_dst, a_dst + Cfg::kABytes, bar);
+                            if (pt.u_lo) load_u_rest(pt, m, (int)(list[q] >> 16), a_dst, bar);
                         }
-                        ctrl->stage_info[stage] = (uint32_t)nk | kStageChunks | (side ? kStageAcc1 : 0u);
+                        ctrl->stage_info[stage] = (pt.u_lo ? 3u | kStageOneB : (uint32_t)nk) | kStageChunks | (side ? kStageAcc1 : 0u);
                         mbar_arrive(bar);
                         advance();
                     }
@@ -1090,7 +1102,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
                 const uint32_t a_addr = tiles_addr + stage * Cfg::kStageBytes;
                 const uint64_t adesc = chunks ? umma_desc_k16(a_addr) : umma_desc_k128(a_addr);
                 const uint64_t bdesc = chunks ? umma_desc_k16(a_addr + Cfg::kABytes) : umma_desc_k128(a_addr + Cfg::kABytes);
-                const uint64_t astep = chunks ? kUBlockBytes / 16 : 2, bstep = chunks ? BN * kChunk * 2 / 16 : 2;
+                const uint64_t astep = chunks ? kUBlockBytes / 16 : 2, bstep = (info & kStageOneB) ? 0 : (chunks ? BN * kChunk * 2 / 16 : 2);
                 tc_fence_after();
                 if ((info & kStageAcc1) == 0) {
 #pragma unroll 4
@@ -1197,7 +1209,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
                 *reinterpret_cast<uint4*>(yout + (size_t)pos * pt.N + col0 + j * 8) = v;
             }
             if (nf_slot >= 0)
-                add_nonfinite(pt, nf_slot, col0, (o ? p.u2 : pt.u) + nf_u, o || !pt.u_lo ? nullptr : pt.u_lo + nf_u, reinterpret_cast<uint8_t*>(yout + (size_t)pos * pt.N + col0), 0);
+                add_nonfinite(pt, nf_slot, col0, (o ? p.u2 : pt.u) + nf_u, pt.u_mid ? pt.u_mid + nf_u : nullptr, pt.u_lo ? pt.u_lo + nf_u : nullptr, reinterpret_cast<uint8_t*>(yout + (size_t)pos * pt.N + col0), 0);
         }
     }
     }   // outputs
@@ -1450,7 +1462,7 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
         } else {
             pt.y = pt.w;
         }
-        pt.bk = pr.ar->Bk; pt.b = pr.ar->B; pt.nonfinite = pr.ar->nonfinite; pt.plan = pr.plan; pt.u = pr.u; pt.u_lo = pr.u_lo; pt.y_ptr = (__nv_bfloat16*)pr.y;
+        pt.bk = pr.ar->Bk; pt.b = pr.ar->B; pt.nonfinite = pr.ar->nonfinite; pt.plan = pr.plan; pt.u = pr.u; pt.u_mid = pr.u_mid; pt.u_lo = pr.u_lo; pt.y_ptr = (__nv_bfloat16*)pr.y;
         pt.live = pt.nch[0] = pt.nch[1] = 0ull;
         for (int s = 0; s < pr.snap->max_slots; ++s)
             if (pr.snap->rank[s] > 0) {

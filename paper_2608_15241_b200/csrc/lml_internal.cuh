@@ -137,7 +137,8 @@ struct BindPart {
     const uint32_t* nonfinite;    // as in Arena
     TilePlan* plan;               // [row tile]
     __nv_bfloat16* u;
-    __nv_bfloat16* u2;            // a second set of blocks (see BindArgs::second)
+    __nv_bfloat16* u2;            // further sets of blocks (see BindArgs::second)
+    __nv_bfloat16* u3;
     int cap;
     int pad;
 };
@@ -145,7 +146,8 @@ struct BindArgs {
     const void* x;
     int T, d_in, P;
     RowSource rows;
-    // what u2 holds: dual calls 1 the second binding's blocks, 2 second minus first; else 3 the rest of u beyond its bf16 value
+    // what u2 holds: dual calls 1 the second binding's blocks, 2 second minus first; else 3: u, u2 and u3 are three bf16 values
+    // whose sum is the fp32 u (zeros in u2 and u3 where u is not finite)
     int second = 0;
     // early start of the GEMM (see bind_starts_gemm_early): the word that says "x may be read" and this call's value of it
     uint32_t* x_flag = nullptr;
@@ -169,7 +171,8 @@ struct GemmProj {
     const SlotSnapshot* snap;
     const TilePlan* plan;
     const __nv_bfloat16* u;
-    const __nv_bfloat16* u_lo;   // or null: the rest of u, multiplied with the same B
+    const __nv_bfloat16* u_mid;   // or null: what the bf16 values in u leave of the fp32 u, in two further sets, multiplied
+    const __nv_bfloat16* u_lo;    // with the same B
     int cap;
 };
 // What the library takes for a call: width of an output tile and CTAs that share one (1: whole-K tiles), CTAs in all, and

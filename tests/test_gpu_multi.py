@@ -199,3 +199,43 @@ def test_projections_of_a_few_blocks_of_tokens_keep_u_beyond_bf16(T, K, Ns):
         ref, _ = oracle.forward(x, W[p], ents[p], np.arange(T + 1, dtype=np.int32), tok)
         err = [np.linalg.norm(wl.bf16_bits_to_f64(y) - ref) / np.linalg.norm(ref) for y in (out[p], sep[p])]
         assert err[0] <= 1.01 * err[1], (p, err)     # (both are the rounding of y; u rounded to bf16 would add 2^-9 / sqrt(3) of the LoRA term)
+
+
+@pytest.mark.parametrize("T", [17, 40, 48])
+def test_projections_of_a_few_blocks_of_tokens_keep_u_in_fp32(T):
+    """Two columns of A that differ in one element by 2^-9 of a typical one, with opposite columns of B, on a zero W0: y is the difference of two u
+    that agree in about 12 bits.  fp32 sums of 520 products leave it some 2^-10 of relative error and y's rounding 2^-9; u of 16
+    bits would leave 2^-4, of 8 bits nothing."""
+    K, Ns = 520, (264, 136)
+    x, W, ents, tok = _case(700 + T, K, Ns, [(2, 2, 2)] * 2, [(1.0, 2.0, 0.5)] * 2, T)
+    W = [np.zeros_like(w) for w in W]
+    for p in range(2):
+        for e in ents[p]:
+            e.A[0, 7] = 0
+            e.A[1] = e.A[0]
+            e.A[1, 7] = wl.f32_to_bf16_bits(np.array([0.02 * 2.0 ** -7], np.float32))[0]
+            e.B[:, 1] = e.B[:, 0] ^ 0x8000
+    out, sep, flags = _run_multi(K, Ns, x, W, ents, tok)
+    assert flags == [0, 0]
+    for p in range(2):
+        ref, _ = oracle.forward(x, W[p], ents[p], np.arange(T + 1, dtype=np.int32), tok)
+        own = tok >= 0
+        for y in (out[p], sep[p]):
+            err = np.linalg.norm(wl.bf16_bits_to_f64(y)[own] - ref[own]) / np.linalg.norm(ref[own])
+            assert err <= 2.0 ** -7, (p, err)
+
+
+@pytest.mark.parametrize("T", [17, 40, 200])
+def test_infinite_u_stays_infinite(T):
+    """An Inf in a row of A, and an Inf in a row of x: y is Inf where the sums have one sign and NaN where they do not, as in separate calls."""
+    K, Ns = 264, (136, 72)
+    x, W, ents, tok = _case(800 + T, K, Ns, [(1, 4, 1)] * 2, [(1.0, 2.0, 0.5)] * 2, T)
+    tok[2], tok[3], tok[5] = 0, 2, 2
+    for p in range(2):
+        ents[p][0].A[0, 3] = 0x7f80          # u of adapter 0 is +-Inf, or NaN with x = 0
+    x[5, 9] = 0x7f80                         # a row of x on a rank-1 adapter
+    out, sep, flags = _run_multi(K, Ns, x, W, ents, tok)
+    for p in range(2):
+        a, b = wl.bf16_bits_to_f64(out[p]), wl.bf16_bits_to_f64(sep[p])
+        assert np.isinf(b).any()
+        assert np.array_equal(np.isnan(a), np.isnan(b)) and np.array_equal(np.where(np.isinf(a), a, 0), np.where(np.isinf(b), b, 0))
