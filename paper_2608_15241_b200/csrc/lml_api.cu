@@ -63,14 +63,13 @@ struct GemmCall {
     const int32_t* ids;     // per token, or per segment
     uint8_t* ws;
     WsLayout layout;
+    bool precise = false;   // u goes into the product as three bf16 values that add up to its fp32 value, two further K-steps per chunk
 };
 
 // The GEMM path: the rows stay in their order; one launch binds them and computes u (unless the GEMM does both itself),
-// one launch multiplies.  P > 1: projections of the same x.  ids2 / y2: the second binding of a dual call.  precise: u goes
-// into the product as three bf16 values that add up to its fp32 value, two further K-steps per chunk.
+// one launch multiplies.  P > 1: projections of the same x.  ids2 / y2: the second binding of a dual call.
 cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, RowMode mode, const int32_t* seg_offsets, int G,
-                          const int32_t* perm, const int32_t* ids2, void* y2, bool by_adapter, cudaStream_t stream, int* launches,
-                          bool precise = false)
+                          const int32_t* perm, const int32_t* ids2, void* y2, bool by_adapter, cudaStream_t stream, int* launches)
 {
     lml_table* t0 = calls[0].t;
     const int num_m = (T + kTileM - 1) / kTileM;
@@ -101,11 +100,11 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         bp.plan = reinterpret_cast<TilePlan*>(c.ws + c.layout.plan_off);
         bp.u = reinterpret_cast<__nv_bfloat16*>(c.ws + c.layout.u_off);
         bp.u2 = reinterpret_cast<__nv_bfloat16*>(c.ws + c.layout.u2_off);
-        bp.u3 = reinterpret_cast<__nv_bfloat16*>(c.ws + c.layout.u3_off);
+        bp.u3 = c.precise ? reinterpret_cast<__nv_bfloat16*>(c.ws + c.layout.u3_off) : nullptr;
         bp.cap = cap;
         GemmProj& gp = g.proj[p];
         gp.W0 = c.W0; gp.y = c.y; gp.d_out = c.t->d_out; gp.ar = &c.t->arena; gp.snap = &snap[p];
-        gp.plan = bp.plan; gp.u = bp.u; gp.u_mid = precise ? bp.u2 : nullptr; gp.u_lo = precise ? bp.u3 : nullptr; gp.cap = cap;
+        gp.plan = bp.plan; gp.u = bp.u; gp.u_mid = c.precise ? bp.u2 : nullptr; gp.u_lo = bp.u3; gp.cap = cap;
     }
     g.num_sms = t0->num_sms;
     if (mode == kRowsSegments && (perm || G > kBindSegs || num_m > kSlabTiles)) {   // a slot per row first
@@ -140,7 +139,6 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
             if (++t0->next_call == 0u) ++t0->next_call;
             b.call_id = g.call_id = t0->next_call;
         }
-        if (precise) b.second = 3;
         if (dual) {
             // (split-K: an accumulator per binding; whole-K tiles: the second output is the first plus the difference)
             b.second = g.shape.split > 1 ? 1 : 2;
@@ -812,17 +810,16 @@ lml_status lora_mixed_linear_multi(lml_table* const* tables, int P, const void* 
         DeviceGuard guard(tables[0]->device);
         if (!guard.ok) return LML_ERR_CUDA;
         GemmCall calls[LML_MAX_PROJECTIONS];
-        // A call of its own would run as blocks of 16 tokens on the decode kernel, which keeps u in fp32: the shared launches
-        // carry it as three bf16 values then, which is as many bits.
-        bool precise = false;
         size_t off = 0;
         for (int p = 0; p < P; ++p) {
             calls[p] = GemmCall{tables[p], W0[p], y[p], token_slots[p], static_cast<uint8_t*>(workspace) + off, tokens_layout(tables[p], T)};
-            precise = precise || T <= decode_block_limit(tables[p]);
+            // (in a call of its own this projection would run as blocks of 16 tokens on the decode kernel, which keeps u in fp32:
+            // the shared launches carry it as three bf16 values then, which is as many bits)
+            calls[p].precise = T <= decode_block_limit(tables[p]);
             off += round_up(calls[p].layout.total, 1024);
         }
         int launches = 0;
-        const cudaError_t e = run_gemm_path(calls, P, x, T, kRowsTokens, nullptr, 0, nullptr, nullptr, nullptr, false, stream, &launches, precise);
+        const cudaError_t e = run_gemm_path(calls, P, x, T, kRowsTokens, nullptr, 0, nullptr, nullptr, nullptr, false, stream, &launches);
         if (e != cudaSuccess) { cudaGetLastError(); return LML_ERR_CUDA; }
         for (int p = P - 1; p >= 0; --p) tables[p]->last_launches = p == 0 ? launches : 0;
         return LML_OK;

@@ -316,7 +316,7 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
             const bool a = ctrl->row[0][tr] == slot, b = dual && ctrl->row[1][tr] == slot;
             const uint2 zero = make_uint2(0u, 0u);
             const size_t at = ((size_t)m * part.cap + c0 + (piece >> 2)) * (kTileM * kChunk) + chunk_elem(tr, (piece & 3) * 4);
-            if (L.second == 3) {
+            if (part.u3) {
                 uint2 hi, mid, lo;
                 split_bf16(v.x, v.y, hi.x, mid.x, lo.x);
                 split_bf16(v.z, v.w, hi.y, mid.y, lo.y);

@@ -209,12 +209,20 @@ __device__ __forceinline__ int list_chunks(const TilePlan* plan, uint32_t who, i
     return n;
 }
 // The terms of one row that the product with the chunks left out, 32 columns from col0: u_j B[n][j] where B is Inf or NaN.
-// u, u_more, u_rest: the row of the slot's first block (the others: to be added to it, or null); out: the row's outputs, bf16, 16-byte
-// pieces in an order given by piece_xor.
-__device__ __noinline__ void add_nonfinite(const GemmPart& pt, int slot, int col0, const __nv_bfloat16* u, const __nv_bfloat16* u_more,
-                                           const __nv_bfloat16* u_rest, uint8_t* out, int piece_xor)
+// slot, index: the row's slot and the number of its first chunk (index < 0: looked up in the tile's plan, and the slot with it,
+// under binding `which`); u, u_more, u_rest: the sets of blocks whose sum is u (the latter two may be null); out: the row's outputs,
+// bf16, 16-byte pieces in an order given by piece_xor.  Out of line, and all of it, so that the epilogue stays as short as it is
+// without.
+__device__ __noinline__ void add_nonfinite(const GemmPart& pt, int m, int row, int which, int slot, int index, int col0, const __nv_bfloat16* u,
+                                           const __nv_bfloat16* u_more, const __nv_bfloat16* u_rest, uint8_t* out, int piece_xor)
 {
     auto value = [](const __nv_bfloat16* p) { return __uint_as_float(ld_after_wait(reinterpret_cast<const uint16_t*>(p)) << 16); };
+    if (index < 0) {
+        slot = ld_after_wait(&pt.plan[m].nonfinite_row[which][row]);
+        if (slot < 0) return;
+        for (index = 0; index < kMaxChunks - 1 && (int)(ld_after_wait(&pt.plan[m].chunk[index]) & 0xfffu) != slot;) ++index;
+    }
+    const size_t u_at = ((size_t)m * pt.cap + index) * (kTileM * kChunk) + chunk_elem(row, 0);
     const int cols = slot_chunks(pt, slot) * kChunk;
     for (int c = 0; c < kEpiChunkCols && col0 + c < pt.N; ++c) {
         const __nv_bfloat16* b = pt.b + ((size_t)slot * pt.N + col0 + c) * kRankPad;
@@ -223,7 +231,7 @@ __device__ __noinline__ void add_nonfinite(const GemmPart& pt, int slot, int col
         for (int j = 0; j < cols; ++j) {
             const float bv = value(b + j);
             if (isfinite(bv)) continue;
-            const size_t at = (size_t)(j / kChunk) * (kTileM * kChunk) + chunk_elem(0, j % kChunk);
+            const size_t at = u_at + (size_t)(j / kChunk) * (kTileM * kChunk) + chunk_elem(0, j % kChunk);
             sum += (value(u + at) + (u_more ? value(u_more + at) : 0.f) + (u_rest ? value(u_rest + at) : 0.f)) * bv;
             any = true;
         }
@@ -231,17 +239,6 @@ __device__ __noinline__ void add_nonfinite(const GemmPart& pt, int slot, int col
         __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(out + ((c >> 3) ^ piece_xor) * 16 + (c & 7) * 2);
         *o = __float2bfloat16_rn(__bfloat162float(*o) + sum);
     }
-}
-// number of the first of a slot's chunks among those of a tile
-__device__ __noinline__ int first_chunk_of(const TilePlan* plan, int slot)
-{
-    int i = 0;
-    while (i < kMaxChunks - 1 && (int)(ld_after_wait(&plan->chunk[i]) & 0xfffu) != slot) ++i;
-    return i;
-}
-__device__ __forceinline__ size_t u_row(const GemmPart& pt, int m, int index, int row)
-{
-    return ((size_t)m * pt.cap + index) * (kTileM * kChunk) + chunk_elem(row, 0);
 }
 // One chunk of a stage: the block of u (number `index` of row tile m) and the chunk's rows of B for columns
 // [n * BN, + BN), each contiguous.  entry = slot | chunk << 8.
@@ -872,20 +869,6 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                 fph ^= 1u;
                 tc_fence_after();
                 const bool last_pass = pass == (dual ? 1 : 0);
-                int nf_slot = -1;   // this row's slot, if its B holds Inf or NaN
-                size_t nf_u = 0;
-                if (nonfinite) {
-                    if (!p.fused) {
-                        nf_slot = ld_after_wait(&pt.plan[m].nonfinite_row[pass][q * 32 + lane]);
-                        if (nf_slot >= 0) nf_u = u_row(pt, m, first_chunk_of(pt.plan + m, nf_slot), q * 32 + lane);
-                    } else {
-                        const int s = row_base + lane < p.T ? row_slot(row_base + lane) : -1;
-                        if (s >= 0 && ((ctrl->nonfinite >> s) & 1ull)) {
-                            nf_slot = s;
-                            nf_u = u_row(pt, m, mask_chunks(pt, tile_mask[m] & ((1ull << s) - 1ull)), q * 32 + lane);
-                        }
-                    }
-                }
                 const uint32_t t_addr = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(acc * BN);
 #pragma unroll 1
                 for (int c = 0; c < BN / kEpiChunkCols; ++c) {
@@ -917,7 +900,15 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                         const int phys = j ^ ((lane >> 1) & 3);
                         *reinterpret_cast<uint4*>(bp + lane * 64 + phys * 16) = v;
                     }
-                    if (nf_slot >= 0) add_nonfinite(pt, nf_slot, col0, pt.u + nf_u, pass ? p.u2 + nf_u : (pt.u_mid ? pt.u_mid + nf_u : nullptr), pt.u_lo ? pt.u_lo + nf_u : nullptr, bp + lane * 64, (lane >> 1) & 3);
+                    if (__builtin_expect(nonfinite, 0)) {
+                        int s = -1, index = -1;
+                        if (p.fused && row_base + lane < p.T) {
+                            s = row_slot(row_base + lane);
+                            if (s >= 0 && ((ctrl->nonfinite >> s) & 1ull)) index = mask_chunks(pt, tile_mask[m] & ((1ull << s) - 1ull));
+                        }
+                        if (!p.fused || index >= 0)
+                            add_nonfinite(pt, m, q * 32 + lane, pass, s, index, col0, pt.u, pass ? p.u2 : pt.u_mid, pt.u_lo, bp + lane * 64, (lane >> 1) & 3);
+                    }
                     fence_proxy_async_smem();
                     __syncwarp();
                     if (lane == 0) {
@@ -1181,8 +1172,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
         const int pos = m * kBM + row;
         const bool row_ok = pos < p.T;
         const int c_first = first_chunk(rank), c_end = first_chunk(rank + 1);
-        const int nf_slot = nonfinite && row_ok ? ld_after_wait(&pt.plan[m].nonfinite_row[o][row]) : -1;   // this row's slot, if its B holds Inf or NaN
-        const size_t nf_u = nf_slot >= 0 ? u_row(pt, m, first_chunk_of(pt.plan + m, nf_slot), row) : 0;
 #pragma unroll 1
         for (int c = c_first; c < c_end; ++c) {
             float acc[32];
@@ -1208,8 +1197,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
                 v.w = pack_bf16(acc[8 * j + 6], acc[8 * j + 7]);
                 *reinterpret_cast<uint4*>(yout + (size_t)pos * pt.N + col0 + j * 8) = v;
             }
-            if (nf_slot >= 0)
-                add_nonfinite(pt, nf_slot, col0, (o ? p.u2 : pt.u) + nf_u, pt.u_mid ? pt.u_mid + nf_u : nullptr, pt.u_lo ? pt.u_lo + nf_u : nullptr, reinterpret_cast<uint8_t*>(yout + (size_t)pos * pt.N + col0), 0);
+            if (__builtin_expect(nonfinite, 0))
+                add_nonfinite(pt, m, row, o, -1, -1, col0, o ? p.u2 : pt.u, pt.u_mid, pt.u_lo, reinterpret_cast<uint8_t*>(yout + (size_t)pos * pt.N + col0), 0);
         }
     }
     }   // outputs

@@ -138,7 +138,7 @@ struct BindPart {
     TilePlan* plan;               // [row tile]
     __nv_bfloat16* u;
     __nv_bfloat16* u2;            // further sets of blocks (see BindArgs::second)
-    __nv_bfloat16* u3;
+    __nv_bfloat16* u3;            // or null
     int cap;
     int pad;
 };
@@ -146,8 +146,8 @@ struct BindArgs {
     const void* x;
     int T, d_in, P;
     RowSource rows;
-    // what u2 holds: dual calls 1 the second binding's blocks, 2 second minus first; else 3: u, u2 and u3 are three bf16 values
-    // whose sum is the fp32 u (zeros in u2 and u3 where u is not finite)
+    // what u2 holds in a dual call: 1 the second binding's blocks, 2 second minus first.  Else, where a part has u3: u, u2 and u3
+    // are three bf16 values whose sum is the fp32 u (zeros in u2 and u3 where u is not finite)
     int second = 0;
     // early start of the GEMM (see bind_starts_gemm_early): the word that says "x may be read" and this call's value of it
     uint32_t* x_flag = nullptr;
