@@ -212,7 +212,7 @@ lml_status lml_segment_tokens(lml_table* t, const int32_t* token_slots, int T, i
  * W0 is the frozen base weight: it must not be written by work on `stream` that may still be running
  * when the call is reached (the decode kernel, and the GEMM of a call of few rows, start fetching W0
  * while the kernel before them is still draining; x, the segment arrays and the adapters are read only
- * after that kernel has finished).
+ * after that kernel has finished, however long that takes).
  * Errors: INVALID_ARG, WORKSPACE, CUDA.
  */
 lml_status lora_mixed_linear(lml_table* t, const void* x, const void* W0, int T,

@@ -24,7 +24,8 @@
 // table's device memory; a producer waits for a tile's flags (a bounded wait) before it loads the tile's u blocks.  The
 // table's epoch, advanced by the last CTA of every such call, tells this call's flags from the last call's.
 // Early start (few rows): the kernel begins while the work before the call is still running.  It asks for the first stages'
-// W0, which is frozen, and reads x once bind_shrink, which waits for that work, has raised a word for it (a bounded wait).
+// W0, which is frozen, and reads x once bind_shrink, which waits for that work, has raised a word for it.  That work may take as
+// long as it likes: no other role, and no limit, starts before x may be read (see wait_x).
 // For few tokens (tiles far fewer than SMs) a split-K variant follows below: a cluster of CTAs shares a
 // tile and exchanges partial sums through distributed shared memory.
 // B's chunks hold zeros where the adapter's B is Inf or NaN (every row of a tile meets the chunks of all its slots).  The terms
@@ -156,25 +157,17 @@ __device__ __forceinline__ int mask_chunks(const GemmPart& pt, unsigned long lon
     for (; mask; mask &= mask - 1ull) n += slot_chunks(pt, __ffsll((long long)mask) - 1);
     return n;
 }
-// Early start: W0 is on its way already; x may be read once the launch that this one overlaps with says so (bounded wait).
-__device__ __forceinline__ bool wait_x(const GemmParams& p, volatile int* abort)
+// Early start: W0 is on its way already; x may be read once bind_shrink, which this launch overlaps with, says so.  The word is
+// polled for a few milliseconds; if the work before the call runs on for longer, the hardware's wait for the whole of bind_shrink
+// (which waits for that work) takes over.  The rest of the CTA is held at a barrier meanwhile, so that the limits of the other
+// waits in this kernel measure this kernel only.
+constexpr long long kPollClocks = 1ll << 22;
+__device__ __forceinline__ void wait_x(const GemmParams& p)
 {
     const long long t0 = clock64();
-    while (ld_acquire_gpu_u32(p.x_flag) != p.call_id) {
-        if (*abort) return false;
-        if (clock64() - t0 > (1ll << 31)) { *abort = 1; return false; }
-    }
+    while (ld_acquire_gpu_u32(p.x_flag) != p.call_id)
+        if (clock64() - t0 > kPollClocks) { grid_dependency_wait(); break; }
     fence_proxy_async_all();
-    return true;
-}
-// A give-up before x: the copies of W0 that are on their way land (again a bounded wait) before the CTA leaves.
-__device__ __forceinline__ void drain_ahead(GemmCtrl* ctrl, int ahead)
-{
-    volatile int never = 0;
-    for (int i = 0; i < ahead; ++i) {
-        mbar_arrive(smem_u32(&ctrl->full[i]));
-        mbar_wait(smem_u32(&ctrl->full[i]), 0u, &never);
-    }
 }
 // ... and its last CTA clears the word: a replay of the same call finds it cleared.
 __device__ __forceinline__ void leave_early_start(const GemmParams& p)
@@ -329,6 +322,21 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
     tc_fence_after();
     const uint32_t tmem_base = ctrl->tmem_base;
     volatile int* abort = &ctrl->abort;
+    if (p.x_flag) {   // early start: the first k-blocks' W0, then x
+        const GemmPart& pt = p.part[part_of(p, (int)blockIdx.x)];
+        const int n0 = ((int)blockIdx.x - pt.tile0) / num_mt;
+        if (warp == 0 && lane == 0) {
+            for (int kb = 0; kb < min(Cfg::kStages, num_kb); ++kb) {
+                const uint32_t bar = smem_u32(&ctrl->full[kb]);
+                mbar_expect_tx(bar, Cfg::kBBytes);
+                tma_load_2d(tiles_addr + kb * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, kb * kBK, n0 * BN);
+            }
+            wait_x(p);
+        } else if (warp == 2) {
+            prefetch_b<BN>(pt, n0, lane, 0, 1);
+        }
+        __syncthreads();
+    }
     if (!p.lora || p.fused) {   // no launch of this call came before this one: wait for foreign work here
         grid_dependency_wait();
         grid_launch_dependents();
@@ -552,18 +560,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                     advance();
                 }
             }
-            int ahead = 0;   // early start: k-blocks of the first tile whose W0 has been asked for already
-            if (p.x_flag) {
-                const GemmPart& pt = *list0_part;
-                ahead = min(Cfg::kStages, num_kb);
-                for (int kb = 0; kb < ahead; ++kb) {
-                    const uint32_t bar = smem_u32(&ctrl->full[kb]);
-                    mbar_expect_tx(bar, Cfg::kBBytes);
-                    tma_load_2d(tiles_addr + kb * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, kb * kBK, list0_n * BN);
-                }
-                ok = wait_x(p, abort);
-                if (!ok) drain_ahead(ctrl, ahead);
-            }
+            const int ahead = p.x_flag ? min(Cfg::kStages, num_kb) : 0;   // early start: k-blocks of the first tile whose W0 has been asked for already
             // k-blocks [k0, k1) of a tile; the ring's place lives in registers here (the lambdas above hold it by reference)
             auto base_blocks = [&](const CUtensorMap* w, int row0, int col0, int k0, int k1, uint32_t acc_flag, uint32_t flags_last, int have_w) {
                 int st = stage;
@@ -796,7 +793,6 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
         bool ok = true;
         if (p.lora && !p.fused && warp == 2) {   // nothing else to do yet: the first tile's chunks, as soon as they are known
             const GemmPart& pt = p.part[part_of(p, (int)blockIdx.x)];
-            if (p.x_flag) prefetch_b<BN>(pt, ((int)blockIdx.x - pt.tile0) / num_mt, lane, 0, 1);
             grid_dependency_wait();
             grid_launch_dependents();
             const int n = list_chunks(pt.plan + ((int)blockIdx.x - pt.tile0) % num_mt * kRowTiles, kChunkFirst | kChunkSecond, 0, 1, lane, list0);
@@ -1000,6 +996,20 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
     tc_fence_after();
     const uint32_t tmem_base = ctrl->tmem_base;
     volatile int* abort = &ctrl->abort;
+    if (p.x_flag) {   // early start: the first k-blocks' W0, then x
+        if (warp == 0 && lane == 0) {
+            const int kb0 = rank * num_kb / S, ahead = min(p.stages, (rank + 1) * num_kb / S - kb0);
+            for (int i = 0; i < ahead; ++i) {
+                const uint32_t bar = smem_u32(&ctrl->full[i]);
+                mbar_expect_tx(bar, Cfg::kBBytes);
+                tma_load_2d(tiles_addr + i * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, (kb0 + i) * kBK, n * BN);
+            }
+            wait_x(p);
+        } else if (warp == 2) {
+            prefetch_b<BN>(pt, n, lane, rank, S);
+        }
+        __syncthreads();
+    }
     if (!p.lora) {   // no launch of this call came before this one: wait for foreign work here
         grid_dependency_wait();
         grid_launch_dependents();
@@ -1016,17 +1026,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
             const int row0 = m * kBM;
             const int kb0 = rank * num_kb / S, kb1 = (rank + 1) * num_kb / S;
             // base k-blocks first: they do not depend on the launch that precedes this one
-            int ahead = 0;   // early start: k-blocks whose W0 has been asked for already
-            if (p.x_flag) {
-                ahead = min(p.stages, kb1 - kb0);
-                for (int i = 0; i < ahead; ++i) {
-                    const uint32_t bar = smem_u32(&ctrl->full[i]);
-                    mbar_expect_tx(bar, Cfg::kBBytes);
-                    tma_load_2d(tiles_addr + i * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, (kb0 + i) * kBK, n * BN);
-                }
-                ok = wait_x(p, abort);
-                if (!ok) drain_ahead(ctrl, ahead);
-            }
+            const int ahead = p.x_flag ? min(p.stages, kb1 - kb0) : 0;   // early start: k-blocks whose W0 has been asked for already
             for (int kb = kb0; kb < kb1 && ok; ++kb) {
                 ok = acquire();
                 if (!ok) break;
@@ -1122,7 +1122,6 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
     bool ok = true, nonfinite = false;
     if (warp >= 2) {
         if (p.lora && warp == 2) {   // nothing else to do yet: this CTA's share of the tile's chunks, as soon as they are known
-            if (p.x_flag) prefetch_b<BN>(pt, n, lane, rank, S);
             grid_dependency_wait();
             grid_launch_dependents();
             for (int side = 0; side < (dual ? 2 : 1); ++side) {

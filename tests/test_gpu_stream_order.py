@@ -101,3 +101,28 @@ def test_a_call_reads_the_x_that_the_call_before_it_wrote(T):
     assert all(np.array_equal(chain(False), want) for _ in range(4))
     assert tbl.device_status() == 0
     tbl.close()
+
+
+def test_a_call_behind_work_that_releases_its_dependents_early_and_runs_on():
+    """The segmentation kernel lets the kernels behind it start at once and then works on millions of tokens for longer than the
+    GEMM polls for x: the call behind it waits as long as that takes, with all its limits counted from there."""
+    import torch
+    T, K, N = 40, 2048, 520
+    tbl, W = _site(K, N)
+    x, ids = to_dev(wl.normal_bf16(1, 1, (T, K), 1.0)), _ids(T, 3)
+    want = to_bits(tbl.lora_mixed_linear_tokens(x, W, ids))
+    many = _ids(4_000_000, 3)
+    torch.cuda.synchronize()
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    a.record()
+    tbl.segment_tokens(many)
+    b.record()
+    torch.cuda.synchronize()
+    print("segmentation", a.elapsed_time(b), "ms")
+    for _ in range(3):
+        tbl.segment_tokens(many)
+        y = tbl.lora_mixed_linear_tokens(x, W, ids)
+        torch.cuda.synchronize()
+        assert np.array_equal(to_bits(y), want)
+    assert tbl.device_status() == 0
+    tbl.close()
