@@ -129,7 +129,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         // With whole-K tiles and few row tiles the shrink runs inside the GEMM kernel (on the CTAs that own the fewest tiles,
         // ahead of their tiles); otherwise a launch goes first and the GEMM is its programmatic dependent.
         g.fused = mode == kRowsSegments && !dual && P == 1 && T == rows && t0->fuse_shrink &&
-                  gemm_can_fuse_shrink(g.shape, T, t0->d_out, G, b.rows.mode == kRowsSegments, b.part[0].cap, t0->num_sms);
+                  gemm_can_fuse_shrink(g.shape, T, t0->d_out, G, b.rows.mode == kRowsSegments, t0->max_slots, t0->num_sms);
         if (g.fused) g.rows = b.rows;
         b.x_flag = g.x_flag = nullptr;
         if (mode != kRowsNone && !g.fused && bind_starts_gemm_early(rows, P, t0->num_sms)) {

@@ -1414,17 +1414,22 @@ bool TmapCache::get_2d(CUtensorMap* out, const void* base, uint64_t inner, uint6
 // the passes on CTAs with a tile's time to spare.  A shrink pass takes about as long as an output tile, whatever its width.
 // It pays where some CTAs have that time and the others do not reach their first chunks before it is over: 256-column
 // tiles in more than one wave, and few enough passes (every segment boundary inside a row tile can add one) that no CTA gets two.
-bool gemm_can_fuse_shrink(const GemmShape& shape, int T, int d_out, int G, bool in_segment_order, int cap, int num_sms)
+// (What counts is T, G and the table's size, not what is registered: the two forms sum x.A^T in different orders, and a call's
+// bits must not change with adapters that it does not use.  Segments in order: a tile has one pass and one more for every segment
+// that begins in it, at most; rows in any order: reckoned with half of the widest adapter for every segment.)
+bool gemm_can_fuse_shrink(const GemmShape& shape, int T, int d_out, int G, bool in_segment_order, int max_slots, int num_sms)
 {
     if (G <= 0 || (in_segment_order && G > kBindSegs)) return false;
     if (shape.split != 1 || shape.bn != 256) return false;
     const int num_m = (T + kBM - 1) / kBM, num_n = (d_out + 255) / 256;
     if (num_m > kFuseTilesInKernel || (!shape.tall && num_m * num_n <= num_sms)) return false;
-    int worst_passes = num_m * ((cap + kShrChunks - 1) / kShrChunks);
-    if (in_segment_order && num_m + G < worst_passes) worst_passes = num_m + G;
+    static_assert(kShrChunks * kChunk == kRankPad, "a slot takes one pass at most");
+    const int slots = G < max_slots ? G : max_slots;
+    if (num_m * slots > kShrMaxPasses * num_sms && !in_segment_order) return false;   // (room for a CTA's passes)
+    const int passes = in_segment_order ? num_m + G : num_m * ((slots + 1) / 2);
     // (tall tiles: only as many passes as there are CTAs with a tile less than the others, or none)
-    if (shape.tall) return worst_passes <= num_sms - (shape.ctas - 1) % num_sms - 1;
-    return worst_passes <= num_sms / 2;
+    if (shape.tall) return passes <= num_sms - (shape.ctas - 1) % num_sms - 1;
+    return passes <= num_sms / 2;
 }
 
 cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* caches, const GemmArgs& a, cudaStream_t stream)

@@ -197,8 +197,8 @@ struct GemmArgs {
 };
 // split_bn, split_s: the table's override (-1 = the library chooses, 0 = whole-K tiles, else the forced shape)
 GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, int num_sms, int split_bn, int split_s);
-// whether the shrink of a plain call of this size and shape runs inside the GEMM kernel; cap: chunks per tile at most
-bool gemm_can_fuse_shrink(const GemmShape& shape, int T, int d_out, int G, bool in_segment_order, int cap, int num_sms);
+// whether the shrink of a plain call of this size and shape runs inside the GEMM kernel
+bool gemm_can_fuse_shrink(const GemmShape& shape, int T, int d_out, int G, bool in_segment_order, int max_slots, int num_sms);
 // Tensor maps of caller buffers, kept per table and found again by (pointer, shape, box).
 struct TmapCache {
     static constexpr int kEntries = 32;

@@ -71,3 +71,39 @@ def test_malformed_offsets_are_caught_by_the_fused_form(monkeypatch):
     good, f3 = site.run(seg_offsets=[0, T // 3, 2 * T // 3, T], raw_slot_ids=[site.slots[0], -1, site.slots[2]])
     assert f3 == 0 and np.array_equal(y2, good)
     site.close()
+
+
+@pytest.mark.parametrize("T,N,G", [(2048, 4096, 8), (700, 8192, 5), (130, 2048, 3), (40, 520, 2)])
+def test_bits_do_not_depend_on_adapters_that_the_call_does_not_use(T, N, G):
+    """More and wider adapters are registered beside those of the call: the form of the shrink, the tiles and the order of the
+    sums stay as they are."""
+    import torch
+    from paper_2608_15241_b200.binding import Table
+    from gpu_util import to_bits, to_dev
+    K = 2048
+    tbl = Table(K, N, 24)
+
+    def add(a, r):
+        return tbl.register_adapter(a, 1, to_dev(wl.normal_bf16(3, 100 + a, (r, K), 0.02)), to_dev(wl.normal_bf16(3, 200 + a, (N, r), 0.02)), 2.0)
+
+    slots = [add(a, 16) for a in range(4)]
+    x, W = to_dev(wl.normal_bf16(3, 1, (T, K), 1.0)), to_dev(wl.normal_bf16(3, 2, (N, K), 0.02))
+    ids = np.array([slots[g % 4] for g in range(G)], np.int32)
+    so = np.linspace(0, T, G + 1).astype(np.int32)
+    tok = torch.from_numpy(np.repeat(ids, np.diff(so))).cuda()
+    so, ids = torch.from_numpy(so).cuda(), torch.from_numpy(ids).cuda()
+
+    def calls():
+        perm, po, pi = tbl.segment_tokens(tok)
+        return [to_bits(y) for y in (tbl.lora_mixed_linear(x, W, so, ids), tbl.lora_mixed_linear_tokens(x, W, tok),
+                                     tbl.lora_mixed_linear(x, W, po, pi, perm=perm), *tbl.lora_mixed_linear_dual(x, W, so, ids, ids.flip(0).contiguous()))]
+
+    want = calls()
+    for a, r in ((4, 16), (5, 64), (6, 33)):
+        add(a, r)
+    for a in range(7, 24):
+        add(a, 64)
+        if a in (8, 23):
+            assert all(np.array_equal(y, w) for y, w in zip(calls(), want))
+    assert tbl.device_status() == 0
+    tbl.close()
