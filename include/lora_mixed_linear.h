@@ -37,7 +37,9 @@
  *     synchronise nor read device memory from the host.
  *   - Calls that use the same workspace, or the same table from different streams without
  *     ordering between them, race; one table may be shared by ordered streams.
- *   - Same inputs give bitwise the same y on every run (no atomics touch y).
+ *   - Same inputs give bitwise the same y on every run (no atomics touch y), whatever else is registered in the
+ *     table: y[t] follows from row t of x and the entry of token t (an adapter that holds Inf or NaN concerns its
+ *     own tokens only) and, in the order of its sums, from the shape of the call.
  */
 #ifndef LORA_MIXED_LINEAR_H_
 #define LORA_MIXED_LINEAR_H_
@@ -81,8 +83,8 @@ const char* lml_status_string(lml_status s);
 
 /*
  * Create the slot table of one linear site on CUDA device `device`.
- * Allocates (once, here) the packed adapter arena: max_slots * 64 * (d_in + d_out) bf16, plus
- * a few hundred bytes.  1 <= max_slots <= LML_MAX_SLOTS; d_in, d_out > 0 and multiples of 8.
+ * Allocates (once, here) the packed adapter arena, max_slots * (64 * d_in + 80 * d_out + 64 * (d_out rounded up
+ * to 256)) bf16 (B is kept three times, in the orders of the kernels that read it), plus about 100 KB.  1 <= max_slots <= LML_MAX_SLOTS; d_in, d_out > 0 and multiples of 8.
  * Errors: INVALID_ARG, UNSUPPORTED (not compute capability 10.x), CUDA.
  */
 lml_status lml_table_create(lml_table** out, int device, int d_in, int d_out, int max_slots);
@@ -95,7 +97,7 @@ lml_status lml_table_destroy(lml_table* t);
  * version": Section 4.2 / 5.3; a newer version is registered while the older one still
  * serves).  A: device bf16 [rank][d_in]; B: device bf16 [d_out][rank]; 1 <= rank <= 64;
  * scale is the final multiplier (the library never divides by rank).  The adapter is copied
- * into the table's arena in the layout the kernels read (rows zero-padded to rank 64) by a
+ * into the table's arena in the layout the kernels read (zero-padded to a multiple of 16 columns) by a
  * small kernel enqueued on `stream`; A and B may be released once that stream work is done.
  * The new entry is visible to calls issued after this returns; work on OTHER streams must be
  * ordered after `stream` by the caller.  *slot_out receives the physical slot index to use in
@@ -386,7 +388,8 @@ lml_status lora_mixed_linear_decode_static(lml_table* t, const void* x, const vo
 /*
  * Read and clear the sticky device status word (LML_FLAG_* bits).  Synchronises `stream`.
  * When the word carries LML_FLAG_TIMEOUT (a launch gave up on a wait), the table's decode exchange blocks
- * (values, marks, counters) are put back to zero as well; no decode call on the table may be in flight then.
+ * (values, marks, counters) and the words through which a GEMM is told that x may be read are put back to zero as
+ * well; no call on the table may be in flight then.
  * Errors: INVALID_ARG, CUDA.
  */
 lml_status lml_device_status(lml_table* t, uint32_t* flags_out, void* stream);

@@ -161,7 +161,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
 
 static void free_table_resources(lml_table* t)
 {
-    cudaFree(t->arena.A); cudaFree(t->arena.B); cudaFree(t->arena.Bc); cudaFree(t->arena.Bk); cudaFree(t->arena.status); cudaFree(t->arena.adapter_map); cudaFree(t->arena.tile_flags); cudaFree(t->arena.dec_u);
+    cudaFree(t->arena.A); cudaFree(t->arena.B); cudaFree(t->arena.Bc); cudaFree(t->arena.Bk); cudaFree(t->arena.status); cudaFree(t->arena.adapter_map); cudaFree(t->arena.pass_flags); cudaFree(t->arena.dec_u);
     if (t->copy_in) cudaStreamDestroy(t->copy_in);
     if (t->copy_out) cudaStreamDestroy(t->copy_out);
     if (t->ev_begin) cudaEventDestroy(t->ev_begin);
@@ -236,8 +236,8 @@ lml_status lml_table_create(lml_table** out, int device, int d_in, int d_out, in
     ok = ok && cudaMalloc(&t->arena.dec_u, dec_u_bytes) == cudaSuccess;
     ok = ok && cudaMemset(t->arena.dec_u, 0, dec_u_bytes) == cudaSuccess;   // mark 0: written by no launch
     ok = ok && cudaMemset(t->arena.adapter_map, 0xff, kMaxAdapterIds * sizeof(int32_t)) == cudaSuccess;   // -1: no serving version
-    ok = ok && cudaMalloc(&t->arena.tile_flags, kFuseMaxTiles * sizeof(int32_t)) == cudaSuccess;
-    ok = ok && cudaMemset(t->arena.tile_flags, 0, kFuseMaxTiles * sizeof(int32_t)) == cudaSuccess;
+    ok = ok && cudaMalloc(&t->arena.pass_flags, kFuseMaxPasses * sizeof(int32_t)) == cudaSuccess;
+    ok = ok && cudaMemset(t->arena.pass_flags, 0, kFuseMaxPasses * sizeof(int32_t)) == cudaSuccess;
     ok = ok && decode_init() == cudaSuccess;   // (first: see there)
     ok = ok && gemm_sm100_init(device) == cudaSuccess;
     ok = ok && shrink_init() == cudaSuccess;
@@ -772,34 +772,26 @@ lml_status lora_mixed_linear_multi(lml_table* const* tables, int P, const void* 
     bool distinct = true;   // (a table's counters serve one projection of a launch)
     for (int p = 0; p < P; ++p)
         for (int q = 0; q < p; ++q) distinct = distinct && tables[p] != tables[q];
-    const int nb = 1;   // (projections times blocks of 16 tokens in one launch was measured: 44.1 us against 42.8 us for q/k/v at 32 tokens as one call per projection)
     if (P > 1 && distinct && T <= kDecodeMaxT) {
         // One launch of the decode kernel for all projections: its CTAs are dealt out over them, each works on its
-        // projection as in a call of its own, and the fixed costs of a call are paid once.
+        // projection as in a call of its own, and the fixed costs of a call are paid once.  (Projections times blocks of 16
+        // tokens in one launch was measured: 44.1 us against 42.8 us for q/k/v at 32 tokens as one call per projection.)
         DeviceGuard guard(tables[0]->device);
         if (!guard.ok) return LML_ERR_CUDA;
-        SlotSnapshot snaps[kDecMaxBlocks];
-        DecodeArgs args[kDecMaxBlocks];
-        const Arena* ars[kDecMaxBlocks];
-        int n = 0;
+        SlotSnapshot snaps[LML_MAX_PROJECTIONS];
+        DecodeArgs args[LML_MAX_PROJECTIONS];
+        const Arena* ars[LML_MAX_PROJECTIONS];
         for (int p = 0; p < P; ++p) {
-            const SlotSnapshot snap = snapshot_locked(tables[p]);
-            for (int bi = 0; bi < nb; ++bi, ++n) {
-                const int t0 = bi * kDecodeMaxT;
-                snaps[n] = snap;
-                ars[n] = &tables[p]->arena;
-                DecodeArgs& a = args[n];
-                a.x = static_cast<const __nv_bfloat16*>(x) + (size_t)t0 * tables[0]->d_in;
-                a.W0 = W0[p];
-                a.y = static_cast<__nv_bfloat16*>(y[p]) + (size_t)t0 * tables[p]->d_out;
-                a.perm = nullptr; a.seg_offsets = nullptr; a.slot_ids = nullptr;
-                a.token_slots = token_slots[p] + t0;
-                a.by_adapter = false;
-                a.T = T - t0 < kDecodeMaxT ? T - t0 : kDecodeMaxT;
-                a.d_in = tables[0]->d_in; a.d_out = tables[p]->d_out; a.G = 1; a.num_sms = tables[0]->num_sms;
-            }
+            snaps[p] = snapshot_locked(tables[p]);
+            ars[p] = &tables[p]->arena;
+            DecodeArgs& a = args[p];
+            a.x = x; a.W0 = W0[p]; a.y = y[p];
+            a.perm = nullptr; a.seg_offsets = nullptr; a.slot_ids = nullptr;
+            a.token_slots = token_slots[p];
+            a.by_adapter = false;
+            a.T = T; a.d_in = tables[0]->d_in; a.d_out = tables[p]->d_out; a.G = 1; a.num_sms = tables[0]->num_sms;
         }
-        const cudaError_t e = launch_decode_multi(ars, snaps, args, n, stream);
+        const cudaError_t e = launch_decode_multi(ars, snaps, args, P, stream);
         if (e != cudaSuccess) { cudaGetLastError(); return LML_ERR_CUDA; }
         for (int p = 0; p < P; ++p) tables[p]->last_launches = p == 0 ? 1 : 0;
         return LML_OK;

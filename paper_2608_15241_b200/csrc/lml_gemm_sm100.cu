@@ -86,8 +86,6 @@ struct GemmCtrl {
 // stage_info flags
 constexpr uint32_t kStageCommit = 0x100u;   // after this stage the accumulator holds an output: commit it to the epilogue
 constexpr uint32_t kStageAcc1 = 0x200u;     // the stage belongs to accumulator 1 (else 0)
-constexpr uint32_t kStageFresh = 0x400u;    // first stage of a tile: wait for the accumulator to be free, overwrite it
-constexpr uint32_t kStageDelta = 0x800u;    // dual form: first stage of a tile's second output: wait until the first was read
 
 static_assert(sizeof(GemmCtrl) <= 256, "control block");
 constexpr uint32_t kStageBoth = 0x2000u;    // split-K dual form: the stage's product goes into both bindings' accumulators
@@ -142,7 +140,7 @@ struct alignas(64) GemmParams {
     int lora;                   // the call has adapters
     int fused;                  // the shrink runs inside this kernel (else a bind_shrink launch came before it)
     RowSource rows;             // fused: where the slot of a row comes from
-    int32_t* tile_flags;        // fused: [pass] = epoch + 1 once its u blocks are written
+    int32_t* pass_flags;        // fused: [pass] = epoch + 1 once its u blocks are written
     uint32_t* x_flag;           // early start (else null): [0] == call_id: x may be read; [1] CTAs that have finished
     uint32_t call_id;
     uint32_t* fuse_sync;        // fused: [0] the table's epoch, [1] CTAs that have finished (the last one advances the epoch)
@@ -415,13 +413,12 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        // Stage order.  A tile is its base k-blocks followed by one stage per LoRA piece; the last of
-        // these carries kStageCommit.  In the dual form every tile has a second output, the same
-        // accumulator plus (second slots' delta minus first slots' delta): its stages ("delta
-        // stages": one per piece of the second slot array, one per piece of the first with the
-        // negated u) can only run once the epilogue has read the first output, so they are slipped
-        // into the middle of the NEXT tile's k-blocks (or follow the last tile), where the MMA thread
-        // does not have to wait for that.
+        // Stage order.  A tile is its base k-blocks followed by its LoRA chunks, up to four to a stage; the last stage
+        // carries kStageCommit.  In the dual form every tile has a second output, the same accumulator plus (second
+        // slots' delta minus first slots' delta): the chunks of both bindings again, with the blocks that hold that
+        // difference.  These "delta stages" can only run once the epilogue has read the first output, so they are slipped
+        // into the middle of the NEXT tile's k-blocks (or follow the last tile), where the MMA thread does not have to
+        // wait for that.
         if (lane == 0) {
             bool lora = false, lora_known = !p.lora;
             // the CTA's first tile: its chunks are listed in shared memory
@@ -454,18 +451,17 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                 const int want = shr->epoch + 1;
                 const long long t0 = clock64();
                 for (int i = shr_base[m]; i < shr_base[m + 1]; ++i)
-                    while (ld_acquire_gpu_s32(p.tile_flags + i) != want) {
+                    while (ld_acquire_gpu_s32(p.pass_flags + i) != want) {
                         if (*abort) { ok = false; return; }
                         if (clock64() - t0 > (1ll << 31)) { *abort = 1; ok = false; return; }
                     }
                 fence_proxy_async_all();   // what those CTAs wrote with ordinary stores is read by bulk copies from here on
                 flag_seen_m = m;
             };
-            // The chunks of row tile m that rows use under the bindings `who`, up to four to a stage; `flags_first` go on the
-            // first stage, `flags_last` on the last.  They are listed in the tile's plan; with the fused shrink, they follow
+            // The chunks of row tile m that rows use under the bindings `who`, up to four to a stage; `flags_last` go on the last
+            // stage.  They are listed in the tile's plan; with the fused shrink, they follow
             // from the tile's slots.
-            auto emit_chunks = [&](const GemmPart& pt, const __nv_bfloat16* u, int m, int n, uint32_t who, uint32_t acc_flag,
-                                   uint32_t flags_first, uint32_t flags_last) {
+            auto emit_chunks = [&](const GemmPart& pt, const __nv_bfloat16* u, int m, int n, uint32_t who, uint32_t acc_flag, uint32_t flags_last) {
                 wait_u(m);
                 int index = -1, c = 0, at = 0;
                 const bool listed = !p.fused && &pt == list0_part && m == list0_m && n == list0_n;
@@ -492,7 +488,6 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                     }
                     return -1;
                 };
-                bool first = true;
                 int e = next();
                 while (e >= 0 && ok) {
                     ok = acquire();
@@ -504,8 +499,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                         if (pt.u_lo) { load_u_rest(pt, m, index, a_dst, bar); k = 4; }   // (a stage to itself)
                         e = next();
                     }
-                    ctrl->stage_info[stage] = (pt.u_lo ? 3u | kStageOneB : (uint32_t)k) | acc_flag | kStageChunks | (first ? flags_first : 0u) | (e < 0 ? flags_last : 0u);
-                    first = false;
+                    ctrl->stage_info[stage] = (pt.u_lo ? 3u | kStageOneB : (uint32_t)k) | acc_flag | kStageChunks | (e < 0 ? flags_last : 0u);
                     mbar_arrive(bar);
                     advance();
                 }
@@ -517,9 +511,13 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                 const bool listed = &pt == list0_part && m == list0_m && n == list0_n;
                 const TilePlan* plan = pt.plan + m;
                 const int count = listed ? ctrl->listed[0] : ld_after_wait(&plan->count);
-                if (!dual) return count > 0;
-                for (int i = 0; i < count; ++i) if ((listed ? list0[i] : ld_after_wait(&plan->chunk[i])) & who) return true;
-                return false;
+                if constexpr (!kTall) {   // (tall tiles have no dual form)
+                    if (dual) {
+                        for (int i = 0; i < count; ++i) if ((listed ? list0[i] : ld_after_wait(&plan->chunk[i])) & who) return true;
+                        return false;
+                    }
+                }
+                return count > 0;
             };
             // a stage without operands: only its flags matter to the MMA thread
             auto emit_marker = [&](uint32_t info) {
@@ -531,8 +529,8 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
             };
             // dual form: the delta stages of tile (m, n) on accumulator flag acc_flag
             auto emit_delta = [&](int m, int n, uint32_t acc_flag) {
-                if (!has_chunks(p.part[0], m, n, kChunkFirst | kChunkSecond)) { emit_marker(acc_flag | kStageDelta | kStageCommit); return; }
-                emit_chunks(p.part[0], p.u2, m, n, kChunkFirst | kChunkSecond, acc_flag, kStageDelta, kStageCommit);
+                if (!has_chunks(p.part[0], m, n, kChunkFirst | kChunkSecond)) { emit_marker(acc_flag | kStageCommit); return; }
+                emit_chunks(p.part[0], p.u2, m, n, kChunkFirst | kChunkSecond, acc_flag, kStageCommit);
             };
             int ordinal = 0, prev_m = -1, prev_n = -1;
             // this CTA's shrink passes: a pass is num_kb stages of [x k-block | A k-blocks of its pieces]
@@ -549,7 +547,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                     const int nsub = min(per_stage, num_kb - kb);
                     const uint32_t bar = smem_u32(&ctrl->full[stage]);
                     ctrl->stage_info[stage] = 4u | acc_flag | ((uint32_t)sp.n << 16) | ((uint32_t)nsub << 20) |
-                                              (kb == 0 ? kStageFresh : 0u) | (kb + nsub >= num_kb ? kStageCommit : 0u);
+                                              (kb + nsub >= num_kb ? kStageCommit : 0u);
                     mbar_arrive_expect_tx(bar, (uint32_t)(nsub * (p.x_bytes + sp.n * (kChunk * kBK * 2))));
                     for (int j = 0; j < nsub; ++j) {
                         const uint32_t a_dst = tiles_addr + stage * Cfg::kStageBytes + j * sub_bytes;
@@ -572,7 +570,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                     const uint32_t a_dst = tiles_addr + st * Cfg::kStageBytes;
                     const uint32_t bar = smem_u32(&ctrl->full[st]);
                     const bool second = kTall && row0 + kBM < p.T;
-                    ctrl->stage_info[st] = 4u | acc_flag | (kb == 0 ? kStageFresh : 0u) | (kb == num_kb - 1 ? flags_last : 0u);
+                    ctrl->stage_info[st] = 4u | acc_flag | (kb == num_kb - 1 ? flags_last : 0u);
                     mbar_arrive_expect_tx(bar, (uint32_t)(p.x_bytes + (second ? p.x_bytes : 0) + (kb < have_w ? 0 : Cfg::kBBytes)));
                     tma_load_2d(a_dst, &p.x, bar, kb * kBK, row0);
                     if (second) tma_load_2d(a_dst + Cfg::kXBytes, &p.x, bar, kb * kBK, row0 + kBM);
@@ -604,11 +602,11 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                 if constexpr (kTall) {
                     const bool chunks1 = m + 1 < p.num_m && has_chunks(pt, m + 1, n, kChunkFirst);
                     base_blocks(&pt.w, row0, n * BN, num_kb - 1, num_kb, 0u, (chunks ? kStageMore0 : 0u) | (chunks1 ? kStageMore1 : 0u), ordinal == 0 ? ahead : 0);
-                    if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, 0u, 0u, kStageCommit);
-                    if (ok && chunks1) emit_chunks(pt, pt.u, m + 1, n, kChunkFirst, 0u, 0u, kStageCommit);
+                    if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, 0u, kStageCommit);
+                    if (ok && chunks1) emit_chunks(pt, pt.u, m + 1, n, kChunkFirst, 0u, kStageCommit);
                 } else {
                     base_blocks(&pt.w, row0, n * BN, num_kb - 1, num_kb, acc_flag, chunks ? 0u : kStageCommit, ordinal == 0 ? ahead : 0);
-                    if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, acc_flag, 0u, kStageCommit);
+                    if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, acc_flag, kStageCommit);
                 }
                 prev_m = m; prev_n = n;
             }
@@ -846,7 +844,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
             fence_proxy_async_all();   // the blocks will be read by TMA
             __threadfence();
             asm volatile("bar.sync %0, 128;" ::"r"(1 + group) : "memory");   // the four epilogue warps of the accumulator
-            if ((ew & 3) == 0 && lane == 0) st_release_gpu_s32(p.tile_flags + sp.flag, shr->epoch + 1);
+            if ((ew & 3) == 0 && lane == 0) st_release_gpu_s32(p.pass_flags + sp.flag, shr->epoch + 1);
             acc ^= 1;
         }
         for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
@@ -1475,7 +1473,7 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
     p.T = a.T; p.K = a.d_in; p.P = a.P; p.num_tiles = tiles;
     p.lora = a.lora ? 1 : 0; p.fused = a.fused ? 1 : 0; p.rows = a.rows;
     p.x_flag = a.x_flag; p.call_id = a.call_id;
-    p.tile_flags = a.proj[0].ar->tile_flags; p.fuse_sync = a.proj[0].ar->status + 4;
+    p.pass_flags = a.proj[0].ar->pass_flags; p.fuse_sync = a.proj[0].ar->status + 4;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     // with adapters the predecessor is the bind_shrink launch of this call, else the kernel waits at its top

@@ -23,8 +23,8 @@ constexpr int kUBlockBytes = kTileM * kChunk * 2;             // u of one row ti
 constexpr int kSlabTiles = 512;       // row tiles worked on at a time: longer calls run in slabs of this many, so that the u blocks stay bounded
 constexpr int kBindSegs = 256;        // segments that the kernels look up in shared memory; more are turned into a slot per row first
 constexpr int kDecodeMaxT = LML_DECODE_MAX_TOKENS;
-constexpr int kMaxAdapterIds = LML_MAX_ADAPTER_IDS;
-constexpr int kFuseMaxTiles = 4096;   // row tiles of a call whose shrink can run inside the GEMM kernel (524288 tokens)   // adapter ids that can be resolved on the device
+constexpr int kMaxAdapterIds = LML_MAX_ADAPTER_IDS;   // adapter ids that can be resolved on the device
+constexpr int kFuseMaxPasses = 4096;   // flags of the fused shrink, one a pass; a call has a few hundred passes at most (gemm_can_fuse_shrink)
 
 // Per-call snapshot of the slot table, passed by value as a kernel parameter so that a later
 // register / retire cannot change a call that is already enqueued.
@@ -48,7 +48,7 @@ struct Arena {
     uint32_t* nonfinite;    // [0] not 0: some registration's B held Inf or NaN; [1 + slot] nonfinite_tag() of the last such one in the slot.  The
                             // GEMM adds those terms to the slot's own rows
     uint32_t* status;   // sticky LML_FLAG_* bits
-    int32_t* tile_flags;    // [kFuseMaxTiles] fused shrink of the prefill GEMM: the u blocks of pass i are written (= epoch + 1; the epoch is word 4 of status)
+    int32_t* pass_flags;    // [kFuseMaxPasses] fused shrink of the prefill GEMM: the u blocks of pass i are written (= epoch + 1; the epoch is word 4 of status)
     int32_t* adapter_map;   // [kMaxAdapterIds] serving entry of each adapter id: slot | generation << 8, -1 = none; written by lml_publish
     unsigned long long* dec_u;   // [kDecMaxBlocks][kDecExchStride] the decode kernel's exchange blocks, one per part of a launch that works on this table
 };
