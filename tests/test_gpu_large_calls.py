@@ -13,7 +13,7 @@ pytestmark = pytest.mark.gpu
 
 def _site(K, N, ranks, seed=17):
     from paper_2608_15241_b200.binding import Table
-    entries = wl.make_entries(seed, K, N, [(a, 1, r, 2.0) for a, r in enumerate(ranks)], std=0.1)
+    entries = wl.make_entries(seed, K, N, [(a, 1, r, 2.0) for a, r in enumerate(ranks)], std=0.05)
     tbl = Table(K, N, len(ranks))
     for e in entries:
         tbl.register_adapter(e.adapter_id, 1, to_dev(e.A), to_dev(e.B), e.scale)

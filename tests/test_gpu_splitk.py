@@ -12,7 +12,7 @@ from gpu_util import Site
 
 pytestmark = pytest.mark.gpu
 
-SHAPES = ["128x2", "128x3", "128x4", "256x2", "256x3", "256x4", "256x5", "256x6", "256x8"]
+SHAPES = ["64x2", "64x3", "64x4", "64x8", "128x2", "128x3", "128x4", "256x2", "256x3", "256x4", "256x5", "256x6", "256x8"]
 
 
 @pytest.mark.parametrize("shape", SHAPES)

@@ -30,3 +30,30 @@ def test_tall_tiles_against_oracle(kw, fuse, monkeypatch):
     assert np.array_equal(y, y2)
     refb, _ = oracle.forward(w.x, w.W0, w.entries, np.array([0, w.T], np.int32), np.array([-1], np.int32), w.perm)
     assert fb == 0 and oracle.compare(yb, refb)["ok"]
+
+
+@pytest.mark.parametrize("T", [130, 300, 700])
+def test_tall_tiles_of_several_projections(T, monkeypatch):
+    """Tiles numbered through three projections of unequal width, an odd number of row tiles among them."""
+    import torch
+    from paper_2608_15241_b200 import binding as b
+    from paper_2608_15241_b200.binding import Table
+    from gpu_util import to_bits, to_dev
+    monkeypatch.setenv("LML_GEMM_SPLIT", "512x1")
+    K, Ns, ranks = 520, (264, 1000, 136), (4, 33, 64)
+    x = wl.normal_bf16(9, 1, (T, K), 1.0)
+    tok = np.random.default_rng(T).integers(-1, len(ranks), size=T).astype(np.int32)
+    tables, W, ents = [], [], []
+    for p, N in enumerate(Ns):
+        W.append(wl.normal_bf16(9, 10 + p, (N, K), 0.02))
+        ents.append(wl.make_entries(9 + p, K, N, [(a, 1, r, 2.0) for a, r in enumerate(ranks)]))
+        tables.append(Table(K, N, len(ranks)))
+        for e in ents[p]:
+            tables[p].register_adapter(e.adapter_id, 1, to_dev(e.A), to_dev(e.B), e.scale)
+    ys = b.multi_projection(tables, to_dev(x), [to_dev(w) for w in W], torch.from_numpy(tok).cuda())
+    torch.cuda.synchronize()
+    for p in range(len(Ns)):
+        ref, _ = oracle.forward(x, W[p], ents[p], np.arange(T + 1, dtype=np.int32), tok)
+        r = oracle.compare(to_bits(ys[p]), ref)
+        assert r["ok"] and tables[p].device_status() == 0, (p, r)
+        tables[p].close()
