@@ -524,8 +524,8 @@ def run_workload(name, steps, warmup, device, world, peaks, want_cpu_baseline, e
     del rot
     torch.cuda.empty_cache()
     if kind != "decode" and "shuffled" in extras:
-        # the same batch with its rows in arrival order: per-token ids through the segmentation pass, the
-        # row gather and the scatter epilogue, all inside the timed step
+        # the same batch with its rows in arrival order: per-token ids through the token form, which binds the rows
+        # where they are
         ws = wl.mlp_up_gate(shuffled=True) if name == "mlp_up_gate" else wl.shuffle_rows(w)
         rot_s = Rotation(ws, device, 4 * L2_BYTES)
         ssteps = max(rot_s.R, min(steps, 200 if ws.flops() < 2e11 else 60))
