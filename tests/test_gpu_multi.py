@@ -188,7 +188,7 @@ def test_seven_b_class_qkv_decode():
 @pytest.mark.parametrize("T", [17, 33, 48])
 @pytest.mark.parametrize("K,Ns", [(520, (264, 136, 1000)), (2048, (2056, 1032))])
 def test_projections_of_a_few_blocks_of_tokens_keep_u_beyond_bf16(T, K, Ns):
-    """17 - 48 tokens: a call of its own keeps u in fp32 (decode kernel); the shared launches carry it as two bf16 values, so
+    """17 - 48 tokens: a call of its own keeps u in fp32 (decode kernel); the shared launches carry it as three bf16 values, so
     the outputs stay as close to the fp64 result."""
     ranks = [(16, 64, 4, 8), (8, 16, 33, 1), (64, 33, 16, 2)][:len(Ns)]
     scales = [(40.0, 50.0, 100.0, 40.0), (100.0, 20.0, 25.0, 300.0), (50.0, 15.0, 200.0, 100.0)][:len(Ns)]
