@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
     // x does not depend on the ids: the first stages' tiles go out here when most groups of chunks are sure to be needed
     const int wide_stage = kBindXBytes + B.group * kBindABytes;
     const int pre = B.early ? min(min(B.ring_bytes / wide_stage, kBindMaxStages), nkb) : 0;
-    if (tid == 0)
+    if (warp == 0 && elect_one())
         for (int i = 0; i < pre; ++i) {
             const uint32_t bar = smem_u32(&ctrl->full[i]);
             mbar_expect_tx(bar, (uint32_t)B.x_bytes);
@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
         int stage = 0;                // producer's and issuer's place in the ring
         uint32_t phase = 0;
         if (warp == 0) {
-            if (lane == 0) {
+            if (elect_one()) {
                 bool ok = true;
                 for (int i = 0; i < nkb && ok; ++i) {
                     ok = mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, abort);
@@ -252,7 +252,7 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
                 }
             }
         } else if (warp == 1) {
-            if (lane == 0) {
+            if (elect_one()) {
                 const uint32_t idesc = umma_idesc_bf16(kTileM, nc * kChunk);
                 bool ok = true;
                 for (int i = 0; i < nkb && ok; ++i) {

@@ -323,13 +323,15 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
     if (p.x_flag) {   // early start: the first k-blocks' W0, then x
         const GemmPart& pt = p.part[part_of(p, (int)blockIdx.x)];
         const int n0 = ((int)blockIdx.x - pt.tile0) / num_mt;
-        if (warp == 0 && lane == 0) {
-            for (int kb = 0; kb < min(Cfg::kStages, num_kb); ++kb) {
-                const uint32_t bar = smem_u32(&ctrl->full[kb]);
-                mbar_expect_tx(bar, Cfg::kBBytes);
-                tma_load_2d(tiles_addr + kb * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, kb * kBK, n0 * BN);
+        if (warp == 0) {
+            if (elect_one()) {
+                for (int kb = 0; kb < min(Cfg::kStages, num_kb); ++kb) {
+                    const uint32_t bar = smem_u32(&ctrl->full[kb]);
+                    mbar_expect_tx(bar, Cfg::kBBytes);
+                    tma_load_2d(tiles_addr + kb * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, kb * kBK, n0 * BN);
+                }
+                wait_x(p);
             }
-            wait_x(p);
         } else if (warp == 2) {
             prefetch_b<BN>(pt, n0, lane, 0, 1);
         }
@@ -419,7 +421,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
         // difference.  These "delta stages" can only run once the epilogue has read the first output, so they are slipped
         // into the middle of the NEXT tile's k-blocks (or follow the last tile), where the MMA thread does not have to
         // wait for that.
-        if (lane == 0) {
+        if (elect_one()) {
             bool lora = false, lora_known = !p.lora;
             // the CTA's first tile: its chunks are listed in shared memory
             const GemmPart* const list0_part = &p.part[part_of(p, (int)blockIdx.x)];
@@ -623,7 +625,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
         // Walks the same schedule as the producer.  The base k-blocks are always four K-steps and need no
         // side-band word; the last one, the LoRA stages after it and the delta stages carry one (how
         // many K-steps, and whether an output is complete after the stage).
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = umma_idesc_bf16(kBM, BN);
             int stage = 0;
             uint32_t phase = 0;
@@ -777,6 +779,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
         const int ew = warp - 2;
         const int group = ew >> 2;              // tall tiles: the row tile, and accumulator, of these four warps
         constexpr int kBufs = Cfg::kEpiBufs;    // staging buffers of a warp
+        const bool one = elect_one();           // the lane that issues the stores
         const uint32_t buf_addr0 = epi_addr + (uint32_t)(ew * kBufs * kEpiBufBytes);
         uint8_t* buf_ptr0 = epi_ptr + ew * kBufs * kEpiBufBytes;
         int acc = 0;
@@ -879,7 +882,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                     const int col0 = n * BN + c * kEpiChunkCols;
                     if (col0 >= pt.N || row_base >= p.T) continue;   // nothing of this chunk is inside y
                     // the buffer we are about to overwrite must have been read by its earlier store
-                    if (lane == 0) tma_store_wait_read<kBufs - 1>();
+                    if (one) tma_store_wait_read<kBufs - 1>();
                     __syncwarp();
                     uint8_t* bp = buf_ptr0 + buf * kEpiBufBytes;
                     const uint32_t ba = buf_addr0 + (uint32_t)(buf * kEpiBufBytes);
@@ -905,7 +908,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                     }
                     fence_proxy_async_smem();
                     __syncwarp();
-                    if (lane == 0) {
+                    if (one) {
                         if (pass == 0) tma_store_2d(&pt.y, ba, col0, row_base);
                         else tma_store_2d(&p.y2, ba, col0, row_base);
                         tma_store_commit();
@@ -915,7 +918,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
             }
             acc ^= 1;
         }
-        if (lane == 0) tma_store_wait_all();
+        if (one) tma_store_wait_all();
     }
 
     __syncthreads();
@@ -995,14 +998,16 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
     const uint32_t tmem_base = ctrl->tmem_base;
     volatile int* abort = &ctrl->abort;
     if (p.x_flag) {   // early start: the first k-blocks' W0, then x
-        if (warp == 0 && lane == 0) {
-            const int kb0 = rank * num_kb / S, ahead = min(p.stages, (rank + 1) * num_kb / S - kb0);
-            for (int i = 0; i < ahead; ++i) {
-                const uint32_t bar = smem_u32(&ctrl->full[i]);
-                mbar_expect_tx(bar, Cfg::kBBytes);
-                tma_load_2d(tiles_addr + i * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, (kb0 + i) * kBK, n * BN);
+        if (warp == 0) {
+            if (elect_one()) {
+                const int kb0 = rank * num_kb / S, ahead = min(p.stages, (rank + 1) * num_kb / S - kb0);
+                for (int i = 0; i < ahead; ++i) {
+                    const uint32_t bar = smem_u32(&ctrl->full[i]);
+                    mbar_expect_tx(bar, Cfg::kBBytes);
+                    tma_load_2d(tiles_addr + i * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, (kb0 + i) * kBK, n * BN);
+                }
+                wait_x(p);
             }
-            wait_x(p);
         } else if (warp == 2) {
             prefetch_b<BN>(pt, n, lane, rank, S);
         }
@@ -1015,7 +1020,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        if (lane == 0) {
+        if (elect_one()) {
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -1076,7 +1081,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        if (elect_one()) {
             constexpr uint32_t idesc = umma_idesc_bf16(kBM, BN);
             int stage = 0;
             uint32_t phase = 0, accumulate = 0, accumulate2 = 0;

@@ -61,6 +61,17 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     }
 }
 
+// One lane of a converged warp, for roles that a single thread plays.  What that thread issues (MMAs, commits, bulk copies) takes its
+// operands from uniform registers; behind elect.sync the compiler knows that one lane is active, behind lane == 0 it does not and loops
+// over the lanes for every such instruction: 40 cycles per MMA, 490 per stage of four MMAs and their barriers against 330.
+__device__ __forceinline__ bool elect_one()
+{
+    uint32_t p;
+    __syncwarp();
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xffffffff;\n\tselp.u32 %0, 1, 0, p;\n\t}" : "=r"(p));
+    return p != 0;
+}
+
 // Pure polling variant for the two single-thread roles on the critical path of the GEMM ring (the
 // TMA producer and the MMA issuer): test_wait never parks the thread, so a barrier flip is seen
 // within a few cycles instead of after a wake-up.  Same bound and give-up protocol as mbar_wait.
