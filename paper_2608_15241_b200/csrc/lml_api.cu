@@ -126,15 +126,17 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         if (r0 > 0 && b.rows.rows) b.rows.rows += kSlabTiles * kTileM;
         if (r0 > 0 && b.rows.rows2) b.rows.rows2 += kSlabTiles * kTileM;
         g.shape = gemm_pick_shape(rows, t0->d_in, d_outs, P, dual, t0->num_sms, t0->split_bn, t0->split_s);
-        // With whole-K tiles and few row tiles the shrink runs inside the GEMM kernel (on the CTAs that own the fewest tiles,
-        // ahead of their tiles); otherwise a launch goes first and the GEMM is its programmatic dependent.
-        g.fused = mode == kRowsSegments && !dual && P == 1 && T == rows && t0->fuse_shrink &&
-                  gemm_can_fuse_shrink(g.shape, T, t0->d_out, G, b.rows.mode == kRowsSegments, t0->max_slots, t0->num_sms);
+        // Small plain calls compute u inside the GEMM kernel (on the CTAs that own the fewest tiles, ahead of their tiles); otherwise a
+        // launch goes first and the GEMM is its programmatic dependent.
+        g.fused = mode == kRowsSegments && !dual && P == 1 && T == rows && t0->fuse_shrink && t0->split_bn <= 0 &&
+                  gemm_can_fuse_shrink(T, t0->d_in, t0->d_out, G, b.rows.mode == kRowsSegments, t0->max_slots, t0->num_sms);
+        if (g.fused) g.shape = {256, 1, ((rows + kTileM - 1) / kTileM) * ((t0->d_out + 255) / 256), false};
         if (g.fused) g.rows = b.rows;
         b.x_flag = g.x_flag = nullptr;
         if (mode != kRowsNone && !g.fused && bind_starts_gemm_early(rows, P, t0->num_sms)) {
             b.x_flag = g.x_flag = t0->arena.status + 8;
-            b.share_sm = g.share_sm = g.shape.ctas + bind_ctas_early(rows, t0->d_in, P, most_chunks, t0->num_sms) > t0->num_sms;
+            b.early = bind_early(rows, t0->d_in, P, most_chunks, g.shape.ctas, t0->num_sms);
+            g.share_sm = b.early.share_sm;
             std::lock_guard<std::mutex> lock(t0->mu);
             if (++t0->next_call == 0u) ++t0->next_call;
             b.call_id = g.call_id = t0->next_call;
@@ -150,7 +152,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
             if (e != cudaSuccess) return e;
             ++*launches;
         }
-        const cudaError_t e = launch_gemm_sm100(t0->tmap_A, caches, g, stream);
+        const cudaError_t e = g.shape.pair ? launch_gemm_pair(caches, g, stream) : launch_gemm_sm100(t0->tmap_A, caches, g, stream);
         if (e != cudaSuccess) return e;
         ++*launches;
     }
@@ -240,6 +242,7 @@ lml_status lml_table_create(lml_table** out, int device, int d_in, int d_out, in
     ok = ok && cudaMemset(t->arena.pass_flags, 0, kFuseMaxPasses * sizeof(int32_t)) == cudaSuccess;
     ok = ok && decode_init() == cudaSuccess;   // (first: see there)
     ok = ok && gemm_sm100_init(device) == cudaSuccess;
+    ok = ok && gemm_pair_init() == cudaSuccess;
     ok = ok && shrink_init() == cudaSuccess;
     ok = ok && aux_init() == cudaSuccess;
     ok = ok && bind_init() == cudaSuccess;

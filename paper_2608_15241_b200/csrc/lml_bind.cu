@@ -219,7 +219,7 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
             if (first_cta) part.plan[m].chunk[before + c] = (uint16_t)((uint32_t)(tid | (c << 8)) | who);
         }
     }
-    if (first_cta && tid == 0) part.plan[m].count = count;
+    if (first_cta && tid == 0) { part.plan[m].count = count; part.plan[m].used = used; }
     __syncthreads();
 
     // ---- x.A^T of this CTA's part of K, a group of chunks at a time
@@ -234,19 +234,24 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
         const int stages = min(B.ring_bytes / stage_bytes, kBindMaxStages);
         int stage = 0;                // producer's and issuer's place in the ring
         uint32_t phase = 0;
-        if (warp == 0) {
+        if (warp != 1) {
+            // Warp 0 brings in x and accounts for the stage's bytes; the four row warps, which have nothing to do yet, share the chunks (an
+            // issue costs its thread some 60 cycles: 17 copies of a k-block from one thread took 0.55 us, longer than their flight).
             if (elect_one()) {
                 bool ok = true;
                 for (int i = 0; i < nkb && ok; ++i) {
                     ok = mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, abort);
                     if (!ok) break;
                     const uint32_t bar = smem_u32(&ctrl->full[stage]), dst = ring + (uint32_t)(stage * stage_bytes);
-                    const bool have_x = first && i < pre;
-                    mbar_arrive_expect_tx(bar, (uint32_t)(nc * kBindABytes + (have_x ? 0 : B.x_bytes)));
-                    if (!have_x) tma_load_2d(dst, &B.x, bar, (kb0 + i) * 64, m * kTileM);
-                    for (int c = 0; c < nc; ++c) {
-                        const int e = ctrl->list[c0 + c];
-                        tma_load_3d(dst + (uint32_t)(kBindXBytes + c * kBindABytes), &B.a[pi], bar, (kb0 + i) * 64, (e >> 8) * kChunk, e & 0xff);
+                    if (warp == 0) {
+                        const bool have_x = first && i < pre;
+                        mbar_arrive_expect_tx(bar, (uint32_t)(nc * kBindABytes + (have_x ? 0 : B.x_bytes)));
+                        if (!have_x) tma_load_2d(dst, &B.x, bar, (kb0 + i) * 64, m * kTileM);
+                    } else {
+                        for (int c = warp - 2; c < nc; c += 4) {
+                            const int e = ctrl->list[c0 + c];
+                            tma_load_3d(dst + (uint32_t)(kBindXBytes + c * kBindABytes), &B.a[pi], bar, (kb0 + i) * 64, (e >> 8) * kChunk, e & 0xff);
+                        }
                     }
                     if (++stage == stages) { stage = 0; phase ^= 1u; }
                 }
@@ -361,22 +366,26 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
     }
 }
 
-constexpr int kBindGroupEarly = 4;
-constexpr int kBindRingSmall = 3 * (kBindXBytes + kBindGroupEarly * kBindABytes), kBindRingLarge = 192 * 1024;   // (the partial sums, 8 KB per chunk of a pass, fit either)
+constexpr int kBindRingSmall = 72 * 1024, kBindRingLarge = 192 * 1024;   // (the partial sums, 8 KB per chunk of a pass, fit either)
 static int bind_smem_bytes(int ring) { return 1024 + ring + (int)sizeof(BindCtrl); }
 
 // CTAs that share K.  It follows from the rows alone: a projection's u has the same bits in a call of its own and beside others.
 static int bind_cluster(int T, int d_in, int num_sms)
 {
     const int num_m = (T + kTileM - 1) / kTileM, num_kb = (d_in + 63) / 64;
-    int S = num_m * 16 <= num_sms ? 8 : (num_m * 8 <= num_sms ? 4 : (num_m * 2 <= num_sms ? 2 : 1));
+    int S = num_m * 24 <= num_sms ? 8 : (num_m * 8 <= num_sms ? 4 : (num_m * 2 <= num_sms ? 2 : 1));
     while (S > 1 && num_kb < S) S >>= 1;
     return S;
 }
 bool bind_starts_gemm_early(int T, int P, int num_sms) { return (T + kTileM - 1) / kTileM * P * 8 <= num_sms; }
-int bind_ctas_early(int T, int d_in, int P, int cap, int num_sms)
+// Few rows: a pass takes eight chunks, or sixteen where only that leaves the GEMM's CTAs (gemm_ctas) SMs of their own.  Layer passes,
+// us, with 4 / 8 / 16: 40 tokens, 16 chunks 169 / 162 / 149, 128 tokens, 18 chunks 145 / 126 / 133.
+BindEarly bind_early(int T, int d_in, int P, int cap, int gemm_ctas, int num_sms)
 {
-    return (T + kTileM - 1) / kTileM * P * bind_cluster(T, d_in, num_sms) * ((cap + kBindGroupEarly - 1) / kBindGroupEarly);
+    const int clusters = (T + kTileM - 1) / kTileM * P * bind_cluster(T, d_in, num_sms);
+    for (int group = 8; group <= 16; group += 8)
+        if (gemm_ctas + clusters * ((cap + group - 1) / group) <= num_sms) return {group, false};
+    return {8, true};
 }
 
 cudaError_t launch_bind_shrink(const BindArgs& a, const CUtensorMap* const* tmap_A, TmapCache* cache, int num_sms, cudaStream_t stream)
@@ -392,14 +401,14 @@ cudaError_t launch_bind_shrink(const BindArgs& a, const CUtensorMap* const* tmap
     }
     const int num_m = b.num_m = (a.T + kTileM - 1) / kTileM;
     const int tiles = num_m * a.P, S = bind_cluster(a.T, a.d_in, num_sms);
-    // Few rows: small groups of chunks, so that the call spreads over many SMs; in a ring small enough to share an SM with
-    // the split-K GEMM, whose base product runs meanwhile, where the two do not find SMs of their own.  Many rows: x is read
+    // Few rows: see bind_early; in a ring small enough to share an SM with the split-K GEMM, whose base product runs meanwhile,
+    // where the two do not find SMs of their own.  Many rows: x is read
     // once for up to 16 chunks, one wave of CTAs.
     int groups;
     b.early = a.x_flag ? 1 : 0;
     if (b.early) {
-        b.group = kBindGroupEarly;
-        b.ring_bytes = a.share_sm ? kBindRingSmall : kBindRingLarge;
+        b.group = a.early.group;
+        b.ring_bytes = a.early.share_sm ? kBindRingSmall : kBindRingLarge;
         groups = (cap + b.group - 1) / b.group;
     } else {
         b.group = 16; b.ring_bytes = kBindRingLarge;

@@ -33,33 +33,24 @@
 // Every wait is bounded; on give-up the CTA sets LML_FLAG_TIMEOUT, drains and frees its TMEM.
 #include <cstdio>
 #include <cstdlib>
+#include <cstring>
 #include <mutex>
 
-#include "lml_internal.cuh"
-#include "lml_ptx_sm100.cuh"
+#include "lml_gemm_common.cuh"
 
 namespace lml {
 
-using namespace ptx;
-
-constexpr int kBM = kTileM;   // 128
-constexpr int kBK = 64;       // bf16 elements per 128-byte swizzled row
 constexpr int kGemmThreads = 192;
-constexpr int kGemmThreadsTall = 320;
-constexpr int kEpiChunkCols = 32;
-constexpr int kEpiBufBytes = 32 * kEpiChunkCols * 2;   // 2 KB: 32 rows x 64 B
 
 constexpr int kFuseTilesInKernel = 80;    // row tiles of a call whose shrink runs inside the kernel (the per-tile tables in shared memory)
 
-template <int BN, bool kTall = false> struct GemmCfg {
-    static constexpr int kRowTiles = kTall ? 2 : 1;
-    static constexpr int kXBytes = kBM * kBK * 2;             // a k-block of one row tile
-    static constexpr int kABytes = kRowTiles * kXBytes;
+template <int BN> struct GemmCfg {
+    static constexpr int kXBytes = kBM * kBK * 2;             // a k-block of the row tile
+    static constexpr int kABytes = kXBytes;
     static constexpr int kBBytes = BN * kBK * 2;
     static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kStages = kTall ? 3 : ((BN == 256) ? 4 : (BN == 128 ? 6 : 8));
-    static constexpr int kEpiBufs = kTall ? 1 : 2;
-    static constexpr int kEpiBytes = 4 * kRowTiles * kEpiBufs * kEpiBufBytes;
+    static constexpr int kStages = BN == 256 ? 4 : (BN == 128 ? 6 : 8);
+    static constexpr int kEpiBytes = 4 * 2 * kEpiBufBytes;
     static constexpr int kTmemCols = 2 * BN;
     static constexpr int kCtrlBytes = 256 + (kBindSegs + 1) * 4 + kBindSegs + 4 + 512 + kFuseTilesInKernel * 10 + 8 + kMaxChunks * 4;   // barriers; fused shrink: segment cache, shrink plan, per-tile masks and first passes; the first tile's chunks
     // The split-K kernel: no staging for the epilogue.  The ring also takes the partial sums that the CTAs exchange; where
@@ -89,7 +80,6 @@ constexpr uint32_t kStageAcc1 = 0x200u;     // the stage belongs to accumulator 
 
 static_assert(sizeof(GemmCtrl) <= 256, "control block");
 constexpr uint32_t kStageBoth = 0x2000u;    // split-K dual form: the stage's product goes into both bindings' accumulators
-constexpr uint32_t kStageMore0 = 0x8000u, kStageMore1 = 0x10000u;   // tall tiles, on the last k-block: LoRA stages follow for the first / second row tile
 constexpr uint32_t kStageOneB = 0x1000u;    // a LoRA chunk whose u is three blocks: a K-step each, with the same block of B
 constexpr uint32_t kStageChunks = 0x4000u;  // LoRA chunks (no-swizzle operands), a K-step each
 
@@ -112,125 +102,6 @@ struct ShrPlan {
 };
 static_assert(sizeof(ShrPlan) <= 512, "shrink plan");
 
-struct alignas(64) GemmPart {
-    CUtensorMap w, y;
-    const __nv_bfloat16* bk;            // the table's packed B, by chunk
-    const __nv_bfloat16* b;             // ... and by row, as registered
-    const uint32_t* nonfinite;
-    const TilePlan* plan;               // [row tile] its chunks
-    const __nv_bfloat16* u;
-    const __nv_bfloat16* u_mid;         // or null: what u's bf16 values leave of the fp32 u, two further K-steps per chunk
-    const __nv_bfloat16* u_lo;
-    __nv_bfloat16* y_ptr;
-    unsigned long long live;            // slots that hold an adapter
-    unsigned long long nch[2];          // ... their chunks less one, two bits each
-    int N, num_n, n_pad, cap;           // n_pad: rows of a chunk of B in memory
-    int tile0;                          // number of its first tile
-};
-struct alignas(64) GemmParams {
-    CUtensorMap x, a, y2;
-    GemmPart part[LML_MAX_PROJECTIONS];
-    const __nv_bfloat16* u2;            // dual form (else null): the second set of u blocks
-    __nv_bfloat16* y2_ptr;              // dual form: the second output
-    uint32_t* status;
-    int T, K, P;
-    int num_m, num_tiles;
-    int x_bytes;                // of one copy of x (a k-block of a row tile)
-    int stages;                 // split-K kernel: stages of the ring
-    int lora;                   // the call has adapters
-    int fused;                  // the shrink runs inside this kernel (else a bind_shrink launch came before it)
-    RowSource rows;             // fused: where the slot of a row comes from
-    int32_t* pass_flags;        // fused: [pass] = epoch + 1 once its u blocks are written
-    uint32_t* x_flag;           // early start (else null): [0] == call_id: x may be read; [1] CTAs that have finished
-    uint32_t call_id;
-    uint32_t* fuse_sync;        // fused: [0] the table's epoch, [1] CTAs that have finished (the last one advances the epoch)
-};
-__device__ __forceinline__ int slot_chunks(const GemmPart& pt, int slot)
-{
-    return 1 + (int)((pt.nch[slot >> 5] >> (2 * (slot & 31))) & 3ull);
-}
-__device__ __forceinline__ int mask_chunks(const GemmPart& pt, unsigned long long mask)
-{
-    int n = 0;
-    for (; mask; mask &= mask - 1ull) n += slot_chunks(pt, __ffsll((long long)mask) - 1);
-    return n;
-}
-// Early start: W0 is on its way already; x may be read once bind_shrink, which this launch overlaps with, says so.  The word is
-// polled for a few milliseconds; if the work before the call runs on for longer, the hardware's wait for the whole of bind_shrink
-// (which waits for that work) takes over.  The rest of the CTA is held at a barrier meanwhile, so that the limits of the other
-// waits in this kernel measure this kernel only.
-constexpr long long kPollClocks = 1ll << 22;
-__device__ __forceinline__ void wait_x(const GemmParams& p)
-{
-    const long long t0 = clock64();
-    while (ld_acquire_gpu_u32(p.x_flag) != p.call_id)
-        if (clock64() - t0 > kPollClocks) { grid_dependency_wait(); break; }
-    fence_proxy_async_all();
-}
-// ... and its last CTA clears the word: a replay of the same call finds it cleared.
-__device__ __forceinline__ void leave_early_start(const GemmParams& p)
-{
-    if (p.x_flag && atomicAdd(p.x_flag + 1, 1u) == gridDim.x * gridDim.y * gridDim.z - 1) {
-        p.x_flag[1] = 0u;
-        p.x_flag[0] = 0u;
-    }
-}
-// the projection that a tile belongs to
-__device__ __forceinline__ int part_of(const GemmParams& p, int tile)
-{
-    int i = 0;
-    while (i + 1 < p.P && tile >= p.part[i + 1].tile0) ++i;
-    return i;
-}
-// A whole warp copies the part of a tile's plan that concerns this CTA into shared memory, number << 16 | chunk word:
-// chunks that rows use under the bindings `who` and (rank, S) its share of them.  Returns how many.
-__device__ __forceinline__ int list_chunks(const TilePlan* plan, uint32_t who, int rank, int S, int lane, uint32_t* out)
-{
-    uint32_t e = ld_after_wait(&plan->chunk[lane]);   // (goes out with the count; what lies past it is not used)
-    const int count = ld_after_wait(&plan->count);
-    int n = 0;
-    for (int i0 = 0; i0 < count; i0 += 32) {
-        const int i = i0 + lane;
-        if (i0 > 0) e = i < count ? ld_after_wait(&plan->chunk[i]) : 0u;
-        const bool keep = i < count && (e & who) && (S == 1 || (int)((e & 0xffu) + ((e >> 8) & 0xfu)) % S == rank);
-        const uint32_t m = __ballot_sync(0xffffffffu, keep);
-        if (keep) out[n + __popc(m & ((1u << lane) - 1u))] = ((uint32_t)i << 16) | e;
-        n += __popc(m);
-    }
-    return n;
-}
-// The terms of one row that the product with the chunks left out, 32 columns from col0: u_j B[n][j] where B is Inf or NaN.
-// slot, index: the row's slot and the number of its first chunk (index < 0: looked up in the tile's plan, and the slot with it,
-// under binding `which`); u, u_more, u_rest: the sets of blocks whose sum is u (the latter two may be null); out: the row's outputs,
-// bf16, 16-byte pieces in an order given by piece_xor.  Out of line, and all of it, so that the epilogue stays as short as it is
-// without.
-__device__ __noinline__ void add_nonfinite(const GemmPart& pt, int m, int row, int which, int slot, int index, int col0, const __nv_bfloat16* u,
-                                           const __nv_bfloat16* u_more, const __nv_bfloat16* u_rest, uint8_t* out, int piece_xor)
-{
-    auto value = [](const __nv_bfloat16* p) { return __uint_as_float(ld_after_wait(reinterpret_cast<const uint16_t*>(p)) << 16); };
-    if (index < 0) {
-        slot = ld_after_wait(&pt.plan[m].nonfinite_row[which][row]);
-        if (slot < 0) return;
-        for (index = 0; index < kMaxChunks - 1 && (int)(ld_after_wait(&pt.plan[m].chunk[index]) & 0xfffu) != slot;) ++index;
-    }
-    const size_t u_at = ((size_t)m * pt.cap + index) * (kTileM * kChunk) + chunk_elem(row, 0);
-    const int cols = slot_chunks(pt, slot) * kChunk;
-    for (int c = 0; c < kEpiChunkCols && col0 + c < pt.N; ++c) {
-        const __nv_bfloat16* b = pt.b + ((size_t)slot * pt.N + col0 + c) * kRankPad;
-        float sum = 0.f;
-        bool any = false;
-        for (int j = 0; j < cols; ++j) {
-            const float bv = value(b + j);
-            if (isfinite(bv)) continue;
-            const size_t at = u_at + (size_t)(j / kChunk) * (kTileM * kChunk) + chunk_elem(0, j % kChunk);
-            sum += (value(u + at) + (u_more ? value(u_more + at) : 0.f) + (u_rest ? value(u_rest + at) : 0.f)) * bv;
-            any = true;
-        }
-        if (!any) continue;
-        __nv_bfloat16* o = reinterpret_cast<__nv_bfloat16*>(out + ((c >> 3) ^ piece_xor) * 16 + (c & 7) * 2);
-        *o = __float2bfloat16_rn(__bfloat162float(*o) + sum);
-    }
-}
 // One chunk of a stage: the block of u (number `index` of row tile m) and the chunk's rows of B for columns
 // [n * BN, + BN), each contiguous.  entry = slot | chunk << 8.
 template <int BN>
@@ -262,18 +133,12 @@ __device__ __forceinline__ void prefetch_b(const GemmPart& pt, int n, int lane, 
     }
 }
 
-// kTall: a tile is two row tiles high (256 x 256).  Both accumulators belong to the tile, each row tile has four epilogue
-// warps of its own, and a stage holds two tiles of x beside one of W0: 64 KB for 1024 cycles of the tensor cores where the
-// single tile moves 48 KB for 512, so the ring covers twice the latency of a copy with the same shared memory (2048 x 4096 x
-// 4096 without adapters 55.9 -> 50.4 us, 0.82 of the 1665 TFLOP/s that a plain library product reaches here).  (No dual form.)
-template <int BN, bool kTall>
-__global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lora_gemm_sm100_kernel(
-    const __grid_constant__ GemmParams p, const __grid_constant__ SlotSnapshot snap)
+template <int BN>
+__global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const __grid_constant__ GemmParams p,
+                                                                           const __grid_constant__ SlotSnapshot snap)
 {
-    using Cfg = GemmCfg<BN, kTall>;
-    constexpr int kRowTiles = Cfg::kRowTiles;
-    constexpr int kThreads = kTall ? kGemmThreadsTall : kGemmThreads;
-    const bool dual = !kTall && p.u2 != nullptr;
+    using Cfg = GemmCfg<BN>;
+    const bool dual = p.u2 != nullptr;
     extern __shared__ uint8_t smem_raw[];
     // 128-byte swizzled tiles need 1024-byte alignment
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -292,7 +157,6 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int num_tiles = p.num_tiles;
     const int num_kb = (p.K + kBK - 1) / kBK;
-    const int num_mt = (p.num_m + kRowTiles - 1) / kRowTiles;   // tiles along the rows
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < Cfg::kStages; ++s) {
@@ -322,7 +186,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
     volatile int* abort = &ctrl->abort;
     if (p.x_flag) {   // early start: the first k-blocks' W0, then x
         const GemmPart& pt = p.part[part_of(p, (int)blockIdx.x)];
-        const int n0 = ((int)blockIdx.x - pt.tile0) / num_mt;
+        const int n0 = ((int)blockIdx.x - pt.tile0) / p.num_m;
         if (warp == 0) {
             if (elect_one()) {
                 for (int kb = 0; kb < min(Cfg::kStages, num_kb); ++kb) {
@@ -330,7 +194,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                     mbar_expect_tx(bar, Cfg::kBBytes);
                     tma_load_2d(tiles_addr + kb * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, kb * kBK, n0 * BN);
                 }
-                wait_x(p);
+                wait_x(p.x_flag, p.call_id);
             }
         } else if (warp == 2) {
             prefetch_b<BN>(pt, n0, lane, 0, 1);
@@ -347,16 +211,16 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
         // the same verdict) or from the slot per row.
         int bad_off = 0, bad_slot = 0;
         const uint32_t any_nonfinite = threadIdx.x < kMaxSlots ? ld_after_wait(p.part[0].nonfinite) : 0u;
-        for (int m = threadIdx.x; m < p.num_m; m += kThreads) tile_mask[m] = 0ull;
+        for (int m = threadIdx.x; m < p.num_m; m += kGemmThreads) tile_mask[m] = 0ull;
         if (by_segment) {
             const int G = p.rows.G;
-            for (int g = threadIdx.x; g <= G; g += kThreads) seg_cache[g] = ld_after_wait(p.rows.seg_offsets + g);
-            for (int g = threadIdx.x; g < G; g += kThreads) {
+            for (int g = threadIdx.x; g <= G; g += kGemmThreads) seg_cache[g] = ld_after_wait(p.rows.seg_offsets + g);
+            for (int g = threadIdx.x; g < G; g += kGemmThreads) {
                 const int s = ld_after_wait(p.rows.ids + g);
                 slot_cache[g] = (int8_t)(slot_rank(snap, s) > 0 ? s : (s == -1 ? -1 : -2));
             }
             __syncthreads();
-            for (int g = threadIdx.x; g < G; g += kThreads) {
+            for (int g = threadIdx.x; g < G; g += kGemmThreads) {
                 const int s0 = seg_cache[g], s1 = seg_cache[g + 1];
                 if (s1 < s0 || s0 < 0 || s1 > p.T) bad_off = 1;
                 if (slot_cache[g] == -2 && s1 > s0) bad_slot = 1;   // an empty segment may name anything
@@ -365,7 +229,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
             bad_off = __syncthreads_or(bad_off);
             bad_slot = __syncthreads_or(bad_slot);
             if (!bad_off)
-                for (int g = threadIdx.x; g < G; g += kThreads) {
+                for (int g = threadIdx.x; g < G; g += kGemmThreads) {
                     const int s0 = seg_cache[g], s1 = seg_cache[g + 1], s = slot_cache[g];
                     if (s >= 0 && s1 > s0)
                         for (int m = s0 / kBM; m <= (s1 - 1) / kBM; ++m) atomicOr(&tile_mask[m], 1ull << s);
@@ -376,7 +240,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
             }
         } else {
             __syncthreads();
-            for (int row = threadIdx.x; row < p.T; row += kThreads) {
+            for (int row = threadIdx.x; row < p.T; row += kGemmThreads) {
                 const int s = p.rows.rows[row];
                 if (slot_rank(snap, s) > 0) atomicOr(&tile_mask[row / kBM], 1ull << s);
             }
@@ -384,7 +248,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
         __syncthreads();
         const GemmPart& pt = p.part[0];
         if (any_nonfinite && ld_after_wait(pt.nonfinite + 1 + threadIdx.x) == nonfinite_tag(snap.gen[threadIdx.x])) atomicOr(&ctrl->nonfinite, 1ull << threadIdx.x);
-        for (int m = threadIdx.x; m < p.num_m; m += kThreads)
+        for (int m = threadIdx.x; m < p.num_m; m += kGemmThreads)
             shr_base[m + 1] = (uint16_t)((mask_chunks(pt, tile_mask[m]) + kShrChunks - 1) / kShrChunks);
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -425,7 +289,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
             bool lora = false, lora_known = !p.lora;
             // the CTA's first tile: its chunks are listed in shared memory
             const GemmPart* const list0_part = &p.part[part_of(p, (int)blockIdx.x)];
-            const int list0_m = ((int)blockIdx.x - list0_part->tile0) % num_mt * kRowTiles, list0_n = ((int)blockIdx.x - list0_part->tile0) / num_mt;
+            const int list0_m = ((int)blockIdx.x - list0_part->tile0) % p.num_m, list0_n = ((int)blockIdx.x - list0_part->tile0) / p.num_m;
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -513,11 +377,9 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                 const bool listed = &pt == list0_part && m == list0_m && n == list0_n;
                 const TilePlan* plan = pt.plan + m;
                 const int count = listed ? ctrl->listed[0] : ld_after_wait(&plan->count);
-                if constexpr (!kTall) {   // (tall tiles have no dual form)
-                    if (dual) {
-                        for (int i = 0; i < count; ++i) if ((listed ? list0[i] : ld_after_wait(&plan->chunk[i])) & who) return true;
-                        return false;
-                    }
+                if (dual) {
+                    for (int i = 0; i < count; ++i) if ((listed ? list0[i] : ld_after_wait(&plan->chunk[i])) & who) return true;
+                    return false;
                 }
                 return count > 0;
             };
@@ -571,11 +433,9 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                     if (!good) break;
                     const uint32_t a_dst = tiles_addr + st * Cfg::kStageBytes;
                     const uint32_t bar = smem_u32(&ctrl->full[st]);
-                    const bool second = kTall && row0 + kBM < p.T;
                     ctrl->stage_info[st] = 4u | acc_flag | (kb == num_kb - 1 ? flags_last : 0u);
-                    mbar_arrive_expect_tx(bar, (uint32_t)(p.x_bytes + (second ? p.x_bytes : 0) + (kb < have_w ? 0 : Cfg::kBBytes)));
+                    mbar_arrive_expect_tx(bar, (uint32_t)(p.x_bytes + (kb < have_w ? 0 : Cfg::kBBytes)));
                     tma_load_2d(a_dst, &p.x, bar, kb * kBK, row0);
-                    if (second) tma_load_2d(a_dst + Cfg::kXBytes, &p.x, bar, kb * kBK, row0 + kBM);
                     if (kb >= have_w) tma_load_2d(a_dst + Cfg::kABytes, w, bar, kb * kBK, col0);
                     if (++st == Cfg::kStages) { st = 0; ph ^= 1u; }
                 }
@@ -583,7 +443,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
             };
             for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++ordinal) {
                 const GemmPart& pt = p.part[part_of(p, tile)];
-                const int m = (tile - pt.tile0) % num_mt * kRowTiles, n = (tile - pt.tile0) / num_mt;
+                const int m = (tile - pt.tile0) % p.num_m, n = (tile - pt.tile0) / p.num_m;
                 const int row0 = m * kBM;
                 const uint32_t acc_flag = (ordinal & 1) ? kStageAcc1 : 0u;
                 const int mid = min((num_kb + 1) / 2, num_kb - 1);
@@ -601,15 +461,8 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                 learn_lora();
                 if (!ok) break;
                 const bool chunks = has_chunks(pt, m, n, kChunkFirst);
-                if constexpr (kTall) {
-                    const bool chunks1 = m + 1 < p.num_m && has_chunks(pt, m + 1, n, kChunkFirst);
-                    base_blocks(&pt.w, row0, n * BN, num_kb - 1, num_kb, 0u, (chunks ? kStageMore0 : 0u) | (chunks1 ? kStageMore1 : 0u), ordinal == 0 ? ahead : 0);
-                    if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, 0u, kStageCommit);
-                    if (ok && chunks1) emit_chunks(pt, pt.u, m + 1, n, kChunkFirst, 0u, kStageCommit);
-                } else {
-                    base_blocks(&pt.w, row0, n * BN, num_kb - 1, num_kb, acc_flag, chunks ? 0u : kStageCommit, ordinal == 0 ? ahead : 0);
-                    if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, acc_flag, kStageCommit);
-                }
+                base_blocks(&pt.w, row0, n * BN, num_kb - 1, num_kb, acc_flag, chunks ? 0u : kStageCommit, ordinal == 0 ? ahead : 0);
+                if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, acc_flag, kStageCommit);
                 prev_m = m; prev_n = n;
             }
             if (ok && dual && prev_m >= 0) {
@@ -647,8 +500,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                 if (++stage == Cfg::kStages) { stage = 0; phase ^= 1u; }
             };
             // `count` k-blocks without a side-band word: the loop that the tensor cores wait for; its state lives in registers
-            // (tall tiles: both halves, the second's product right behind the first's)
-            auto base_stages = [&](uint32_t d_tmem, int count, uint32_t& accumulate, bool second) {
+            auto base_stages = [&](uint32_t d_tmem, int count, uint32_t& accumulate) {
                 int st = stage;
                 uint32_t ph = phase, on = accumulate;
                 bool good = true;
@@ -661,11 +513,6 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
                         umma_bf16(d_tmem, adesc0 + at + (uint64_t)(k * 2), bdesc0 + at + (uint64_t)(k * 2), idesc, k == 0 ? on : 1u);
-                    if (kTall && second) {
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            umma_bf16(d_tmem + (uint32_t)BN, adesc0 + at + (uint64_t)(Cfg::kXBytes / 16 + k * 2), bdesc0 + at + (uint64_t)(k * 2), idesc, k == 0 ? on : 1u);
-                    }
                     on = 1u;
                     umma_commit(empty0 + 8u * (uint32_t)st);
                     if (++st == Cfg::kStages) { st = 0; ph ^= 1u; }
@@ -729,29 +576,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                 }
                 if (ok) umma_commit(smem_u32(&ctrl->tmem_full[acc]));
             }
-            for (int tile = blockIdx.x; kTall && tile < num_tiles && ok; tile += gridDim.x) {
-                const GemmPart& pt = p.part[part_of(p, tile)];
-                const bool second = (tile - pt.tile0) % num_mt * kRowTiles + 1 < p.num_m;
-                ok = mbar_wait(smem_u32(&ctrl->tmem_empty[0]), empty_ph0 ^ 1u, abort);
-                if (ok && second) ok = mbar_wait(smem_u32(&ctrl->tmem_empty[1]), empty_ph1 ^ 1u, abort);
-                if (!ok) break;
-                empty_ph0 ^= 1u;
-                if (second) empty_ph1 ^= 1u;
-                tc_fence_after();
-                uint32_t accumulate = 0;
-                base_stages(tmem_base, num_kb - 1, accumulate, second);
-                if (!ok) break;
-                ok = mbar_wait(smem_u32(&ctrl->full[stage]), phase, abort);
-                if (!ok) break;
-                const uint32_t info = ctrl->stage_info[stage];
-                base_stages(tmem_base, 1, accumulate, second);
-                if (info & kStageMore0) flagged_stages(0, accumulate);
-                else umma_commit(smem_u32(&ctrl->tmem_full[0]));
-                if (!ok || !second) continue;
-                if (info & kStageMore1) flagged_stages(1, accumulate);
-                else umma_commit(smem_u32(&ctrl->tmem_full[1]));
-            }
-            for (int tile = blockIdx.x; !kTall && tile < num_tiles && ok; tile += gridDim.x, ++ordinal) {
+            for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++ordinal) {
                 const int acc = ordinal & 1;
                 uint32_t& eph = acc ? empty_ph1 : empty_ph0;
                 ok = mbar_wait(smem_u32(&ctrl->tmem_empty[acc]), eph ^ 1u, abort);
@@ -763,11 +588,11 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                 int from = 0;
                 if (dual && ordinal > 0) {
                     from = min((num_kb + 1) / 2, num_kb - 1);
-                    base_stages(d_tmem, from, accumulate, false);
+                    base_stages(d_tmem, from, accumulate);
                     if (ok) delta_stages(acc ^ 1);
                     if (!ok) break;
                 }
-                base_stages(d_tmem, num_kb - 1 - from, accumulate, false);
+                base_stages(d_tmem, num_kb - 1 - from, accumulate);
                 if (!ok) break;
                 flagged_stages(acc, accumulate);   // the last k-block and the tile's LoRA pieces
             }
@@ -777,8 +602,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
         // ------------------------------------------------------------------ epilogue warps
         const int q = warp & 3;                 // TMEM lane quarter this warp may read
         const int ew = warp - 2;
-        const int group = ew >> 2;              // tall tiles: the row tile, and accumulator, of these four warps
-        constexpr int kBufs = Cfg::kEpiBufs;    // staging buffers of a warp
+        constexpr int kBufs = 2;                // staging buffers of a warp
         const bool one = elect_one();           // the lane that issues the stores
         const uint32_t buf_addr0 = epi_addr + (uint32_t)(ew * kBufs * kEpiBufBytes);
         uint8_t* buf_ptr0 = epi_ptr + ew * kBufs * kEpiBufBytes;
@@ -796,7 +620,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
             const GemmPart& pt = p.part[part_of(p, (int)blockIdx.x)];
             grid_dependency_wait();
             grid_launch_dependents();
-            const int n = list_chunks(pt.plan + ((int)blockIdx.x - pt.tile0) % num_mt * kRowTiles, kChunkFirst | kChunkSecond, 0, 1, lane, list0);
+            const int n = list_chunks(pt.plan + ((int)blockIdx.x - pt.tile0) % p.num_m, kChunkFirst | kChunkSecond, 0, 1, lane, list0);
             __syncwarp();
             if (lane == 0) { ctrl->listed[0] = n; mbar_arrive(smem_u32(&ctrl->plan_full)); }
         } else if (p.lora && !p.fused) {
@@ -806,7 +630,6 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
         // flag goes up (release: the four warps' stores are complete)
         for (int ps = 0; p.fused && ps < shr->npass && ok; ++ps) {
             const ShrPass& sp = shr->pass[ps];
-            if (kTall && (ps & 1) != group) { acc ^= 1; continue; }
             uint32_t& fph = acc ? full_ph1 : full_ph0;
             ok = mbar_wait_warp(smem_u32(&ctrl->tmem_full[acc]), fph, abort);
             if (!ok) break;
@@ -846,17 +669,13 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
             if (lane == 0) mbar_arrive(smem_u32(&ctrl->tmem_empty[acc]));
             fence_proxy_async_all();   // the blocks will be read by TMA
             __threadfence();
-            asm volatile("bar.sync %0, 128;" ::"r"(1 + group) : "memory");   // the four epilogue warps of the accumulator
-            if ((ew & 3) == 0 && lane == 0) st_release_gpu_s32(p.pass_flags + sp.flag, shr->epoch + 1);
+            asm volatile("bar.sync 1, 128;" ::: "memory");   // the four epilogue warps
+            if (ew == 0 && lane == 0) st_release_gpu_s32(p.pass_flags + sp.flag, shr->epoch + 1);
             acc ^= 1;
         }
         for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
             const GemmPart& pt = p.part[part_of(p, tile)];
-            const int m = (tile - pt.tile0) % num_mt * kRowTiles + group, n = (tile - pt.tile0) / num_mt;
-            if (kTall) {
-                acc = group;
-                if (m >= p.num_m) continue;
-            }
+            const int m = (tile - pt.tile0) % p.num_m, n = (tile - pt.tile0) / p.num_m;
             const int row_base = m * kBM + q * 32;
             const bool nonfinite = p.lora && (p.fused ? (tile_mask[m] & ctrl->nonfinite) != 0ull : ld_after_wait(pt.nonfinite) != 0u);
             for (int pass = 0; pass < (dual ? 2 : 1) && ok; ++pass) {
@@ -913,7 +732,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
                         else tma_store_2d(&p.y2, ba, col0, row_base);
                         tma_store_commit();
                     }
-                    buf = kBufs == 2 ? buf ^ 1 : 0;
+                    buf ^= 1;
                 }
             }
             acc ^= 1;
@@ -923,7 +742,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
 
     __syncthreads();
     if (threadIdx.x == 0 && ctrl->abort) atomicOr(p.status, LML_FLAG_TIMEOUT);
-    if (threadIdx.x == 0) leave_early_start(p);
+    if (threadIdx.x == 0) leave_early_start(p.x_flag);
     if (threadIdx.x == 0 && p.fused) {
         // the last CTA to finish moves the table's epoch on: the flags of this call mean nothing to the next one
         __threadfence();
@@ -1006,7 +825,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
                     mbar_expect_tx(bar, Cfg::kBBytes);
                     tma_load_2d(tiles_addr + i * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, (kb0 + i) * kBK, n * BN);
                 }
-                wait_x(p);
+                wait_x(p.x_flag, p.call_id);
             }
         } else if (warp == 2) {
             prefetch_b<BN>(pt, n, lane, rank, S);
@@ -1206,7 +1025,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
     }   // outputs
     __syncthreads();
     if (threadIdx.x == 0 && ctrl->abort) atomicOr(p.status, LML_FLAG_TIMEOUT);
-    if (threadIdx.x == 0) leave_early_start(p);
+    if (threadIdx.x == 0) leave_early_start(p.x_flag);
     if (warp == 1) {
         tc_fence_after();
         tmem_dealloc(tmem_base, dual ? 2 * BN : BN);
@@ -1240,7 +1059,7 @@ static CUtensorMapSwizzle swizzle_for(uint32_t box_inner_elems)
 }
 
 bool encode_tmap_2d(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer, uint64_t row_stride_bytes,
-                    uint32_t box_inner, uint32_t box_outer)
+                    uint32_t box_inner, uint32_t box_outer, bool swizzle)
 {
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return false;
@@ -1249,7 +1068,7 @@ bool encode_tmap_2d(CUtensorMap* m, const void* base, uint64_t inner, uint64_t o
     cuuint32_t box[2] = {box_inner, box_outer};
     cuuint32_t estr[2] = {1, 1};
     return fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle_for(box_inner), CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+              CU_TENSOR_MAP_INTERLEAVE_NONE, swizzle ? swizzle_for(box_inner) : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
               CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
@@ -1272,11 +1091,9 @@ cudaError_t gemm_sm100_init(int /*device*/)
     cudaError_t e = cudaFuncSetAttribute(lora_gemm_sm100_splitk_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          GemmCfg<64>::split_smem(GemmCfg<64>::kStages));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<64>::kSmemBytes);
+    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<64>::kSmemBytes);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<256, true>::kSmemBytes);
-    if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          GemmCfg<256>::kSmemBytes);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(lora_gemm_sm100_splitk_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1285,19 +1102,23 @@ cudaError_t gemm_sm100_init(int /*device*/)
     e = cudaFuncSetAttribute(lora_gemm_sm100_splitk_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              GemmCfg<128>::split_smem(GemmCfg<128>::kStages));
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(lora_gemm_sm100_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(lora_gemm_sm100_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 GemmCfg<128>::kSmemBytes);
 }
 
 // The table's override (LML_GEMM_SPLIT, read once when the table is created; a test knob): "<bn>x<split>"
-// forces that shape, 0 switches the split-K kernel off.  Returns false when the variable is not set.
+// forces that shape, "<bn>p" CTA pairs of that width ("512x1": the same as 256p), 0 switches the split-K kernel off.  Returns false
+// when the variable is not set.  split_out: 0 for pairs.
 bool gemm_split_override(int* bn_out, int* split_out)
 {
     *bn_out = -1; *split_out = -1;
     const char* e = getenv("LML_GEMM_SPLIT");
     if (!e) return false;
     int bn = 0, sp = 0;
-    if (sscanf(e, "%dx%d", &bn, &sp) == 2 && (bn == 64 || bn == 128 || bn == 256 || (bn == 512 && sp == 1)) && sp >= 1 && sp <= kSplitMaxS &&
+    char c = 0;
+    if (!strcmp(e, "512x1")) e = "256p";
+    if (sscanf(e, "%d%c", &bn, &c) == 2 && c == 'p' && bn >= 64 && bn <= 256 && bn % 32 == 0) { *bn_out = bn; *split_out = 0; return true; }
+    if (sscanf(e, "%dx%d", &bn, &sp) == 2 && (bn == 64 || bn == 128 || bn == 256) && sp >= 1 && sp <= kSplitMaxS &&
         (sp == 1 ? 0 : sp) * ((bn / 32 + sp - 1) / sp) * 16384 <= GemmCfg<128>::kStages * GemmCfg<128>::kStageBytes) {
         *bn_out = bn; *split_out = sp;
     } else {
@@ -1314,10 +1135,12 @@ static int gemm_stages_short(int bn)
 static int gemm_stage_bytes(int bn) { return (kBM + bn) * kBK * 2; }
 static int gemm_exchange_bytes(int bn, int split) { return split * ((bn / 32 + split - 1) / split) * 16384; }
 
-// The shape of a call: the smallest estimated time (us) over whole-K tiles of three widths and over the splits that the
-// machine can hold.  More tiles than SMs: rounds of tiles times the tensor time of a k-block.  Fewer: a CTA's k-blocks come
-// through its ring at one round of the ring per trip to memory, 1.5 us while W0 streams (measured at 128 tokens, us per
-// k-block: 256 columns whole-K 0.37, 128 columns 0.265; with the short rings of the split-K kernel 0.52 and 0.40).
+// The shape of a call: the smallest estimated time (us) over whole-K tiles of three widths, the splits that the machine can hold, and
+// CTA pairs.  A fixed part and so much per k-block and round of tiles, from single calls with four adapters, W0 out of HBM (us per call):
+// whole-K tiles of 64 / 128 / 256 columns 16.0 / 19.1 / 28.5 at 128 x 4096 -> 4096, 12.2 / 12.6 / 16.8 at 2048 -> 2048, 33.7 / 42.7 / 68.0 at
+// 11008 -> 4096; splits there 128x2 34.7, 128x3 27.0, 256x4 32.5, 256x6 30.0; pairs of 256 / 160 / 128 columns 26.8 / 21.4 / 21.3 at 512 x
+// 4096 -> 4096, and where the tiles take several rounds, at the power that the tensor cores may draw, 96.6 at 1300 x 4096 -> 11008 (256
+// columns, four rounds), 109.3 at 1600 (224 columns, five; with 256 columns 115.9), against 111 and 128.6 for single tiles of 128.
 GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, int num_sms, int split_bn, int split_s)
 {
     static int max_clusters[3][kSplitMaxS + 1];   // for 64, 128 and 256 columns
@@ -1348,44 +1171,44 @@ GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, 
         for (int p = 0; p < P; ++p) tiles += num_m * ((d_outs[p] + bn - 1) / bn);
         return tiles;
     };
-    if (split_bn == 512 && !dual) {   // (a test knob: tall tiles)
+    auto pair_tiles_of = [&](int bn) {
         int tiles = 0;
-        for (int p = 0; p < P; ++p) tiles += (num_m + 1) / 2 * ((d_outs[p] + 255) / 256);
-        return {256, 1, tiles, true};
+        for (int p = 0; p < P; ++p) tiles += (num_m + 1) / 2 * ((d_outs[p] + bn - 1) / bn);
+        return tiles;
+    };
+    if (split_bn > 0 && split_s == 0) {
+        if (!dual) return {split_bn, 1, 2 * pair_tiles_of(split_bn), true};
+        split_bn = 0;
     }
-    if (split_bn == 512) split_bn = 0;
     if (split_bn > 0) return {split_bn, split_s, tiles_of(split_bn) * split_s, false};
-    const bool crowded = tiles_of(256) > num_sms;
+    float w0_bytes = 0.f;
+    for (int p = 0; p < P; ++p) w0_bytes += 2.f * (float)d_in * (float)d_outs[p];
+    const float stream_us = 7.5f + w0_bytes / 5.45e6f;   // no shape reads W0 faster
     GemmShape best = {256, 1, tiles_of(256), false};
     float best_us = 1e30f;
-    for (int w = 2; w >= (crowded ? 1 : 0); --w) {
+    auto consider = [&](const GemmShape& shape, float us) {
+        us = (us > stream_us ? us : stream_us) + 0.1f * us;
+        if (us < best_us * 0.999f) { best_us = us; best = shape; }
+    };
+    for (int w = 2; w >= 0; --w) {
         const int bn = 64 << w, tiles = tiles_of(bn);
-        for (int S = 1; S <= (split_bn == 0 ? 1 : kSplitMaxS); ++S) {
-            if (S > 1 && (max_clusters[w][S] <= 0 || num_kb < 8 * S || gemm_exchange_bytes(bn, S) > gemm_stages(bn) * gemm_stage_bytes(bn))) continue;
+        const int waves = (tiles + num_sms - 1) / num_sms;
+        const float t1[3] = {0.145f, 0.21f, 0.365f}, t2[3] = {0.185f, 0.25f, 0.41f}, a1[3] = {7.f, 5.5f, 5.f};
+        consider({bn, 1, tiles, false}, a1[w] + (float)(waves * num_kb) * (waves > 1 ? t2[w] : t1[w]));
+        for (int S = 2; S <= kSplitMaxS && split_bn != 0; ++S) {
+            if (max_clusters[w][S] < tiles || num_kb < 8 * S || gemm_exchange_bytes(bn, S) > gemm_stages(bn) * gemm_stage_bytes(bn)) continue;
             // (a cluster needs its CTAs on one part of the chip: where they do not all find a place beside bind_shrink's, about
             // 40 CTAs, some wait for it to end)
-            const int fit = S > 1 ? max_clusters[w][S] : num_sms;
-            if (S > 1 && tiles > fit) continue;
-            const bool beside = tiles * num_sms <= fit * (num_sms - 40);
-            const int waves = (tiles + fit - 1) / fit;
-            float us;
-            if (crowded) {
-                us = (float)(waves * num_kb) * (w == 2 ? 0.415f : 0.34f);
-            } else {
-                const int stages = S > 1 && !beside ? gemm_stages_short(bn) : gemm_stages(bn);
-                us = (w == 2 ? 12.5f : (w == 1 ? 10.f : 8.f)) + (S > 1 ? 1.f : 0.f) + (S > 1 && !beside ? 4.f : 0.f) +
-                     (float)waves * (float)((num_kb + S - 1) / S) * 1.55f / (float)stages;
-            }
-            if (us < best_us * 0.999f) { best_us = us; best = {bn, S, tiles * S, false}; }
+            const bool beside = tiles * num_sms <= max_clusters[w][S] * (num_sms - 40);
+            consider({bn, S, tiles * S, false}, (S <= 4 ? 5.f + 2.f * (float)S : 18.5f) + (float)((num_kb + S - 1) / S) * (w == 2 ? 0.43f : 0.29f) +
+                                                    (beside ? 0.f : (S == 2 ? 1.5f : (S == 3 ? 4.f : 6.f))));
         }
     }
-    if (crowded && !dual && num_m > 1 && best.split == 1) {
-        // Tall tiles: 0.71 us per k-block against twice 0.415 (2048 tokens, us per call without adapters, single / tall:
-        // 4096 x 4096 55.9 / 50.4, 4096 x 11008 145.5 / 127.0; 8192 tokens, 11008 x 4096 581 / 546).
-        int tiles = 0;
-        for (int p = 0; p < P; ++p) tiles += (num_m + 1) / 2 * ((d_outs[p] + 255) / 256);
-        const float us = (float)((tiles + num_sms - 1) / num_sms) * ((float)num_kb * 0.71f);
-        if (us < best_us) best = {256, 1, tiles, true};
+    if (!dual && num_m > 1 && best.split == 1) {   // CTA pairs (lml_gemm_pair.cu), tiles of 256 rows
+        for (int bn = 256; bn >= 64; bn -= 32) {
+            const int tiles = pair_tiles_of(bn), waves = (tiles + num_sms / 2 - 1) / (num_sms / 2);
+            consider({bn, 1, 2 * tiles, true}, 10.f + (float)(waves * num_kb) * (waves > 1 ? 0.12f + 0.00082f * (float)bn : 0.035f + 0.00097f * (float)bn));
+        }
     }
     return best;
 }
@@ -1393,46 +1216,44 @@ GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, 
 // Tensor maps of the caller's buffers are kept per table: a serving loop calls with the same few
 // (pointer, shape) combinations over and over, and encoding a map costs a driver call each time.
 bool TmapCache::get_2d(CUtensorMap* out, const void* base, uint64_t inner, uint64_t outer, uint64_t stride_bytes,
-                       uint32_t box_inner, uint32_t box_outer)
+                       uint32_t box_inner, uint32_t box_outer, bool swizzle)
 {
     std::lock_guard<std::mutex> lock(mu);
     for (int i = 0; i < used; ++i) {
         const Key& k = keys[i];
         if (k.base == base && k.inner == inner && k.outer == outer && k.stride == stride_bytes && k.box_inner == box_inner &&
-            k.box_outer == box_outer) {
+            k.box_outer == box_outer && k.swizzle == swizzle) {
             *out = maps[i];
             return true;
         }
     }
     CUtensorMap m;
-    if (!encode_tmap_2d(&m, base, inner, outer, stride_bytes, box_inner, box_outer)) return false;
+    if (!encode_tmap_2d(&m, base, inner, outer, stride_bytes, box_inner, box_outer, swizzle)) return false;
     const int slot = used < kEntries ? used++ : (next = (next + 1) % kEntries);
-    keys[slot] = Key{base, inner, outer, stride_bytes, box_inner, box_outer};
+    keys[slot] = Key{base, inner, outer, stride_bytes, box_inner, box_outer, swizzle};
     maps[slot] = m;
     *out = m;
     return true;
 }
 
-// Whether the shrink can run inside the GEMM kernel for this call: whole-K tiles, few enough row tiles for its tables, and
-// the passes on CTAs with a tile's time to spare.  A shrink pass takes about as long as an output tile, whatever its width.
-// It pays where some CTAs have that time and the others do not reach their first chunks before it is over: 256-column
-// tiles in more than one wave, and few enough passes (every segment boundary inside a row tile can add one) that no CTA gets two.
+// Whether the shrink runs inside the GEMM kernel: a plain call with little x (1.4 M elements), whole-K tiles of 256 columns in more than
+// one wave, so that CTAs have time to spare, few enough row tiles for the kernel's tables and few enough passes (a pass per row tile and
+// four chunks; every segment boundary inside a row tile can add one) that no CTA gets two.  One launch instead of two, in about the same
+// time on the device (us, inside / bind_shrink ahead: 700 x 520 -> 8192 19.6 / 20.2, 700 x 264 -> 8192 16.9 / 17.0, 1300 x 1032 -> 4104 26.6 /
+// 25.1, 2100 x 264 -> 5000 27.6 / 23.0); with more x bind_shrink, which shares K among the CTAs that the tiles leave, is done
+// sooner (2048 x 4096 -> 4096 61.4 / 49.9).
 // (What counts is T, G and the table's size, not what is registered: the two forms sum x.A^T in different orders, and a call's
 // bits must not change with adapters that it does not use.  Segments in order: a tile has one pass and one more for every segment
 // that begins in it, at most; rows in any order: reckoned with half of the widest adapter for every segment.)
-bool gemm_can_fuse_shrink(const GemmShape& shape, int T, int d_out, int G, bool in_segment_order, int max_slots, int num_sms)
+bool gemm_can_fuse_shrink(int T, int d_in, int d_out, int G, bool in_segment_order, int max_slots, int num_sms)
 {
     if (G <= 0 || (in_segment_order && G > kBindSegs)) return false;
-    if (shape.split != 1 || shape.bn != 256) return false;
     const int num_m = (T + kBM - 1) / kBM, num_n = (d_out + 255) / 256;
-    if (num_m > kFuseTilesInKernel || (!shape.tall && num_m * num_n <= num_sms)) return false;
+    if ((long long)T * d_in > 1400000ll || num_m > kFuseTilesInKernel || num_m * num_n <= num_sms) return false;
     static_assert(kShrChunks * kChunk == kRankPad, "a slot takes one pass at most");
     const int slots = G < max_slots ? G : max_slots;
     if (num_m * slots > kShrMaxPasses * num_sms && !in_segment_order) return false;   // (room for a CTA's passes)
-    const int passes = in_segment_order ? num_m + G : num_m * ((slots + 1) / 2);
-    // (tall tiles: only as many passes as there are CTAs with a tile less than the others, or none)
-    if (shape.tall) return passes <= num_sms - (shape.ctas - 1) % num_sms - 1;
-    return passes <= num_sms / 2;
+    return (in_segment_order ? num_m + G : num_m * ((slots + 1) / 2)) <= num_sms / 2;
 }
 
 cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* caches, const GemmArgs& a, cudaStream_t stream)
@@ -1440,17 +1261,18 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
     const bool dual = a.u2 != nullptr;
     if (dual && (!a.lora || !a.y2 || a.P != 1 || a.fused)) return cudaErrorInvalidValue;
     const int bn = a.shape.bn, split = a.shape.split;
-    if (a.fused && (split != 1 || bn != 256 || a.P != 1)) return cudaErrorInvalidValue;   // (the caller asked gemm_can_fuse_shrink first)
+    if (a.fused && (split != 1 || bn != 256 || a.P != 1)) return cudaErrorInvalidValue;
     GemmParams p;
+    p.a = tmap_A;
     p.num_m = (a.T + kBM - 1) / kBM;
     const uint64_t xs = (uint64_t)a.d_in * 2;
     if (!caches[0]->get_2d(&p.x, a.x, (uint64_t)a.d_in, (uint64_t)a.T, xs, kBK, (uint32_t)x_box_rows(a.T))) return cudaErrorInvalidValue;
     p.x_bytes = x_box_rows(a.T) * kBK * 2;
-    p.a = tmap_A;
     int tiles = 0, columns = 0;
     for (int i = 0; i < a.P; ++i) {
         const GemmProj& pr = a.proj[i];
         GemmPart& pt = p.part[i];
+        fill_gemm_part(pt, pr, bn, tiles);
         const uint64_t ys = (uint64_t)pr.d_out * 2;
         if (!caches[i]->get_2d(&pt.w, pr.W0, (uint64_t)a.d_in, (uint64_t)pr.d_out, xs, kBK, (uint32_t)bn)) return cudaErrorInvalidValue;
         if (split == 1) {   // (the split-K kernel stores its outputs with plain stores)
@@ -1458,16 +1280,7 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
         } else {
             pt.y = pt.w;
         }
-        pt.bk = pr.ar->Bk; pt.b = pr.ar->B; pt.nonfinite = pr.ar->nonfinite; pt.plan = pr.plan; pt.u = pr.u; pt.u_mid = pr.u_mid; pt.u_lo = pr.u_lo; pt.y_ptr = (__nv_bfloat16*)pr.y;
-        pt.live = pt.nch[0] = pt.nch[1] = 0ull;
-        for (int s = 0; s < pr.snap->max_slots; ++s)
-            if (pr.snap->rank[s] > 0) {
-                pt.live |= 1ull << s;
-                pt.nch[s >> 5] |= (unsigned long long)(chunks_of_rank(pr.snap->rank[s]) - 1) << (2 * (s & 31));
-            }
-        pt.N = pr.d_out; pt.num_n = (pr.d_out + bn - 1) / bn; pt.n_pad = b_rows_padded(pr.d_out); pt.cap = pr.cap;
-        pt.tile0 = tiles;
-        tiles += (a.shape.tall ? (p.num_m + 1) / 2 : p.num_m) * pt.num_n;
+        tiles += p.num_m * pt.num_n;
         columns += pt.num_n;
     }
     p.y2 = p.part[0].y;
@@ -1477,15 +1290,13 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
     p.status = a.proj[0].ar->status;
     p.T = a.T; p.K = a.d_in; p.P = a.P; p.num_tiles = tiles;
     p.lora = a.lora ? 1 : 0; p.fused = a.fused ? 1 : 0; p.rows = a.rows;
-    p.x_flag = a.x_flag; p.call_id = a.call_id;
     p.pass_flags = a.proj[0].ar->pass_flags; p.fuse_sync = a.proj[0].ar->status + 4;
+    p.x_flag = a.x_flag; p.call_id = a.call_id;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     // with adapters the predecessor is the bind_shrink launch of this call, else the kernel waits at its top
-    const bool tall = a.shape.tall;
-    // (tall tiles with the shrink inside: the SMs without a tile take its passes)
-    pdl_config(cfg, attr, dim3((unsigned)(tiles < a.num_sms && !(tall && a.fused) ? tiles : a.num_sms)), dim3(tall ? kGemmThreadsTall : kGemmThreads),
-               tall ? GemmCfg<256, true>::kSmemBytes : bn == 256 ? GemmCfg<256>::kSmemBytes : (bn == 128 ? GemmCfg<128>::kSmemBytes : GemmCfg<64>::kSmemBytes), stream);
+    pdl_config(cfg, attr, dim3((unsigned)(tiles < a.num_sms ? tiles : a.num_sms)), dim3(kGemmThreads),
+               bn == 256 ? GemmCfg<256>::kSmemBytes : (bn == 128 ? GemmCfg<128>::kSmemBytes : GemmCfg<64>::kSmemBytes), stream);
     p.stages = 0;
     if (split > 1) {
         p.stages = a.share_sm && gemm_exchange_bytes(bn, split) <= gemm_stages_short(bn) * gemm_stage_bytes(bn) ? gemm_stages_short(bn) : gemm_stages(bn);
@@ -1500,10 +1311,9 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
         if (bn == 64) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_splitk_kernel<64>, p);
         return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_splitk_kernel<128>, p);
     }
-    if (tall) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<256, true>, p, *a.proj[0].snap);
-    if (bn == 256) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<256, false>, p, *a.proj[0].snap);
-    if (bn == 64) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<64, false>, p, *a.proj[0].snap);
-    return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<128, false>, p, *a.proj[0].snap);
+    if (bn == 256) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<256>, p, *a.proj[0].snap);
+    if (bn == 64) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<64>, p, *a.proj[0].snap);
+    return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<128>, p, *a.proj[0].snap);
 }
 
 }  // namespace lml

@@ -110,7 +110,8 @@ inline int b_rows_padded(int d_out) { return (d_out + 255) / 256 * 256; }
 // What bind_shrink writes for the GEMM, per row tile: the tile's chunks in the order of their blocks.
 struct alignas(16) TilePlan {
     int32_t count;
-    int32_t pad[3];
+    int32_t pad;
+    unsigned long long used;      // the slots that rows of the tile use, under either binding
     uint16_t chunk[kMaxChunks];   // slot | chunk << 8 | kChunkFirst, kChunkSecond
     int8_t nonfinite_row[2][kTileM];   // [binding][row] the row's slot if its B holds Inf or NaN, else -1 (written only where the table has seen such a B)
 };
@@ -142,6 +143,8 @@ struct BindPart {
     int cap;
     int pad;
 };
+// Early start: chunks of a pass, and whether the GEMM's CTAs and this launch's have to fit an SM together.
+struct BindEarly { int group = 8; bool share_sm = false; };
 struct BindArgs {
     const void* x;
     int T, d_in, P;
@@ -152,7 +155,7 @@ struct BindArgs {
     // early start of the GEMM (see bind_starts_gemm_early): the word that says "x may be read" and this call's value of it
     uint32_t* x_flag = nullptr;
     uint32_t call_id = 0;
-    bool share_sm = false;   // the GEMM's CTAs and this launch's have to fit an SM together
+    BindEarly early;
     BindPart part[LML_MAX_PROJECTIONS];
     SlotSnapshot snap[LML_MAX_PROJECTIONS];
 };
@@ -176,8 +179,8 @@ struct GemmProj {
     int cap;
 };
 // What the library takes for a call: width of an output tile and CTAs that share one (1: whole-K tiles), CTAs in all, and
-// whether a whole-K tile is two row tiles high.
-struct GemmShape { int bn, split, ctas; bool tall; };
+// whether a whole-K tile is the work of a pair of CTAs, two row tiles high.
+struct GemmShape { int bn, split, ctas; bool pair; };
 struct GemmArgs {
     const void* x;
     int T, d_in, P;
@@ -197,33 +200,35 @@ struct GemmArgs {
 };
 // split_bn, split_s: the table's override (-1 = the library chooses, 0 = whole-K tiles, else the forced shape)
 GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, int num_sms, int split_bn, int split_s);
-// whether the shrink of a plain call of this size and shape runs inside the GEMM kernel
-bool gemm_can_fuse_shrink(const GemmShape& shape, int T, int d_out, int G, bool in_segment_order, int max_slots, int num_sms);
+// whether the shrink of a plain call of this size runs inside the GEMM kernel, on whole-K tiles of 256 columns
+bool gemm_can_fuse_shrink(int T, int d_in, int d_out, int G, bool in_segment_order, int max_slots, int num_sms);
 // Tensor maps of caller buffers, kept per table and found again by (pointer, shape, box).
 struct TmapCache {
     static constexpr int kEntries = 32;
-    struct Key { const void* base; uint64_t inner, outer, stride; uint32_t box_inner, box_outer; };
+    struct Key { const void* base; uint64_t inner, outer, stride; uint32_t box_inner, box_outer; bool swizzle; };
     Key keys[kEntries];
     CUtensorMap maps[kEntries];
     int used = 0, next = 0;
     std::mutex mu;
     bool get_2d(CUtensorMap* out, const void* base, uint64_t inner, uint64_t outer, uint64_t stride_bytes,
-                uint32_t box_inner, uint32_t box_outer);
+                uint32_t box_inner, uint32_t box_outer, bool swizzle = true);
 };
 bool gemm_split_override(int* bn_out, int* split_out);
 // bind_starts_gemm_early: for calls of few rows the GEMM may start while the work before the call is still running; it then
 // reads nothing but W0 until bind_shrink, which waits for that work, has said that x may be read.
 bool bind_starts_gemm_early(int T, int P, int num_sms);
-int bind_ctas_early(int T, int d_in, int P, int cap, int num_sms);   // ... and how many CTAs bind_shrink has then
+BindEarly bind_early(int T, int d_in, int P, int cap, int gemm_ctas, int num_sms);   // ... beside a GEMM of so many CTAs
 // tmap_A[p]: the map of projection p's packed A arena ([max_slots][64][d_in], box 64 x 16 x 1)
 cudaError_t launch_bind_shrink(const BindArgs& a, const CUtensorMap* const* tmap_A, TmapCache* cache, int num_sms, cudaStream_t stream);
 // tmap_A: the same of the (first) table, for the fused shrink; caches[p]: the tensor maps of the buffers of projection p.
-// Returns cudaErrorInvalidValue if one cannot be encoded.
+// Return cudaErrorInvalidValue if one cannot be encoded.
 cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* caches, const GemmArgs& a, cudaStream_t stream);
+cudaError_t launch_gemm_pair(TmapCache* const* caches, const GemmArgs& a, cudaStream_t stream);   // shapes of CTA pairs
 cudaError_t gemm_sm100_init(int device);
+cudaError_t gemm_pair_init();
 cudaError_t shrink_init();   // these set the dynamic shared memory attributes of their kernels
 bool encode_tmap_2d(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer,
-                    uint64_t row_stride_bytes, uint32_t box_inner, uint32_t box_outer);
+                    uint64_t row_stride_bytes, uint32_t box_inner, uint32_t box_outer, bool swizzle = true);
 bool encode_tmap_3d(CUtensorMap* m, const void* base, uint64_t d0, uint64_t d1, uint64_t d2,
                     uint64_t stride1_bytes, uint64_t stride2_bytes, uint32_t b0, uint32_t b1,
                     uint32_t b2);
@@ -309,6 +314,12 @@ __device__ __forceinline__ uint32_t ld_after_wait(const uint16_t* p)
     return v;
 }
 
+__device__ __forceinline__ unsigned long long ld_after_wait(const unsigned long long* p)
+{
+    unsigned long long v;
+    asm volatile("ld.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
+    return v;
+}
 __device__ __forceinline__ uint32_t ld_after_wait(const uint32_t* p) { return (uint32_t)ld_after_wait(reinterpret_cast<const int32_t*>(p)); }
 __device__ __forceinline__ int ld_after_wait(const int8_t* p)
 {
