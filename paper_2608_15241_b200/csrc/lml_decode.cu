@@ -241,6 +241,7 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_main_kernel(const __gri
         if (lane < 16) { ctrl->slot_of_row[lane] = -1; ctrl->b_of_row[lane] = -1; ctrl->b_lead[lane] = 0; ctrl->b_rows[lane] = 0; }
         asm volatile("bar.sync 4, %0;" ::"n"(kDecThreads) : "memory");   // the barriers are set up
         grid_launch_dependents();
+        const uint64_t once = policy_evict_first();
         for (int round_begin = row_begin; round_begin < row_end && ok; round_begin += kDecRoundUnits * kDecUnitRows) {
             const int round_rows = min(kDecRoundUnits * kDecUnitRows, row_end - round_begin);
             const int nunits = (round_rows + kDecUnitRows - 1) / kDecUnitRows;
@@ -260,9 +261,9 @@ __global__ void __launch_bounds__(kDecThreads, 1) decode_main_kernel(const __gri
                         if (lane == 0) mbar_arrive_expect_tx(smem_u32(&ctrl->full[stage]), (uint32_t)(rows * cols * 2));
                         __syncwarp();
                         if (lane < rows)
-                            bulk_copy_g2s(ring + stage * kDecStageBytes + lane * kDecRowPitch,
+                            bulk_copy_g2s_once(ring + stage * kDecStageBytes + lane * kDecRowPitch,
                                           W0 + (size_t)(r0 + lane) * K + k_begin + kc * kDecChunk,
-                                          (uint32_t)(cols * 2), smem_u32(&ctrl->full[stage]));
+                                          (uint32_t)(cols * 2), smem_u32(&ctrl->full[stage]), once);
                         if (++stage == kS) { stage = 0; phase ^= 1u; }
                     }
                 }

@@ -184,6 +184,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
     tc_fence_after();
     const uint32_t tmem_base = ctrl->tmem_base;
     volatile int* abort = &ctrl->abort;
+    const uint64_t once = policy_evict_first();   // W0 passes through L2 once and must not push out what the next launches begin with
     if (p.x_flag) {   // early start: the first k-blocks' W0, then x
         const GemmPart& pt = p.part[part_of(p, (int)blockIdx.x)];
         const int n0 = ((int)blockIdx.x - pt.tile0) / p.num_m;
@@ -192,7 +193,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                 for (int kb = 0; kb < min(Cfg::kStages, num_kb); ++kb) {
                     const uint32_t bar = smem_u32(&ctrl->full[kb]);
                     mbar_expect_tx(bar, Cfg::kBBytes);
-                    tma_load_2d(tiles_addr + kb * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, kb * kBK, n0 * BN);
+                    tma_load_2d_once(tiles_addr + kb * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, kb * kBK, n0 * BN, once);
                 }
                 wait_x(p.x_flag, p.call_id);
             }
@@ -436,7 +437,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                     ctrl->stage_info[st] = 4u | acc_flag | (kb == num_kb - 1 ? flags_last : 0u);
                     mbar_arrive_expect_tx(bar, (uint32_t)(p.x_bytes + (kb < have_w ? 0 : Cfg::kBBytes)));
                     tma_load_2d(a_dst, &p.x, bar, kb * kBK, row0);
-                    if (kb >= have_w) tma_load_2d(a_dst + Cfg::kABytes, w, bar, kb * kBK, col0);
+                    if (kb >= have_w) tma_load_2d_once(a_dst + Cfg::kABytes, w, bar, kb * kBK, col0, once);
                     if (++st == Cfg::kStages) { st = 0; ph ^= 1u; }
                 }
                 stage = st; phase = ph; ok = good;
@@ -816,6 +817,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
     tc_fence_after();
     const uint32_t tmem_base = ctrl->tmem_base;
     volatile int* abort = &ctrl->abort;
+    const uint64_t once = policy_evict_first();   // W0 passes through L2 once and must not push out what the next launches begin with
     if (p.x_flag) {   // early start: the first k-blocks' W0, then x
         if (warp == 0) {
             if (elect_one()) {
@@ -823,7 +825,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
                 for (int i = 0; i < ahead; ++i) {
                     const uint32_t bar = smem_u32(&ctrl->full[i]);
                     mbar_expect_tx(bar, Cfg::kBBytes);
-                    tma_load_2d(tiles_addr + i * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, (kb0 + i) * kBK, n * BN);
+                    tma_load_2d_once(tiles_addr + i * Cfg::kStageBytes + Cfg::kABytes, &pt.w, bar, (kb0 + i) * kBK, n * BN, once);
                 }
                 wait_x(p.x_flag, p.call_id);
             }
@@ -858,7 +860,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
                 const bool have_w = kb - kb0 < ahead;
                 mbar_arrive_expect_tx(bar, (uint32_t)(p.x_bytes + (have_w ? 0 : Cfg::kBBytes)));
                 tma_load_2d(a_dst, &p.x, bar, kb * kBK, row0);
-                if (!have_w) tma_load_2d(a_dst + Cfg::kABytes, &pt.w, bar, kb * kBK, n * BN);
+                if (!have_w) tma_load_2d_once(a_dst + Cfg::kABytes, &pt.w, bar, kb * kBK, n * BN, once);
                 advance();
             }
             // This CTA's share of the tile's LoRA chunks: chunk c of slot s goes to CTA (s + c) mod S.  Which CTA adds a
