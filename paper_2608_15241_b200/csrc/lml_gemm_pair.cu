@@ -320,6 +320,8 @@ __global__ void __launch_bounds__(kPairThreads, 1) lora_gemm_pair_kernel(const _
         const uint32_t acc_free0 = mapa_shared(smem_u32(&ctrl->tmem_empty[0]), 0);   // the first CTA's
         int acc = 0;
         uint32_t fph = 0;   // bit a: phase of tmem_full[a]
+        int buf = 0;        // staging buffer of the next store: it alternates from store to store, through all tiles (a tile may store
+                            // an odd number of chunks)
         bool ok = true;
         if (p.lora) grid_dependency_wait();   // (the plans are read here too)
         for (int tile = pair; tile < p.num_tiles && ok; tile += npairs) {
@@ -340,8 +342,8 @@ __global__ void __launch_bounds__(kPairThreads, 1) lora_gemm_pair_kernel(const _
             auto put = [&](int c, const uint32_t (&v32)[32]) {   // 32 columns: to bf16, into shared memory, out
                 const int col0 = n * p.bn + c * kEpiChunkCols;
                 if (col0 >= pt.N || row_base >= p.T) return;   // nothing of this chunk is inside y
-                const int at = last ? (ew * (kPairAcc / kEpiChunkCols) + c) * kEpiBufBytes : kPairRingBytes + (ew * 2 + (c & 1)) * kEpiBufBytes;
-                if (!last) {   // the buffer we are about to overwrite must have been read by its earlier store
+                const int at = last ? (ew * (kPairAcc / kEpiChunkCols) + c) * kEpiBufBytes : kPairRingBytes + (ew * 2 + buf) * kEpiBufBytes;
+                if (!last) {   // the buffer we are about to overwrite must have been read by its earlier store: all but the newest have
                     if (one) tma_store_wait_read<1>();
                     __syncwarp();
                 }
@@ -365,6 +367,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) lora_gemm_pair_kernel(const _
                     tma_store_2d(&pt.y, ring + (uint32_t)at, col0, row_base);
                     tma_store_commit();
                 }
+                buf ^= 1;
             };
             auto fetched = [&](int c) {   // chunk c is in registers; behind the last one the accumulator goes back to the MMA issuer
                 tmem_ld_wait();
