@@ -237,7 +237,9 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
         if (warp != 1) {
             // Warp 0 brings in x and accounts for the stage's bytes; the four row warps, which have nothing to do yet, share the chunks (an
             // issue costs its thread some 60 cycles: 17 copies of a k-block from one thread took 0.55 us, longer than their flight).
-            if (elect_one()) {
+            // A warp without a chunk stays out: no stage waits for it, so nothing would keep it within a lap of the ring, and a parity read
+            // a lap late says "not yet" for good.
+            if ((warp == 0 || warp - 2 < nc) && elect_one()) {
                 bool ok = true;
                 for (int i = 0; i < nkb && ok; ++i) {
                     ok = mbar_wait(smem_u32(&ctrl->empty[stage]), phase ^ 1u, abort);

@@ -11,13 +11,13 @@ from gpu_util import Guarded, to_bits, to_dev
 pytestmark = pytest.mark.gpu
 
 
-def _site(K, N, ranks, seed=17):
+def _site(K, N, ranks, seed=17, std=0.05):
     from paper_2608_15241_b200.binding import Table
-    entries = wl.make_entries(seed, K, N, [(a, 1, r, 2.0) for a, r in enumerate(ranks)], std=0.05)
+    entries = wl.make_entries(seed, K, N, [(a, 1, r, 2.0) for a, r in enumerate(ranks)], std=std)
     tbl = Table(K, N, len(ranks))
     for e in entries:
         tbl.register_adapter(e.adapter_id, 1, to_dev(e.A), to_dev(e.B), e.scale)
-    return tbl, entries, wl.normal_bf16(seed, 2, (N, K), 0.05)
+    return tbl, entries, wl.normal_bf16(seed, 2, (N, K), std)
 
 
 def _sample(T, seed=0):
@@ -32,6 +32,26 @@ def _check(y, x, W, entries, entry, pos):
     ref, _ = oracle.forward(x[pos], W, entries, np.arange(len(pos) + 1, dtype=np.int32), entry[pos])
     r = oracle.compare(to_bits(y)[pos], ref)
     assert r["ok"], r
+
+
+@pytest.mark.parametrize("T", [300, 5000])
+@pytest.mark.parametrize("ranks", [(16,), (16, 9), (33,), (64, 4), (16,) * 18])
+def test_few_chunks_on_many_laps_of_the_ring(T, ranks):
+    """Passes of one, two, three and five chunks, and of two after full ones, over 129 k-blocks: fewer chunks than bind_shrink has warps that
+    copy them, and a ring that goes round many times.  (Adapters of N(0, 0.02): u is 2 x.A, of size 2 sqrt(8200) 0.02 = 3.6, and its rounding to
+    bf16, 2^-9 of it in the mean, reaches y through at most 64 entries of B: 3.6 2^-9 0.02 8 = 1.1e-3, a ninth of the tolerance.)"""
+    import torch
+    K, N = 8200, 136
+    tbl, entries, W = _site(K, N, ranks, std=0.02)
+    x = wl.normal_bf16(31, 1, (T, K), 1.0)
+    entry = np.random.default_rng(T).integers(-1, len(ranks), size=T).astype(np.int32)
+    tok = torch.from_numpy(entry).cuda()
+    ys = [tbl.lora_mixed_linear_tokens(to_dev(x), to_dev(W), tok) for _ in range(3)]
+    torch.cuda.synchronize()
+    assert tbl.device_status() == 0
+    _check(ys[0], x, W, entries, entry, _sample(T))
+    assert all(torch.equal(ys[0], y) for y in ys[1:])
+    tbl.close()
 
 
 @pytest.mark.parametrize("T", [5000, 9600])
