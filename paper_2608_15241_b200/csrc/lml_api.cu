@@ -74,6 +74,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
     lml_table* t0 = calls[0].t;
     const int num_m = (T + kTileM - 1) / kTileM;
     const bool dual = y2 != nullptr;
+    bool precise = false;
     SlotSnapshot snap[LML_MAX_PROJECTIONS];
     BindArgs b;
     GemmArgs g;
@@ -89,6 +90,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         snap[p] = snapshot_locked(c.t);
         b.snap[p] = snap[p];
         caches[p] = &c.t->tmaps;
+        precise = precise || c.precise;
         tmaps_A[p] = &c.t->tmap_A;
         d_outs[p] = c.t->d_out;
         int live = 0;   // chunks of all live slots: no tile needs more
@@ -125,7 +127,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         }
         if (r0 > 0 && b.rows.rows) b.rows.rows += kSlabTiles * kTileM;
         if (r0 > 0 && b.rows.rows2) b.rows.rows2 += kSlabTiles * kTileM;
-        g.shape = gemm_pick_shape(rows, t0->d_in, d_outs, P, dual, t0->num_sms, t0->split_bn, t0->split_s);
+        g.shape = gemm_pick_shape(rows, t0->d_in, d_outs, P, dual, precise, t0->num_sms, t0->split_bn, t0->split_s);
         // Small plain calls compute u inside the GEMM kernel (on the CTAs that own the fewest tiles, ahead of their tiles); otherwise a
         // launch goes first and the GEMM is its programmatic dependent.
         g.fused = mode == kRowsSegments && !dual && P == 1 && T == rows && t0->fuse_shrink && t0->split_bn <= 0 &&

@@ -480,6 +480,7 @@ cudaError_t launch_gemm_pair(TmapCache* const* caches, const GemmArgs& a, cudaSt
     int tiles = 0;
     for (int i = 0; i < a.P; ++i) {
         const GemmProj& pr = a.proj[i];
+        if (pr.u_lo) return cudaErrorInvalidValue;   // (gemm_pick_shape chooses no pairs for such a call)
         PairPart& pp = p.part[i];
         GemmPart& pt = pp.g;
         fill_gemm_part(pt, pr, bn, tiles);

@@ -198,8 +198,9 @@ struct GemmArgs {
     bool share_sm = false;        // as in BindArgs
     int num_sms;
 };
-// split_bn, split_s: the table's override (-1 = the library chooses, 0 = whole-K tiles, else the forced shape)
-GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, int num_sms, int split_bn, int split_s);
+// split_bn, split_s: the table's override (-1 = the library chooses, 0 = whole-K tiles, else the forced shape); precise: some projection's
+// u is three bf16 values
+GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, bool precise, int num_sms, int split_bn, int split_s);
 // whether the shrink of a plain call of this size runs inside the GEMM kernel, on whole-K tiles of 256 columns
 bool gemm_can_fuse_shrink(int T, int d_in, int d_out, int G, bool in_segment_order, int max_slots, int num_sms);
 // Tensor maps of caller buffers, kept per table and found again by (pointer, shape, box).

@@ -66,3 +66,34 @@ def test_several_panels_of_rows(monkeypatch):
     rows = pos if w.perm is None else w.perm[pos]
     r = oracle.compare(y[rows], ref[rows])
     assert flags == 0 and r["ok"], r
+
+
+@pytest.mark.parametrize("T", [17, 48])
+def test_u_of_three_values_does_not_take_pairs(T, monkeypatch):
+    """A call of several projections at 17 - 48 tokens multiplies u as three bf16 values, which the pair kernel has no place for: with pairs
+    asked for it runs on whole-K tiles, and keeps its bits."""
+    import torch
+    from paper_2608_15241_b200 import binding as b
+    from paper_2608_15241_b200.binding import Table
+    from gpu_util import to_bits, to_dev
+    K, Ns, ranks = 520, (264, 1000), (4, 33, 64)
+    x, tok = wl.normal_bf16(9, 1, (T, K), 1.0), np.random.default_rng(T).integers(-1, len(ranks), size=T).astype(np.int32)
+    W = [wl.normal_bf16(9, 10 + p, (N, K), 0.02) for p, N in enumerate(Ns)]
+    ents = [wl.make_entries(9 + p, K, N, [(a, 1, r, 2.0) for a, r in enumerate(ranks)]) for p, N in enumerate(Ns)]
+    out = []
+    for shape in ("0", "128p"):
+        monkeypatch.setenv("LML_GEMM_SPLIT", shape)
+        tables = [Table(K, N, len(ranks)) for N in Ns]
+        for t, es in zip(tables, ents):
+            for e in es:
+                t.register_adapter(e.adapter_id, 1, to_dev(e.A), to_dev(e.B), e.scale)
+        ys = b.multi_projection(tables, to_dev(x), [to_dev(w) for w in W], torch.from_numpy(tok).cuda())
+        torch.cuda.synchronize()
+        assert all(t.device_status() == 0 for t in tables)
+        out.append([to_bits(y) for y in ys])
+        for t in tables:
+            t.close()
+    for p in range(len(Ns)):
+        assert np.array_equal(out[0][p], out[1][p]), p
+        ref, _ = oracle.forward(x, W[p], ents[p], np.arange(T + 1, dtype=np.int32), tok)
+        assert oracle.compare(out[1][p], ref)["ok"], p
