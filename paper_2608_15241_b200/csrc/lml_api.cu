@@ -109,6 +109,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         gp.plan = bp.plan; gp.u = bp.u; gp.u_mid = c.precise ? bp.u2 : nullptr; gp.u_lo = bp.u3; gp.cap = cap;
     }
     g.num_sms = t0->num_sms;
+    g.num_pairs = t0->num_pairs;
     if (mode == kRowsSegments && (perm || G > kBindSegs || num_m > kSlabTiles)) {   // a slot per row first
         int8_t* rows = reinterpret_cast<int8_t*>(calls[0].ws + calls[0].layout.rows_off);
         int8_t* rows2 = dual ? reinterpret_cast<int8_t*>(calls[0].ws + calls[0].layout.rows2_off) : nullptr;
@@ -127,7 +128,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         }
         if (r0 > 0 && b.rows.rows) b.rows.rows += kSlabTiles * kTileM;
         if (r0 > 0 && b.rows.rows2) b.rows.rows2 += kSlabTiles * kTileM;
-        g.shape = gemm_pick_shape(rows, t0->d_in, d_outs, P, dual, precise, t0->num_sms, t0->split_bn, t0->split_s);
+        g.shape = gemm_pick_shape(rows, t0->d_in, d_outs, P, dual, precise, t0->num_sms, t0->num_pairs, t0->split_bn, t0->split_s);
         // Small plain calls compute u inside the GEMM kernel (on the CTAs that own the fewest tiles, ahead of their tiles); otherwise a
         // launch goes first and the GEMM is its programmatic dependent.
         g.fused = mode == kRowsSegments && !dual && P == 1 && T == rows && t0->fuse_shrink && t0->split_bn <= 0 &&
@@ -244,7 +245,7 @@ lml_status lml_table_create(lml_table** out, int device, int d_in, int d_out, in
     ok = ok && cudaMemset(t->arena.pass_flags, 0, kFuseMaxPasses * sizeof(int32_t)) == cudaSuccess;
     ok = ok && decode_init() == cudaSuccess;   // (first: see there)
     ok = ok && gemm_sm100_init(device) == cudaSuccess;
-    ok = ok && gemm_pair_init() == cudaSuccess;
+    ok = ok && gemm_pair_init(t->num_sms, &t->num_pairs) == cudaSuccess;
     ok = ok && shrink_init() == cudaSuccess;
     ok = ok && aux_init() == cudaSuccess;
     ok = ok && bind_init() == cudaSuccess;

@@ -20,8 +20,6 @@
 //            whose own row tile does not use a chunk multiplies zeros (a copy from behind the end of the u blocks).
 //
 // Early start as in lml_gemm_sm100.cu.  Every wait is bounded; on give-up the CTA sets LML_FLAG_TIMEOUT and frees its TMEM.
-#include <mutex>
-
 #include "lml_gemm_common.cuh"
 
 namespace lml {
@@ -442,33 +440,26 @@ __global__ void __launch_bounds__(kPairThreads, 1) lora_gemm_pair_kernel(const _
     }
 }
 
-// Pairs of CTAs that are resident at once.
-static int pairs_resident(int num_sms)
+// pairs: the pairs of CTAs that are resident at once; 0, and no call takes pairs, where the runtime does not say.
+cudaError_t gemm_pair_init(int num_sms, int* pairs)
 {
-    static int pairs;
-    static std::once_flag probed;
-    std::call_once(probed, [&]() {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3((unsigned)(num_sms / 2 * 2));
-        cfg.blockDim = dim3(kPairThreads);
-        cfg.dynamicSmemBytes = kPairSmemBytes;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr; cfg.numAttrs = 1;
-        if (cudaOccupancyMaxActiveClusters(&pairs, lora_gemm_pair_kernel, &cfg) != cudaSuccess || pairs < 1) { (void)cudaGetLastError(); pairs = 1; }
-    });
-    return pairs;
-}
-
-cudaError_t gemm_pair_init()
-{
-    return cudaFuncSetAttribute(lora_gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes);
+    const cudaError_t e = cudaFuncSetAttribute(lora_gemm_pair_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kPairSmemBytes);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)(num_sms / 2 * 2));
+    cfg.blockDim = dim3(kPairThreads);
+    cfg.dynamicSmemBytes = kPairSmemBytes;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 2; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr; cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(pairs, lora_gemm_pair_kernel, &cfg) != cudaSuccess) { *pairs = 0; (void)cudaGetLastError(); }
+    return cudaSuccess;
 }
 
 cudaError_t launch_gemm_pair(TmapCache* const* caches, const GemmArgs& a, cudaStream_t stream)
 {
-    if (a.u2 || a.fused) return cudaErrorInvalidValue;
+    if (a.u2 || a.fused || a.num_pairs < 1) return cudaErrorInvalidValue;
     PairParams p;
     const int bn = a.shape.bn;
     p.num_m = (a.T + kBM - 1) / kBM;
@@ -509,8 +500,7 @@ cudaError_t launch_gemm_pair(TmapCache* const* caches, const GemmArgs& a, cudaSt
     p.stages = kPairRingBytes / p.stage_bytes < kPairMaxStages ? kPairRingBytes / p.stage_bytes : kPairMaxStages;
     p.lora = a.lora ? 1 : 0;
     p.x_flag = a.x_flag; p.call_id = a.call_id;
-    const int pairs_max = pairs_resident(a.num_sms);
-    const int pairs = tiles < pairs_max ? tiles : pairs_max;
+    const int pairs = tiles < a.num_pairs ? tiles : a.num_pairs;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     pdl_config(cfg, attr, dim3((unsigned)(2 * pairs)), dim3(kPairThreads), kPairSmemBytes, stream);

@@ -1143,7 +1143,7 @@ static int gemm_exchange_bytes(int bn, int split) { return split * ((bn / 32 + s
 // 11008 -> 4096; splits there 128x2 34.7, 128x3 27.0, 256x4 32.5, 256x6 30.0; pairs of 256 / 160 / 128 columns 26.8 / 21.4 / 21.3 at 512 x
 // 4096 -> 4096, and where the tiles take several rounds, at the power that the tensor cores may draw, 96.6 at 1300 x 4096 -> 11008 (256
 // columns, four rounds), 109.3 at 1600 (224 columns, five; with 256 columns 115.9), against 111 and 128.6 for single tiles of 128.
-GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, bool precise, int num_sms, int split_bn, int split_s)
+GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, bool precise, int num_sms, int num_pairs, int split_bn, int split_s)
 {
     static int max_clusters[3][kSplitMaxS + 1];   // for 64, 128 and 256 columns
     static std::once_flag probed;
@@ -1178,7 +1178,7 @@ GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, 
         for (int p = 0; p < P; ++p) tiles += (num_m + 1) / 2 * ((d_outs[p] + bn - 1) / bn);
         return tiles;
     };
-    const bool pairs = !dual && !precise;   // (the pair kernel has neither a second output nor a u of three values)
+    const bool pairs = num_pairs > 0 && !dual && !precise;   // (the pair kernel has neither a second output nor a u of three values)
     if (split_bn > 0 && split_s == 0) {
         if (pairs) return {split_bn, 1, 2 * pair_tiles_of(split_bn), true};
         split_bn = 0;
@@ -1209,7 +1209,7 @@ GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, 
     }
     if (pairs && num_m > 1 && best.split == 1) {   // CTA pairs (lml_gemm_pair.cu), tiles of 256 rows
         for (int bn = 256; bn >= 64; bn -= 32) {
-            const int tiles = pair_tiles_of(bn), waves = (tiles + num_sms / 2 - 1) / (num_sms / 2);
+            const int tiles = pair_tiles_of(bn), waves = (tiles + num_pairs - 1) / num_pairs;
             consider({bn, 1, 2 * tiles, true}, 10.f + (float)(waves * num_kb) * (waves > 1 ? 0.12f + 0.00082f * (float)bn : 0.035f + 0.00097f * (float)bn));
         }
     }

@@ -197,10 +197,11 @@ struct GemmArgs {
     uint32_t call_id = 0;
     bool share_sm = false;        // as in BindArgs
     int num_sms;
+    int num_pairs;                // pairs of the pair kernel's CTAs that are resident at once
 };
 // split_bn, split_s: the table's override (-1 = the library chooses, 0 = whole-K tiles, else the forced shape); precise: some projection's
 // u is three bf16 values
-GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, bool precise, int num_sms, int split_bn, int split_s);
+GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, bool precise, int num_sms, int num_pairs, int split_bn, int split_s);
 // whether the shrink of a plain call of this size runs inside the GEMM kernel, on whole-K tiles of 256 columns
 bool gemm_can_fuse_shrink(int T, int d_in, int d_out, int G, bool in_segment_order, int max_slots, int num_sms);
 // Tensor maps of caller buffers, kept per table and found again by (pointer, shape, box).
@@ -226,7 +227,7 @@ cudaError_t launch_bind_shrink(const BindArgs& a, const CUtensorMap* const* tmap
 cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* caches, const GemmArgs& a, cudaStream_t stream);
 cudaError_t launch_gemm_pair(TmapCache* const* caches, const GemmArgs& a, cudaStream_t stream);   // shapes of CTA pairs
 cudaError_t gemm_sm100_init(int device);
-cudaError_t gemm_pair_init();
+cudaError_t gemm_pair_init(int num_sms, int* pairs);
 cudaError_t shrink_init();   // these set the dynamic shared memory attributes of their kernels
 bool encode_tmap_2d(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer,
                     uint64_t row_stride_bytes, uint32_t box_inner, uint32_t box_outer, bool swizzle = true);

@@ -7,6 +7,7 @@
 
 struct lml_table {
     int device = 0, d_in = 0, d_out = 0, max_slots = 0, num_sms = 0;
+    int num_pairs = 0;                  // pairs of the GEMM's CTAs that the device holds at once
     struct Entry {
         bool live = false;
         int adapter_id = 0, version = 0, rank = 0;
