@@ -282,6 +282,7 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
         bool ok = true;
         if (warp >= 2) {
             ok = mbar_wait_warp(smem_u32(&ctrl->tmem_full), tmem_ph, abort);   // this CTA's products are complete: so are its loads
+            if (!ok) __nanosleep(50000);   // gave up: let copies still in flight land before the ring takes the partial sums
             tc_fence_after();
         }
         tmem_ph ^= 1u;

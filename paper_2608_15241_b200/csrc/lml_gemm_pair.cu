@@ -430,6 +430,7 @@ __global__ void __launch_bounds__(kPairThreads, 1) lora_gemm_pair_kernel(const _
     }
 
     __syncthreads();
+    if (ctrl->abort) __nanosleep(50000);   // gave up: let copies still in flight land before the CTA goes away
     if (threadIdx.x == 0 && ctrl->abort) atomicOr(p.status, LML_FLAG_TIMEOUT);
     if (threadIdx.x == 0) leave_early_start(p.x_flag);
     __syncwarp();

@@ -742,6 +742,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
     }
 
     __syncthreads();
+    if (ctrl->abort) __nanosleep(50000);   // gave up: let copies still in flight land before the CTA goes away
     if (threadIdx.x == 0 && ctrl->abort) atomicOr(p.status, LML_FLAG_TIMEOUT);
     if (threadIdx.x == 0) leave_early_start(p.x_flag);
     if (threadIdx.x == 0 && p.fused) {
@@ -959,6 +960,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
         }
         if (p.lora) nonfinite = ld_after_wait(pt.nonfinite) != 0u;
         ok = mbar_wait_warp(smem_u32(&ctrl->tmem_full[0]), 0u, abort);   // this CTA's MMAs are complete: so are its loads
+        if (!ok) __nanosleep(50000);   // gave up: let copies still in flight land before the stages take the partial sums
         tc_fence_after();
     }
     const int q = warp & 3;   // TMEM lane quarter an epilogue warp may read
