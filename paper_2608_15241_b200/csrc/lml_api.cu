@@ -131,9 +131,10 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         g.shape = gemm_pick_shape(rows, t0->d_in, d_outs, P, dual, precise, t0->num_sms, t0->num_pairs, t0->split_bn, t0->split_s);
         // Small plain calls compute u inside the GEMM kernel (on the CTAs that own the fewest tiles, ahead of their tiles); otherwise a
         // launch goes first and the GEMM is its programmatic dependent.
-        g.fused = mode == kRowsSegments && !dual && P == 1 && T == rows && t0->fuse_shrink && t0->split_bn <= 0 &&
-                  gemm_can_fuse_shrink(T, t0->d_in, t0->d_out, G, b.rows.mode == kRowsSegments, t0->max_slots, t0->num_sms);
-        if (g.fused) g.shape = {256, 1, ((rows + kTileM - 1) / kTileM) * ((t0->d_out + 255) / 256), false};
+        GemmShape inside;
+        g.fused = mode == kRowsSegments && !dual && P == 1 && T == rows && t0->fuse_shrink &&
+                  gemm_fused_shape(&inside, T, t0->d_in, t0->d_out, G, b.rows.mode == kRowsSegments, t0->max_slots, t0->num_sms, t0->split_bn);
+        if (g.fused) g.shape = inside;
         if (g.fused) g.rows = b.rows;
         b.x_flag = g.x_flag = nullptr;
         if (mode != kRowsNone && !g.fused && bind_starts_gemm_early(rows, P, t0->num_sms)) {

@@ -18,7 +18,8 @@
 // then adds (second binding's delta - first binding's delta) on top, as further K-steps whose u
 // operands come from a second set of u blocks, and the epilogue reads the second output.  The producer slips
 // those stages into the middle of the next tile's k-blocks, by when the first read is long done.
-// Fused shrink (the plain call on a few row tiles): no launch goes ahead of this one.  Every CTA works out the slots of
+// Tall tiles (two row tiles to a CTA): see the kernel.
+// Fused shrink (the plain call on a few row tiles, on tall tiles): no launch goes ahead of this one.  Every CTA works out the slots of
 // all row tiles; the CTAs at the end of the grid, which own the fewest output tiles, first compute u = scale * x.A^T,
 // four chunks of a row tile to a pass, as 128 x 64 tcgen05 products, write the u blocks and raise the pass's flag in the
 // table's device memory; a producer waits for a tile's flags (a bounded wait) before it loads the tile's u blocks.  The
@@ -33,7 +34,6 @@
 // Every wait is bounded; on give-up the CTA sets LML_FLAG_TIMEOUT, drains and frees its TMEM.
 #include <cstdio>
 #include <cstdlib>
-#include <cstring>
 #include <mutex>
 
 #include "lml_gemm_common.cuh"
@@ -41,16 +41,20 @@
 namespace lml {
 
 constexpr int kGemmThreads = 192;
+constexpr int kGemmThreadsTall = 320;
+constexpr int kTallOverride = 512;        // the shape knob's width for tall tiles
 
 constexpr int kFuseTilesInKernel = 80;    // row tiles of a call whose shrink runs inside the kernel (the per-tile tables in shared memory)
 
-template <int BN> struct GemmCfg {
-    static constexpr int kXBytes = kBM * kBK * 2;             // a k-block of the row tile
-    static constexpr int kABytes = kXBytes;
+template <int BN, bool kTall = false> struct GemmCfg {
+    static constexpr int kRowTiles = kTall ? 2 : 1;
+    static constexpr int kXBytes = kBM * kBK * 2;             // a k-block of one row tile
+    static constexpr int kABytes = kRowTiles * kXBytes;
     static constexpr int kBBytes = BN * kBK * 2;
     static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kStages = BN == 256 ? 4 : (BN == 128 ? 6 : 8);
-    static constexpr int kEpiBytes = 4 * 2 * kEpiBufBytes;
+    static constexpr int kStages = kTall ? 3 : (BN == 256 ? 4 : (BN == 128 ? 6 : 8));
+    static constexpr int kEpiBufs = kTall ? 1 : 2;            // staging buffers of an epilogue warp
+    static constexpr int kEpiBytes = 4 * kRowTiles * kEpiBufs * kEpiBufBytes;
     static constexpr int kTmemCols = 2 * BN;
     static constexpr int kCtrlBytes = 256 + (kBindSegs + 1) * 4 + kBindSegs + 4 + 512 + kFuseTilesInKernel * 10 + 8 + kMaxChunks * 4;   // barriers; fused shrink: segment cache, shrink plan, per-tile masks and first passes; the first tile's chunks
     // The split-K kernel: no staging for the epilogue.  The ring also takes the partial sums that the CTAs exchange; where
@@ -80,6 +84,7 @@ constexpr uint32_t kStageAcc1 = 0x200u;     // the stage belongs to accumulator 
 
 static_assert(sizeof(GemmCtrl) <= 256, "control block");
 constexpr uint32_t kStageBoth = 0x2000u;    // split-K dual form: the stage's product goes into both bindings' accumulators
+constexpr uint32_t kStageMore0 = 0x8000u, kStageMore1 = 0x10000u;   // tall tiles, on the last k-block: LoRA stages follow for the first / second row tile
 constexpr uint32_t kStageOneB = 0x1000u;    // a LoRA chunk whose u is three blocks: a K-step each, with the same block of B
 constexpr uint32_t kStageChunks = 0x4000u;  // LoRA chunks (no-swizzle operands), a K-step each
 
@@ -133,12 +138,18 @@ __device__ __forceinline__ void prefetch_b(const GemmPart& pt, int n, int lane, 
     }
 }
 
-template <int BN>
-__global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const __grid_constant__ GemmParams p,
-                                                                           const __grid_constant__ SlotSnapshot snap)
+// kTall: a tile is two row tiles high (256 x 256).  Both accumulators belong to the tile, each row tile has four epilogue
+// warps of its own, and a stage holds two tiles of x beside one of W0: 64 KB for 1024 cycles of the tensor cores where the
+// single tile moves 48 KB for 512.  A CTA covers what a pair of CTAs does, so a call whose tall tiles take no more than a round leaves
+// SMs to bind_shrink, or to the shrink's passes, which only this form takes inside.  (No dual form.)
+template <int BN, bool kTall>
+__global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lora_gemm_sm100_kernel(
+    const __grid_constant__ GemmParams p, const __grid_constant__ SlotSnapshot snap)
 {
-    using Cfg = GemmCfg<BN>;
-    const bool dual = p.u2 != nullptr;
+    using Cfg = GemmCfg<BN, kTall>;
+    constexpr int kRowTiles = Cfg::kRowTiles;
+    constexpr int kThreads = kTall ? kGemmThreadsTall : kGemmThreads;
+    const bool dual = !kTall && p.u2 != nullptr, fused = kTall && p.fused;
     extern __shared__ uint8_t smem_raw[];
     // 128-byte swizzled tiles need 1024-byte alignment
     const uint32_t raw_addr = smem_u32(smem_raw);
@@ -157,6 +168,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int num_tiles = p.num_tiles;
     const int num_kb = (p.K + kBK - 1) / kBK;
+    const int num_mt = (p.num_m + kRowTiles - 1) / kRowTiles;   // tiles along the rows
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < Cfg::kStages; ++s) {
@@ -187,7 +199,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
     const uint64_t once = policy_evict_first();   // W0 passes through L2 once and must not push out what the next launches begin with
     if (p.x_flag) {   // early start: the first k-blocks' W0, then x
         const GemmPart& pt = p.part[part_of(p, (int)blockIdx.x)];
-        const int n0 = ((int)blockIdx.x - pt.tile0) / p.num_m;
+        const int n0 = ((int)blockIdx.x - pt.tile0) / num_mt;
         if (warp == 0) {
             if (elect_one()) {
                 for (int kb = 0; kb < min(Cfg::kStages, num_kb); ++kb) {
@@ -202,26 +214,26 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
         }
         __syncthreads();
     }
-    if (!p.lora || p.fused) {   // no launch of this call came before this one: wait for foreign work here
+    if (!p.lora || fused) {   // no launch of this call came before this one: wait for foreign work here
         grid_dependency_wait();
         grid_launch_dependents();
     }
     const bool by_segment = p.rows.mode == kRowsSegments;
-    if (p.fused) {
+    if (fused) {
         // Every CTA works out the slots of all row tiles from its own copy of the segment arrays (checked here: all reach
         // the same verdict) or from the slot per row.
         int bad_off = 0, bad_slot = 0;
         const uint32_t any_nonfinite = threadIdx.x < kMaxSlots ? ld_after_wait(p.part[0].nonfinite) : 0u;
-        for (int m = threadIdx.x; m < p.num_m; m += kGemmThreads) tile_mask[m] = 0ull;
+        for (int m = threadIdx.x; m < p.num_m; m += kThreads) tile_mask[m] = 0ull;
         if (by_segment) {
             const int G = p.rows.G;
-            for (int g = threadIdx.x; g <= G; g += kGemmThreads) seg_cache[g] = ld_after_wait(p.rows.seg_offsets + g);
-            for (int g = threadIdx.x; g < G; g += kGemmThreads) {
+            for (int g = threadIdx.x; g <= G; g += kThreads) seg_cache[g] = ld_after_wait(p.rows.seg_offsets + g);
+            for (int g = threadIdx.x; g < G; g += kThreads) {
                 const int s = ld_after_wait(p.rows.ids + g);
                 slot_cache[g] = (int8_t)(slot_rank(snap, s) > 0 ? s : (s == -1 ? -1 : -2));
             }
             __syncthreads();
-            for (int g = threadIdx.x; g < G; g += kGemmThreads) {
+            for (int g = threadIdx.x; g < G; g += kThreads) {
                 const int s0 = seg_cache[g], s1 = seg_cache[g + 1];
                 if (s1 < s0 || s0 < 0 || s1 > p.T) bad_off = 1;
                 if (slot_cache[g] == -2 && s1 > s0) bad_slot = 1;   // an empty segment may name anything
@@ -230,7 +242,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             bad_off = __syncthreads_or(bad_off);
             bad_slot = __syncthreads_or(bad_slot);
             if (!bad_off)
-                for (int g = threadIdx.x; g < G; g += kGemmThreads) {
+                for (int g = threadIdx.x; g < G; g += kThreads) {
                     const int s0 = seg_cache[g], s1 = seg_cache[g + 1], s = slot_cache[g];
                     if (s >= 0 && s1 > s0)
                         for (int m = s0 / kBM; m <= (s1 - 1) / kBM; ++m) atomicOr(&tile_mask[m], 1ull << s);
@@ -241,7 +253,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             }
         } else {
             __syncthreads();
-            for (int row = threadIdx.x; row < p.T; row += kGemmThreads) {
+            for (int row = threadIdx.x; row < p.T; row += kThreads) {
                 const int s = p.rows.rows[row];
                 if (slot_rank(snap, s) > 0) atomicOr(&tile_mask[row / kBM], 1ull << s);
             }
@@ -249,7 +261,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
         __syncthreads();
         const GemmPart& pt = p.part[0];
         if (any_nonfinite && ld_after_wait(pt.nonfinite + 1 + threadIdx.x) == nonfinite_tag(snap.gen[threadIdx.x])) atomicOr(&ctrl->nonfinite, 1ull << threadIdx.x);
-        for (int m = threadIdx.x; m < p.num_m; m += kGemmThreads)
+        for (int m = threadIdx.x; m < p.num_m; m += kThreads)
             shr_base[m + 1] = (uint16_t)((mask_chunks(pt, tile_mask[m]) + kShrChunks - 1) / kShrChunks);
         __syncthreads();
         if (threadIdx.x == 0) {
@@ -290,7 +302,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             bool lora = false, lora_known = !p.lora;
             // the CTA's first tile: its chunks are listed in shared memory
             const GemmPart* const list0_part = &p.part[part_of(p, (int)blockIdx.x)];
-            const int list0_m = ((int)blockIdx.x - list0_part->tile0) % p.num_m, list0_n = ((int)blockIdx.x - list0_part->tile0) / p.num_m;
+            const int list0_m = ((int)blockIdx.x - list0_part->tile0) % num_mt * kRowTiles, list0_n = ((int)blockIdx.x - list0_part->tile0) / num_mt;
             int stage = 0;
             uint32_t phase = 0;
             bool ok = true;
@@ -302,7 +314,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                 // Everything the launch before this one wrote (plans, u blocks) is first touched after the
                 // base k-blocks of the first tile are already in flight.
                 if (!lora_known) {
-                    if (!p.fused) {   // (warp 2 has waited for that launch, and has let the next one go)
+                    if (!fused) {   // (warp 2 has waited for that launch, and has let the next one go)
                         ok = mbar_wait(smem_u32(&ctrl->plan_full), 0u, abort);
                         grid_dependency_wait();
                     }
@@ -314,7 +326,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             // passes' flags when they are complete (bounded wait; the flags' writers run their passes first thing)
             int flag_seen_m = -1;
             auto wait_u = [&](int m) {
-                if (!p.fused || m == flag_seen_m) return;
+                if (!fused || m == flag_seen_m) return;
                 const int want = shr->epoch + 1;
                 const long long t0 = clock64();
                 for (int i = shr_base[m]; i < shr_base[m + 1]; ++i)
@@ -331,12 +343,12 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             auto emit_chunks = [&](const GemmPart& pt, const __nv_bfloat16* u, int m, int n, uint32_t who, uint32_t acc_flag, uint32_t flags_last) {
                 wait_u(m);
                 int index = -1, c = 0, at = 0;
-                const bool listed = !p.fused && &pt == list0_part && m == list0_m && n == list0_n;
-                unsigned long long mk = p.fused ? tile_mask[m] : 0ull;
+                const bool listed = !fused && &pt == list0_part && m == list0_m && n == list0_n;
+                unsigned long long mk = fused ? tile_mask[m] : 0ull;
                 const TilePlan* plan = pt.plan + m;
-                const int count = p.fused ? 0 : (listed ? ctrl->listed[0] : ld_after_wait(&plan->count));
+                const int count = fused ? 0 : (listed ? ctrl->listed[0] : ld_after_wait(&plan->count));
                 auto next = [&]() -> int {   // the next chunk, or -1; index is its number
-                    if (p.fused) {
+                    if (fused) {
                         if (!mk) return -1;
                         const int s = __ffsll((long long)mk) - 1, e = s | (c << 8);
                         if (++c == slot_chunks(pt, s)) { c = 0; mk &= mk - 1ull; }
@@ -374,13 +386,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             // whether any rows of tile m use a slot under the bindings `who`
             auto has_chunks = [&](const GemmPart& pt, int m, int n, uint32_t who) -> bool {
                 if (!lora) return false;
-                if (p.fused) return tile_mask[m] != 0ull;
+                if (fused) return tile_mask[m] != 0ull;
                 const bool listed = &pt == list0_part && m == list0_m && n == list0_n;
                 const TilePlan* plan = pt.plan + m;
                 const int count = listed ? ctrl->listed[0] : ld_after_wait(&plan->count);
-                if (dual) {
-                    for (int i = 0; i < count; ++i) if ((listed ? list0[i] : ld_after_wait(&plan->chunk[i])) & who) return true;
-                    return false;
+                if constexpr (!kTall) {   // (tall tiles have no dual form)
+                    if (dual) {
+                        for (int i = 0; i < count; ++i) if ((listed ? list0[i] : ld_after_wait(&plan->chunk[i])) & who) return true;
+                        return false;
+                    }
                 }
                 return count > 0;
             };
@@ -399,7 +413,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             };
             int ordinal = 0, prev_m = -1, prev_n = -1;
             // this CTA's shrink passes: a pass is num_kb stages of [x k-block | A k-blocks of its pieces]
-            for (int ps = 0; p.fused && ps < shr->npass && ok; ++ps, ++ordinal) {
+            for (int ps = 0; fused && ps < shr->npass && ok; ++ps, ++ordinal) {
                 const ShrPass& sp = shr->pass[ps];
                 const uint32_t acc_flag = (ordinal & 1) ? kStageAcc1 : 0u;
                 // (a k-block of a pass is at most 24 KB: two share a stage, so that as many bytes are on their way
@@ -434,9 +448,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                     if (!good) break;
                     const uint32_t a_dst = tiles_addr + st * Cfg::kStageBytes;
                     const uint32_t bar = smem_u32(&ctrl->full[st]);
+                    const bool second = kTall && row0 + kBM < p.T;
                     ctrl->stage_info[st] = 4u | acc_flag | (kb == num_kb - 1 ? flags_last : 0u);
-                    mbar_arrive_expect_tx(bar, (uint32_t)(p.x_bytes + (kb < have_w ? 0 : Cfg::kBBytes)));
+                    mbar_arrive_expect_tx(bar, (uint32_t)(p.x_bytes + (second ? p.x_bytes : 0) + (kb < have_w ? 0 : Cfg::kBBytes)));
                     tma_load_2d(a_dst, &p.x, bar, kb * kBK, row0);
+                    if (second) tma_load_2d(a_dst + Cfg::kXBytes, &p.x, bar, kb * kBK, row0 + kBM);
                     if (kb >= have_w) tma_load_2d_once(a_dst + Cfg::kABytes, w, bar, kb * kBK, col0, once);
                     if (++st == Cfg::kStages) { st = 0; ph ^= 1u; }
                 }
@@ -444,7 +460,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             };
             for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++ordinal) {
                 const GemmPart& pt = p.part[part_of(p, tile)];
-                const int m = (tile - pt.tile0) % p.num_m, n = (tile - pt.tile0) / p.num_m;
+                const int m = (tile - pt.tile0) % num_mt * kRowTiles, n = (tile - pt.tile0) / num_mt;
                 const int row0 = m * kBM;
                 const uint32_t acc_flag = (ordinal & 1) ? kStageAcc1 : 0u;
                 const int mid = min((num_kb + 1) / 2, num_kb - 1);
@@ -462,8 +478,15 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                 learn_lora();
                 if (!ok) break;
                 const bool chunks = has_chunks(pt, m, n, kChunkFirst);
-                base_blocks(&pt.w, row0, n * BN, num_kb - 1, num_kb, acc_flag, chunks ? 0u : kStageCommit, ordinal == 0 ? ahead : 0);
-                if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, acc_flag, kStageCommit);
+                if constexpr (kTall) {
+                    const bool chunks1 = m + 1 < p.num_m && has_chunks(pt, m + 1, n, kChunkFirst);
+                    base_blocks(&pt.w, row0, n * BN, num_kb - 1, num_kb, 0u, (chunks ? kStageMore0 : 0u) | (chunks1 ? kStageMore1 : 0u), ordinal == 0 ? ahead : 0);
+                    if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, 0u, kStageCommit);
+                    if (ok && chunks1) emit_chunks(pt, pt.u, m + 1, n, kChunkFirst, 0u, kStageCommit);
+                } else {
+                    base_blocks(&pt.w, row0, n * BN, num_kb - 1, num_kb, acc_flag, chunks ? 0u : kStageCommit, ordinal == 0 ? ahead : 0);
+                    if (ok && chunks) emit_chunks(pt, pt.u, m, n, kChunkFirst, acc_flag, kStageCommit);
+                }
                 prev_m = m; prev_n = n;
             }
             if (ok && dual && prev_m >= 0) {
@@ -501,7 +524,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                 if (++stage == Cfg::kStages) { stage = 0; phase ^= 1u; }
             };
             // `count` k-blocks without a side-band word: the loop that the tensor cores wait for; its state lives in registers
-            auto base_stages = [&](uint32_t d_tmem, int count, uint32_t& accumulate) {
+            // (tall tiles: both halves, the second's product right behind the first's)
+            auto base_stages = [&](uint32_t d_tmem, int count, uint32_t& accumulate, bool second) {
                 int st = stage;
                 uint32_t ph = phase, on = accumulate;
                 bool good = true;
@@ -514,6 +538,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
 #pragma unroll
                     for (int k = 0; k < 4; ++k)
                         umma_bf16(d_tmem, adesc0 + at + (uint64_t)(k * 2), bdesc0 + at + (uint64_t)(k * 2), idesc, k == 0 ? on : 1u);
+                    if (kTall && second) {
+#pragma unroll
+                        for (int k = 0; k < 4; ++k)
+                            umma_bf16(d_tmem + (uint32_t)BN, adesc0 + at + (uint64_t)(Cfg::kXBytes / 16 + k * 2), bdesc0 + at + (uint64_t)(k * 2), idesc, k == 0 ? on : 1u);
+                    }
                     on = 1u;
                     umma_commit(empty0 + 8u * (uint32_t)st);
                     if (++st == Cfg::kStages) { st = 0; ph ^= 1u; }
@@ -545,7 +574,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             };
             int ordinal = 0;
             // this CTA's shrink passes: 128 x (16 per chunk) products
-            for (int ps = 0; p.fused && ps < shr->npass && ok; ++ps, ++ordinal) {
+            for (int ps = 0; fused && ps < shr->npass && ok; ++ps, ++ordinal) {
                 const int acc = ordinal & 1;
                 uint32_t& eph = acc ? empty_ph1 : empty_ph0;
                 ok = mbar_wait(smem_u32(&ctrl->tmem_empty[acc]), eph ^ 1u, abort);
@@ -577,7 +606,29 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                 }
                 if (ok) umma_commit(smem_u32(&ctrl->tmem_full[acc]));
             }
-            for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x, ++ordinal) {
+            for (int tile = blockIdx.x; kTall && tile < num_tiles && ok; tile += gridDim.x) {
+                const GemmPart& pt = p.part[part_of(p, tile)];
+                const bool second = (tile - pt.tile0) % num_mt * kRowTiles + 1 < p.num_m;
+                ok = mbar_wait(smem_u32(&ctrl->tmem_empty[0]), empty_ph0 ^ 1u, abort);
+                if (ok && second) ok = mbar_wait(smem_u32(&ctrl->tmem_empty[1]), empty_ph1 ^ 1u, abort);
+                if (!ok) break;
+                empty_ph0 ^= 1u;
+                if (second) empty_ph1 ^= 1u;
+                tc_fence_after();
+                uint32_t accumulate = 0;
+                base_stages(tmem_base, num_kb - 1, accumulate, second);
+                if (!ok) break;
+                ok = mbar_wait(smem_u32(&ctrl->full[stage]), phase, abort);
+                if (!ok) break;
+                const uint32_t info = ctrl->stage_info[stage];
+                base_stages(tmem_base, 1, accumulate, second);
+                if (info & kStageMore0) flagged_stages(0, accumulate);
+                else umma_commit(smem_u32(&ctrl->tmem_full[0]));
+                if (!ok || !second) continue;
+                if (info & kStageMore1) flagged_stages(1, accumulate);
+                else umma_commit(smem_u32(&ctrl->tmem_full[1]));
+            }
+            for (int tile = blockIdx.x; !kTall && tile < num_tiles && ok; tile += gridDim.x, ++ordinal) {
                 const int acc = ordinal & 1;
                 uint32_t& eph = acc ? empty_ph1 : empty_ph0;
                 ok = mbar_wait(smem_u32(&ctrl->tmem_empty[acc]), eph ^ 1u, abort);
@@ -589,11 +640,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                 int from = 0;
                 if (dual && ordinal > 0) {
                     from = min((num_kb + 1) / 2, num_kb - 1);
-                    base_stages(d_tmem, from, accumulate);
+                    base_stages(d_tmem, from, accumulate, false);
                     if (ok) delta_stages(acc ^ 1);
                     if (!ok) break;
                 }
-                base_stages(d_tmem, num_kb - 1 - from, accumulate);
+                base_stages(d_tmem, num_kb - 1 - from, accumulate, false);
                 if (!ok) break;
                 flagged_stages(acc, accumulate);   // the last k-block and the tile's LoRA pieces
             }
@@ -603,7 +654,8 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
         // ------------------------------------------------------------------ epilogue warps
         const int q = warp & 3;                 // TMEM lane quarter this warp may read
         const int ew = warp - 2;
-        constexpr int kBufs = 2;                // staging buffers of a warp
+        const int group = ew >> 2;              // tall tiles: the row tile, and accumulator, of these four warps
+        constexpr int kBufs = Cfg::kEpiBufs;
         const bool one = elect_one();           // the lane that issues the stores
         const uint32_t buf_addr0 = epi_addr + (uint32_t)(ew * kBufs * kEpiBufBytes);
         uint8_t* buf_ptr0 = epi_ptr + ew * kBufs * kEpiBufBytes;
@@ -617,20 +669,21 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             return lo < p.rows.G ? slot_cache[lo] : -1;
         };
         bool ok = true;
-        if (p.lora && !p.fused && warp == 2) {   // nothing else to do yet: the first tile's chunks, as soon as they are known
+        if (p.lora && !fused && warp == 2) {   // nothing else to do yet: the first tile's chunks, as soon as they are known
             const GemmPart& pt = p.part[part_of(p, (int)blockIdx.x)];
             grid_dependency_wait();
             grid_launch_dependents();
-            const int n = list_chunks(pt.plan + ((int)blockIdx.x - pt.tile0) % p.num_m, kChunkFirst | kChunkSecond, 0, 1, lane, list0);
+            const int n = list_chunks(pt.plan + ((int)blockIdx.x - pt.tile0) % num_mt * kRowTiles, kChunkFirst | kChunkSecond, 0, 1, lane, list0);
             __syncwarp();
             if (lane == 0) { ctrl->listed[0] = n; mbar_arrive(smem_u32(&ctrl->plan_full)); }
-        } else if (p.lora && !p.fused) {
+        } else if (p.lora && !fused) {
             grid_dependency_wait();   // (this warp reads the plans too)
         }
         // this CTA's shrink passes: scale, zero the rows of other slots, round, write the u blocks; then the pass's
         // flag goes up (release: the four warps' stores are complete)
-        for (int ps = 0; p.fused && ps < shr->npass && ok; ++ps) {
+        for (int ps = 0; fused && ps < shr->npass && ok; ++ps) {
             const ShrPass& sp = shr->pass[ps];
+            if (kTall && (ps & 1) != group) { acc ^= 1; continue; }
             uint32_t& fph = acc ? full_ph1 : full_ph0;
             ok = mbar_wait_warp(smem_u32(&ctrl->tmem_full[acc]), fph, abort);
             if (!ok) break;
@@ -670,15 +723,19 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
             if (lane == 0) mbar_arrive(smem_u32(&ctrl->tmem_empty[acc]));
             fence_proxy_async_all();   // the blocks will be read by TMA
             __threadfence();
-            asm volatile("bar.sync 1, 128;" ::: "memory");   // the four epilogue warps
-            if (ew == 0 && lane == 0) st_release_gpu_s32(p.pass_flags + sp.flag, shr->epoch + 1);
+            asm volatile("bar.sync %0, 128;" ::"r"(1 + group) : "memory");   // the four epilogue warps of the accumulator
+            if ((ew & 3) == 0 && lane == 0) st_release_gpu_s32(p.pass_flags + sp.flag, shr->epoch + 1);
             acc ^= 1;
         }
         for (int tile = blockIdx.x; tile < num_tiles && ok; tile += gridDim.x) {
             const GemmPart& pt = p.part[part_of(p, tile)];
-            const int m = (tile - pt.tile0) % p.num_m, n = (tile - pt.tile0) / p.num_m;
+            const int m = (tile - pt.tile0) % num_mt * kRowTiles + group, n = (tile - pt.tile0) / num_mt;
+            if (kTall) {
+                acc = group;
+                if (m >= p.num_m) continue;
+            }
             const int row_base = m * kBM + q * 32;
-            const bool nonfinite = p.lora && (p.fused ? (tile_mask[m] & ctrl->nonfinite) != 0ull : ld_after_wait(pt.nonfinite) != 0u);
+            const bool nonfinite = p.lora && (fused ? (tile_mask[m] & ctrl->nonfinite) != 0ull : ld_after_wait(pt.nonfinite) != 0u);
             for (int pass = 0; pass < (dual ? 2 : 1) && ok; ++pass) {
                 uint32_t& fph = acc ? full_ph1 : full_ph0;
                 ok = mbar_wait_warp(smem_u32(&ctrl->tmem_full[acc]), fph, abort);
@@ -719,11 +776,11 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                     }
                     if (__builtin_expect(nonfinite, 0)) {
                         int s = -1, index = -1;
-                        if (p.fused && row_base + lane < p.T) {
+                        if (fused && row_base + lane < p.T) {
                             s = row_slot(row_base + lane);
                             if (s >= 0 && ((ctrl->nonfinite >> s) & 1ull)) index = mask_chunks(pt, tile_mask[m] & ((1ull << s) - 1ull));
                         }
-                        if (!p.fused || index >= 0)
+                        if (!fused || index >= 0)
                             add_nonfinite(pt, m, q * 32 + lane, pass, s, index, col0, pt.u, pass ? p.u2 : pt.u_mid, pt.u_lo, bp + lane * 64, (lane >> 1) & 3);
                     }
                     fence_proxy_async_smem();
@@ -733,7 +790,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
                         else tma_store_2d(&p.y2, ba, col0, row_base);
                         tma_store_commit();
                     }
-                    buf ^= 1;
+                    buf = kBufs == 2 ? buf ^ 1 : 0;
                 }
             }
             acc ^= 1;
@@ -745,7 +802,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_kernel(const 
     if (ctrl->abort) __nanosleep(50000);   // gave up: let copies still in flight land before the CTA goes away
     if (threadIdx.x == 0 && ctrl->abort) atomicOr(p.status, LML_FLAG_TIMEOUT);
     if (threadIdx.x == 0) leave_early_start(p.x_flag);
-    if (threadIdx.x == 0 && p.fused) {
+    if (threadIdx.x == 0 && fused) {
         // the last CTA to finish moves the table's epoch on: the flags of this call mean nothing to the next one
         __threadfence();
         if (atomicAdd(p.fuse_sync + 1, 1u) == gridDim.x - 1) {
@@ -1095,9 +1152,11 @@ cudaError_t gemm_sm100_init(int /*device*/)
     cudaError_t e = cudaFuncSetAttribute(lora_gemm_sm100_splitk_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          GemmCfg<64>::split_smem(GemmCfg<64>::kStages));
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<64>::kSmemBytes);
+    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<64, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<64>::kSmemBytes);
     if (e != cudaSuccess) return e;
-    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<256, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, GemmCfg<256, true>::kSmemBytes);
+    if (e != cudaSuccess) return e;
+    e = cudaFuncSetAttribute(lora_gemm_sm100_kernel<256, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          GemmCfg<256>::kSmemBytes);
     if (e != cudaSuccess) return e;
     e = cudaFuncSetAttribute(lora_gemm_sm100_splitk_kernel<256>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1106,12 +1165,12 @@ cudaError_t gemm_sm100_init(int /*device*/)
     e = cudaFuncSetAttribute(lora_gemm_sm100_splitk_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              GemmCfg<128>::split_smem(GemmCfg<128>::kStages));
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(lora_gemm_sm100_kernel<128>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    return cudaFuncSetAttribute(lora_gemm_sm100_kernel<128, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 GemmCfg<128>::kSmemBytes);
 }
 
 // The table's override (LML_GEMM_SPLIT, read once when the table is created; a test knob): "<bn>x<split>"
-// forces that shape, "<bn>p" CTA pairs of that width ("512x1": the same as 256p), 0 switches the split-K kernel off.  Returns false
+// forces that shape, "512x1" tall tiles, "<bn>p" CTA pairs of that width, 0 switches the split-K kernel off.  Returns false
 // when the variable is not set.  split_out: 0 for pairs.
 bool gemm_split_override(int* bn_out, int* split_out)
 {
@@ -1120,9 +1179,8 @@ bool gemm_split_override(int* bn_out, int* split_out)
     if (!e) return false;
     int bn = 0, sp = 0;
     char c = 0;
-    if (!strcmp(e, "512x1")) e = "256p";
     if (sscanf(e, "%d%c", &bn, &c) == 2 && c == 'p' && bn >= 64 && bn <= 256 && bn % 32 == 0) { *bn_out = bn; *split_out = 0; return true; }
-    if (sscanf(e, "%dx%d", &bn, &sp) == 2 && (bn == 64 || bn == 128 || bn == 256) && sp >= 1 && sp <= kSplitMaxS &&
+    if (sscanf(e, "%dx%d", &bn, &sp) == 2 && (bn == 64 || bn == 128 || bn == 256 || (bn == kTallOverride && sp == 1)) && sp >= 1 && sp <= kSplitMaxS &&
         (sp == 1 ? 0 : sp) * ((bn / 32 + sp - 1) / sp) * 16384 <= GemmCfg<128>::kStages * GemmCfg<128>::kStageBytes) {
         *bn_out = bn; *split_out = sp;
     } else {
@@ -1185,6 +1243,10 @@ GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, 
         if (pairs) return {split_bn, 1, 2 * pair_tiles_of(split_bn), true};
         split_bn = 0;
     }
+    if (split_bn == kTallOverride) {
+        if (!dual) return {256, 1, pair_tiles_of(256), false, true};
+        split_bn = 0;
+    }
     if (split_bn > 0) return {split_bn, split_s, tiles_of(split_bn) * split_s, false};
     float w0_bytes = 0.f;
     for (int p = 0; p < P; ++p) w0_bytes += 2.f * (float)d_in * (float)d_outs[p];
@@ -1241,24 +1303,27 @@ bool TmapCache::get_2d(CUtensorMap* out, const void* base, uint64_t inner, uint6
     return true;
 }
 
-// Whether the shrink runs inside the GEMM kernel: a plain call with little x (1.4 M elements), whole-K tiles of 256 columns in more than
-// one wave, so that CTAs have time to spare, few enough row tiles for the kernel's tables and few enough passes (a pass per row tile and
-// four chunks; every segment boundary inside a row tile can add one) that no CTA gets two.  One launch instead of two, in about the same
-// time on the device (us, inside / bind_shrink ahead: 700 x 520 -> 8192 19.6 / 20.2, 700 x 264 -> 8192 16.9 / 17.0, 1300 x 1032 -> 4104 26.6 /
-// 25.1, 2100 x 264 -> 5000 27.6 / 23.0); with more x bind_shrink, which shares K among the CTAs that the tiles leave, is done
-// sooner (2048 x 4096 -> 4096 61.4 / 49.9).
+// Whether the shrink runs inside the GEMM kernel: a plain call with little x (1.4 M elements) of more than one wave of 256-column tiles, as
+// tall tiles; few enough row tiles for the kernel's tables, and no more passes (a pass per row tile and four chunks; every segment
+// boundary inside a row tile can add one) than there are CTAs with a tile less than the others, or none: those compute u while the others'
+// tiles run.  us per call back to back, inside / the same tiles behind bind_shrink / single 256-column tiles with the shrink inside: 700 x
+// 520 -> 8192 18.4 / 15.2 / 26.0, 700 x 264 -> 8192 15.9 / 15.0 / 20.8, 1300 x 1032 -> 4104 24.9 / 21.0 / 32.7, 2048 x 520 -> 8192 33.1 / 28.8 /
+// 42.3.  One launch instead of two: what it is for is a call alone, issued from the host.
 // (What counts is T, G and the table's size, not what is registered: the two forms sum x.A^T in different orders, and a call's
 // bits must not change with adapters that it does not use.  Segments in order: a tile has one pass and one more for every segment
 // that begins in it, at most; rows in any order: reckoned with half of the widest adapter for every segment.)
-bool gemm_can_fuse_shrink(int T, int d_in, int d_out, int G, bool in_segment_order, int max_slots, int num_sms)
+bool gemm_fused_shape(GemmShape* shape, int T, int d_in, int d_out, int G, bool in_segment_order, int max_slots, int num_sms, int split_bn)
 {
     if (G <= 0 || (in_segment_order && G > kBindSegs)) return false;
-    const int num_m = (T + kBM - 1) / kBM, num_n = (d_out + 255) / 256;
-    if ((long long)T * d_in > 1400000ll || num_m > kFuseTilesInKernel || num_m * num_n <= num_sms) return false;
+    if (split_bn > 0 && split_bn != kTallOverride) return false;
+    const int num_m = (T + kBM - 1) / kBM, num_n = (d_out + 255) / 256, tall_tiles = (num_m + 1) / 2 * num_n;
+    if (num_m > kFuseTilesInKernel) return false;
+    if (split_bn != kTallOverride && ((long long)T * d_in > 1400000ll || num_m * num_n <= num_sms)) return false;
     static_assert(kShrChunks * kChunk == kRankPad, "a slot takes one pass at most");
     const int slots = G < max_slots ? G : max_slots;
     if (num_m * slots > kShrMaxPasses * num_sms && !in_segment_order) return false;   // (room for a CTA's passes)
-    return (in_segment_order ? num_m + G : num_m * ((slots + 1) / 2)) <= num_sms / 2;
+    *shape = {256, 1, tall_tiles, false, true};
+    return (in_segment_order ? num_m + G : num_m * ((slots + 1) / 2)) <= num_sms - (tall_tiles - 1) % num_sms - 1;
 }
 
 cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* caches, const GemmArgs& a, cudaStream_t stream)
@@ -1266,7 +1331,7 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
     const bool dual = a.u2 != nullptr;
     if (dual && (!a.lora || !a.y2 || a.P != 1 || a.fused)) return cudaErrorInvalidValue;
     const int bn = a.shape.bn, split = a.shape.split;
-    if (a.fused && (split != 1 || bn != 256 || a.P != 1)) return cudaErrorInvalidValue;
+    if ((a.fused && (!a.shape.tall || a.P != 1)) || (a.shape.tall && dual)) return cudaErrorInvalidValue;
     GemmParams p;
     p.a = tmap_A;
     p.num_m = (a.T + kBM - 1) / kBM;
@@ -1285,7 +1350,7 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
         } else {
             pt.y = pt.w;
         }
-        tiles += p.num_m * pt.num_n;
+        tiles += (a.shape.tall ? (p.num_m + 1) / 2 : p.num_m) * pt.num_n;
         columns += pt.num_n;
     }
     p.y2 = p.part[0].y;
@@ -1300,8 +1365,10 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     // with adapters the predecessor is the bind_shrink launch of this call, else the kernel waits at its top
-    pdl_config(cfg, attr, dim3((unsigned)(tiles < a.num_sms ? tiles : a.num_sms)), dim3(kGemmThreads),
-               bn == 256 ? GemmCfg<256>::kSmemBytes : (bn == 128 ? GemmCfg<128>::kSmemBytes : GemmCfg<64>::kSmemBytes), stream);
+    // (tall tiles with the shrink inside: the SMs without a tile take its passes)
+    const bool tall = a.shape.tall;
+    pdl_config(cfg, attr, dim3((unsigned)(tiles < a.num_sms && !(tall && a.fused) ? tiles : a.num_sms)), dim3(tall ? kGemmThreadsTall : kGemmThreads),
+               tall ? GemmCfg<256, true>::kSmemBytes : bn == 256 ? GemmCfg<256>::kSmemBytes : (bn == 128 ? GemmCfg<128>::kSmemBytes : GemmCfg<64>::kSmemBytes), stream);
     p.stages = 0;
     if (split > 1) {
         p.stages = a.share_sm && gemm_exchange_bytes(bn, split) <= gemm_stages_short(bn) * gemm_stage_bytes(bn) ? gemm_stages_short(bn) : gemm_stages(bn);
@@ -1316,9 +1383,10 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
         if (bn == 64) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_splitk_kernel<64>, p);
         return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_splitk_kernel<128>, p);
     }
-    if (bn == 256) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<256>, p, *a.proj[0].snap);
-    if (bn == 64) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<64>, p, *a.proj[0].snap);
-    return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<128>, p, *a.proj[0].snap);
+    if (tall) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<256, true>, p, *a.proj[0].snap);
+    if (bn == 256) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<256, false>, p, *a.proj[0].snap);
+    if (bn == 64) return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<64, false>, p, *a.proj[0].snap);
+    return cudaLaunchKernelEx(&cfg, lora_gemm_sm100_kernel<128, false>, p, *a.proj[0].snap);
 }
 
 }  // namespace lml

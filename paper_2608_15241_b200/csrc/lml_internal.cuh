@@ -24,7 +24,7 @@ constexpr int kSlabTiles = 512;       // row tiles worked on at a time: longer c
 constexpr int kBindSegs = 256;        // segments that the kernels look up in shared memory; more are turned into a slot per row first
 constexpr int kDecodeMaxT = LML_DECODE_MAX_TOKENS;
 constexpr int kMaxAdapterIds = LML_MAX_ADAPTER_IDS;   // adapter ids that can be resolved on the device
-constexpr int kFuseMaxPasses = 4096;   // flags of the fused shrink, one a pass; a call has a few hundred passes at most (gemm_can_fuse_shrink)
+constexpr int kFuseMaxPasses = 4096;   // flags of the fused shrink, one a pass; a call has a few hundred passes at most (gemm_fused_shape)
 
 // Per-call snapshot of the slot table, passed by value as a kernel parameter so that a later
 // register / retire cannot change a call that is already enqueued.
@@ -179,8 +179,8 @@ struct GemmProj {
     int cap;
 };
 // What the library takes for a call: width of an output tile and CTAs that share one (1: whole-K tiles), CTAs in all, and
-// whether a whole-K tile is the work of a pair of CTAs, two row tiles high.
-struct GemmShape { int bn, split, ctas; bool pair; };
+// whether a whole-K tile is two row tiles high: the work of a pair of CTAs, or of one (tall).
+struct GemmShape { int bn, split, ctas; bool pair, tall = false; };
 struct GemmArgs {
     const void* x;
     int T, d_in, P;
@@ -202,8 +202,8 @@ struct GemmArgs {
 // split_bn, split_s: the table's override (-1 = the library chooses, 0 = whole-K tiles, else the forced shape); precise: some projection's
 // u is three bf16 values
 GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, bool precise, int num_sms, int num_pairs, int split_bn, int split_s);
-// whether the shrink of a plain call of this size runs inside the GEMM kernel, on whole-K tiles of 256 columns
-bool gemm_can_fuse_shrink(int T, int d_in, int d_out, int G, bool in_segment_order, int max_slots, int num_sms);
+// whether the shrink of a plain call of this size runs inside the GEMM kernel, and on which shape
+bool gemm_fused_shape(GemmShape* shape, int T, int d_in, int d_out, int G, bool in_segment_order, int max_slots, int num_sms, int split_bn);
 // Tensor maps of caller buffers, kept per table and found again by (pointer, shape, box).
 struct TmapCache {
     static constexpr int kEntries = 32;
