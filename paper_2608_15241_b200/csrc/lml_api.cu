@@ -139,7 +139,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         b.x_flag = g.x_flag = nullptr;
         if (mode != kRowsNone && !g.fused && bind_starts_gemm_early(rows, P, t0->num_sms)) {
             b.x_flag = g.x_flag = t0->arena.status + 8;
-            b.early = bind_early(rows, t0->d_in, P, most_chunks, g.shape.ctas, t0->num_sms);
+            b.early = bind_early(rows, t0->d_in, P, most_chunks, g.shape.ctas, g.shape.split > 1, t0->num_sms);
             g.share_sm = b.early.share_sm;
             std::lock_guard<std::mutex> lock(t0->mu);
             if (++t0->next_call == 0u) ++t0->next_call;

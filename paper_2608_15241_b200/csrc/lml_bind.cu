@@ -369,7 +369,8 @@ __global__ void __launch_bounds__(kBindThreads) bind_shrink_kernel(const __grid_
     }
 }
 
-constexpr int kBindRingSmall = 72 * 1024, kBindRingLarge = 192 * 1024;   // (the partial sums, 8 KB per chunk of a pass, fit either)
+// (the partial sums, 8 KB per chunk of a pass, fit each)
+constexpr int kBindRingShared = 72 * 1024, kBindRingTwo = 96 * 1024, kBindRingLarge = 192 * 1024;
 static int bind_smem_bytes(int ring) { return 1024 + ring + (int)sizeof(BindCtrl); }
 
 // CTAs that share K.  It follows from the rows alone: a projection's u has the same bits in a call of its own and beside others.
@@ -381,14 +382,20 @@ static int bind_cluster(int T, int d_in, int num_sms)
     return S;
 }
 bool bind_starts_gemm_early(int T, int P, int num_sms) { return (T + kTileM - 1) / kTileM * P * 8 <= num_sms; }
-// Few rows: a pass takes eight chunks, or sixteen where only that leaves the GEMM's CTAs (gemm_ctas) SMs of their own.  Layer passes,
-// us, with 4 / 8 / 16: 40 tokens, 16 chunks 169 / 162 / 149, 128 tokens, 18 chunks 145 / 126 / 133.
-BindEarly bind_early(int T, int d_in, int P, int cap, int gemm_ctas, int num_sms)
+// Few rows: a pass takes eight chunks (or all there are), or sixteen where only that leaves the GEMM's CTAs (gemm_ctas) SMs of their own.
+// Layer passes, us, with 4 / 8 / 16: 40 tokens, 16 chunks 169 / 162 / 149, 128 tokens, 18 chunks 145 / 126 / 133.  Where the two do not
+// find SMs of their own, bind_shrink shares SMs with the split-K GEMM, each with a short ring; no other GEMM fits beside it, so two
+// of its own CTAs share an SM, with three stages of eight chunks, and leave the other SMs to the GEMM.  us per call, 16 adapters of rank 8
+// ... 64, with two stages of eight (three to an SM) / three (two) / six (one): 160 x 11008 -> 4096 63.5 / 59.3 / 57.5, 500 x 4096 -> 4096 37.4 / 36.0 /
+// 36.0, but with four adapters of rank 16 500 x 4096 -> 4096 20.9 / 20.9 / 26.9, 1000 x 2048 -> 2048 15.8 / 15.8 / 20.2.
+BindEarly bind_early(int T, int d_in, int P, int cap, int gemm_ctas, bool split, int num_sms)
 {
     const int clusters = (T + kTileM - 1) / kTileM * P * bind_cluster(T, d_in, num_sms);
-    for (int group = 8; group <= 16; group += 8)
-        if (gemm_ctas + clusters * ((cap + group - 1) / group) <= num_sms) return {group, false};
-    return {8, true};
+    for (int most = 8; most <= 16; most += 8) {
+        const int group = cap < most ? cap : most;
+        if (gemm_ctas + clusters * ((cap + group - 1) / group) <= num_sms) return {group, kBindRingLarge, false};
+    }
+    return {cap < 8 ? cap : 8, split ? kBindRingShared : kBindRingTwo, split};
 }
 
 cudaError_t launch_bind_shrink(const BindArgs& a, const CUtensorMap* const* tmap_A, TmapCache* cache, int num_sms, cudaStream_t stream)
@@ -404,14 +411,12 @@ cudaError_t launch_bind_shrink(const BindArgs& a, const CUtensorMap* const* tmap
     }
     const int num_m = b.num_m = (a.T + kTileM - 1) / kTileM;
     const int tiles = num_m * a.P, S = bind_cluster(a.T, a.d_in, num_sms);
-    // Few rows: see bind_early; in a ring small enough to share an SM with the split-K GEMM, whose base product runs meanwhile,
-    // where the two do not find SMs of their own.  Many rows: x is read
-    // once for up to 16 chunks, one wave of CTAs.
+    // Few rows: see bind_early.  Many rows: x is read once for up to 16 chunks, one wave of CTAs.
     int groups;
     b.early = a.x_flag ? 1 : 0;
     if (b.early) {
         b.group = a.early.group;
-        b.ring_bytes = a.early.share_sm ? kBindRingSmall : kBindRingLarge;
+        b.ring_bytes = a.early.ring_bytes;
         groups = (cap + b.group - 1) / b.group;
     } else {
         b.group = 16; b.ring_bytes = kBindRingLarge;
@@ -419,7 +424,7 @@ cudaError_t launch_bind_shrink(const BindArgs& a, const CUtensorMap* const* tmap
         const int most = num_sms / (tiles * S);   // (one wave: what is over goes in turn)
         groups = groups < most ? groups : (most < 1 ? 1 : most);
     }
-    b.tmem_cols = b.group * kChunk;
+    for (b.tmem_cols = 32; b.tmem_cols < b.group * kChunk;) b.tmem_cols *= 2;
     cudaLaunchConfig_t cfg = {};
     cudaLaunchAttribute attr[2];
     pdl_config(cfg, attr, dim3((unsigned)S, (unsigned)groups, (unsigned)tiles), dim3(kBindThreads), (size_t)bind_smem_bytes(b.ring_bytes), stream);

@@ -143,8 +143,8 @@ struct BindPart {
     int cap;
     int pad;
 };
-// Early start: chunks of a pass, and whether the GEMM's CTAs and this launch's have to fit an SM together.
-struct BindEarly { int group = 8; bool share_sm = false; };
+// Early start: chunks of a pass, bytes of the ring, and whether the GEMM's CTAs and this launch's have to fit an SM together.
+struct BindEarly { int group = 8, ring_bytes = 0; bool share_sm = false; };
 struct BindArgs {
     const void* x;
     int T, d_in, P;
@@ -219,7 +219,7 @@ bool gemm_split_override(int* bn_out, int* split_out);
 // bind_starts_gemm_early: for calls of few rows the GEMM may start while the work before the call is still running; it then
 // reads nothing but W0 until bind_shrink, which waits for that work, has said that x may be read.
 bool bind_starts_gemm_early(int T, int P, int num_sms);
-BindEarly bind_early(int T, int d_in, int P, int cap, int gemm_ctas, int num_sms);   // ... beside a GEMM of so many CTAs
+BindEarly bind_early(int T, int d_in, int P, int cap, int gemm_ctas, bool split, int num_sms);   // ... beside a GEMM of so many CTAs, split-K or not
 // tmap_A[p]: the map of projection p's packed A arena ([max_slots][64][d_in], box 64 x 16 x 1)
 cudaError_t launch_bind_shrink(const BindArgs& a, const CUtensorMap* const* tmap_A, TmapCache* cache, int num_sms, cudaStream_t stream);
 // tmap_A: the same of the (first) table, for the fused shrink; caches[p]: the tensor maps of the buffers of projection p.
