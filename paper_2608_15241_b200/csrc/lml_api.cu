@@ -75,6 +75,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
     const int num_m = (T + kTileM - 1) / kTileM;
     const bool dual = y2 != nullptr;
     bool precise = false;
+    int slots = 0;
     SlotSnapshot snap[LML_MAX_PROJECTIONS];
     BindArgs b;
     GemmArgs g;
@@ -91,6 +92,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         b.snap[p] = snap[p];
         caches[p] = &c.t->tmaps;
         precise = precise || c.precise;
+        slots = c.t->max_slots > slots ? c.t->max_slots : slots;
         tmaps_A[p] = &c.t->tmap_A;
         d_outs[p] = c.t->d_out;
         int live = 0;   // chunks of all live slots: no tile needs more
@@ -128,7 +130,7 @@ cudaError_t run_gemm_path(const GemmCall* calls, int P, const void* x, int T, Ro
         }
         if (r0 > 0 && b.rows.rows) b.rows.rows += kSlabTiles * kTileM;
         if (r0 > 0 && b.rows.rows2) b.rows.rows2 += kSlabTiles * kTileM;
-        g.shape = gemm_pick_shape(rows, t0->d_in, d_outs, P, dual, precise, t0->num_sms, t0->num_pairs, t0->split_bn, t0->split_s);
+        g.shape = gemm_pick_shape(rows, t0->d_in, d_outs, P, dual, precise, g.lora ? slots : 0, t0->num_sms, t0->num_pairs, t0->split_bn, t0->split_s);
         // Small plain calls compute u inside the GEMM kernel (on the CTAs that own the fewest tiles, ahead of their tiles); otherwise a
         // launch goes first and the GEMM is its programmatic dependent.
         GemmShape inside;

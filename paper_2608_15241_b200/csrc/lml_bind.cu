@@ -381,6 +381,12 @@ static int bind_cluster(int T, int d_in, int num_sms)
     while (S > 1 && num_kb < S) S >>= 1;
     return S;
 }
+// A chunk per slot, 16 chunks at most, whatever the table holds.
+int bind_ctas_reckoned(int T, int d_in, int P, int slots, int num_sms)
+{
+    const int clusters = (T + kTileM - 1) / kTileM * P * bind_cluster(T, d_in, num_sms);
+    return clusters * (slots > 8 && bind_starts_gemm_early(T, P, num_sms) ? 2 : 1);
+}
 bool bind_starts_gemm_early(int T, int P, int num_sms) { return (T + kTileM - 1) / kTileM * P * 8 <= num_sms; }
 // Few rows: a pass takes eight chunks (or all there are), or sixteen where only that leaves the GEMM's CTAs (gemm_ctas) SMs of their own.
 // Layer passes, us, with 4 / 8 / 16: 40 tokens, 16 chunks 169 / 162 / 149, 128 tokens, 18 chunks 145 / 126 / 133.  Where the two do not

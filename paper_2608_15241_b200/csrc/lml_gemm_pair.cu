@@ -441,6 +441,12 @@ __global__ void __launch_bounds__(kPairThreads, 1) lora_gemm_pair_kernel(const _
     }
 }
 
+int gemm_pair_stages(int bn)
+{
+    const int stages = kPairRingBytes / (kPairXBytes + bn / 2 * kBK * 2);
+    return stages < kPairMaxStages ? stages : kPairMaxStages;
+}
+
 // pairs: the pairs of CTAs that are resident at once; 0, and no call takes pairs, where the runtime does not say.
 cudaError_t gemm_pair_init(int num_sms, int* pairs)
 {
@@ -498,7 +504,7 @@ cudaError_t launch_gemm_pair(TmapCache* const* caches, const GemmArgs& a, cudaSt
     const int panels = (int)((uint64_t)p.num_mp * 2 * kBM * xs / (48u << 20)) + 1;
     p.panel = (p.num_mp + panels - 1) / panels;
     p.stage_bytes = kPairXBytes + bn / 2 * kBK * 2;
-    p.stages = kPairRingBytes / p.stage_bytes < kPairMaxStages ? kPairRingBytes / p.stage_bytes : kPairMaxStages;
+    p.stages = gemm_pair_stages(bn);
     p.lora = a.lora ? 1 : 0;
     p.x_flag = a.x_flag; p.call_id = a.call_id;
     const int pairs = tiles < a.num_pairs ? tiles : a.num_pairs;

@@ -1203,7 +1203,12 @@ static int gemm_exchange_bytes(int bn, int split) { return split * ((bn / 32 + s
 // 11008 -> 4096; splits there 128x2 34.7, 128x3 27.0, 256x4 32.5, 256x6 30.0; pairs of 256 / 160 / 128 columns 26.8 / 21.4 / 21.3 at 512 x
 // 4096 -> 4096, and where the tiles take several rounds, at the power that the tensor cores may draw, 96.6 at 1300 x 4096 -> 11008 (256
 // columns, four rounds), 109.3 at 1600 (224 columns, five; with 256 columns 115.9), against 111 and 128.6 for single tiles of 128.
-GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, bool precise, int num_sms, int num_pairs, int split_bn, int split_s)
+// A pair's k-block also takes a share of a trip to memory, 1.4 us over the stages of its ring, which is what narrow pairs are bound by (256 x
+// 11008 -> 4096: 64p 39.7, 64x1 32.8).  And 2 us where the tiles' CTAs and bind_shrink's do not find SMs of their own, so that some start when
+// bind_shrink leaves (3000 x 3072 -> 1024: 192p, 144 CTAs, 29.7; 256x1, 96 CTAs, 21.1).  With these two, over 14 layers from 264 -> 8192 to
+// 5120 -> 13824, 64 ... 4096 tokens, 4 and 16 adapters, the choice is 1.046 times the best of all shapes in the mean, 1.067 without.
+// slots: of the largest table, 0 without adapters; what the tables hold must not choose between sums of different order.
+GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, bool precise, int slots, int num_sms, int num_pairs, int split_bn, int split_s)
 {
     static int max_clusters[3][kSplitMaxS + 1];   // for 64, 128 and 256 columns
     static std::once_flag probed;
@@ -1253,8 +1258,10 @@ GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, 
     const float stream_us = 7.5f + w0_bytes / 5.45e6f;   // no shape reads W0 faster
     GemmShape best = {256, 1, tiles_of(256), false};
     float best_us = 1e30f;
+    const int bind_ctas = slots > 0 ? bind_ctas_reckoned(T, d_in, P, slots, num_sms) : 0;
     auto consider = [&](const GemmShape& shape, float us) {
         us = (us > stream_us ? us : stream_us) + 0.1f * us;
+        if (bind_ctas > 0 && shape.ctas + bind_ctas > num_sms) us += 2.f;
         if (us < best_us * 0.999f) { best_us = us; best = shape; }
     };
     for (int w = 2; w >= 0; --w) {
@@ -1271,10 +1278,13 @@ GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, 
                                                     (beside ? 0.f : (S == 2 ? 1.5f : (S == 3 ? 4.f : 6.f))));
         }
     }
+    // Whether K is split is settled among the single tiles, which a dual call has too: its first output has the bits of the plain call.  Whole-K
+    // tiles of every form add up in one order.
     if (pairs && num_m > 1 && best.split == 1) {   // CTA pairs (lml_gemm_pair.cu), tiles of 256 rows
         for (int bn = 256; bn >= 64; bn -= 32) {
             const int tiles = pair_tiles_of(bn), waves = (tiles + num_pairs - 1) / num_pairs;
-            consider({bn, 1, 2 * tiles, true}, 10.f + (float)(waves * num_kb) * (waves > 1 ? 0.12f + 0.00082f * (float)bn : 0.035f + 0.00097f * (float)bn));
+            const float trip = 1.4f / (float)gemm_pair_stages(bn), one = 0.035f + 0.00097f * (float)bn;
+            consider({bn, 1, 2 * tiles, true}, 10.f + (float)(waves * num_kb) * (waves > 1 ? 0.12f + 0.00082f * (float)bn : (one > trip ? one : trip)));
         }
     }
     return best;

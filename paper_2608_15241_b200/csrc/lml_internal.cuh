@@ -200,8 +200,8 @@ struct GemmArgs {
     int num_pairs;                // pairs of the pair kernel's CTAs that are resident at once
 };
 // split_bn, split_s: the table's override (-1 = the library chooses, 0 = whole-K tiles, else the forced shape); precise: some projection's
-// u is three bf16 values
-GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, bool precise, int num_sms, int num_pairs, int split_bn, int split_s);
+// u is three bf16 values; slots: of the largest table, 0 without adapters
+GemmShape gemm_pick_shape(int T, int d_in, const int* d_outs, int P, bool dual, bool precise, int slots, int num_sms, int num_pairs, int split_bn, int split_s);
 // whether the shrink of a plain call of this size runs inside the GEMM kernel, and on which shape
 bool gemm_fused_shape(GemmShape* shape, int T, int d_in, int d_out, int G, bool in_segment_order, int max_slots, int num_sms, int split_bn);
 // Tensor maps of caller buffers, kept per table and found again by (pointer, shape, box).
@@ -219,6 +219,7 @@ bool gemm_split_override(int* bn_out, int* split_out);
 // bind_starts_gemm_early: for calls of few rows the GEMM may start while the work before the call is still running; it then
 // reads nothing but W0 until bind_shrink, which waits for that work, has said that x may be read.
 bool bind_starts_gemm_early(int T, int P, int num_sms);
+int bind_ctas_reckoned(int T, int d_in, int P, int slots, int num_sms);   // what bind_shrink is likely to launch
 BindEarly bind_early(int T, int d_in, int P, int cap, int gemm_ctas, bool split, int num_sms);   // ... beside a GEMM of so many CTAs, split-K or not
 // tmap_A[p]: the map of projection p's packed A arena ([max_slots][64][d_in], box 64 x 16 x 1)
 cudaError_t launch_bind_shrink(const BindArgs& a, const CUtensorMap* const* tmap_A, TmapCache* cache, int num_sms, cudaStream_t stream);
@@ -228,6 +229,7 @@ cudaError_t launch_gemm_sm100(const CUtensorMap& tmap_A, TmapCache* const* cache
 cudaError_t launch_gemm_pair(TmapCache* const* caches, const GemmArgs& a, cudaStream_t stream);   // shapes of CTA pairs
 cudaError_t gemm_sm100_init(int device);
 cudaError_t gemm_pair_init(int num_sms, int* pairs);
+int gemm_pair_stages(int bn);
 cudaError_t shrink_init();   // these set the dynamic shared memory attributes of their kernels
 bool encode_tmap_2d(CUtensorMap* m, const void* base, uint64_t inner, uint64_t outer,
                     uint64_t row_stride_bytes, uint32_t box_inner, uint32_t box_outer, bool swizzle = true);

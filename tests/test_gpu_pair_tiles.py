@@ -97,3 +97,29 @@ def test_u_of_three_values_does_not_take_pairs(T, monkeypatch):
         assert np.array_equal(out[0][p], out[1][p]), p
         ref, _ = oracle.forward(x, W[p], ents[p], np.arange(T + 1, dtype=np.int32), tok)
         assert oracle.compare(out[1][p], ref)["ok"], p
+
+
+def test_whole_k_tiles_of_every_form_agree_bit_for_bit(monkeypatch):
+    """Which whole-K tiles a call takes follows from estimates; its bits do not: single tiles, tall tiles and pairs of every width add up in
+    one order.  So does a dual call's first output, although a dual call takes no pairs."""
+    import torch
+    from gpu_util import to_bits
+    w = wl.ragged(T=700, d_in=1032, d_out=1000, ranks=(4, 16, 1, 33, 64))
+    monkeypatch.setenv("LML_FUSE_SHRINK", "0")   # (inside the GEMM kernel u is summed in another order)
+    ys = {}
+    for shape in ("64x1", "128x1", "256x1", "512x1", "64p", "160p", "256p", None):
+        if shape:
+            monkeypatch.setenv("LML_GEMM_SPLIT", shape)
+        else:
+            monkeypatch.delenv("LML_GEMM_SPLIT")
+        site = Site(w)
+        ys[shape], flags = site.run()
+        assert flags == 0
+        if shape in ("256x1", None):
+            so, ids = torch.from_numpy(w.seg_offsets).cuda(), torch.from_numpy(site.slot_ids()).cuda()
+            ys["dual", shape] = to_bits(site.table.lora_mixed_linear_dual(site.x, site.W0, so, ids, ids.flip(0).contiguous())[0])
+        site.close()
+    ref, _ = oracle.forward_workload(w)
+    assert oracle.compare(ys["64x1"], ref)["ok"]
+    for shape, y in ys.items():
+        assert np.array_equal(y, ys["64x1"]), shape
