@@ -11,7 +11,7 @@ __device__ __forceinline__ void bulk_copy_g2s(uint32_t dst, const void* src, uin
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];"
                  ::"r"(dst), "l"(src), "r"(bytes), "r"(bar) : "memory");
 }
-// Of what is read once: it leaves L2 first.
+// Of what leaves L2 first (policy_evict_first).
 __device__ __forceinline__ void bulk_copy_g2s_once(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar, uint64_t policy)
 {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1], %2, [%3], %4;"
@@ -27,10 +27,6 @@ __device__ __forceinline__ void ldg_nc_v8(const void* p, uint4& a, uint4& b)   /
 {
     asm volatile("ld.global.nc.v8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
                  : "=r"(a.x), "=r"(a.y), "=r"(a.z), "=r"(a.w), "=r"(b.x), "=r"(b.y), "=r"(b.z), "=r"(b.w) : "l"(p));
-}
-__device__ __forceinline__ void red_release_gpu_add(unsigned* p, unsigned v)
-{
-    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 __device__ __forceinline__ void red_relaxed_gpu_add(unsigned* p, unsigned v)
 {
@@ -55,12 +51,6 @@ __device__ __forceinline__ void st_relaxed_gpu_b64(unsigned long long* p, unsign
 __device__ __forceinline__ void ld_relaxed_gpu_v2_b64(const unsigned long long* p, unsigned long long& a, unsigned long long& b)   // 16-byte aligned
 {
     asm volatile("ld.relaxed.gpu.global.v2.b64 {%0, %1}, [%2];" : "=l"(a), "=l"(b) : "l"(p) : "memory");
-}
-__device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned* p)
-{
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
 }
 __device__ __forceinline__ void bulk_prefetch_l2(const void* src, uint32_t bytes)   // 16-byte aligned, multiple of 16
 {

@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(kTall ? kGemmThreadsTall : kGemmThreads, 1) lo
     tc_fence_after();
     const uint32_t tmem_base = ctrl->tmem_base;
     volatile int* abort = &ctrl->abort;
-    const uint64_t once = policy_evict_first();   // W0 passes through L2 once and must not push out what the next launches begin with
+    const uint64_t once = policy_evict_first();   // (see there)
     if (p.x_flag) {   // early start: the first k-blocks' W0, then x
         const GemmPart& pt = p.part[part_of(p, (int)blockIdx.x)];
         const int n0 = ((int)blockIdx.x - pt.tile0) / num_mt;
@@ -875,7 +875,7 @@ __global__ void __launch_bounds__(kGemmThreads, 1) lora_gemm_sm100_splitk_kernel
     tc_fence_after();
     const uint32_t tmem_base = ctrl->tmem_base;
     volatile int* abort = &ctrl->abort;
-    const uint64_t once = policy_evict_first();   // W0 passes through L2 once and must not push out what the next launches begin with
+    const uint64_t once = policy_evict_first();   // (see there)
     if (p.x_flag) {   // early start: the first k-blocks' W0, then x
         if (warp == 0) {
             if (elect_one()) {

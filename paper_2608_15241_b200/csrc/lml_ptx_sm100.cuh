@@ -63,7 +63,7 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
 
 // One lane of a converged warp, for roles that a single thread plays.  What that thread issues (MMAs, commits, bulk copies) takes its
 // operands from uniform registers; behind elect.sync the compiler knows that one lane is active, behind lane == 0 it does not and loops
-// over the lanes for every such instruction: 40 cycles per MMA, 490 per stage of four MMAs and their barriers against 330.
+// over the lanes for every such instruction: 310 cycles for the four MMAs of a stage and 58 for its commit, against 153 for all five.
 __device__ __forceinline__ bool elect_one()
 {
     uint32_t p;
@@ -143,6 +143,12 @@ __device__ __forceinline__ void st_release_gpu_s32(int* p, int v)
 }
 
 // ---- TMA ------------------------------------------------------------------------------------------
+// For W0 in the decode kernel and the single-tile GEMMs: a pass over a model's weights must not push out of L2 what the next launches begin
+// with (code, parameters, ids, x, the adapters' rows).  It holds as well where several CTAs read a line, the halves of a dual call, blocks of
+// 16 tokens, row tiles: they walk W0 together and find it.  us per call, weights of 1.5 GB in turn, lines of normal priority / evict-first: 4096 ->
+// 4096 with 16 adapters 8 tokens 8.9 / 8.6, 48 tokens (three blocks) 26.3 / 25.4; dual 4096 -> 11008 300 tokens 38 / 35, 2048 tokens 164 / 156 (but
+// 144 against 148 without any hint); 84 MB of weights beside 40 MB of other traffic a pass, 8 tokens 8.6 / 8.2.  Weights that fit L2 with nothing
+// beside them lose a little: 68 MB of 520 -> 8192 in turn 8.2 / 8.45.
 __device__ __forceinline__ uint64_t policy_evict_first()
 {
     uint64_t policy;
@@ -159,7 +165,7 @@ __device__ __forceinline__ void tma_load_2d(uint32_t dst, const CUtensorMap* m, 
         "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1) : "memory");
 }
-// ... of what is read once: it leaves L2 first
+// ... of what leaves L2 first (policy_evict_first)
 __device__ __forceinline__ void tma_load_2d_once(uint32_t dst, const CUtensorMap* m, uint32_t bar, int c0, int c1, uint64_t policy)
 {
     asm volatile(
@@ -182,12 +188,6 @@ __device__ __forceinline__ void bulk_load(uint32_t dst, const void* src, uint32_
 __device__ __forceinline__ void bulk_prefetch_to_l2(const void* src, uint32_t bytes)
 {
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
-}
-// Pull a tile into L2 only (no shared-memory destination, no barrier).
-__device__ __forceinline__ void tma_prefetch_2d(const CUtensorMap* m, int c0, int c1)
-{
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];"
-                 ::"l"(reinterpret_cast<uint64_t>(m)), "r"(c0), "r"(c1) : "memory");
 }
 __device__ __forceinline__ void tma_store_2d(const CUtensorMap* m, uint32_t src, int c0, int c1)
 {
@@ -288,64 +288,6 @@ __device__ __forceinline__ void cluster_sync_all()
     asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
-__device__ __forceinline__ uint32_t cluster_nctarank()
-{
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
-    return r;
-}
-// The two halves of the cluster barrier, for code that has work to do between them.  Every thread of
-// the cluster that has not exited takes part.
-__device__ __forceinline__ void cluster_arrive()
-{
-    asm volatile("barrier.cluster.arrive.release;" ::: "memory");
-}
-__device__ __forceinline__ void cluster_wait()
-{
-    asm volatile("barrier.cluster.wait.acquire;" ::: "memory");
-}
-__device__ __forceinline__ void fence_acq_rel_cluster()
-{
-    asm volatile("fence.acq_rel.cluster;" ::: "memory");
-}
-__device__ __forceinline__ float ld_shared_cluster_f32(uint32_t cluster_addr)
-{
-    float v;
-    asm volatile("ld.shared::cluster.f32 %0, [%1];" : "=f"(v) : "r"(cluster_addr) : "memory");
-    return v;
-}
-// Bounded wait on a barrier of this CTA that other CTAs of the cluster arrive on: acquire at cluster
-// scope, so what they wrote to their shared memory before arriving is visible afterwards.  Lane 0
-// polls, the warp gets one verdict (see mbar_wait_warp).
-__device__ __forceinline__ bool mbar_try_wait_cluster(uint32_t bar, uint32_t parity)
-{
-    uint32_t ok;
-    asm volatile(
-        "{\n\t.reg .pred p;\n\t"
-        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
-        "selp.u32 %0, 1, 0, p;\n\t}"
-        : "=r"(ok) : "r"(bar), "r"(parity) : "memory");
-    return ok != 0;
-}
-__device__ __forceinline__ bool mbar_wait_cluster_warp(uint32_t bar, uint32_t parity, volatile int* abort)
-{
-    int ok = 1;
-    if ((threadIdx.x & 31) == 0) {
-        if (!mbar_try_wait_cluster(bar, parity)) {
-            const long long t0 = clock64();
-            for (uint32_t it = 1;; ++it) {
-                if (mbar_try_wait_cluster(bar, parity)) break;
-                if ((it & 63u) == 0u) {
-                    if (*abort) { ok = 0; break; }
-                    if (clock64() - t0 > (1ll << 31)) { *abort = 1; ok = 0; break; }
-                }
-            }
-        }
-    }
-    ok = __shfl_sync(0xffffffffu, ok, 0);
-    fence_acq_rel_cluster();   // the other lanes did not poll: order their reads after lane 0's acquire
-    return ok != 0;
-}
 // Address of the same shared-memory offset in CTA `rank` of the cluster.
 __device__ __forceinline__ uint32_t mapa_shared(uint32_t addr, uint32_t rank)
 {
@@ -377,12 +319,6 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
     asm volatile(
         "cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];"
         ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1) : "memory");
-}
-__device__ __forceinline__ void tma_load_3d_pair(uint32_t dst, const CUtensorMap* m, uint32_t bar, int c0, int c1, int c2)
-{
-    asm volatile(
-        "cp.async.bulk.tensor.3d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4, %5}], [%2];"
-        ::"r"(dst), "l"(reinterpret_cast<uint64_t>(m)), "r"(bar), "r"(c0), "r"(c1), "r"(c2) : "memory");
 }
 // D (256 rows, 128 in each CTA's TMEM) (+)= A (128 rows in each CTA) * B^T (half of the N rows in each CTA); one thread of the
 // pair's first CTA issues, for both.
