@@ -19,7 +19,8 @@
 //   warp 6   lists the chunks of the next tile: those that either row tile of the pair uses, in order of slot and chunk; a CTA
 //            whose own row tile does not use a chunk multiplies zeros (a copy from behind the end of the u blocks).
 //
-// Early start as in lml_gemm_sm100.cu.  Every wait is bounded; on give-up the CTA sets LML_FLAG_TIMEOUT and frees its TMEM.
+// Early start as in lml_gemm_sm100.cu.  Every wait is bounded; on give-up the CTA sets LML_FLAG_TIMEOUT, gives its copies in
+// flight time to land and frees its TMEM.
 #include "lml_gemm_common.cuh"
 
 namespace lml {

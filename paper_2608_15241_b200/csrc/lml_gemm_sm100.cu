@@ -31,7 +31,7 @@
 // tile and exchanges partial sums through distributed shared memory.
 // B's chunks hold zeros where the adapter's B is Inf or NaN (every row of a tile meets the chunks of all its slots).  The terms
 // left out are added by the epilogue, element by element, to the rows that are bound to such a slot; other tiles pay one word.
-// Every wait is bounded; on give-up the CTA sets LML_FLAG_TIMEOUT, drains and frees its TMEM.
+// Every wait is bounded; on give-up the CTA sets LML_FLAG_TIMEOUT, gives its copies in flight time to land and frees its TMEM.
 #include <cstdio>
 #include <cstdlib>
 #include <mutex>
